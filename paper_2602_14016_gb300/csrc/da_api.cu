@@ -102,14 +102,20 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   A(dalloc(c, &d.Sum, comp));
   A(dalloc(c, &d.Mx, B * 2 * N * ops->Kc));
   A(dalloc(c, &d.Mn, B * 2 * N * ops->Kc));
+  A(dalloc(c, &d.eX, B * 2 * ops->Kc));
+  A(dalloc(c, &d.eN, B * N));
   A(dalloc(c, &d.obs, B * c->nt * P2 * 2));
   A(dalloc(c, (double**)&d.mobs, B * c->nt * P2 * 2));
   A(dalloc(c, &d.res, B * c->nt * P2 * 2));
   A(dalloc(c, &d.J, B));
   A(dalloc(c, (double**)&d.mult, comp));
-  size_t fold_max = 0;  // room for the folded table of any plan variant
-  for (int v = 0; v < da::plan_count(n); ++v) fold_max = std::max(fold_max, (size_t)da::ops_for(n, v)->fold_doubles);
+  size_t fold_max = 0, fx_max = 0;  // room for the twiddle tables of any plan variant
+  for (int v = 0; v < da::plan_count(n); ++v) {
+    fold_max = std::max(fold_max, (size_t)da::ops_for(n, v)->fold_doubles);
+    fx_max = std::max(fx_max, (size_t)da::ops_for(n, v)->fx_entries);
+  }
   A(dalloc(c, (double**)&d.fold, fold_max));
+  A(dalloc(c, (int4**)&d.fxtw, fx_max));
   A(dalloc(c, (double2**)&d.twP, (size_t)64));
   A(dalloc(c, (da::Sym4**)&d.symF, comp / B));
   A(dalloc(c, (da::Sym4**)&d.symA, comp / B));
@@ -132,7 +138,10 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
     c->nckpt = (c->nsteps + c->ckpt - 1) / c->ckpt;
     A(dalloc(c, &c->ckpt_buf, (size_t)c->nckpt * comp));
   }
-  if (c->ckpt >= 0) A(dalloc(c, &d.traj, B * (size_t)d.traj_steps * 8 * N * N));
+  if (c->ckpt >= 0) {
+    A(dalloc(c, &d.traj, B * (size_t)d.traj_steps * 4 * N * N));
+    A(dalloc(c, &d.eT, B * (size_t)d.traj_steps * 4 * N));
+  }
   A(dalloc(c, &c->d_kind, B));
   A(dalloc(c, &c->d_param, B));
   bool any_table = false;
@@ -149,6 +158,8 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   // lattice
   std::vector<double> fold(ops->fold_doubles);
   ops->fold_table(fold.data());
+  std::vector<int4> fxtw(ops->fx_entries);
+  ops->fx_table(fxtw.data());
   std::vector<double2> twP = roots_of_unity(64);
   std::vector<int>& kind = c->h_kind;
   std::vector<double>& param = c->h_param;
@@ -159,6 +170,7 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
     param[b] = kernels[b].param;
   }
   cudaError_t e = cudaMemcpy((void*)d.fold, fold.data(), fold.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy((void*)d.fxtw, fxtw.data(), fxtw.size() * sizeof(int4), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy((void*)d.twP, twP.data(), 64 * sizeof(double2), cudaMemcpyHostToDevice);
   // per-mode symbols of the column passes, column-major [Kc][Kr]
   const int K = ops->K, Kr = ops->Kr, Kc = ops->Kc;

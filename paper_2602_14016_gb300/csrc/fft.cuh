@@ -1,4 +1,5 @@
-// fft.cuh -- FP64 shared-memory FFT engine for the pass kernels.
+// fft.cuh -- FP64 shared-memory FFT engine of the control maps, and the radix
+// plans and gap masks it shares with the integer engine (fx.cuh).
 //
 // A CTA transforms a batch of F complex sequences of length N held in shared
 // memory, with a mixed-radix Stockham auto-sort algorithm: stage s with
@@ -11,13 +12,12 @@
 // written out by even/odd splitting so that multiplications by +-i and +-1
 // cost nothing.
 //
-// GB300's FP64 pipe is the bottleneck of every kernel here (about 1.6 FP64
-// instructions per clock per SM for this mix), so the engine counts FP64
-// instructions.  The pass kernels use fft_folded: the twiddles' cosines are
-// folded into the butterflies' FMAs (see "Folded twiddles" below), from a
-// per-N table in shared memory.  fft_batch, with a plain table of
-// W_N^t = exp(-2 pi i t / N) (conjugated for the inverse sign), serves the
-// allocation-free control map, whose scratch is static.
+// GB300's FP64 pipe is the bottleneck here (about 1.6 FP64 instructions per
+// clock per SM for this mix), so the engine counts FP64 instructions:
+// fft_folded folds the twiddles' cosines into the butterflies' FMAs (see
+// "Folded twiddles" below), from a per-N table in shared memory.  fft_batch,
+// with a plain table of W_N^t = exp(-2 pi i t / N) (conjugated for the inverse
+// sign), serves the allocation-free control map, whose scratch is static.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -595,69 +595,6 @@ template <int N, int V, int S, int F, int KIN = -1, int KOUT = -1>
 __device__ __forceinline__ void fft_folded(double2* buf, const double* T) {
   static_assert(F == 1 || F == 2, "batches of one or two transforms");
   run_stages_folded<N, V, S, F, 1, KIN, KOUT>(buf, T, typename Plan<N, V>::two{});
-}
-
-// Whether an inverse transform, a pointwise map and a forward transform of the
-// same sequences can hand the data over in registers: when the plan's first
-// and last radix agree, the thread that forms outputs k + m N/R of the last
-// inverse stage is the thread that needs inputs i + m N/R (i = k) of the
-// first forward stage.
-template <int N, int V>
-struct Fusable {
-  using P = typename Plan<N, V>::two;
-  static constexpr bool value = FirstRadix<P>::value == LastRadix<P>::value;
-};
-
-// Inverse transform (S = +1, input band-limited to KIN), then op applied to
-// every output point, then forward transform (S = -1, output needed on the
-// band KOUT) of F sequences in buf: the last inverse stage, op and the first
-// forward stage run on registers, between one pair of barriers.  op(f, x, z)
-// gets sequence f, position x and the inverse transform's value there, and
-// returns the forward transform's input there.  Same contract as two
-// fft_folded calls with op applied in between; requires Fusable<N, V>.
-template <int N, int V, int F, int KIN, int KOUT, typename Op>
-__device__ __forceinline__ void fft_folded_turn(double2* buf, const double* T, Op op) {
-  using P = typename Plan<N, V>::two;
-  static_assert(Fusable<N, V>::value, "first and last radix must agree");
-  constexpr int R = LastRadix<P>::value, NB = N / R, L = N / R;
-  constexpr int Th = PlanInfo<N, V>::THREADS, TOT = F * NB, J = (TOT + Th - 1) / Th;
-  // inverse stages but the last
-  run_stages_folded<N, V, +1, F, 1, KIN, -1>(buf, T, typename InitRadices<P>::type{});
-  const double* Tl = T + FoldSize<1, typename InitRadices<P>::type>::value;
-  double2 a[J][R];
-  int base[J], ii[J];
-#pragma unroll
-  for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * Th;
-    base[jb] = 0;
-    ii[jb] = 0;
-    if (TOT % Th == 0 || u < TOT) {
-      const int f = u / NB;
-      const int i = u - f * NB;
-      base[jb] = f * N;
-      ii[jb] = i;
-#pragma unroll
-      for (int m = 0; m < R; ++m) a[jb][m] = buf[base[jb] + i + m * NB];
-      stage_butterfly<R, +1, L, 0, 0>(a[jb], Tl, i);  // last inverse stage: class k = i
-    }
-  }
-  __syncthreads();  // every thread has read buf
-#pragma unroll
-  for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * Th;
-    if (TOT % Th == 0 || u < TOT) {
-      const int f = u / NB;
-#pragma unroll
-      for (int m = 0; m < R; ++m) a[jb][m] = op(f, ii[jb] + m * L, a[jb][m]);
-      dftR<R, -1, 0>(a[jb]);  // first forward stage
-#pragma unroll
-      for (int m = 0; m < R; ++m) buf[base[jb] + ii[jb] * R + m] = a[jb][m];
-    }
-  }
-  __syncthreads();
-  // forward stages after the first (its table slots start at 0: the first
-  // stage has none)
-  run_stages_folded<N, V, -1, F, R, -1, KOUT>(buf, T, typename TailRadices<P>::type{});
 }
 
 // Host side: flops of one band-limited transform of N points under Plan<N,

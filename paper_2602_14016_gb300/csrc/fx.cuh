@@ -1,0 +1,646 @@
+// fx.cuh -- block fixed-point FFT engine of the pass kernels.
+//
+// GB300 issues about 1.7 FP64 instructions per clock per SM but 64 lanes of
+// 32-bit integer additions and of 32 x 32 + 64-bit multiply-adds, so a 64-bit
+// integer addition (two instructions) costs a sixteenth of an FP64 one and a
+// 64 x 64-bit high product (four multiply-adds) a tenth.  The transforms of
+// the pass kernels therefore run on 64-bit integers with one power-of-two
+// exponent per sequence: a value is v 2^e.  Additions are exact; a product
+// with a twiddle rounds once, at the unit of the sequence's integers.
+//
+// Error.  A sequence enters a forward transform normalised so that its
+// largest component has 62 - log2 G bits, G the largest growth of a component
+// over the stages, or over the first stage only where that leaves two bits
+// more: the second stage then starts with a measured shift.  A sequence enters an inverse transform, whose inputs are
+// spectra with few large coefficients, normalised by the sum of its
+// components' magnitudes, which bounds every partial sum (inv_shift).  Every
+// rounding is at most one unit, against results whose root mean square is
+// 2^54 units or more on the fields of the path (FP64's roundings are 2^-53 of
+// the values themselves).
+//
+// Stages are those of fft.cuh (Stockham, mixed radix, in place, R points per
+// butterfly in registers).  The inverse transform runs the plan's radices in
+// reverse, so its last radix is the forward transform's first, and the row
+// passes hand the data over in registers (fx_turn).  A twiddled stage of
+// radix 4 or 8 scales by 1/4, one of radix 2 by 1/2: the twiddles are 62-bit
+// integers, and no shift follows the product.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cmath>
+
+#include "fft.cuh"
+
+namespace da {
+
+typedef long long i64;
+typedef longlong2 q2;  // complex integer
+
+__host__ __device__ __forceinline__ q2 mkq(i64 x, i64 y) {
+  q2 r;
+  r.x = x;
+  r.y = y;
+  return r;
+}
+__device__ __forceinline__ q2 qadd(q2 a, q2 b) { return mkq(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ q2 qsub(q2 a, q2 b) { return mkq(a.x - b.x, a.y - b.y); }
+
+// (S i) a, S = +-1
+template <int S>
+__device__ __forceinline__ q2 qmul_si(q2 a) {
+  return S > 0 ? mkq(-a.y, a.x) : mkq(a.y, -a.x);
+}
+
+// Sum and difference where ZX, ZY mark an operand known to be zero (its
+// register holds nothing).
+template <bool ZX, bool ZY>
+__device__ __forceinline__ q2 qadd_z(q2 x, q2 y) {
+  if constexpr (ZX && ZY) return mkq(0, 0);
+  else if constexpr (ZY) return x;
+  else if constexpr (ZX) return y;
+  else return qadd(x, y);
+}
+template <bool ZX, bool ZY>
+__device__ __forceinline__ q2 qsub_z(q2 x, q2 y) {
+  if constexpr (ZX && ZY) return mkq(0, 0);
+  else if constexpr (ZY) return x;
+  else if constexpr (ZX) return mkq(-y.x, -y.y);
+  else return qsub(x, y);
+}
+
+// d = hi 2^32 + lo with a signed low word (-2^31 <= lo < 2^31), so that both
+// words enter signed multiply-adds.
+__device__ __forceinline__ int lo_word(i64 d) { return (int)d; }
+__device__ __forceinline__ int hi_word(i64 d) { return (int)(d >> 32) + (int)((unsigned)d >> 31); }
+
+__device__ __forceinline__ i64 madw(int a, int b, i64 c) { return (i64)a * b + c; }
+
+constexpr i64 kHalfWord = 0x80000000LL;  // rounds the discarded low word of a middle sum
+
+// a b / 2^64, the product of the low words left out (below one unit).
+// |a|, |b| <= 2^62.
+__device__ __forceinline__ i64 mul_hi(i64 a, i64 b) {
+  const int ah = hi_word(a), al = lo_word(a), bh = hi_word(b), bl = lo_word(b);
+  const i64 mid = madw(ah, bl, madw(al, bh, kHalfWord));
+  return madw(ah, bh, (i64)(int)(mid >> 32));
+}
+
+// (a b +- c d) / 2^64, |.| <= 2^62 each.
+template <int SG>
+__device__ __forceinline__ i64 mul_hi2(int ah, int al, int bh, int bl, int ch, int cl, int dh, int dl) {
+  const int sh = SG > 0 ? dh : -dh, sl = SG > 0 ? dl : -dl;
+  const i64 mid = madw(ch, sl, madw(cl, sh, madw(ah, bl, madw(al, bh, kHalfWord))));
+  return madw(ch, sh, madw(ah, bh, (i64)(int)(mid >> 32)));
+}
+
+// Twiddle: (cos, sin) as 62-bit integers, each split in signed words.
+// a w / 4 for S = -1, a conj(w) / 4 for S = +1 (the tables hold S = -1).
+template <int S>
+__device__ __forceinline__ q2 qtwiddle(q2 a, int4 w) {
+  const int xh = hi_word(a.x), xl = lo_word(a.x), yh = hi_word(a.y), yl = lo_word(a.y);
+  const int sh = S < 0 ? w.z : -w.z, sl = S < 0 ? w.w : -w.w;  // imaginary part for this sign
+  const int nh = S < 0 ? -w.z : w.z, nl = S < 0 ? -w.w : w.w;
+  const i64 mr = madw(yh, nl, madw(yl, nh, madw(xh, w.y, madw(xl, w.x, kHalfWord))));
+  const i64 mi = madw(yh, w.y, madw(yl, w.x, madw(xh, sl, madw(xl, sh, kHalfWord))));
+  return mkq(madw(yh, nh, madw(xh, w.x, (i64)(int)(mr >> 32))), madw(yh, w.x, madw(xh, sh, (i64)(int)(mi >> 32))));
+}
+
+// x c for a constant c in (1/2, 1): x + x (c - 1), with c - 1 in 64 bits.
+template <unsigned long long CM1>
+__device__ __forceinline__ i64 mul_near_one(i64 x) {
+  constexpr int cl = (int)(unsigned)CM1;
+  constexpr int ch = (int)((i64)CM1 >> 32) + (int)((unsigned)CM1 >> 31);
+  const int h = hi_word(x), l = lo_word(x);
+  const i64 mid = madw(h, cl, madw(l, ch, kHalfWord));
+  return madw(h, ch, x + (i64)(int)(mid >> 32));
+}
+
+// 2^64 (cos(pi/4) - 1), 2^64 (cos(pi/8) - 1), 2^64 sin(pi/8), rounded.
+constexpr unsigned long long kFxR2m1 = 0xB504F333F9DE6484ULL;
+constexpr unsigned long long kFxC8m1 = 0xEC835E79946A3145ULL;
+constexpr unsigned long long kFxS8 = 0x61F78A9ABAA58B47ULL;
+
+__device__ __forceinline__ q2 q_r2(q2 a) { return mkq(mul_near_one<kFxR2m1>(a.x), mul_near_one<kFxR2m1>(a.y)); }
+
+// a (cos(pi/8) + S i sin(pi/8))
+template <int S>
+__device__ __forceinline__ q2 q_rot8(q2 a) {
+  constexpr int cl = (int)(unsigned)kFxC8m1, ch = (int)((i64)kFxC8m1 >> 32) + (int)((unsigned)kFxC8m1 >> 31);
+  constexpr int sl0 = (int)(unsigned)kFxS8, sh0 = (int)((i64)kFxS8 >> 32) + (int)((unsigned)kFxS8 >> 31);
+  constexpr int sl = S > 0 ? sl0 : -sl0, sh = S > 0 ? sh0 : -sh0;
+  const int xh = hi_word(a.x), xl = lo_word(a.x), yh = hi_word(a.y), yl = lo_word(a.y);
+  const i64 mr = madw(yh, -sl, madw(yl, -sh, madw(xh, cl, madw(xl, ch, kHalfWord))));
+  const i64 mi = madw(xh, sl, madw(xl, sh, madw(yh, cl, madw(yl, ch, kHalfWord))));
+  return mkq(madw(yh, -sh, madw(xh, ch, a.x + (i64)(int)(mr >> 32))),
+             madw(xh, sh, madw(yh, ch, a.y + (i64)(int)(mi >> 32))));
+}
+
+template <int S, int Z = 0>
+__device__ __forceinline__ void qdft2(q2* a) {
+  constexpr bool z0 = Z & 1, z1 = (Z >> 1) & 1;
+  const q2 t = a[0];
+  a[0] = qadd_z<z0, z1>(t, a[1]);
+  a[1] = qsub_z<z0, z1>(t, a[1]);
+}
+
+// X_k = sum_m a_m exp(S 2 pi i m k / R), in place; bit m of Z: input m is
+// zero (not loaded).
+template <int S, int Z = 0>
+__device__ __forceinline__ void qdft4(q2* a) {
+  constexpr bool z0 = Z & 1, z1 = (Z >> 1) & 1, z2 = (Z >> 2) & 1, z3 = (Z >> 3) & 1;
+  constexpr bool ze = z0 && z2, zo = z1 && z3;
+  const q2 t0 = qadd_z<z0, z2>(a[0], a[2]), t1 = qsub_z<z0, z2>(a[0], a[2]);
+  const q2 t2 = qadd_z<z1, z3>(a[1], a[3]), t3 = qsub_z<z1, z3>(a[1], a[3]);
+  a[0] = qadd_z<ze, zo>(t0, t2);
+  a[2] = qsub_z<ze, zo>(t0, t2);
+  // t1 +- S i t3
+  if constexpr (S > 0) {
+    a[1] = mkq(t1.x - t3.y, t1.y + t3.x);
+    a[3] = mkq(t1.x + t3.y, t1.y - t3.x);
+  } else {
+    a[1] = mkq(t1.x + t3.y, t1.y - t3.x);
+    a[3] = mkq(t1.x - t3.y, t1.y + t3.x);
+  }
+}
+
+template <int S, int Z = 0>
+__device__ __forceinline__ void qdft8(q2* a) {
+  q2 e[4] = {a[0], a[2], a[4], a[6]};
+  q2 o[4] = {a[1], a[3], a[5], a[7]};
+  qdft4<S, even_bits(Z, 8)>(e);
+  qdft4<S, odd_bits(Z, 8)>(o);
+  a[0] = qadd(e[0], o[0]);
+  a[4] = qsub(e[0], o[0]);
+  const q2 o2 = qmul_si<S>(o[2]);
+  a[2] = qadd(e[2], o2);
+  a[6] = qsub(e[2], o2);
+  const q2 w1 = q_r2(mkq(S > 0 ? o[1].x - o[1].y : o[1].x + o[1].y, S > 0 ? o[1].y + o[1].x : o[1].y - o[1].x));
+  a[1] = qadd(e[1], w1);
+  a[5] = qsub(e[1], w1);
+  const q2 w3 = q_r2(mkq(S > 0 ? o[3].x + o[3].y : o[3].x - o[3].y, S > 0 ? o[3].y - o[3].x : o[3].y + o[3].x));
+  a[3] = qsub(e[3], w3);
+  a[7] = qadd(e[3], w3);
+}
+
+template <int S, int Z = 0>
+__device__ __forceinline__ void qdft16(q2* a) {
+  q2 e[8], o[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    e[k] = a[2 * k];
+    o[k] = a[2 * k + 1];
+  }
+  qdft8<S, even_bits(Z, 16)>(e);
+  qdft8<S, odd_bits(Z, 16)>(o);
+  // o_k exp(S i k pi / 8)
+  o[1] = q_rot8<S>(o[1]);
+  o[2] = q_r2(mkq(S > 0 ? o[2].x - o[2].y : o[2].x + o[2].y, S > 0 ? o[2].y + o[2].x : o[2].y - o[2].x));
+  o[3] = qmul_si<S>(q_rot8<-S>(o[3]));  // 3 pi/8 = pi/2 - pi/8
+  o[4] = qmul_si<S>(o[4]);
+  o[5] = qmul_si<S>(q_rot8<S>(o[5]));  // 5 pi/8 = pi/2 + pi/8
+  o[6] = qmul_si<S>(q_r2(mkq(S > 0 ? o[6].x - o[6].y : o[6].x + o[6].y, S > 0 ? o[6].y + o[6].x : o[6].y - o[6].x)));
+  const q2 r7 = q_rot8<-S>(o[7]);  // 7 pi/8 = pi - pi/8
+  o[7] = mkq(-r7.x, -r7.y);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    a[k] = qadd(e[k], o[k]);
+    a[k + 8] = qsub(e[k], o[k]);
+  }
+}
+
+template <int R, int S, int Z = 0>
+__device__ __forceinline__ void qdftR(q2* a) {
+  if constexpr (R == 2) qdft2<S, Z>(a);
+  if constexpr (R == 4) qdft4<S, Z>(a);
+  if constexpr (R == 8) qdft8<S, Z>(a);
+  if constexpr (R == 16) qdft16<S, Z>(a);
+}
+
+// ---------------------------------------------------------------------------
+// Plans, scaling and twiddle tables
+// ---------------------------------------------------------------------------
+
+template <typename P, typename Q> struct ReverseOnto;
+template <typename Q> struct ReverseOnto<Radices<>, Q> { using type = Q; };
+template <int R, int... Rs, int... Qs> struct ReverseOnto<Radices<R, Rs...>, Radices<Qs...>> {
+  using type = typename ReverseOnto<Radices<Rs...>, Radices<R, Qs...>>::type;
+};
+
+// log2 of the scaling of one twiddled stage (1/4, radix 2: 1/2)
+constexpr int stage_shift(int r) { return r == 2 ? 1 : 2; }
+
+template <int L, typename P> struct FxSum;
+template <int L> struct FxSum<L, Radices<>> { static constexpr int shift = 0, entries = 0; };
+template <int L, int R, int... Rs> struct FxSum<L, Radices<R, Rs...>> {
+  using Next = FxSum<L * R, Radices<Rs...>>;
+  static constexpr int shift = (L > 1 ? stage_shift(R) : 0) + Next::shift;
+  static constexpr int entries = (L > 1 ? (R - 1) * L : 0) + Next::entries;
+};
+
+constexpr int log2c(int n) { return n <= 1 ? 0 : 1 + log2c(n / 2); }
+
+template <int N, int V = 0>
+struct FxPlan {
+  using fwd = typename Plan<N, V>::two;
+  using inv = typename ReverseOnto<fwd, Radices<>>::type;
+  // both directions scale by 2^-SHIFT in all
+  static constexpr int SHIFT = FxSum<1, fwd>::shift;
+  static constexpr int SHIFT_INV = FxSum<1, inv>::shift;
+  static constexpr int ENTRIES = FxSum<1, fwd>::entries, ENTRIES_INV = FxSum<1, inv>::entries;
+  static constexpr int TABLE = ENTRIES + ENTRIES_INV;  // forward table, then inverse
+  // Bits of the largest input component of a forward transform: a component
+  // of a partial sum is at most sqrt2 times the largest input component times
+  // the product of the radices so far, scaled; it stays below 2^63.
+  template <int L, typename P> struct Growth;
+  template <int L> struct Growth<L, Radices<>> { static constexpr int most(int) { return 0; } };
+  template <int L, int R, int... Rs> struct Growth<L, Radices<R, Rs...>> {
+    static constexpr int most(int g) {
+      const int here = g + log2c(R) - (L > 1 ? stage_shift(R) : 0);
+      const int next = Growth<L * R, Radices<Rs...>>::most(here);
+      return here > next ? here : next;
+    }
+  };
+  static constexpr int GROWTH = Growth<1, fwd>::most(0);
+  static constexpr int R1 = FirstRadix<fwd>::value;
+  static constexpr int GROWTH1 = log2c(R1);                                          // first stage
+  static constexpr int GROWTH2 = Growth<R1, typename TailRadices<fwd>::type>::most(0);  // the others
+  static constexpr int BITS_FWD = 62 - GROWTH;
+};
+
+template <int L>
+inline void fx_fill(int4*, Radices<>) {}
+
+// exp(-2 pi i m k / (L R)) for m = 1..R-1, k < L, entry (m - 1) L + k of each
+// twiddled stage: round(2^62 cos), round(2^62 sin), each hi, lo signed words.
+template <int L, int R, int... Rs>
+inline void fx_fill(int4* out, Radices<R, Rs...>) {
+  if (L > 1) {
+    const long double pi = 3.141592653589793238462643383279502884L;
+    const long double s = 4611686018427387904.0L;
+    for (int m = 1; m < R; ++m)
+      for (int k = 0; k < L; ++k) {
+        const long double th = -2.0L * pi * (long double)(m * k) / (long double)(L * R);
+        const i64 c = llroundl(s * cosl(th)), n = llroundl(s * sinl(th));
+        auto lo = [](i64 v) { return (int)(unsigned)(v & 0xffffffffLL); };
+        auto hi = [&](i64 v) { return (int)((v - (i64)lo(v)) >> 32); };
+        out[(m - 1) * L + k] = make_int4(hi(c), lo(c), hi(n), lo(n));
+      }
+    out += (R - 1) * L;
+  }
+  fx_fill<L * R>(out, Radices<Rs...>{});
+}
+
+template <int N, int V>
+inline void fx_table(int4* out) {
+  using P = FxPlan<N, V>;
+  fx_fill<1>(out, typename P::fwd{});
+  fx_fill<1>(out + P::ENTRIES, typename P::inv{});
+}
+
+// ---------------------------------------------------------------------------
+// Exponents and conversions
+// ---------------------------------------------------------------------------
+
+// Exponent of an all-zero sequence, and of one that holds an infinity or a
+// NaN; sums of two exponents are brought back to these by clamp_exp.
+constexpr int kZeroExp = -100000, kBadExp = 100000;
+
+__device__ __forceinline__ int clamp_exp(int e) { return e < kZeroExp / 2 ? kZeroExp : e > kBadExp / 2 ? kBadExp : e; }
+
+// Magnitude bits of an integer's high word: |v| < 2^(32 + bits).
+__device__ __forceinline__ int mag32(i64 v) {
+  const int h = (int)(v >> 32);
+  return h ^ (h >> 31);
+}
+__device__ __forceinline__ int bits32(int m) { return 32 - __clz(m); }
+
+// v 2^s: left for s >= 0 (the caller knows that it fits), right with
+// rounding for s < 0.
+struct Shift {
+  int l, r;
+  i64 half;
+  __device__ __forceinline__ explicit Shift(int s) {
+    l = max(s, 0);
+    r = min(max(-s, 0), 62);
+    l = min(l, 62);
+    half = (1LL << r) >> 1;
+  }
+  __device__ __forceinline__ i64 operator()(i64 v) const { return ((v << l) + half) >> r; }
+  __device__ __forceinline__ q2 operator()(q2 v) const { return mkq((*this)(v.x), (*this)(v.y)); }
+};
+
+// Largest key over the CTA, for each of the two sequences (a, b).  scratch:
+// 2 ints per warp, not in use by another call since the last barrier but
+// one.  Ends with a barrier.
+template <int T>
+__device__ __forceinline__ int2 block_max2(int a, int b, int* scratch) {
+  a = __reduce_max_sync(0xffffffffu, a);
+  b = __reduce_max_sync(0xffffffffu, b);
+  if constexpr (T <= 32) {
+    __syncthreads();
+    return make_int2(a, b);
+  } else {
+    if ((threadIdx.x & 31) == 0) {
+      scratch[(threadIdx.x >> 5) * 2] = a;
+      scratch[(threadIdx.x >> 5) * 2 + 1] = b;
+    }
+    __syncthreads();
+    int2 r = make_int2(scratch[0], scratch[1]);
+#pragma unroll
+    for (int w = 1; w < T / 32; ++w) {
+      r.x = max(r.x, scratch[2 * w]);
+      r.y = max(r.y, scratch[2 * w + 1]);
+    }
+    return r;
+  }
+}
+
+// Sums over the CTA of two counts (one per sequence) are left in scratch, one
+// pair per warp, and read back by sum2 after the caller's next barrier.
+// scratch: as for block_max2.
+__device__ __forceinline__ void block_sum2_put(unsigned a, unsigned b, int* scratch) {
+  a = __reduce_add_sync(0xffffffffu, a);
+  b = __reduce_add_sync(0xffffffffu, b);
+  if ((threadIdx.x & 31) == 0) {
+    scratch[(threadIdx.x >> 5) * 2] = (int)a;
+    scratch[(threadIdx.x >> 5) * 2 + 1] = (int)b;
+  }
+}
+template <int T>
+__device__ __forceinline__ int2 block_sum2_get(const int* scratch) {
+  int2 r = make_int2(scratch[0], scratch[1]);
+#pragma unroll
+  for (int w = 1; w < (T + 31) / 32; ++w) {
+    r.x += scratch[2 * w];
+    r.y += scratch[2 * w + 1];
+  }
+  return r;
+}
+
+// Inputs of an inverse transform are first brought to kInvBits bits, then,
+// as the first stage reads them, shifted right (rounded) until the sum of
+// their magnitudes has 62 bits.  The sum is counted in units of
+// 2^(32 + kSumDrop): mag32 >> kSumDrop, at most 4 x 683 terms of 2^18 each,
+// one unit more a term for the part dropped.
+//
+// The second stage scales by 2^-G before it adds, so the sum may have 62 + G
+// bits where the first stage's own sums, at most R sqrt2 times the largest
+// component (61 bits), stay below 2^62.5: from a shift of log2 R - 1 on.
+constexpr int kInvBits = 61, kSumDrop = 12;
+template <int N, int V>
+__device__ __forceinline__ int inv_shift(int sum) {
+  using I = typename FxPlan<N, V>::inv;
+  constexpr int first = log2c(FirstRadix<I>::value) - 1;
+  constexpr int G = stage_shift(FirstRadix<typename TailRadices<I>::type>::value);
+  const int r = bits32(sum) + 32 + kSumDrop - 62;
+  return max(0, min(r, max(r - G, first)));
+}
+__device__ __forceinline__ unsigned mag_units(q2 v) { return (unsigned)(((mag32(v.x) + mag32(v.y)) >> kSumDrop) + 1); }
+
+// v 2^e as a double (one rounding).
+__device__ __forceinline__ double pow2_double(int e) {  // 2^e, -1022 <= e <= 1023
+  return __hiloint2double((e + 1023) << 20, 0);
+}
+__device__ __forceinline__ double fx_to_double(i64 v, int e) {
+  if (e >= kBadExp) return __hiloint2double(0x7ff80000, 0);
+  const double d = (double)v;
+  if (e >= -960 && e <= 960) return d * pow2_double(e);
+  if (v == 0) return 0.0;
+  // outside that range the scaling goes in steps, each within a double's
+  int left = max(min(e, 2200), -2200);
+  double r = d;
+  while (left != 0) {
+    const int s = max(min(left, 900), -900);
+    r *= pow2_double(s);
+    left -= s;
+  }
+  return r;
+}
+
+// Biased exponent field of a double (0: zero or subnormal, 2047: not finite).
+__device__ __forceinline__ int exp_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
+
+// Exponent e for a sequence whose largest exponent field is f, so that every
+// component has at most BITS bits: |d| < 2^(f - 1022) = 2^(BITS + e).
+template <int BITS>
+__device__ __forceinline__ int exp_for(int f) {
+  return f == 0 ? kZeroExp : f == 2047 ? kBadExp : f - 1022 - BITS;
+}
+
+// d / 2^e as an integer, rounded towards zero; e from exp_for<BITS> (BITS <=
+// 62).  Subnormals count as zero.
+__device__ __forceinline__ i64 double_to_fx(double d, int e) {
+  const int hi = __double2hiint(d), lo = __double2loint(d);
+  const int f = (hi >> 20) & 0x7ff;
+  // 53-bit significand m, value m 2^(f - 1075): m 2^9 >> r
+  const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
+  const int r = min(9 - (f - 1075 - e), 63);
+  const i64 q = f == 0 ? 0 : (m << 9) >> r;
+  return hi < 0 ? -q : q;
+}
+
+// ---------------------------------------------------------------------------
+// Stages
+// ---------------------------------------------------------------------------
+
+// a / 2^s, rounded
+__device__ __forceinline__ i64 shr_round(i64 v, int s) { return (v + (1LL << (s - 1))) >> s; }
+
+// The butterfly of one stage: twiddles (L > 1), then the R-point DFT.
+template <int R, int S, int L, int Z>
+__device__ __forceinline__ void fx_butterfly(q2* a, const int4* __restrict__ T, int k) {
+  if constexpr (L > 1) {
+    a[0] = mkq(shr_round(a[0].x, stage_shift(R)), shr_round(a[0].y, stage_shift(R)));
+#pragma unroll
+    for (int m = 1; m < R; ++m) {
+      a[m] = qtwiddle<S>(a[m], __ldg(T + (m - 1) * L + k));
+      if constexpr (R == 2) a[m] = mkq(a[m].x * 2, a[m].y * 2);
+    }
+  }
+  qdftR<R, S, Z>(a);
+}
+
+// Runs the first stage's butterfly for the warp's mask of zero inputs.
+template <int R, int S, typename G>
+__device__ __forceinline__ void fx_masked_first(q2* a, int w) {
+  constexpr int C = G::C, A = G::A, B = G::B;
+  if constexpr (A == 0) {
+    qdftR<R, S, C>(a);
+  } else if constexpr (B == 0) {
+    if (w & A) qdftR<R, S, C | A>(a);
+    else qdftR<R, S, C>(a);
+  } else {
+    if ((w & (A | B)) == (A | B)) qdftR<R, S, C | A | B>(a);
+    else if (w & A) qdftR<R, S, C | A>(a);
+    else if (w & B) qdftR<R, S, C | B>(a);
+    else qdftR<R, S, C>(a);
+  }
+}
+
+// One in-place Stockham stage on F sequences.  KIN >= 0: zero outside the
+// band (first stage of an inverse transform, which also applies the right
+// shifts pre of the sequences); KOUT >= 0: only the band is needed (last
+// stage).  SHR: a later stage that starts with the right shifts pre.
+template <int N, int V, int R, int S, int F, int L, int KIN, int KOUT, bool SHR = false>
+__device__ __forceinline__ void fx_stage(q2* buf, const int4* __restrict__ T, int2 pre) {
+  constexpr int NB = N / R, Th = PlanInfo<N, V>::THREADS, TOT = F * NB, J = (TOT + Th - 1) / Th;
+  constexpr bool FIRST = L == 1, LAST = L * R == N;
+  using GI = GapMask<N, R, FIRST ? KIN : -1>;
+  using GO = GapMask<N, R, LAST ? KOUT : -1>;
+  q2 a[J][R];
+  int base[J], dst[J], om[J];
+#pragma unroll
+  for (int jb = 0; jb < J; ++jb) {
+    const int u = threadIdx.x + jb * Th;
+    base[jb] = dst[jb] = om[jb] = 0;
+    if (TOT % Th == 0 || u < TOT) {
+      const int f = u / NB;
+      const int i = u - f * NB;
+      const int k = i & (L - 1);
+      base[jb] = f * N;
+      const int zm = GI::warp(i);
+#pragma unroll
+      for (int m = 0; m < R; ++m)
+        if (!((zm >> m) & 1)) a[jb][m] = buf[base[jb] + i + m * NB];
+      if constexpr (FIRST) {
+        if constexpr (KIN >= 0) {
+          const int r = f ? pre.y : pre.x;
+          const i64 half = (1LL << r) >> 1;
+#pragma unroll
+          for (int m = 0; m < R; ++m)
+            if (!((zm >> m) & 1)) a[jb][m] = mkq((a[jb][m].x + half) >> r, (a[jb][m].y + half) >> r);
+        }
+        fx_masked_first<R, S, GI>(a[jb], zm);
+      } else {
+        om[jb] = GO::warp(i);
+        if constexpr (SHR) {
+          const int r = f ? pre.y : pre.x;
+          if (r > 0) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) a[jb][m] = mkq(shr_round(a[jb][m].x, r), shr_round(a[jb][m].y, r));
+          }
+        }
+        fx_butterfly<R, S, L, 0>(a[jb], T, k);
+      }
+      dst[jb] = (i - k) * R + k;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int jb = 0; jb < J; ++jb) {
+    const int u = threadIdx.x + jb * Th;
+    if (TOT % Th == 0 || u < TOT) {
+#pragma unroll
+      for (int m = 0; m < R; ++m)
+        if (!((om[jb] >> m) & 1)) buf[base[jb] + dst[jb] + m * L] = a[jb][m];
+    }
+  }
+  __syncthreads();
+}
+
+template <int N, int V, int S, int F, int L, int KIN, int KOUT>
+__device__ __forceinline__ void fx_run(q2*, const int4*, int2, Radices<>) {}
+template <int N, int V, int S, int F, int L, int KIN, int KOUT, int R, int... Rs>
+__device__ __forceinline__ void fx_run(q2* buf, const int4* T, int2 pre, Radices<R, Rs...>) {
+  fx_stage<N, V, R, S, F, L, KIN, KOUT>(buf, T, pre);
+  fx_run<N, V, S, F, L * R, KIN, KOUT>(buf, T + (L > 1 ? (R - 1) * L : 0), pre, Radices<Rs...>{});
+}
+
+// The stages after the first of a forward transform, whose first stage's
+// results have at most 32 + bits32(m) bits (m.x, m.y for the two sequences).
+// SPARE: bits of the results to leave free.  Returns the shifts taken.
+template <int N, int V, int KB, int SPARE>
+__device__ __forceinline__ int2 fx_forward_rest(q2* buf, const int4* tw, int2 m) {
+  using P = FxPlan<N, V>;
+  constexpr int most = 62 - SPARE - P::GROWTH2 - 32;
+  const int2 r = make_int2(max(0, bits32(m.x) - most), max(0, bits32(m.y) - most));
+  using Tail = typename TailRadices<typename P::fwd>::type;
+  constexpr int R2 = FirstRadix<Tail>::value;
+  fx_stage<N, V, R2, -1, 2, P::R1, -1, (P::R1 * R2 == N) ? KB : -1, true>(buf, tw, r);
+  fx_run<N, V, -1, 2, P::R1 * R2, -1, KB>(buf, tw + (R2 - 1) * P::R1, r, typename TailRadices<Tail>::type{});
+  return r;
+}
+
+// Transforms, in place, of two sequences of N points back to back in buf:
+// inverse (S = +1) of sequences zero outside the band KB, and forward, of
+// which only the band KB is formed.  The gap positions must hold zeros on
+// input of the inverse (warps that straddle the gap read it) and are
+// undefined after the forward.  Inputs have at most kInvBits bits and are
+// shifted right by pre first (inverse), or have at most BITS_FWD bits
+// (forward); the result is the transform times 2^-SHIFT.  tw: FxPlan's
+// tables.
+template <int N, int V, int KB>
+__device__ __forceinline__ void fx_inverse(q2* buf, const int4* tw, int2 pre) {
+  using P = FxPlan<N, V>;
+  fx_run<N, V, +1, 2, 1, KB, -1>(buf, tw + P::ENTRIES, pre, typename P::inv{});
+}
+template <int N, int V, int KB>
+__device__ __forceinline__ void fx_forward(q2* buf, const int4* tw) {
+  fx_run<N, V, -1, 2, 1, -1, KB>(buf, tw, make_int2(0, 0), typename FxPlan<N, V>::fwd{});
+}
+
+// Inverse transform, a pointwise map, and forward transform of two sequences:
+// the last inverse stage, the map and the first forward stage run on
+// registers.  prep(m0, m1) gets the largest high-word magnitude (mag32) of
+// each sequence's inverse transform, on every thread after a barrier;
+// op(f, x, z) gets sequence f, position x and the value there and returns
+// the forward transform's input.  MEASURE: the inputs leave room for the first
+// forward stage only (fx_forward_rest).  The results leave one bit free;
+// returns the shifts taken.
+template <int N, int V, int KB, bool MEASURE, typename Prep, typename Op>
+__device__ __forceinline__ int2 fx_turn(q2* buf, const int4* tw, int2 pre, int* scratch, Prep prep, Op op) {
+  using P = FxPlan<N, V>;
+  constexpr int R = FirstRadix<typename P::fwd>::value, NB = N / R, L = N / R;
+  constexpr int Th = PlanInfo<N, V>::THREADS, TOT = 2 * NB, J = (TOT + Th - 1) / Th;
+  using Init = typename InitRadices<typename P::inv>::type;
+  fx_run<N, V, +1, 2, 1, KB, -1>(buf, tw + P::ENTRIES, pre, Init{});
+  const int4* Tl = tw + P::ENTRIES + FxSum<1, Init>::entries;
+  q2 a[J][R];
+  int m0 = 0, m1 = 0;
+#pragma unroll
+  for (int jb = 0; jb < J; ++jb) {
+    const int u = threadIdx.x + jb * Th;
+    if (TOT % Th == 0 || u < TOT) {
+      const int f = u / NB;
+      const int i = u - f * NB;
+#pragma unroll
+      for (int m = 0; m < R; ++m) a[jb][m] = buf[f * N + i + m * NB];
+      fx_butterfly<R, +1, L, 0>(a[jb], Tl, i);
+      int mm = 0;
+#pragma unroll
+      for (int m = 0; m < R; ++m) mm = max(mm, max(mag32(a[jb][m].x), mag32(a[jb][m].y)));
+      if (f == 0) m0 = max(m0, mm);
+      else m1 = max(m1, mm);
+    }
+  }
+  const int2 mx = block_max2<Th>(m0, m1, scratch);  // every thread has read buf
+  prep(mx.x, mx.y);
+  m0 = m1 = 0;
+#pragma unroll
+  for (int jb = 0; jb < J; ++jb) {
+    const int u = threadIdx.x + jb * Th;
+    if (TOT % Th == 0 || u < TOT) {
+      const int f = u / NB;
+      const int i = u - f * NB;
+#pragma unroll
+      for (int m = 0; m < R; ++m) a[jb][m] = op(f, i + m * L, a[jb][m]);
+      qdftR<R, -1, 0>(a[jb]);
+      int mm = 0;
+#pragma unroll
+      for (int m = 0; m < R; ++m) {
+        if constexpr (MEASURE) mm = max(mm, max(mag32(a[jb][m].x), mag32(a[jb][m].y)));
+        buf[f * N + i * R + m] = a[jb][m];
+      }
+      if (f == 0) m0 = max(m0, mm);
+      else m1 = max(m1, mm);
+    }
+  }
+  if constexpr (MEASURE) {
+    return fx_forward_rest<N, V, KB, 1>(buf, tw, block_max2<Th>(m0, m1, scratch + 16));
+  }
+  __syncthreads();
+  fx_run<N, V, -1, 2, R, -1, KB>(buf, tw, pre, typename TailRadices<typename P::fwd>::type{});
+  return make_int2(0, 0);
+}
+
+}  // namespace da

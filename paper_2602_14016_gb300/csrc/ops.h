@@ -15,6 +15,8 @@ struct Ops {
   double flops_inverse;             // nominal flops of one band-limited inverse transform
   double flops_forward;             // ... and forward transform (band_transform_flops)
   void (*fold_table)(double* out);  // fills it on the host
+  int fx_entries;                   // entries of the integer twiddle tables
+  void (*fx_table)(int4* out);      // fills them on the host
   cudaError_t (*setup)();
   void (*r2c_rows)(const Dev&, const double* in, cudaStream_t);
   void (*c2r_rows)(const Dev&, double* out, cudaStream_t);

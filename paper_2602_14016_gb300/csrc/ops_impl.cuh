@@ -18,16 +18,17 @@ Ops make_ops() {
   o.flops_inverse = band_transform_flops<N, V, G::K>(true);
   o.flops_forward = band_transform_flops<N, V, G::K>(false);
   o.fold_table = [](double* out) { fold_table<N, V>(out); };
+  o.fx_entries = FxPlan<N, V>::TABLE;
+  o.fx_table = [](int4* out) { fx_table<N, V>(out); };
   o.setup = []() -> cudaError_t {
-    const int s = (int)G::SMEM;
     cudaError_t e = cudaSuccess;
-    auto set = [&](const void* f) {
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s);
+    auto set = [&](const void* f, size_t s = G::SMEM_FX) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s);
     };
-    set((const void*)k_r2c_rows<N, V>);
-    set((const void*)k_c2r_rows<N, V>);
-    set((const void*)k_spec_to_mixed<N, V>);
-    set((const void*)k_ctrl_cols<N, V>);
+    set((const void*)k_r2c_rows<N, V>, G::SMEM);
+    set((const void*)k_c2r_rows<N, V>, G::SMEM);
+    set((const void*)k_spec_to_mixed<N, V>, G::SMEM);
+    set((const void*)k_ctrl_cols<N, V>, G::SMEM);
     set((const void*)k_fwd_rows<N, V>);
     set((const void*)k_fwd_cols<N, V>);
     set((const void*)k_state_cols<N, V>);
@@ -55,22 +56,22 @@ Ops make_ops() {
     k_ctrl_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d, flags);
   };
   o.fwd_rows = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_fwd_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM, st>>>(d, n, stage, flags);
+    k_fwd_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
   };
   o.fwd_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_fwd_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d, n, stage, flags);
+    k_fwd_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
   };
   o.state_cols = [](const Dev& d, cudaStream_t st) {
-    k_state_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d);
+    k_state_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d);
   };
   o.adj_init = [](const Dev& d, int mode, cudaStream_t st) {
-    k_adj_init<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d, mode);
+    k_adj_init<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, mode);
   };
   o.adj_rows = [](const Dev& d, int n, int stage, cudaStream_t st) {
-    k_adj_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM, st>>>(d, n, stage);
+    k_adj_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
   };
   o.adj_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_adj_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d, n, stage, flags);
+    k_adj_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
   };
   o.make_mult = [](const Dev& d, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                    cudaStream_t st) {

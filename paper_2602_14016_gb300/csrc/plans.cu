@@ -27,6 +27,9 @@ static da_status set_plan(da_ctx* c, int v) {
   std::vector<double> fold(o->fold_doubles);
   o->fold_table(fold.data());
   DA_TRY_CUDA(c, cudaMemcpy((void*)c->dev.fold, fold.data(), fold.size() * sizeof(double), cudaMemcpyHostToDevice));
+  std::vector<int4> fxtw(o->fx_entries);
+  o->fx_table(fxtw.data());
+  DA_TRY_CUDA(c, cudaMemcpy((void*)c->dev.fxtw, fxtw.data(), fxtw.size() * sizeof(int4), cudaMemcpyHostToDevice));
   DA_TRY_CUDA(c, o->setup());
   c->ops = o;
   drop_graphs(c);
@@ -68,6 +71,8 @@ static da_status clear_state(da_ctx* c, cudaStream_t st) {
     DA_TRY_CUDA(c, cudaMemsetAsync(p, 0, comp, st));
   DA_TRY_CUDA(c, cudaMemsetAsync(d.Mx, 0, mixed, st));
   DA_TRY_CUDA(c, cudaMemsetAsync(d.Mn, 0, mixed, st));
+  DA_TRY_CUDA(c, cudaMemsetAsync(d.eX, 0, (size_t)c->B * 2 * c->ops->Kc * sizeof(int), st));
+  DA_TRY_CUDA(c, cudaMemsetAsync(d.eN, 0, (size_t)c->B * c->n * sizeof(int), st));
   return DA_OK;
 }
 
