@@ -274,7 +274,11 @@ class CoBatchServer:
     of its grid into free slots (their windows, kernels, observations and
     first guesses), runs one step (da_lbfgs_iterate: one evaluation shared by
     every member, whatever point of its iteration it is at), and retires the
-    members that finished.
+    members that finished.  A retired member takes no part in later steps; it
+    keeps its slot until another job needs one, so that retiring costs no
+    blocking call between steps (idling a slot waits for the stream and
+    uploads its tables).  `peak_members` of a run's summary is the most member
+    slots that were held at once, retired members included.
     Plan variant `plan` on every pool, so a job's result equals its result in
     a batch-1 context on that variant; plan=None lets the autotuner pick each
     pool's variant for its slot count (results then equal the batch-1 ones to
@@ -304,7 +308,7 @@ class CoBatchServer:
                 for b in range(p["slots"]):
                     ctx.set_member(b, 0)
                 self.pools[n] = {"ctx": ctx, "slots": p["slots"], "stream": torch.cuda.Stream(device),
-                                 "jobs": [None] * p["slots"], "steps": 0}
+                                 "jobs": [None] * p["slots"], "held": set(), "steps": 0}
         self.peak_members = 0
 
     @staticmethod
@@ -315,6 +319,7 @@ class CoBatchServer:
         torch, api = self.torch, self.api
         ctx, st = pool["ctx"], pool["stream"]
         slots = pool["jobs"]
+        held = pool["held"]  # slots whose last member finished and was not replaced
         try:
             with torch.cuda.device(self.device), torch.cuda.stream(st):
                 while True:
@@ -324,7 +329,9 @@ class CoBatchServer:
                         for j in arrived:
                             if None not in slots:
                                 break
-                            b = slots.index(None)
+                            free = [b for b, x in enumerate(slots) if x is None]
+                            b = min(free, key=lambda b: b in held)
+                            held.discard(b)
                             queue.remove(j)
                             slots[b] = j
                             j.t_admit = now
@@ -333,7 +340,7 @@ class CoBatchServer:
                                            torch.from_numpy(j.m[0]), stream=st)
                             ctx.lbfgs_start(b, torch.from_numpy(j.s0[0]).to(ctx.device), j.iters, stream=st)
                         busy = sum(x is not None for x in slots)
-                        self.peak_members = max(self.peak_members, busy)
+                        self.peak_members = max(self.peak_members, busy + len(held))
                         remaining = len(queue)
                     if busy == 0:
                         if remaining == 0:
@@ -354,8 +361,8 @@ class CoBatchServer:
                         j.s = s.cpu().numpy()[None]
                         j.t_done = time.perf_counter() - t0
                         ctx.lbfgs_release(b)
-                        ctx.set_member(b, 0, stream=st)
                         slots[b] = None
+                        held.add(b)
         except Exception as e:  # recorded; the run reports it
             errors.append((n, repr(e)))
 
