@@ -73,7 +73,14 @@ __device__ __forceinline__ q2 qsub_z(q2 x, q2 y) {
 __device__ __forceinline__ int lo_word(i64 d) { return (int)d; }
 __device__ __forceinline__ int hi_word(i64 d) { return (int)(d >> 32) + (int)((unsigned)d >> 31); }
 
-__device__ __forceinline__ i64 madw(int a, int b, i64 c) { return (i64)a * b + c; }
+// a b + c as the one instruction it is: written in C++, the compiler reorders
+// the sums of a product's parts and needs twice the instructions (a twiddle:
+// 50 against 28).
+__device__ __forceinline__ i64 madw(int a, int b, i64 c) {
+  i64 r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
 
 constexpr i64 kHalfWord = 0x80000000LL;  // rounds the discarded low word of a middle sum
 
@@ -239,9 +246,11 @@ template <int L, int R, int... Rs> struct FxSum<L, Radices<R, Rs...>> {
 
 constexpr int log2c(int n) { return n <= 1 ? 0 : 1 + log2c(n / 2); }
 
-template <int N, int V = 0>
-struct FxPlan {
-  using fwd = typename Plan<N, V>::two;
+// A plan of N points on TPS threads a sequence; fwd: its radices.
+template <int N_, int TPS_, typename Fwd>
+struct FxPlanOf {
+  static constexpr int N = N_, TPS = TPS_;
+  using fwd = Fwd;
   using inv = typename ReverseOnto<fwd, Radices<>>::type;
   // both directions scale by 2^-SHIFT in all
   static constexpr int SHIFT = FxSum<1, fwd>::shift;
@@ -265,7 +274,13 @@ struct FxPlan {
   static constexpr int GROWTH1 = log2c(R1);                                          // first stage
   static constexpr int GROWTH2 = Growth<R1, typename TailRadices<fwd>::type>::most(0);  // the others
   static constexpr int BITS_FWD = 62 - GROWTH;
+  // q2 of one buffer of a sequence: a stage reads one and writes the other
+  static constexpr int SEQ = N + N / 8;
+  static constexpr int WARPS = (TPS + 31) / 32;
 };
+
+template <int N, int V = 0>
+using FxPlan = FxPlanOf<N, PlanInfo<N, V>::THREADS / 2, typename Plan<N, V>::two>;
 
 template <int L>
 inline void fx_fill(int4*, Radices<>) {}
@@ -290,9 +305,8 @@ inline void fx_fill(int4* out, Radices<R, Rs...>) {
   fx_fill<L * R>(out, Radices<Rs...>{});
 }
 
-template <int N, int V>
+template <typename P>
 inline void fx_table(int4* out) {
-  using P = FxPlan<N, V>;
   fx_fill<1>(out, typename P::fwd{});
   fx_fill<1>(out + P::ENTRIES, typename P::inv{});
 }
@@ -329,52 +343,56 @@ struct Shift {
   __device__ __forceinline__ q2 operator()(q2 v) const { return mkq((*this)(v.x), (*this)(v.y)); }
 };
 
-// Largest key over the CTA, for each of the two sequences (a, b).  scratch:
-// 2 ints per warp, not in use by another call since the last barrier but
-// one.  Ends with a barrier.
-template <int T>
-__device__ __forceinline__ int2 block_max2(int a, int b, int* scratch) {
-  a = __reduce_max_sync(0xffffffffu, a);
-  b = __reduce_max_sync(0xffffffffu, b);
-  if constexpr (T <= 32) {
-    __syncthreads();
-    return make_int2(a, b);
-  } else {
-    if ((threadIdx.x & 31) == 0) {
-      scratch[(threadIdx.x >> 5) * 2] = a;
-      scratch[(threadIdx.x >> 5) * 2 + 1] = b;
-    }
-    __syncthreads();
-    int2 r = make_int2(scratch[0], scratch[1]);
-#pragma unroll
-    for (int w = 1; w < T / 32; ++w) {
-      r.x = max(r.x, scratch[2 * w]);
-      r.y = max(r.y, scratch[2 * w + 1]);
-    }
-    return r;
-  }
+// The threads of one sequence: TPS of them, whole warps or an aligned part of
+// one.  Threads of several sequences share a warp where TPS < 32; they run in
+// lockstep.  id: the sequence's index in the CTA.
+template <int TPS>
+__device__ __forceinline__ void seq_sync(int id) {
+  if constexpr (TPS <= 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "n"(TPS) : "memory");
 }
 
-// Sums over the CTA of two counts (one per sequence) are left in scratch, one
-// pair per warp, and read back by sum2 after the caller's next barrier.
-// scratch: as for block_max2.
-__device__ __forceinline__ void block_sum2_put(unsigned a, unsigned b, int* scratch) {
-  a = __reduce_add_sync(0xffffffffu, a);
-  b = __reduce_add_sync(0xffffffffu, b);
-  if ((threadIdx.x & 31) == 0) {
-    scratch[(threadIdx.x >> 5) * 2] = (int)a;
-    scratch[(threadIdx.x >> 5) * 2 + 1] = (int)b;
-  }
+// Reductions over a sequence: put leaves each warp's part in scratch (TPS/32
+// ints of the sequence's own; unused where one warp holds the sequence), and
+// get, after the next seq_sync, returns the whole.
+template <int TPS>
+__device__ __forceinline__ unsigned seq_mask(int t) {
+  if constexpr (TPS >= 32) return 0xffffffffu;
+  else return ((1u << TPS) - 1) << ((threadIdx.x & 31) - t);
 }
-template <int T>
-__device__ __forceinline__ int2 block_sum2_get(const int* scratch) {
-  int2 r = make_int2(scratch[0], scratch[1]);
-#pragma unroll
-  for (int w = 1; w < (T + 31) / 32; ++w) {
-    r.x += scratch[2 * w];
-    r.y += scratch[2 * w + 1];
+template <int TPS>
+__device__ __forceinline__ int seq_max_put(int v, int t, int* scratch) {
+  v = __reduce_max_sync(seq_mask<TPS>(t), v);
+  if constexpr (TPS > 32) {
+    if ((t & 31) == 0) scratch[t >> 5] = v;
   }
-  return r;
+  return v;
+}
+template <int TPS>
+__device__ __forceinline__ int seq_max_get(int v, const int* scratch) {
+  if constexpr (TPS > 32) {
+    v = scratch[0];
+#pragma unroll
+    for (int w = 1; w < TPS / 32; ++w) v = max(v, scratch[w]);
+  }
+  return v;
+}
+template <int TPS>
+__device__ __forceinline__ int seq_sum_put(int v, int t, int* scratch) {
+  v = (int)__reduce_add_sync(seq_mask<TPS>(t), (unsigned)v);
+  if constexpr (TPS > 32) {
+    if ((t & 31) == 0) scratch[t >> 5] = v;
+  }
+  return v;
+}
+template <int TPS>
+__device__ __forceinline__ int seq_sum_get(int v, const int* scratch) {
+  if constexpr (TPS > 32) {
+    v = scratch[0];
+#pragma unroll
+    for (int w = 1; w < TPS / 32; ++w) v += scratch[w];
+  }
+  return v;
 }
 
 // Inputs of an inverse transform are first brought to kInvBits bits, then,
@@ -387,11 +405,14 @@ __device__ __forceinline__ int2 block_sum2_get(const int* scratch) {
 // bits where the first stage's own sums, at most R sqrt2 times the largest
 // component (61 bits), stay below 2^62.5: from a shift of log2 R - 1 on.
 constexpr int kInvBits = 61, kSumDrop = 12;
-template <int N, int V>
+// Nor may it have more than 60 + SHIFT_INV bits: the results then have 60,
+// and the row passes only ever shift them left (RowBits).
+template <typename P>
 __device__ __forceinline__ int inv_shift(int sum) {
-  using I = typename FxPlan<N, V>::inv;
+  using I = typename P::inv;
   constexpr int first = log2c(FirstRadix<I>::value) - 1;
-  constexpr int G = stage_shift(FirstRadix<typename TailRadices<I>::type>::value);
+  constexpr int G0 = stage_shift(FirstRadix<typename TailRadices<I>::type>::value);
+  constexpr int G = G0 < P::SHIFT_INV - 2 ? G0 : P::SHIFT_INV - 2;
   const int r = bits32(sum) + 32 + kSumDrop - 62;
   return max(0, min(r, max(r - G, first)));
 }
@@ -460,187 +481,175 @@ __device__ __forceinline__ void fx_butterfly(q2* a, const int4* __restrict__ T, 
   qdftR<R, S, Z>(a);
 }
 
-// Runs the first stage's butterfly for the warp's mask of zero inputs.
-template <int R, int S, typename G>
-__device__ __forceinline__ void fx_masked_first(q2* a, int w) {
-  constexpr int C = G::C, A = G::A, B = G::B;
-  if constexpr (A == 0) {
-    qdftR<R, S, C>(a);
-  } else if constexpr (B == 0) {
-    if (w & A) qdftR<R, S, C | A>(a);
-    else qdftR<R, S, C>(a);
-  } else {
-    if ((w & (A | B)) == (A | B)) qdftR<R, S, C | A | B>(a);
-    else if (w & A) qdftR<R, S, C | A>(a);
-    else if (w & B) qdftR<R, S, C | B>(a);
-    else qdftR<R, S, C>(a);
-  }
+// Position of element i of a sequence in its buffer: one element of padding
+// after every eight (128 bytes), so that the strided stores of a stage meet
+// few bank conflicts.  Every i + m c used below adds pad(m c) exactly.
+__host__ __device__ constexpr int pad(int i) { return i + i / 8; }
+
+// Butterflies of a stage of radix R held by one thread: i = t + jb TPS, jb <
+// J; where there are fewer butterflies than threads, threads t < N / R hold
+// one each.
+template <typename P, int R>
+struct Bfly {
+  static constexpr int NB = P::N / R;
+  static constexpr int J = NB >= P::TPS ? NB / P::TPS : 1;
+  static constexpr int POINTS = J * R;
+  static_assert(NB < P::TPS || NB % P::TPS == 0, "whole butterflies per thread");
+  __device__ static __forceinline__ bool active(int t) { return NB >= P::TPS || t < NB; }
+};
+
+// Inputs i + m NB of butterfly i, out of src; Z: inputs left out.
+template <typename P, int R, int Z = 0>
+__device__ __forceinline__ void fx_load(q2* a, const q2* src, int i) {
+  const q2* s = src + pad(i);
+#pragma unroll
+  for (int m = 0; m < R; ++m)
+    if (!((Z >> m) & 1)) a[m] = s[pad(m * (P::N / R))];
 }
 
-// One in-place Stockham stage on F sequences.  KIN >= 0: zero outside the
-// band (first stage of an inverse transform, which also applies the right
-// shifts pre of the sequences); KOUT >= 0: only the band is needed (last
-// stage).  SHR: a later stage that starts with the right shifts pre.
-template <int N, int V, int R, int S, int F, int L, int KIN, int KOUT, bool SHR = false>
-__device__ __forceinline__ void fx_stage(q2* buf, const int4* __restrict__ T, int2 pre) {
-  constexpr int NB = N / R, Th = PlanInfo<N, V>::THREADS, TOT = F * NB, J = (TOT + Th - 1) / Th;
-  constexpr bool FIRST = L == 1, LAST = L * R == N;
-  using GI = GapMask<N, R, FIRST ? KIN : -1>;
-  using GO = GapMask<N, R, LAST ? KOUT : -1>;
-  q2 a[J][R];
-  int base[J], dst[J], om[J];
+// Outputs of butterfly i of the stage with sub-length L, into dst.
+template <typename P, int R, int L>
+__device__ __forceinline__ void fx_store(const q2* a, q2* dst, int i) {
+  const int k = i & (L - 1);
+  q2* d = dst + pad((i - k) * R + k);
 #pragma unroll
-  for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * Th;
-    base[jb] = dst[jb] = om[jb] = 0;
-    if (TOT % Th == 0 || u < TOT) {
-      const int f = u / NB;
-      const int i = u - f * NB;
-      const int k = i & (L - 1);
-      base[jb] = f * N;
-      const int zm = GI::warp(i);
+  for (int m = 0; m < R; ++m) d[pad(m * L)] = a[m];
+}
+
+__device__ __forceinline__ void swap_bufs(q2*& a, q2*& b) {
+  q2* c = a;
+  a = b;
+  b = c;
+}
+
+// Middle stages with sub-lengths from L on: src -> dst, sync, swap.  SHR: the
+// first of them starts with a right shift by r.
+template <typename P, int S, int L, bool SHR>
+__device__ __forceinline__ void fx_middle(q2*&, q2*&, const int4*, int, int, int, Radices<>) {}
+template <typename P, int S, int L, bool SHR, int R, int... Rs>
+__device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int t, int id, int r, Radices<R, Rs...>) {
+  using B = Bfly<P, R>;
+  if (B::active(t)) {
 #pragma unroll
-      for (int m = 0; m < R; ++m)
-        if (!((zm >> m) & 1)) a[jb][m] = buf[base[jb] + i + m * NB];
-      if constexpr (FIRST) {
-        if constexpr (KIN >= 0) {
-          const int r = f ? pre.y : pre.x;
-          const i64 half = (1LL << r) >> 1;
+    for (int jb = 0; jb < B::J; ++jb) {
+      const int i = t + jb * P::TPS;
+      q2 a[R];
+      fx_load<P, R>(a, src, i);
+      if constexpr (SHR) {
+        if (r > 0) {
 #pragma unroll
-          for (int m = 0; m < R; ++m)
-            if (!((zm >> m) & 1)) a[jb][m] = mkq((a[jb][m].x + half) >> r, (a[jb][m].y + half) >> r);
+          for (int m = 0; m < R; ++m) a[m] = mkq(shr_round(a[m].x, r), shr_round(a[m].y, r));
         }
-        fx_masked_first<R, S, GI>(a[jb], zm);
-      } else {
-        om[jb] = GO::warp(i);
-        if constexpr (SHR) {
-          const int r = f ? pre.y : pre.x;
-          if (r > 0) {
-#pragma unroll
-            for (int m = 0; m < R; ++m) a[jb][m] = mkq(shr_round(a[jb][m].x, r), shr_round(a[jb][m].y, r));
-          }
-        }
-        fx_butterfly<R, S, L, 0>(a[jb], T, k);
       }
-      dst[jb] = (i - k) * R + k;
+      fx_butterfly<R, S, L, 0>(a, T, i & (L - 1));
+      fx_store<P, R, L>(a, dst, i);
     }
   }
-  __syncthreads();
+  seq_sync<P::TPS>(id);
+  swap_bufs(src, dst);
+  fx_middle<P, S, L * R, false>(src, dst, T + (R - 1) * L, t, id, r, Radices<Rs...>{});
+}
+
+// Inverse transform (S = +1) of the sequence in src, zero outside the band
+// KB: the inputs, of at most kInvBits bits, are shifted right by pre first,
+// and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
+// is left in registers: out[jb R + m] is position t + jb TPS + m N / R for R
+// the last radix.  dst is free afterwards, src not before the next sync.
+template <typename P, int KB>
+__device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, int t, int id, int pre, q2* out) {
+  using I = typename P::inv;
+  constexpr int R1 = FirstRadix<I>::value, RL = LastRadix<I>::value;
+  constexpr int Z = gap_common(P::N, R1, KB);  // inputs in the gap for every butterfly
+  using B1 = Bfly<P, R1>;
+  using BL = Bfly<P, RL>;
+  const int4* T = tw + P::ENTRIES;
+  if (B1::active(t)) {
+    const i64 half = (1LL << pre) >> 1;
 #pragma unroll
-  for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * Th;
-    if (TOT % Th == 0 || u < TOT) {
+    for (int jb = 0; jb < B1::J; ++jb) {
+      const int i = t + jb * P::TPS;
+      q2 a[R1];
+      fx_load<P, R1, Z>(a, src, i);
 #pragma unroll
-      for (int m = 0; m < R; ++m)
-        if (!((om[jb] >> m) & 1)) buf[base[jb] + dst[jb] + m * L] = a[jb][m];
+      for (int m = 0; m < R1; ++m)
+        if (!((Z >> m) & 1)) a[m] = mkq((a[m].x + half) >> pre, (a[m].y + half) >> pre);
+      qdftR<R1, +1, Z>(a);
+      fx_store<P, R1, 1>(a, dst, i);
     }
   }
-  __syncthreads();
+  seq_sync<P::TPS>(id);
+  swap_bufs(src, dst);
+  using Mid = typename InitRadices<typename TailRadices<I>::type>::type;
+  fx_middle<P, +1, R1, false>(src, dst, T, t, id, 0, Mid{});
+  constexpr int L = P::N / RL;
+  if (BL::active(t)) {
+    const int4* Tl = T + P::ENTRIES_INV - (RL - 1) * L;
+#pragma unroll
+    for (int jb = 0; jb < BL::J; ++jb) {
+      const int i = t + jb * P::TPS;
+      fx_load<P, RL>(out + jb * RL, src, i);
+      fx_butterfly<RL, +1, L, 0>(out + jb * RL, Tl, i);
+    }
+  }
 }
 
-template <int N, int V, int S, int F, int L, int KIN, int KOUT>
-__device__ __forceinline__ void fx_run(q2*, const int4*, int2, Radices<>) {}
-template <int N, int V, int S, int F, int L, int KIN, int KOUT, int R, int... Rs>
-__device__ __forceinline__ void fx_run(q2* buf, const int4* T, int2 pre, Radices<R, Rs...>) {
-  fx_stage<N, V, R, S, F, L, KIN, KOUT>(buf, T, pre);
-  fx_run<N, V, S, F, L * R, KIN, KOUT>(buf, T + (L > 1 ? (R - 1) * L : 0), pre, Radices<Rs...>{});
-}
-
-// The stages after the first of a forward transform, whose first stage's
-// results have at most 32 + bits32(m) bits (m.x, m.y for the two sequences).
-// SPARE: bits of the results to leave free.  Returns the shifts taken.
-template <int N, int V, int KB, int SPARE>
-__device__ __forceinline__ int2 fx_forward_rest(q2* buf, const int4* tw, int2 m) {
-  using P = FxPlan<N, V>;
-  constexpr int most = 62 - SPARE - P::GROWTH2 - 32;
-  const int2 r = make_int2(max(0, bits32(m.x) - most), max(0, bits32(m.y) - most));
-  using Tail = typename TailRadices<typename P::fwd>::type;
-  constexpr int R2 = FirstRadix<Tail>::value;
-  fx_stage<N, V, R2, -1, 2, P::R1, -1, (P::R1 * R2 == N) ? KB : -1, true>(buf, tw, r);
-  fx_run<N, V, -1, 2, P::R1 * R2, -1, KB>(buf, tw + (R2 - 1) * P::R1, r, typename TailRadices<Tail>::type{});
+// Forward transform (S = -1) of the sequence in registers: in[jb R + m] is
+// position t + jb TPS + m N / R for R the first radix.  MEASURE: the inputs
+// leave room for the first stage only, and a shift measured after it makes
+// room for the others, with SPARE bits of the result free; the shift is
+// returned.  The result, times 2^-SHIFT, is left in src, in natural order,
+// synchronised; only the band KB is formed.
+template <typename P, int KB, bool MEASURE, int SPARE>
+__device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4* tw, int t, int id, int* scratch) {
+  using F = typename P::fwd;
+  using Tail = typename TailRadices<F>::type;
+  constexpr int R1 = FirstRadix<F>::value, RL = LastRadix<F>::value, L = P::N / RL;
+  constexpr int C = gap_common(P::N, RL, KB);  // outputs in the gap for every butterfly
+  using B1 = Bfly<P, R1>;
+  using BL = Bfly<P, RL>;
+  int big = 0, r = 0;
+  if (B1::active(t)) {
+#pragma unroll
+    for (int jb = 0; jb < B1::J; ++jb) {
+      q2* a = in + jb * R1;
+      qdftR<R1, -1, 0>(a);
+      if constexpr (MEASURE) {
+#pragma unroll
+        for (int m = 0; m < R1; ++m) big = max(big, max(mag32(a[m].x), mag32(a[m].y)));
+      }
+      fx_store<P, R1, 1>(a, dst, t + jb * P::TPS);
+    }
+  }
+  if constexpr (MEASURE) big = seq_max_put<P::TPS>(big, t, scratch);
+  seq_sync<P::TPS>(id);
+  swap_bufs(src, dst);
+  if constexpr (MEASURE) r = max(0, bits32(seq_max_get<P::TPS>(big, scratch)) - (62 - SPARE - P::GROWTH2 - 32));
+  using Mid = typename InitRadices<Tail>::type;
+  constexpr bool MIDDLE = L > R1;  // there are middle stages
+  fx_middle<P, -1, R1, MEASURE && MIDDLE>(src, dst, tw, t, id, r, Mid{});
+  if (BL::active(t)) {
+    const int4* Tl = tw + P::ENTRIES - (RL - 1) * L;
+#pragma unroll
+    for (int jb = 0; jb < BL::J; ++jb) {
+      const int i = t + jb * P::TPS;
+      q2 a[RL];
+      fx_load<P, RL>(a, src, i);
+      if constexpr (MEASURE && !MIDDLE) {
+        if (r > 0) {
+#pragma unroll
+          for (int m = 0; m < RL; ++m) a[m] = mkq(shr_round(a[m].x, r), shr_round(a[m].y, r));
+        }
+      }
+      fx_butterfly<RL, -1, L, 0>(a, Tl, i);
+      q2* d = dst + pad(i);
+#pragma unroll
+      for (int m = 0; m < RL; ++m)
+        if (!((C >> m) & 1)) d[pad(m * L)] = a[m];
+    }
+  }
+  seq_sync<P::TPS>(id);
+  swap_bufs(src, dst);
   return r;
-}
-
-// Transforms, in place, of two sequences of N points back to back in buf:
-// inverse (S = +1) of sequences zero outside the band KB, and forward, of
-// which only the band KB is formed.  The gap positions must hold zeros on
-// input of the inverse (warps that straddle the gap read it) and are
-// undefined after the forward.  Inputs have at most kInvBits bits and are
-// shifted right by pre first (inverse), or have at most BITS_FWD bits
-// (forward); the result is the transform times 2^-SHIFT.  tw: FxPlan's
-// tables.
-template <int N, int V, int KB>
-__device__ __forceinline__ void fx_inverse(q2* buf, const int4* tw, int2 pre) {
-  using P = FxPlan<N, V>;
-  fx_run<N, V, +1, 2, 1, KB, -1>(buf, tw + P::ENTRIES, pre, typename P::inv{});
-}
-template <int N, int V, int KB>
-__device__ __forceinline__ void fx_forward(q2* buf, const int4* tw) {
-  fx_run<N, V, -1, 2, 1, -1, KB>(buf, tw, make_int2(0, 0), typename FxPlan<N, V>::fwd{});
-}
-
-// Inverse transform, a pointwise map, and forward transform of two sequences:
-// the last inverse stage, the map and the first forward stage run on
-// registers.  prep(m0, m1) gets the largest high-word magnitude (mag32) of
-// each sequence's inverse transform, on every thread after a barrier;
-// op(f, x, z) gets sequence f, position x and the value there and returns
-// the forward transform's input.  MEASURE: the inputs leave room for the first
-// forward stage only (fx_forward_rest).  The results leave one bit free;
-// returns the shifts taken.
-template <int N, int V, int KB, bool MEASURE, typename Prep, typename Op>
-__device__ __forceinline__ int2 fx_turn(q2* buf, const int4* tw, int2 pre, int* scratch, Prep prep, Op op) {
-  using P = FxPlan<N, V>;
-  constexpr int R = FirstRadix<typename P::fwd>::value, NB = N / R, L = N / R;
-  constexpr int Th = PlanInfo<N, V>::THREADS, TOT = 2 * NB, J = (TOT + Th - 1) / Th;
-  using Init = typename InitRadices<typename P::inv>::type;
-  fx_run<N, V, +1, 2, 1, KB, -1>(buf, tw + P::ENTRIES, pre, Init{});
-  const int4* Tl = tw + P::ENTRIES + FxSum<1, Init>::entries;
-  q2 a[J][R];
-  int m0 = 0, m1 = 0;
-#pragma unroll
-  for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * Th;
-    if (TOT % Th == 0 || u < TOT) {
-      const int f = u / NB;
-      const int i = u - f * NB;
-#pragma unroll
-      for (int m = 0; m < R; ++m) a[jb][m] = buf[f * N + i + m * NB];
-      fx_butterfly<R, +1, L, 0>(a[jb], Tl, i);
-      int mm = 0;
-#pragma unroll
-      for (int m = 0; m < R; ++m) mm = max(mm, max(mag32(a[jb][m].x), mag32(a[jb][m].y)));
-      if (f == 0) m0 = max(m0, mm);
-      else m1 = max(m1, mm);
-    }
-  }
-  const int2 mx = block_max2<Th>(m0, m1, scratch);  // every thread has read buf
-  prep(mx.x, mx.y);
-  m0 = m1 = 0;
-#pragma unroll
-  for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * Th;
-    if (TOT % Th == 0 || u < TOT) {
-      const int f = u / NB;
-      const int i = u - f * NB;
-#pragma unroll
-      for (int m = 0; m < R; ++m) a[jb][m] = op(f, i + m * L, a[jb][m]);
-      qdftR<R, -1, 0>(a[jb]);
-      int mm = 0;
-#pragma unroll
-      for (int m = 0; m < R; ++m) {
-        if constexpr (MEASURE) mm = max(mm, max(mag32(a[jb][m].x), mag32(a[jb][m].y)));
-        buf[f * N + i * R + m] = a[jb][m];
-      }
-      if (f == 0) m0 = max(m0, mm);
-      else m1 = max(m1, mm);
-    }
-  }
-  if constexpr (MEASURE) {
-    return fx_forward_rest<N, V, KB, 1>(buf, tw, block_max2<Th>(m0, m1, scratch + 16));
-  }
-  __syncthreads();
-  fx_run<N, V, -1, 2, R, -1, KB>(buf, tw, pre, typename TailRadices<typename P::fwd>::type{});
-  return make_int2(0, 0);
 }
 
 }  // namespace da

@@ -131,14 +131,18 @@ struct Geo {
   static constexpr int NH = N / 2 + 1;
   // threads: two transforms at a time (fft.cuh)
   static constexpr int THREADS = PlanInfo<N, V>::THREADS;
-  // shared memory: folded twiddle table + one buffer of two sequences +
-  // probe sums
   static constexpr int PMAX = 64;
-  static constexpr int SCRATCH = 4 * 2 * 8;  // ints: four reductions of two values over at most 8 warps
-  static constexpr size_t SMEM =
-      sizeof(double) * FoldInfo<N, V>::PADDED + sizeof(double2) * (2 * N + 2 * PMAX) + sizeof(int) * SCRATCH;
-  // passes that run the integer transforms only: two sequences, probe sums, scratch
-  static constexpr size_t SMEM_FX = sizeof(q2) * (2 * N + 2 * PMAX) + sizeof(int) * SCRATCH;
+  // shared memory of the control maps: folded twiddle table + one sequence
+  static constexpr size_t SMEM = sizeof(double2) * 2 * N;  // static_ctrl.cu: plain table and one sequence
+  static constexpr size_t SMEM_FOLD = sizeof(double) * FoldInfo<N, V>::PADDED + sizeof(double2) * (N + 2);
+  // passes that run the integer transforms: two buffers of each of two
+  // sequences, probe sums, scratch of the reductions (three of WARPS ints for
+  // each sequence, two of a pair per warp for the CTA)
+  static constexpr int SCRATCH = (3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS;
+  static constexpr size_t SMEM_FX =
+      sizeof(q2) * (4 * FxPlan<N, V>::SEQ) + sizeof(double2) * 2 * PMAX + sizeof(int) * ((SCRATCH + 3) / 4 * 4);
+  // k_ctrl_cols runs both: the FP64 part first, in the same memory
+  static constexpr size_t SMEM_CTRL = SMEM_FOLD > SMEM_FX ? SMEM_FOLD : SMEM_FX;
   // column passes load their epilogue inputs before the transforms (about
   // 60 more registers a thread) where a CTA is at most 128 threads
   static constexpr bool PREFETCH = THREADS <= 128;
@@ -335,142 +339,178 @@ __global__ void k_half_to_compact(const double2* __restrict__ in, double2* __res
 // Control map and the inverse column transforms of a stage state
 // ---------------------------------------------------------------------------
 
-// Shared memory of the pass kernels: the two sequences, the probe sums and
-// the scratch of the reductions.
-template <int N>
-struct FxSmem {
-  q2* a;
+// A thread's place in a pass kernel's CTA of two sequences: sequence f,
+// thread t of it; the sequence's two buffers and its scratch; the probe sums.
+template <int N, int V>
+struct FxThread {
+  using P = FxPlan<N, V>;
+  int t, f;
+  q2 *src, *dst;
+  int* scratch;  // three reductions of WARPS ints
   double2 *Tu, *Tv;
-  int* scratch;
-  __device__ __forceinline__ explicit FxSmem(void* base) {
-    a = static_cast<q2*>(base);
-    Tu = reinterpret_cast<double2*>(a + 2 * N);
-    Tv = Tu + Geo<N>::PMAX;
-    scratch = reinterpret_cast<int*>(Tv + Geo<N>::PMAX);
+  __device__ __forceinline__ explicit FxThread(void* base) {
+    f = threadIdx.x / P::TPS;
+    t = threadIdx.x - f * P::TPS;
+    q2* a = static_cast<q2*>(base);
+    src = a + f * 2 * P::SEQ;
+    dst = src + P::SEQ;
+    Tu = reinterpret_cast<double2*>(a + 4 * P::SEQ);
+    Tv = Tu + Geo<N, V>::PMAX;
+    scratch = reinterpret_cast<int*>(Tv + Geo<N, V>::PMAX) + f * 3 * P::WARPS;
   }
+  // the other sequence's buffer at the same place as p (of this sequence)
+  __device__ __forceinline__ q2* other(q2* p) const { return f ? p - 2 * P::SEQ : p + 2 * P::SEQ; }
 };
 
-// A column under construction: complex doubles, as raw bits, at the retained
-// positions of two sequences, and the largest exponent field of each.
-template <int N>
+// A column under construction: the doubles a thread puts at its retained rows
+// rr = threadIdx.x + j THREADS of the two fields, and the largest exponent
+// fields.
+template <int N, int V>
 struct ColumnPut {
-  q2* a;
+  static constexpr int MT = (Geo<N, V>::Kr + Geo<N, V>::THREADS - 1) / Geo<N, V>::THREADS;
+  double2 v0[MT], v1[MT];
   int f0 = 0, f1 = 0;
-  __device__ __forceinline__ explicit ColumnPut(q2* a_) : a(a_) {}
-  __device__ __forceinline__ void put(int q, double2 v0, double2 v1) {
-    a[q] = mkq(__double_as_longlong(v0.x), __double_as_longlong(v0.y));
-    a[N + q] = mkq(__double_as_longlong(v1.x), __double_as_longlong(v1.y));
-    f0 = max(f0, max(exp_field(v0.x), exp_field(v0.y)));
-    f1 = max(f1, max(exp_field(v1.x), exp_field(v1.y)));
+  __device__ __forceinline__ void put(int j, double2 a, double2 b) {
+    v0[j] = a;
+    v1[j] = b;
+    f0 = max(f0, max(exp_field(a.x), exp_field(a.y)));
+    f1 = max(f1, max(exp_field(b.x), exp_field(b.y)));
   }
 };
 
 // The two column values u = i ky/k^2 Yv, v = -i kx/k^2 Yv (scaled by 1/N^2;
-// f = symF entry of the mode) at position q.
-template <int N>
-__device__ __forceinline__ void put_stage_columns(ColumnPut<N>& c, int q, const Sym4& f, double2 Yv) {
-  c.put(q, make_double2(-f.a * Yv.y, f.a * Yv.x),  // u:  i ky / k^2
+// f = symF entry of the mode) as entry j.
+template <int N, int V>
+__device__ __forceinline__ void put_stage_columns(ColumnPut<N, V>& c, int j, const Sym4& f, double2 Yv) {
+  c.put(j, make_double2(-f.a * Yv.y, f.a * Yv.x),  // u:  i ky / k^2
         make_double2(f.b * Yv.y, -f.b * Yv.x));    // v: -i kx / k^2
 }
 
 // The two column values of the adjoint fields of an adjoint stage value kb:
 // 2a = 2 d_xy kb = -2 kx ky kb and b = (d_xx - d_yy) kb = (ky^2 - kx^2) kb,
-// scaled by 1/N^2 (g = symA entry of the mode), at q.
-template <int N>
-__device__ __forceinline__ void put_adjoint_columns(ColumnPut<N>& c, int q, const Sym4& g, double2 kb) {
-  c.put(q, cscale(kb, g.c), cscale(kb, g.d));
+// scaled by 1/N^2 (g = symA entry of the mode).
+template <int N, int V>
+__device__ __forceinline__ void put_adjoint_columns(ColumnPut<N, V>& c, int j, const Sym4& g, double2 kb) {
+  c.put(j, cscale(kb, g.c), cscale(kb, g.d));
 }
 
-// Zeroes the positions outside the retained set in both sequences.
-template <int N, int V>
-__device__ __forceinline__ void zero_outside(q2* seq) {
-  constexpr int K = Geo<N, V>::K, GAP = N - 2 * K - 1;
-  for (int u = threadIdx.x; u < 2 * GAP; u += Geo<N, V>::THREADS) {
-    const int f = u / GAP, q = K + 1 + (u - f * GAP);
-    seq[f * N + q] = mkq(0, 0);
+// Two reductions over the whole CTA at once, (a, b) -> (A, B): `scratch` has
+// a pair per warp, not in use since the barrier before last.  Ends with a
+// barrier.
+template <int T, bool SUM>
+__device__ __forceinline__ int2 cta_reduce2(int a, int b, int* scratch) {
+  if constexpr (SUM) {
+    a = (int)__reduce_add_sync(0xffffffffu, (unsigned)a);
+    b = (int)__reduce_add_sync(0xffffffffu, (unsigned)b);
+  } else {
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
   }
+  if constexpr (T > 32) {
+    if ((threadIdx.x & 31) == 0) {
+      scratch[(threadIdx.x >> 5) * 2] = a;
+      scratch[(threadIdx.x >> 5) * 2 + 1] = b;
+    }
+    __syncthreads();
+    a = scratch[0];
+    b = scratch[1];
+#pragma unroll
+    for (int w = 1; w < T / 32; ++w) {
+      a = SUM ? a + scratch[2 * w] : max(a, scratch[2 * w]);
+      b = SUM ? b + scratch[2 * w + 1] : max(b, scratch[2 * w + 1]);
+    }
+  } else {
+    __syncthreads();
+  }
+  return make_int2(a, b);
 }
 
-// Both columns put in c by this CTA (each thread its rows rr = threadIdx.x +
-// t THREADS, as in the loops that put them): to integers, inverse transform
-// along y, into column kx of both fields of Mx.
+// Both columns put in c: to integers in x's src buffers, inverse transform
+// along y, into column kx of both fields of Mx.  buf0: sequence 0's buffer to
+// start from, free to write (sequence 1's lies 2 SEQ further).
 template <int N, int V>
-__device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N>& c, int bm, int kx, int* scratch) {
+__device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, V>& c, FxThread<N, V> x, int bm, int kx) {
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
-  q2* a = c.a;
-  const int2 f = block_max2<G::THREADS>(c.f0, c.f1, scratch);
+  constexpr int T = G::THREADS, GAP = N - 2 * G::K - 1;
+  int* scratch = x.scratch + (2 - x.f) * 3 * P::WARPS;  // after the two sequences' own
+  const int2 f = cta_reduce2<T, false>(c.f0, c.f1, scratch);
   const int e0 = exp_for<kInvBits>(f.x), e1 = exp_for<kInvBits>(f.y);
+  q2 *a0 = x.f ? x.other(x.src) : x.src, *a1 = a0 + 2 * P::SEQ;
   unsigned s0 = 0, s1 = 0;
 #pragma unroll
-  for (int t = 0; t < (G::Kr + G::THREADS - 1) / G::THREADS; ++t) {
-    const int rr = threadIdx.x + t * G::THREADS;
+  for (int j = 0; j < ColumnPut<N, V>::MT; ++j) {
+    const int rr = threadIdx.x + j * T;
     if (rr >= G::Kr) break;
-    const int q = ky_of_row(rr, G::K) & (N - 1);
-    const q2 x = a[q], y = a[N + q];
-    const q2 u = mkq(double_to_fx(__longlong_as_double(x.x), e0), double_to_fx(__longlong_as_double(x.y), e0));
-    const q2 v = mkq(double_to_fx(__longlong_as_double(y.x), e1), double_to_fx(__longlong_as_double(y.y), e1));
+    const int q = pad(ky_of_row(rr, G::K) & (N - 1));
+    const q2 u = mkq(double_to_fx(c.v0[j].x, e0), double_to_fx(c.v0[j].y, e0));
+    const q2 v = mkq(double_to_fx(c.v1[j].x, e1), double_to_fx(c.v1[j].y, e1));
     s0 += mag_units(u);
     s1 += mag_units(v);
-    a[q] = u;
-    a[N + q] = v;
+    a0[q] = u;
+    a1[q] = v;
   }
-  zero_outside<N, V>(a);
-  block_sum2_put(s0, s1, scratch + 16);
-  __syncthreads();
-  const int2 sum = block_sum2_get<G::THREADS>(scratch + 16);
-  const int2 pre = make_int2(inv_shift<N, V>(sum.x), inv_shift<N, V>(sum.y));
-  fx_inverse<N, V, G::K>(a, d.fxtw, pre);
-  q2* M = d.Mx + (size_t)bm * 2 * N * G::Kc + kx;
+  for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(G::K + 1 + u)] = mkq(0, 0);
+  const int2 sum = cta_reduce2<T, true>(s0, s1, scratch + 4 * P::WARPS);
+  const int pre = inv_shift<P>(x.f ? sum.y : sum.x);
+  constexpr int R = LastRadix<typename P::inv>::value;
+  using B = Bfly<P, R>;
+  q2 out[B::POINTS];
+  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, pre, out);
+  if (B::active(x.t)) {
+    q2* M = d.Mx + (size_t)bm * 2 * N * G::Kc + (size_t)(x.f * N + x.t) * G::Kc + kx;
 #pragma unroll
-  for (int t = 0; t < (2 * N + G::THREADS - 1) / G::THREADS; ++t) {
-    const int u = threadIdx.x + t * G::THREADS;
-    if (u < 2 * N) M[(size_t)u * G::Kc] = a[u];
+    for (int jb = 0; jb < B::J; ++jb)
+#pragma unroll
+      for (int m = 0; m < R; ++m) M[(size_t)(jb * P::TPS + m * B::NB) * G::Kc] = out[jb * R + m];
   }
-  if (threadIdx.x < 2)
-    d.eX[(bm * 2 + threadIdx.x) * G::Kc + kx] = clamp_exp((threadIdx.x ? e1 + pre.y : e0 + pre.x) + P::SHIFT_INV);
+  if (x.t == 0) d.eX[(bm * 2 + x.f) * G::Kc + kx] = clamp_exp((x.f ? e1 : e0) + pre + P::SHIFT_INV);
 }
 
 // Column kx of both fields of the column-major Mn (M points at the column,
-// eN at the member's row exponents) into a, forward transform along y.
-// Returns the exponents of the two results.  `between` runs after the loads
-// are issued.
+// eN at the member's row exponents), forward transform along y, left in the
+// src buffers, synchronised over the CTA.  `between` runs after the loads are
+// issued.  Returns the exponents of the two results.
 template <int N, int V, typename Between>
-__device__ __forceinline__ int2 forward_columns(const q2* __restrict__ M, const int* __restrict__ eN, q2* a,
-                                                const int4* tw, int* scratch, Between between) {
+__device__ __forceinline__ int2 forward_columns(const q2* __restrict__ M, const int* __restrict__ eN,
+                                                FxThread<N, V>& x, const int4* tw, Between between) {
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
-  constexpr int T = G::THREADS, J = (2 * N + T - 1) / T;
-  q2 v[J];
-  int e[J], k0 = kZeroExp, k1 = kZeroExp;
+  constexpr int R = FirstRadix<typename P::fwd>::value;
+  // the first stage only must leave room where that gives two bits more
+  constexpr bool MEASURE = P::GROWTH >= P::GROWTH1 + 2;
+  constexpr int BITS = MEASURE ? 62 - P::GROWTH1 : P::BITS_FWD;
+  using B = Bfly<P, R>;
+  q2 v[B::POINTS];
+  int e[B::POINTS], key = kZeroExp;
+  if (B::active(x.t)) {
 #pragma unroll
-  for (int t = 0; t < J; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < 2 * N) {
-      v[t] = M[u];
-      e[t] = eN[u & (N - 1)];
+    for (int j = 0; j < B::POINTS; ++j) {
+      const int y = x.t + (j / R) * P::TPS + (j % R) * B::NB;
+      v[j] = M[x.f * N + y];
+      e[j] = eN[y];
     }
   }
   between();
+  if (B::active(x.t)) {
 #pragma unroll
-  for (int t = 0; t < J; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < 2 * N) {
-      const int k = bits32(max(mag32(v[t].x), mag32(v[t].y))) + 32 + e[t];
-      if (u < N) k0 = max(k0, k);
-      else k1 = max(k1, k);
-    }
+    for (int j = 0; j < B::POINTS; ++j) key = max(key, bits32(max(mag32(v[j].x), mag32(v[j].y))) + 32 + e[j]);
   }
-  const int2 k = block_max2<T>(k0, k1, scratch);
-  const int e0 = k.x - P::BITS_FWD, e1 = k.y - P::BITS_FWD;
+  key = seq_max_put<P::TPS>(key, x.t, x.scratch);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  key = seq_max_get<P::TPS>(key, x.scratch);
+  const int e0 = key - BITS;
+  if (B::active(x.t)) {
 #pragma unroll
-  for (int t = 0; t < J; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < 2 * N) a[u] = Shift(e[t] - (u < N ? e0 : e1))(v[t]);
+    for (int j = 0; j < B::POINTS; ++j) v[j] = Shift(e[j] - e0)(v[j]);
   }
+  const int r = fx_forward<P, G::K, MEASURE, 0>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
+  // both sequences' results and exponents, to the whole CTA
+  const int out = clamp_exp(e0 + r + P::SHIFT);
+  if (x.t == 0) x.scratch[0] = out;
   __syncthreads();
-  fx_forward<N, V, G::K>(a, tw);
-  return make_int2(clamp_exp(e0 + P::SHIFT), clamp_exp(e1 + P::SHIFT));
+  const int* s0 = x.scratch - x.f * 3 * P::WARPS;
+  return make_int2(s0[0], s0[3 * P::WARPS]);
 }
 
 // Integers of one exponent to doubles, with the power of two folded into the
@@ -494,7 +534,6 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d, int fla
   extern __shared__ double2 sm[];
   double* T = reinterpret_cast<double*>(sm);
   double2* a = sm + FoldInfo<N, V>::PADDED / 2;
-  const FxSmem<N> fs(a);
   const int kx = blockIdx.x, bm = blockIdx.y;
   load_fold<N, V>(T, d.fold);
   const double2* M = reinterpret_cast<const double2*>(d.Mn) + ((size_t)bm * G::Kc + kx) * 2 * N;
@@ -502,19 +541,21 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d, int fla
   for (int y = threadIdx.x; y < N; y += G::THREADS) a[y] = M[y];
   __syncthreads();
   fft_folded<N, V, -1, 1, -1, G::K>(a, T);
-  ColumnPut<N> put(fs.a);
-  // each retained position is read and rewritten by one thread only
-  #pragma unroll
-  for (int rr = threadIdx.x; rr < G::Kr; rr += G::THREADS) {
+  ColumnPut<N, V> put;
+#pragma unroll
+  for (int j = 0; j < put.MT; ++j) {
+    const int rr = threadIdx.x + j * G::THREADS;
+    if (rr >= G::Kr) break;
     const int ky = ky_of_row(rr, G::K);
     const size_t idx = cidx<N>(bm, rr, kx);
     const double2 w0 = cscale(a[ky & (N - 1)], d.mult[idx]);
     d.W[idx] = w0;
     d.Y[idx] = w0;
-    put_stage_columns<N>(put, ky & (N - 1), d.symF[kx * G::Kr + rr], w0);
+    put_stage_columns<N, V>(put, j, d.symF[kx * G::Kr + rr], w0);
   }
   if (flags & F_NO_NEXT) return;
-  finish_columns<N, V>(d, put, bm, kx, fs.scratch);
+  __syncthreads();  // the FP64 part's memory is read no more
+  finish_columns<N, V>(d, put, FxThread<N, V>(sm), bm, kx);
 }
 
 // Restart from the compact state in W (a checkpoint): Y = W and the inverse
@@ -523,110 +564,108 @@ template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_state_cols(Dev d) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
-  const FxSmem<N> fs(sm);
   const int kx = blockIdx.x, bm = blockIdx.y;
-  ColumnPut<N> put(fs.a);
-  #pragma unroll
-  for (int rr = threadIdx.x; rr < G::Kr; rr += G::THREADS) {
-    const int ky = ky_of_row(rr, G::K);
+  ColumnPut<N, V> put;
+#pragma unroll
+  for (int j = 0; j < put.MT; ++j) {
+    const int rr = threadIdx.x + j * G::THREADS;
+    if (rr >= G::Kr) break;
     const size_t idx = cidx<N>(bm, rr, kx);
     const double2 w = d.W[idx];
     d.Y[idx] = w;
-    put_stage_columns<N>(put, ky & (N - 1), d.symF[kx * G::Kr + rr], w);
+    put_stage_columns<N, V>(put, j, d.symF[kx * G::Kr + rr], w);
   }
-  finish_columns<N, V>(d, put, bm, kx, fs.scratch);
+  finish_columns<N, V>(d, put, FxThread<N, V>(sm), bm, kx);
 }
 
 // ---------------------------------------------------------------------------
 // Row passes
 // ---------------------------------------------------------------------------
 
-// Rows y0, y0 + 1 of the two fields of Mx, packed for the inverse transform
-// along x as field 0 + i field 1: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B)
-// for the mixed half spectra A, B (kx = 0..K); the DC bin keeps real parts
-// only; the gap is zeroed.  Ends with a barrier.
+// Row y of the two fields of Mx, packed for the inverse transform along x as
+// field 0 + i field 1: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B) for the
+// mixed half spectra A, B (kx = 0..K); the DC bin keeps real parts only; the
+// gap is zeroed.  Into the sequence's src buffer, synchronised.
 struct RowLoad {
-  int e;     // exponent of both rows as they stand in a
-  int2 pre;  // right shifts their inverse transforms start with
+  int e;    // exponent of the row as it stands in src
+  int pre;  // right shift its inverse transform starts with
 };
 template <int N, int V>
-__device__ __forceinline__ RowLoad load_row_pair(const Dev& d, int bm, int y0, q2* a, int* scratch) {
+__device__ __forceinline__ RowLoad load_row(const Dev& d, int bm, int y, const FxThread<N, V>& x) {
   using G = Geo<N, V>;
-  constexpr int T = G::THREADS, K = G::K, Kc = G::Kc, GAP = N - 2 * K - 1, J = (2 * Kc + T - 1) / T;
-  const q2* M = d.Mx + (size_t)bm * 2 * N * Kc;
+  using P = FxPlan<N, V>;
+  constexpr int K = G::K, Kc = G::Kc, GAP = N - 2 * K - 1, J = (Kc + P::TPS - 1) / P::TPS;
+  const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
+  const q2* MB = MA + (size_t)N * Kc;
   const int* eX = d.eX + (size_t)bm * 2 * Kc;
   q2 p[J], q[J];
   int ep[J], eq[J], key = kZeroExp;
 #pragma unroll
-  for (int t = 0; t < J; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < 2 * Kc) {
-      const int rr = u / Kc, kx = u - rr * Kc;
-      p[t] = M[(size_t)(y0 + rr) * Kc + kx];
-      q[t] = M[((size_t)N + y0 + rr) * Kc + kx];
-      ep[t] = eX[kx];
-      eq[t] = eX[Kc + kx];
+  for (int j = 0; j < J; ++j) {
+    const int kx = x.t + j * P::TPS;
+    if (kx < Kc) {
+      p[j] = MA[kx];
+      q[j] = MB[kx];
+      ep[j] = eX[kx];
+      eq[j] = eX[Kc + kx];
     }
   }
-  for (int u = threadIdx.x; u < 2 * GAP; u += T) {
-    const int rr = u / GAP;
-    a[rr * N + K + 1 + (u - rr * GAP)] = mkq(0, 0);
-  }
+  for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(K + 1 + u)] = mkq(0, 0);
 #pragma unroll
-  for (int t = 0; t < J; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < 2 * Kc) {
-      key = max(key, bits32(max(mag32(p[t].x), mag32(p[t].y))) + 32 + ep[t]);
-      key = max(key, bits32(max(mag32(q[t].x), mag32(q[t].y))) + 32 + eq[t]);
+  for (int j = 0; j < J; ++j) {
+    if (x.t + j * P::TPS < Kc) {
+      key = max(key, bits32(max(mag32(p[j].x), mag32(p[j].y))) + 32 + ep[j]);
+      key = max(key, bits32(max(mag32(q[j].x), mag32(q[j].y))) + 32 + eq[j]);
     }
   }
-  const int e = block_max2<T>(key, key, scratch).x - (kInvBits - 1);  // sums of two below kInvBits bits
-  unsigned s0 = 0, s1 = 0;
+  key = seq_max_put<P::TPS>(key, x.t, x.scratch);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  key = seq_max_get<P::TPS>(key, x.scratch);
+  const int e = key - (kInvBits - 1);  // sums of two below kInvBits bits
+  int sum = 0;
 #pragma unroll
-  for (int t = 0; t < J; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < 2 * Kc) {
-      const int rr = u / Kc, kx = u - rr * Kc;
-      const q2 A = Shift(ep[t] - e)(p[t]), B = Shift(eq[t] - e)(q[t]);
-      q2* seq = a + rr * N;
-      const unsigned units = 2 * (mag_units(A) + mag_units(B));  // of Z(kx) and Z(-kx)
-      if (rr == 0) s0 += units;
-      else s1 += units;
+  for (int j = 0; j < J; ++j) {
+    const int kx = x.t + j * P::TPS;
+    if (kx < Kc) {
+      const q2 A = Shift(ep[j] - e)(p[j]), B = Shift(eq[j] - e)(q[j]);
+      sum += 2 * (mag_units(A) + mag_units(B));  // of Z(kx) and Z(-kx)
       if (kx == 0) {
-        seq[0] = mkq(A.x, B.x);
+        x.src[0] = mkq(A.x, B.x);
       } else {
-        seq[kx] = mkq(A.x - B.y, A.y + B.x);
-        seq[N - kx] = mkq(A.x + B.y, B.x - A.y);
+        x.src[pad(kx)] = mkq(A.x - B.y, A.y + B.x);
+        x.src[pad(N - kx)] = mkq(A.x + B.y, B.x - A.y);
       }
     }
   }
-  block_sum2_put(s0, s1, scratch + 16);
-  __syncthreads();
-  const int2 sum = block_sum2_get<T>(scratch + 16);
-  return {e, make_int2(inv_shift<N, V>(sum.x), inv_shift<N, V>(sum.y))};
+  sum = seq_sum_put<P::TPS>(sum, x.t, x.scratch + P::WARPS);
+  seq_sync<P::TPS>(x.f);
+  return {e, inv_shift<P>(seq_sum_get<P::TPS>(sum, x.scratch + P::WARPS))};
 }
 
-// Forward transforms along x of rows y0, y0+1, sequence rr packed as
-// (field 0 of row y0+rr) + i (field 1 of row y0+rr) -> twice the two fields
-// of both rows (A = Z(k) + conj Z(-k), B = -i (Z(k) - conj Z(-k)); the column
-// pass's symbols carry the 1/2) in the column-major Mn of the member: entry
-// (kx, f, y) at (kx * 2 + f) * N + y, with the rows' exponents e0, e1.
+// Forward transforms along x of rows y0, y0+1, sequence f packed as (field 0
+// of row y0+f) + i (field 1 of row y0+f) -> twice the two fields of both rows
+// (A = Z(k) + conj Z(-k), B = -i (Z(k) - conj Z(-k)); the column pass's
+// symbols carry the 1/2) in the column-major Mn of the member: entry
+// (kx, f, y) at (kx * 2 + f) * N + y; e: this sequence's exponent.
 template <int N, int V>
-__device__ __forceinline__ void store_row_pair(const Dev& d, int bm, int y0, const q2* a, int e0, int e1) {
+__device__ __forceinline__ void store_row_pair(const Dev& d, int bm, int y0, const FxThread<N, V>& x, int e) {
   using G = Geo<N, V>;
+  using P = FxPlan<N, V>;
+  __syncthreads();  // both rows are in
+  const q2* a = x.f ? x.other(x.src) : x.src;
   q2* O = d.Mn + (size_t)bm * G::Kc * 2 * N;
 #pragma unroll
-  for (int t = 0; t < (2 * G::Kc + G::THREADS - 1) / G::THREADS; ++t) {
-    const int u = threadIdx.x + t * G::THREADS;
+  for (int j = 0; j < (2 * G::Kc + G::THREADS - 1) / G::THREADS; ++j) {
+    const int u = threadIdx.x + j * G::THREADS;
     if (u < 2 * G::Kc) {
       const int rr = u & 1, kx = u >> 1;
-      const q2 zk = a[rr * N + kx], zm = a[rr * N + ((N - kx) & (N - 1))];
+      const q2 zk = a[rr * 2 * P::SEQ + pad(kx)], zm = a[rr * 2 * P::SEQ + pad((N - kx) & (N - 1))];
       q2* o = O + (size_t)kx * 2 * N + y0 + rr;
       o[0] = mkq(zk.x + zm.x, zk.y - zm.y);
       o[N] = mkq(zk.y + zm.y, zm.x - zk.x);
     }
   }
-  if (threadIdx.x < 2) d.eN[bm * N + y0 + threadIdx.x] = clamp_exp(threadIdx.x ? e1 : e0);
+  if (x.t == 0) d.eN[bm * N + y0 + x.f] = clamp_exp(e);
 }
 
 // Bits that a row pass brings u, v and 2a, b to, so that the products, less
@@ -653,50 +692,49 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
-  const FxSmem<N> fs(sm);
-  const int bm = blockIdx.y, y0 = 2 * blockIdx.x;
+  FxThread<N, V> x(sm);
+  const int bm = blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;  // the member's window has not begun
-  const RowLoad in = load_row_pair<N, V>(d, bm, y0, fs.a, fs.scratch);
+  constexpr int R = LastRadix<typename P::inv>::value;
+  using B = Bfly<P, R>;
+  const RowLoad in = load_row<N, V>(d, bm, y, x);
   const int Pp = mw.P, st = N / Pp;
   const int slot = (flags & (F_OBS | F_OBS_ONLY)) ? obs_slot(d, n - mw.start) : -1;
-  const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y0;
-  const bool store = (flags & F_STORE) != 0;
-  int ex[2];  // exponents of u, v of the two rows, once normalised
-  int sh[2];
-  auto prep = [&](int m0, int m1) {
+  q2 z[B::POINTS];
+  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, in.pre, z);
+  // u, v to UV bits
+  int m = 0;
+  if (B::active(x.t)) {
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int m = r ? m1 : m0;
-      sh[r] = m == 0 ? 0 : RowBits<N, V>::UV - 32 - bits32(m);
-      ex[r] = clamp_exp(in.e + (r ? in.pre.y : in.pre.x) + P::SHIFT_INV - sh[r]);
-    }
-    if (store && threadIdx.x < 2) d.eT[trow + threadIdx.x] = threadIdx.x ? ex[1] : ex[0];
-  };
-  // (u, v) at column x of row y0 + rr: stage-field store, probe gather, and
-  // the products P = u v, Q = v^2 - u^2 as P + i Q
-  auto products = [&](int rr, int x, q2 uv) {
-    const int y = y0 + rr;
-    uv = Shift(rr ? sh[1] : sh[0])(uv);
-    if (store) d.traj[(trow + rr) * N + x] = uv;
-    if (slot >= 0 && (y % st) == 0 && (x % st) == 0) {
-      const int p = (y / st) * Pp + x / st;
-      double* o = d.obs + bm * d.obs_stride + ((size_t)slot * Pp * Pp + p) * 2;
-      o[0] = fx_to_double(uv.x, rr ? ex[1] : ex[0]);
-      o[1] = fx_to_double(uv.y, rr ? ex[1] : ex[0]);
-    }
-    return mkq(mul_hi(uv.x, uv.y), mul_hi(uv.y - uv.x, uv.y + uv.x));
-  };
-  if (flags & F_OBS_ONLY) {  // the final state: probes only
-    fx_inverse<N, V, G::K>(fs.a, d.fxtw, in.pre);
-    sh[0] = sh[1] = 0;
-    ex[0] = clamp_exp(in.e + in.pre.x + P::SHIFT_INV);
-    ex[1] = clamp_exp(in.e + in.pre.y + P::SHIFT_INV);
-    for (int u = threadIdx.x; u < 2 * N; u += G::THREADS) products(u / N, u & (N - 1), fs.a[u]);
-    return;
+    for (int j = 0; j < B::POINTS; ++j) m = max(m, max(mag32(z[j].x), mag32(z[j].y)));
   }
-  const int2 r = fx_turn<N, V, G::K, RowBits<N, V>::MEASURE>(fs.a, d.fxtw, in.pre, fs.scratch + 32, prep, products);
-  store_row_pair<N, V>(d, bm, y0, fs.a, 2 * ex[0] + 64 + P::SHIFT + r.x, 2 * ex[1] + 64 + P::SHIFT + r.y);
+  m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
+  const int sh = m == 0 ? 0 : RowBits<N, V>::UV - 32 - bits32(m);
+  const int ex = clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
+  const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y;
+  const bool store = (flags & F_STORE) != 0;
+  if (store && x.t == 0) d.eT[trow] = ex;
+  const bool probes = slot >= 0 && (y % st) == 0;
+  if (B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < B::POINTS; ++j) {
+      const int xx = x.t + (j / R) * P::TPS + (j % R) * B::NB;
+      const i64 u = z[j].x << sh, v = z[j].y << sh;
+      if (store) d.traj[trow * N + xx] = mkq(u, v);
+      if (probes && (xx % st) == 0) {
+        double* o = d.obs + bm * d.obs_stride + ((size_t)slot * Pp * Pp + (y / st) * Pp + xx / st) * 2;
+        o[0] = fx_to_double(u, ex);
+        o[1] = fx_to_double(v, ex);
+      }
+      z[j] = mkq(mul_hi(u, v), mul_hi(v - u, v + u));
+    }
+  }
+  if (flags & F_OBS_ONLY) return;  // the final state: probes only
+  const int r = fx_forward<P, G::K, RowBits<N, V>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+  store_row_pair<N, V>(d, bm, y0, x, 2 * ex + 64 + P::SHIFT + r);
 }
 
 // ---------------------------------------------------------------------------
@@ -712,8 +750,7 @@ template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, int stage, int flags) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
-  const FxSmem<N> fs(sm);
-  q2* a = fs.a;
+  FxThread<N, V> x(sm);
   const int kx = blockIdx.x, bm = blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
@@ -735,19 +772,17 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
       nk2[t] = mw.nu * d.k2[kx * G::Kr + rr];
     }
   };
-  const int2 e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, a, d.fxtw, fs.scratch,
-                                       [&] {
-                                         if constexpr (G::PREFETCH) {
+  const int2 e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
+    if constexpr (G::PREFETCH) {
 #pragma unroll
-                                           for (int t = 0; t < MT; ++t) load_inputs(t);
-                                         }
-                                       });
+      for (int t = 0; t < MT; ++t) load_inputs(t);
+    }
+  });
+  const q2 *a0 = x.f ? x.other(x.src) : x.src, *a1 = a0 + 2 * FxPlan<N, V>::SEQ;
   const FxScale s0(e.x), s1(e.y);
   const double dt = d.dt;
   const double fval = -d.amp * d.nf * (double)N * N / 2.0;
-  ColumnPut<N> put(a);
-  // each retained position is read and rewritten (both sequences) by one
-  // thread only
+  ColumnPut<N, V> put;
 #pragma unroll
   for (int t = 0; t < MT; ++t) {
     const int rr = threadIdx.x + t * G::THREADS;
@@ -756,7 +791,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
     const int ky = ky_of_row(rr, G::K);
     const int qi = ky & (N - 1);
     const size_t idx = cidx<N>(bm, rr, kx);
-    const q2 pq = a[qi], qq = a[N + qi];
+    const q2 pq = a0[pad(qi)], qq = a1[pad(qi)];
     const double2 ph = make_double2(s0(pq.x), s0(pq.y)), qh = make_double2(s1(qq.x), s1(qq.y));
     const double cp = f[t].c * s0.s, cq = f[t].d * s1.s;
     // F = -(cp P + cq Q) - nu k^2 y
@@ -779,10 +814,11 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
       d.W[idx] = ynext;
     }
     d.Y[idx] = ynext;
-    put_stage_columns<N>(put, qi, f[t], ynext);
+    put_stage_columns<N, V>(put, t, f[t], ynext);
   }
   if (flags & F_NO_NEXT) return;
-  finish_columns<N, V>(d, put, bm, kx, fs.scratch + 16);
+  swap_bufs(x.src, x.dst);
+  finish_columns<N, V>(d, put, x, bm, kx);
 }
 
 // r = model observations - data and J = 1/2 sum r^2 per member, in a fixed
@@ -864,8 +900,8 @@ template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
-  const FxSmem<N> fs(sm);
-  double2 *Tu = fs.Tu, *Tv = fs.Tv;
+  const FxThread<N, V> x(sm);
+  double2 *Tu = x.Tu, *Tv = x.Tv;
   const int kx = blockIdx.x, bm = blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   // an idle member starts (and stays) at lambda = 0
@@ -874,9 +910,11 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode
   const int slot = (!resume && (mode & INIT_SRC)) ? obs_slot(d, d.nsteps - mw.start) : -1;
   if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, Tu, Tv);
   __syncthreads();
-  ColumnPut<N> put(fs.a);
-  #pragma unroll
-  for (int rr = threadIdx.x; rr < G::Kr; rr += G::THREADS) {
+  ColumnPut<N, V> put;
+#pragma unroll
+  for (int j = 0; j < put.MT; ++j) {
+    const int rr = threadIdx.x + j * G::THREADS;
+    if (rr >= G::Kr) break;
     const int ky = ky_of_row(rr, G::K);
     const size_t idx = cidx<N>(bm, rr, kx);
     double2 kb;
@@ -889,9 +927,9 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode
       kb = cscale(lam, d.dt6);
       d.KB[idx] = kb;
     }
-    put_adjoint_columns<N>(put, ky & (N - 1), d.symA[kx * G::Kr + rr], kb);
+    put_adjoint_columns<N, V>(put, j, d.symA[kx * G::Kr + rr], kb);
   }
-  finish_columns<N, V>(d, put, bm, kx, fs.scratch);
+  finish_columns<N, V>(d, put, x, bm, kx);
 }
 
 // Adjoint row pass of stage `stage` of step n: 2a, b of rows y0, y0+1
@@ -903,32 +941,42 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
   using P = FxPlan<N, V>;
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
-  const FxSmem<N> fs(sm);
-  const int bm = blockIdx.y, y0 = 2 * blockIdx.x;
+  FxThread<N, V> x(sm);
+  const int bm = blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
   if (d.ragged && n < d.mstart[bm]) return;
-  const RowLoad in = load_row_pair<N, V>(d, bm, y0, fs.a, fs.scratch);
-  const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y0;
-  int sh[2], ex[2];
-  auto prep = [&](int m0, int m1) {
+  constexpr int R = LastRadix<typename P::inv>::value;
+  using B = Bfly<P, R>;
+  const RowLoad in = load_row<N, V>(d, bm, y, x);
+  const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y;
+  q2 z[B::POINTS];
+  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, in.pre, z);
+  // 2a, b to AB bits
+  int m = 0;
+  q2 uv[B::POINTS];
+  if (B::active(x.t)) {
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int m = r ? m1 : m0;
-      sh[r] = m == 0 ? 0 : RowBits<N, V>::AB - 32 - bits32(m);
-      ex[r] = clamp_exp(in.e + (r ? in.pre.y : in.pre.x) + P::SHIFT_INV - sh[r]);
+    for (int j = 0; j < B::POINTS; ++j) uv[j] = d.traj[trow * N + x.t + (j / R) * P::TPS + (j % R) * B::NB];
+#pragma unroll
+    for (int j = 0; j < B::POINTS; ++j) m = max(m, max(mag32(z[j].x), mag32(z[j].y)));
+  }
+  m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
+  const int sh = m == 0 ? 0 : RowBits<N, V>::AB - 32 - bits32(m);
+  const int ex = clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
+  // rho_u = v b - u 2a, rho_v = u b + v 2a with the stored u, v
+  if (B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < B::POINTS; ++j) {
+      const i64 aa = z[j].x << sh, bb = z[j].y << sh;
+      const int uh = hi_word(uv[j].x), ul = lo_word(uv[j].x), vh = hi_word(uv[j].y), vl = lo_word(uv[j].y);
+      const int ah = hi_word(aa), al = lo_word(aa), bh = hi_word(bb), bl = lo_word(bb);
+      z[j] = mkq(mul_hi2<-1>(vh, vl, bh, bl, uh, ul, ah, al), mul_hi2<+1>(uh, ul, bh, bl, vh, vl, ah, al));
     }
-  };
-  // (2a, b) at column x of row y0 + rr -> rho_u + i rho_v with the stored
-  // u, v: rho_u = v b - u 2a, rho_v = u b + v 2a
-  auto rho = [&](int rr, int x, q2 ab) {
-    const q2 uv = d.traj[(trow + rr) * N + x];
-    ab = Shift(rr ? sh[1] : sh[0])(ab);
-    const int uh = hi_word(uv.x), ul = lo_word(uv.x), vh = hi_word(uv.y), vl = lo_word(uv.y);
-    const int ah = hi_word(ab.x), al = lo_word(ab.x), bh = hi_word(ab.y), bl = lo_word(ab.y);
-    return mkq(mul_hi2<-1>(vh, vl, bh, bl, uh, ul, ah, al), mul_hi2<+1>(uh, ul, bh, bl, vh, vl, ah, al));
-  };
-  const int2 r = fx_turn<N, V, G::K, RowBits<N, V>::MEASURE>(fs.a, d.fxtw, in.pre, fs.scratch + 32, prep, rho);
-  store_row_pair<N, V>(d, bm, y0, fs.a, clamp_exp(ex[0] + d.eT[trow]) + 64 + P::SHIFT + r.x,
-                       clamp_exp(ex[1] + d.eT[trow + 1]) + 64 + P::SHIFT + r.y);
+  }
+  const int eT = d.eT[trow];
+  const int r = fx_forward<P, G::K, RowBits<N, V>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+  store_row_pair<N, V>(d, bm, y0, x, clamp_exp(ex + eT) + 64 + P::SHIFT + r);
 }
 
 // Adjoint column pass of stage `stage` of step n:
@@ -940,9 +988,8 @@ template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, int stage, int flags) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
-  const FxSmem<N> fs(sm);
-  q2* a = fs.a;
-  double2 *Tu = fs.Tu, *Tv = fs.Tv;
+  FxThread<N, V> x(sm);
+  double2 *Tu = x.Tu, *Tv = x.Tv;
   const int kx = blockIdx.x, bm = blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
@@ -964,19 +1011,17 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
     }
   };
   const int slot = (flags & F_SRC) ? obs_slot(d, n - mw.start) : -1;
-  const int2 e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, a, d.fxtw, fs.scratch,
-                                       [&] {
-                                         if constexpr (G::PREFETCH) {
+  const int2 e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
+    if constexpr (G::PREFETCH) {
 #pragma unroll
-                                           for (int t = 0; t < MT; ++t) load_inputs(t);
-                                         }
-                                         if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, Tu, Tv);
-                                       });
+      for (int t = 0; t < MT; ++t) load_inputs(t);
+    }
+    if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, Tu, Tv);
+  });
+  const q2 *a0 = x.f ? x.other(x.src) : x.src, *a1 = a0 + 2 * FxPlan<N, V>::SEQ;
   const FxScale s0(e.x), s1(e.y);
   const double dt = d.dt;
-  ColumnPut<N> put(a);
-  // each retained position is read and rewritten (both sequences) by one
-  // thread only
+  ColumnPut<N, V> put;
 #pragma unroll
   for (int t = 0; t < MT; ++t) {
     const int rr = threadIdx.x + t * G::THREADS;
@@ -985,7 +1030,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
     const int ky = ky_of_row(rr, G::K);
     const int qi = ky & (N - 1);
     const size_t idx = cidx<N>(bm, rr, kx);
-    const q2 qu = a[qi], qv = a[N + qi];
+    const q2 qu = a0[pad(qi)], qv = a1[pad(qi)];
     const double2 Ru = make_double2(s0(qu.x), s0(qu.y)), Rv = make_double2(s1(qv.x), s1(qv.y));
     const double a1 = g[t].a * s0.s, c1 = g[t].b * s1.s;
     // t = (-i ky/k^2) Ru + (i kx/k^2) Rv (the 1/2 of the row unpack in a1, c1)
@@ -1012,10 +1057,11 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
       nk = cscale(lam, d.dt6);
     }
     d.KB[idx] = nk;
-    put_adjoint_columns<N>(put, qi, g[t], nk);
+    put_adjoint_columns<N, V>(put, t, g[t], nk);
   }
   if (stage == 1 && n == mw.start) return;  // the member's first step: lambda_0 stays in LamBar
-  finish_columns<N, V>(d, put, bm, kx, fs.scratch + 16);
+  swap_bufs(x.src, x.dst);
+  finish_columns<N, V>(d, put, x, bm, kx);
 }
 
 // Control multipliers m(k) = |k| W(k)^{1/2} on the retained set (0 at k = 0),

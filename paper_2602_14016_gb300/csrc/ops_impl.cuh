@@ -19,16 +19,16 @@ Ops make_ops() {
   o.flops_forward = band_transform_flops<N, V, G::K>(false);
   o.fold_table = [](double* out) { fold_table<N, V>(out); };
   o.fx_entries = FxPlan<N, V>::TABLE;
-  o.fx_table = [](int4* out) { fx_table<N, V>(out); };
+  o.fx_table = [](int4* out) { fx_table<FxPlan<N, V>>(out); };
   o.setup = []() -> cudaError_t {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* f, size_t s = G::SMEM_FX) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s);
     };
-    set((const void*)k_r2c_rows<N, V>, G::SMEM);
-    set((const void*)k_c2r_rows<N, V>, G::SMEM);
-    set((const void*)k_spec_to_mixed<N, V>, G::SMEM);
-    set((const void*)k_ctrl_cols<N, V>, G::SMEM);
+    set((const void*)k_r2c_rows<N, V>, G::SMEM_FOLD);
+    set((const void*)k_c2r_rows<N, V>, G::SMEM_FOLD);
+    set((const void*)k_spec_to_mixed<N, V>, G::SMEM_FOLD);
+    set((const void*)k_ctrl_cols<N, V>, G::SMEM_CTRL);
     set((const void*)k_fwd_rows<N, V>);
     set((const void*)k_fwd_cols<N, V>);
     set((const void*)k_state_cols<N, V>);
@@ -38,13 +38,13 @@ Ops make_ops() {
     return e;
   };
   o.r2c_rows = [](const Dev& d, const double* in, cudaStream_t st) {
-    k_r2c_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM, st>>>(d, in);
+    k_r2c_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FOLD, st>>>(d, in);
   };
   o.c2r_rows = [](const Dev& d, double* out, cudaStream_t st) {
-    k_c2r_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM, st>>>(d, out);
+    k_c2r_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FOLD, st>>>(d, out);
   };
   o.spec_to_mixed = [](const Dev& d, const double2* src, int mode, cudaStream_t st) {
-    k_spec_to_mixed<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d, src, mode);
+    k_spec_to_mixed<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FOLD, st>>>(d, src, mode);
   };
   o.compact_to_half = [](const Dev& d, const double2* src, double2* out, cudaStream_t st) {
     k_compact_to_half<N, V><<<dim3((N * G::NH + 255) / 256, d.B), 256, 0, st>>>(src, out);
@@ -53,7 +53,7 @@ Ops make_ops() {
     k_half_to_compact<N, V><<<dim3((G::Kr * G::Kc + 255) / 256, d.B), 256, 0, st>>>(in, dst);
   };
   o.ctrl_cols = [](const Dev& d, int flags, cudaStream_t st) {
-    k_ctrl_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM, st>>>(d, flags);
+    k_ctrl_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_CTRL, st>>>(d, flags);
   };
   o.fwd_rows = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
     k_fwd_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
