@@ -117,8 +117,12 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   A(dalloc(c, (double**)&d.fold, fold_max));
   A(dalloc(c, (int4**)&d.fxtw, fx_max));
   A(dalloc(c, (double2**)&d.twP, (size_t)64));
-  A(dalloc(c, (da::Sym4**)&d.symF, comp / B));
-  A(dalloc(c, (da::Sym4**)&d.symA, comp / B));
+  A(dalloc(c, (da::Sym2**)&d.symF, comp / B));
+  A(dalloc(c, (da::Sym2**)&d.symA, comp / B));
+  A(dalloc(c, (da::FxPair**)&d.fxF, comp / B));
+  A(dalloc(c, (da::FxPair**)&d.fxA, comp / B));
+  A(dalloc(c, (int**)&d.fxFe, comp / B));
+  A(dalloc(c, (int**)&d.fxAe, comp / B));
   A(dalloc(c, (double**)&d.k2, comp / B));
   A(dalloc(c, &c->d_mstart, B));
   A(dalloc(c, &c->d_mnt, B));
@@ -174,8 +178,11 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   if (e == cudaSuccess) e = cudaMemcpy((void*)d.twP, twP.data(), 64 * sizeof(double2), cudaMemcpyHostToDevice);
   // per-mode symbols of the column passes, column-major [Kc][Kr]
   const int K = ops->K, Kr = ops->Kr, Kc = ops->Kc;
-  std::vector<da::Sym4> symF((size_t)Kr * Kc), symA((size_t)Kr * Kc);
-  std::vector<double> k2tab((size_t)Kr * Kc);
+  const size_t modes = (size_t)Kr * Kc;
+  std::vector<da::Sym2> symF(modes), symA(modes);
+  std::vector<da::FxPair> fxF(modes), fxA(modes);
+  std::vector<int> fxFe(modes), fxAe(modes);
+  std::vector<double> k2tab(modes);
   const double s2 = 1.0 / ((double)n * n);
   for (int kx = 0; kx < Kc; ++kx)
     for (int r = 0; r < Kr; ++r) {
@@ -183,12 +190,21 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
       const double k2 = (double)(kx * kx + ky * ky);
       const double ik2 = k2 > 0.0 ? 1.0 / k2 : 0.0;
       const size_t i = (size_t)kx * Kr + r;
-      symF[i] = {ky * ik2 * s2, kx * ik2 * s2, 0.5 * (ky * ky - kx * kx), -0.5 * kx * ky};
-      symA[i] = {0.5 * ky * ik2, 0.5 * kx * ik2, -2.0 * kx * ky * s2, (double)(ky * ky - kx * kx) * s2};
+      symF[i] = {ky * ik2 * s2, kx * ik2 * s2};
+      symA[i] = {-2.0 * kx * ky * s2, (double)(ky * ky - kx * kx) * s2};
+      fxF[i] = da::fx_pair(0.5 * (ky * ky - kx * kx), -0.5 * kx * ky, &fxFe[i]);
+      fxA[i] = da::fx_pair(0.5 * ky * ik2, 0.5 * kx * ik2, &fxAe[i]);
       k2tab[i] = k2;
     }
-  if (e == cudaSuccess) e = cudaMemcpy((void*)d.symF, symF.data(), symF.size() * sizeof(da::Sym4), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy((void*)d.symA, symA.data(), symA.size() * sizeof(da::Sym4), cudaMemcpyHostToDevice);
+  auto upload = [&](const void* dst, const void* src, size_t bytes) {
+    if (e == cudaSuccess) e = cudaMemcpy((void*)dst, src, bytes, cudaMemcpyHostToDevice);
+  };
+  upload(d.symF, symF.data(), modes * sizeof(da::Sym2));
+  upload(d.symA, symA.data(), modes * sizeof(da::Sym2));
+  upload(d.fxF, fxF.data(), modes * sizeof(da::FxPair));
+  upload(d.fxA, fxA.data(), modes * sizeof(da::FxPair));
+  upload(d.fxFe, fxFe.data(), modes * sizeof(int));
+  upload(d.fxAe, fxAe.data(), modes * sizeof(int));
   if (e == cudaSuccess) e = cudaMemcpy((void*)d.k2, k2tab.data(), k2tab.size() * sizeof(double), cudaMemcpyHostToDevice);
   {
     const std::vector<int> zeros(B, 0), nts(B, c->nt), pxs(B, c->P), forces(B, d.force);

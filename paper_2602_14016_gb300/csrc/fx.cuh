@@ -69,7 +69,9 @@ __device__ __forceinline__ q2 qsub_z(q2 x, q2 y) {
 }
 
 // d = hi 2^32 + lo with a signed low word (-2^31 <= lo < 2^31), so that both
-// words enter signed multiply-adds.
+// words enter signed multiply-adds.  Data are negated before they are split,
+// never by words: a low word of -2^31 has no negative.  The words of a
+// coefficient may be negated (fx_words leaves that one out).
 __device__ __forceinline__ int lo_word(i64 d) { return (int)d; }
 __device__ __forceinline__ int hi_word(i64 d) { return (int)(d >> 32) + (int)((unsigned)d >> 31); }
 
@@ -92,12 +94,18 @@ __device__ __forceinline__ i64 mul_hi(i64 a, i64 b) {
   return madw(ah, bh, (i64)(int)(mid >> 32));
 }
 
-// (a b +- c d) / 2^64, |.| <= 2^62 each.
-template <int SG>
-__device__ __forceinline__ i64 mul_hi2(int ah, int al, int bh, int bl, int ch, int cl, int dh, int dl) {
-  const int sh = SG > 0 ? dh : -dh, sl = SG > 0 ? dl : -dl;
-  const i64 mid = madw(ch, sl, madw(cl, sh, madw(ah, bl, madw(al, bh, kHalfWord))));
-  return madw(ch, sh, madw(ah, bh, (i64)(int)(mid >> 32)));
+// A 64-bit factor in words.
+struct Words {
+  int h, l;
+  __device__ __forceinline__ explicit Words(i64 d) : h(hi_word(d)), l(lo_word(d)) {}
+  __device__ __forceinline__ Words(int h_, int l_) : h(h_), l(l_) {}
+};
+
+// (a b + c d) / 2^64: |.| < 2^62 each, the sum of either pair's magnitudes
+// below 2^62.5.
+__device__ __forceinline__ i64 mul_hi2(Words a, Words b, Words c, Words d) {
+  const i64 mid = madw(c.h, d.l, madw(c.l, d.h, madw(a.h, b.l, madw(a.l, b.h, kHalfWord))));
+  return madw(c.h, d.h, madw(a.h, b.h, (i64)(int)(mid >> 32)));
 }
 
 // Twiddle: (cos, sin) as 62-bit integers, each split in signed words.
@@ -274,13 +282,25 @@ struct FxPlanOf {
   static constexpr int GROWTH1 = log2c(R1);                                          // first stage
   static constexpr int GROWTH2 = Growth<R1, typename TailRadices<fwd>::type>::most(0);  // the others
   static constexpr int BITS_FWD = 62 - GROWTH;
-  // q2 of one buffer of a sequence: a stage reads one and writes the other
-  static constexpr int SEQ = N + N / 8;
+  static constexpr int SEQ = N + N / 8;  // q2 of one buffer of a sequence
+  // Threads of several warps read one buffer and write another (one barrier a
+  // stage); a warp alone works in place, since its barriers cost nothing and
+  // half the shared memory lets more of its kind run.
+  static constexpr bool PING = TPS > 32;
+  static constexpr int BUFS = PING ? 2 : 1;
   static constexpr int WARPS = (TPS + 31) / 32;
 };
 
 template <int N, int V = 0>
 using FxPlan = FxPlanOf<N, PlanInfo<N, V>::THREADS / 2, typename Plan<N, V>::two>;
+
+// Signed words (hi, lo) of a coefficient; a low word of -2^31, which could
+// not be negated, is moved by one unit (2^-62).
+inline int2 fx_words(i64 v) {
+  if ((unsigned)v == 0x80000000u) ++v;
+  const int lo = (int)(unsigned)v;
+  return make_int2((int)((v - lo) >> 32), lo);
+}
 
 template <int L>
 inline void fx_fill(int4*, Radices<>) {}
@@ -296,9 +316,8 @@ inline void fx_fill(int4* out, Radices<R, Rs...>) {
       for (int k = 0; k < L; ++k) {
         const long double th = -2.0L * pi * (long double)(m * k) / (long double)(L * R);
         const i64 c = llroundl(s * cosl(th)), n = llroundl(s * sinl(th));
-        auto lo = [](i64 v) { return (int)(unsigned)(v & 0xffffffffLL); };
-        auto hi = [&](i64 v) { return (int)((v - (i64)lo(v)) >> 32); };
-        out[(m - 1) * L + k] = make_int4(hi(c), lo(c), hi(n), lo(n));
+        const int2 cw = fx_words(c), nw = fx_words(n);
+        out[(m - 1) * L + k] = make_int4(cw.x, cw.y, nw.x, nw.y);
       }
     out += (R - 1) * L;
   }
@@ -438,6 +457,27 @@ __device__ __forceinline__ double fx_to_double(i64 v, int e) {
   return r;
 }
 
+// Two real coefficients of a mode, a and b, as integers of one exponent: the
+// larger of |a|, |b| has 62 bits; words (a_hi, a_lo, b_hi, b_lo).
+struct __align__(16) FxPair {
+  int ah, al, bh, bl;
+};
+inline FxPair fx_pair(double a, double b, int* e) {
+  const double big = std::fmax(std::fabs(a), std::fabs(b));
+  *e = 0;
+  if (big == 0.0) return {0, 0, 0, 0};
+  std::frexp(big, e);
+  *e -= 62;
+  const i64 x = (i64)std::ldexp(a, -*e), y = (i64)std::ldexp(b, -*e);  // the smaller may lose what lies below a unit
+  const int2 a2 = fx_words(x), b2 = fx_words(y);
+  return {a2.x, a2.y, b2.x, b2.y};
+}
+// (a p + SG b q) / 2^64, |p|, |q| < 2^61.5.
+template <int SG>
+__device__ __forceinline__ i64 fx_pair_sum(const FxPair& c, i64 p, i64 q) {
+  return mul_hi2(Words(p), Words(c.ah, c.al), Words(q), SG > 0 ? Words(c.bh, c.bl) : Words(-c.bh, -c.bl));
+}
+
 // Biased exponent field of a double (0: zero or subnormal, 2047: not finite).
 __device__ __forceinline__ int exp_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
 
@@ -516,10 +556,19 @@ __device__ __forceinline__ void fx_store(const q2* a, q2* dst, int i) {
   for (int m = 0; m < R; ++m) d[pad(m * L)] = a[m];
 }
 
+// src and dst are the same buffer where P works in place.
+template <typename P>
 __device__ __forceinline__ void swap_bufs(q2*& a, q2*& b) {
-  q2* c = a;
-  a = b;
-  b = c;
+  if constexpr (P::PING) {
+    q2* c = a;
+    a = b;
+    b = c;
+  }
+}
+// Between a stage's loads and its stores in place.
+template <typename P>
+__device__ __forceinline__ void in_place_sync(int id) {
+  if constexpr (!P::PING) seq_sync<P::TPS>(id);
 }
 
 // Middle stages with sub-lengths from L on: src -> dst, sync, swap.  SHR: the
@@ -529,24 +578,31 @@ __device__ __forceinline__ void fx_middle(q2*&, q2*&, const int4*, int, int, int
 template <typename P, int S, int L, bool SHR, int R, int... Rs>
 __device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int t, int id, int r, Radices<R, Rs...>) {
   using B = Bfly<P, R>;
+  q2 a[B::POINTS];
   if (B::active(t)) {
 #pragma unroll
     for (int jb = 0; jb < B::J; ++jb) {
       const int i = t + jb * P::TPS;
-      q2 a[R];
-      fx_load<P, R>(a, src, i);
+      fx_load<P, R>(a + jb * R, src, i);
       if constexpr (SHR) {
         if (r > 0) {
 #pragma unroll
-          for (int m = 0; m < R; ++m) a[m] = mkq(shr_round(a[m].x, r), shr_round(a[m].y, r));
+          for (int m = 0; m < R; ++m) a[jb * R + m] = mkq(shr_round(a[jb * R + m].x, r), shr_round(a[jb * R + m].y, r));
         }
       }
-      fx_butterfly<R, S, L, 0>(a, T, i & (L - 1));
-      fx_store<P, R, L>(a, dst, i);
+      fx_butterfly<R, S, L, 0>(a + jb * R, T, i & (L - 1));
+      if constexpr (P::PING) fx_store<P, R, L>(a + jb * R, dst, i);
+    }
+  }
+  if constexpr (!P::PING) {
+    seq_sync<P::TPS>(id);
+    if (B::active(t)) {
+#pragma unroll
+      for (int jb = 0; jb < B::J; ++jb) fx_store<P, R, L>(a + jb * R, dst, t + jb * P::TPS);
     }
   }
   seq_sync<P::TPS>(id);
-  swap_bufs(src, dst);
+  swap_bufs<P>(src, dst);
   fx_middle<P, S, L * R, false>(src, dst, T + (R - 1) * L, t, id, r, Radices<Rs...>{});
 }
 
@@ -554,7 +610,8 @@ __device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int
 // KB: the inputs, of at most kInvBits bits, are shifted right by pre first,
 // and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
 // is left in registers: out[jb R + m] is position t + jb TPS + m N / R for R
-// the last radix.  dst is free afterwards, src not before the next sync.
+// the last radix.  dst is free afterwards if it is another buffer than src;
+// src is not before the next sync.
 template <typename P, int KB>
 __device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, int t, int id, int pre, q2* out) {
   using I = typename P::inv;
@@ -563,22 +620,26 @@ __device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, i
   using B1 = Bfly<P, R1>;
   using BL = Bfly<P, RL>;
   const int4* T = tw + P::ENTRIES;
+  q2 a[B1::POINTS];
   if (B1::active(t)) {
     const i64 half = (1LL << pre) >> 1;
 #pragma unroll
     for (int jb = 0; jb < B1::J; ++jb) {
-      const int i = t + jb * P::TPS;
-      q2 a[R1];
-      fx_load<P, R1, Z>(a, src, i);
+      q2* b = a + jb * R1;
+      fx_load<P, R1, Z>(b, src, t + jb * P::TPS);
 #pragma unroll
       for (int m = 0; m < R1; ++m)
-        if (!((Z >> m) & 1)) a[m] = mkq((a[m].x + half) >> pre, (a[m].y + half) >> pre);
-      qdftR<R1, +1, Z>(a);
-      fx_store<P, R1, 1>(a, dst, i);
+        if (!((Z >> m) & 1)) b[m] = mkq((b[m].x + half) >> pre, (b[m].y + half) >> pre);
+      qdftR<R1, +1, Z>(b);
     }
   }
+  in_place_sync<P>(id);
+  if (B1::active(t)) {
+#pragma unroll
+    for (int jb = 0; jb < B1::J; ++jb) fx_store<P, R1, 1>(a + jb * R1, dst, t + jb * P::TPS);
+  }
   seq_sync<P::TPS>(id);
-  swap_bufs(src, dst);
+  swap_bufs<P>(src, dst);
   using Mid = typename InitRadices<typename TailRadices<I>::type>::type;
   fx_middle<P, +1, R1, false>(src, dst, T, t, id, 0, Mid{});
   constexpr int L = P::N / RL;
@@ -608,6 +669,7 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
   using B1 = Bfly<P, R1>;
   using BL = Bfly<P, RL>;
   int big = 0, r = 0;
+  in_place_sync<P>(id);  // the registers were loaded from this buffer
   if (B1::active(t)) {
 #pragma unroll
     for (int jb = 0; jb < B1::J; ++jb) {
@@ -622,33 +684,40 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
   }
   if constexpr (MEASURE) big = seq_max_put<P::TPS>(big, t, scratch);
   seq_sync<P::TPS>(id);
-  swap_bufs(src, dst);
+  swap_bufs<P>(src, dst);
   if constexpr (MEASURE) r = max(0, bits32(seq_max_get<P::TPS>(big, scratch)) - (62 - SPARE - P::GROWTH2 - 32));
   using Mid = typename InitRadices<Tail>::type;
   constexpr bool MIDDLE = L > R1;  // there are middle stages
   fx_middle<P, -1, R1, MEASURE && MIDDLE>(src, dst, tw, t, id, r, Mid{});
+  q2 a[BL::POINTS];
   if (BL::active(t)) {
     const int4* Tl = tw + P::ENTRIES - (RL - 1) * L;
 #pragma unroll
     for (int jb = 0; jb < BL::J; ++jb) {
       const int i = t + jb * P::TPS;
-      q2 a[RL];
-      fx_load<P, RL>(a, src, i);
+      q2* b = a + jb * RL;
+      fx_load<P, RL>(b, src, i);
       if constexpr (MEASURE && !MIDDLE) {
         if (r > 0) {
 #pragma unroll
-          for (int m = 0; m < RL; ++m) a[m] = mkq(shr_round(a[m].x, r), shr_round(a[m].y, r));
+          for (int m = 0; m < RL; ++m) b[m] = mkq(shr_round(b[m].x, r), shr_round(b[m].y, r));
         }
       }
-      fx_butterfly<RL, -1, L, 0>(a, Tl, i);
-      q2* d = dst + pad(i);
+      fx_butterfly<RL, -1, L, 0>(b, Tl, i);
+    }
+  }
+  in_place_sync<P>(id);
+  if (BL::active(t)) {
+#pragma unroll
+    for (int jb = 0; jb < BL::J; ++jb) {
+      q2* d = dst + pad(t + jb * P::TPS);
 #pragma unroll
       for (int m = 0; m < RL; ++m)
-        if (!((C >> m) & 1)) d[pad(m * L)] = a[m];
+        if (!((C >> m) & 1)) d[pad(m * L)] = a[jb * RL + m];
     }
   }
   seq_sync<P::TPS>(id);
-  swap_bufs(src, dst);
+  swap_bufs<P>(src, dst);
   return r;
 }
 

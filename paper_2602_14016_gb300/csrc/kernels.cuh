@@ -70,15 +70,18 @@ enum : int { M_ONE = 0, M_CTRL = 1, M_FILTERED = 2, M_INV_CTRL = 3 };
 // Per-mode constants of the column passes, column-major [Kc][Kr] (entry
 // kx * Kr + r), computed once on the host so that no column pass divides or
 // converts integers in FP64:
-//   fwd: su = ky/k^2/N^2, sv = kx/k^2/N^2 (u, v columns of a state value),
-//        cp = (ky^2 - kx^2)/2, cq = -kx ky/2 (advection symbols; the 1/2 is
-//        the one the row pass leaves out when it unpacks two real rows);
-//   adj: a1 = ky/k^2/2, c1 = kx/k^2/2 (transposed velocity symbols, same
-//        1/2), ca = -2 kx ky/N^2, cb = (ky^2 - kx^2)/N^2 (adjoint-field
-//        columns; ca carries the 2 of rho_u, rho_v);
+//   fwd: symF = su = ky/k^2/N^2, sv = kx/k^2/N^2 (u, v columns of a state
+//        value); fxF = cp = (ky^2 - kx^2)/2, cq = -kx ky/2 (advection symbols;
+//        the 1/2 is the one the row pass leaves out when it unpacks two real
+//        rows);
+//   adj: symA = ca = -2 kx ky/N^2, cb = (ky^2 - kx^2)/N^2 (adjoint-field
+//        columns; ca carries the 2 of rho_u, rho_v); fxA = a1 = ky/k^2/2, c1 =
+//        kx/k^2/2 (transposed velocity symbols, same 1/2);
 //   k2 = k^2 (the column passes multiply it by the member's viscosity).
-struct __align__(32) Sym4 {
-  double a, b, c, d;
+// fxF and fxA multiply integer transforms before the conversion to doubles:
+// one conversion per component instead of two, and no FP64 products.
+struct __align__(16) Sym2 {
+  double a, b;
 };
 
 // Everything a kernel needs, passed by value.
@@ -117,8 +120,12 @@ struct Dev {
   const double* fold;                        // folded twiddles of Plan<N> (fft.cuh)
   const int4* fxtw;                          // integer twiddles of FxPlan<N> (fx.cuh)
   const double2* twP;                        // W_64^t, t < 64 (W_P^t = W_64^{t 64/P})
-  const Sym4* symF;                          // [Kc][Kr] su, sv, cp, cq
-  const Sym4* symA;                          // [Kc][Kr] a1, c1, ca, cb
+  const Sym2* symF;                          // [Kc][Kr] su, sv
+  const Sym2* symA;                          // [Kc][Kr] ca, cb
+  const FxPair* fxF;                         // [Kc][Kr] cp, cq
+  const FxPair* fxA;                         // [Kc][Kr] a1, c1
+  const int* fxFe;                           // [Kc][Kr] exponents of fxF
+  const int* fxAe;                           // [Kc][Kr] exponents of fxA
   const double* k2;                          // [Kc][Kr] k^2 (times nu of the member)
   double dt2, dt3, dt6;                      // dt/2, dt/3, dt/6
 };
@@ -135,12 +142,12 @@ struct Geo {
   // shared memory of the control maps: folded twiddle table + one sequence
   static constexpr size_t SMEM = sizeof(double2) * 2 * N;  // static_ctrl.cu: plain table and one sequence
   static constexpr size_t SMEM_FOLD = sizeof(double) * FoldInfo<N, V>::PADDED + sizeof(double2) * (N + 2);
-  // passes that run the integer transforms: two buffers of each of two
-  // sequences, probe sums, scratch of the reductions (three of WARPS ints for
-  // each sequence, two of a pair per warp for the CTA)
-  static constexpr int SCRATCH = (3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS;
-  static constexpr size_t SMEM_FX =
-      sizeof(q2) * (4 * FxPlan<N, V>::SEQ) + sizeof(double2) * 2 * PMAX + sizeof(int) * ((SCRATCH + 3) / 4 * 4);
+  // passes that run the integer transforms: the buffers of two sequences,
+  // scratch of the reductions (three of WARPS ints for each sequence, two of a
+  // pair per warp for the CTA), and probe sums (adjoint column passes)
+  static constexpr int SCRATCH = ((3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS + 3) / 4 * 4;
+  static constexpr size_t SMEM_FX = sizeof(q2) * (2 * FxPlan<N, V>::BUFS * FxPlan<N, V>::SEQ) + sizeof(int) * SCRATCH;
+  static constexpr size_t SMEM_FXP = SMEM_FX + sizeof(double2) * 2 * PMAX;
   // k_ctrl_cols runs both: the FP64 part first, in the same memory
   static constexpr size_t SMEM_CTRL = SMEM_FOLD > SMEM_FX ? SMEM_FOLD : SMEM_FX;
   // column passes load their epilogue inputs before the transforms (about
@@ -347,19 +354,21 @@ struct FxThread {
   int t, f;
   q2 *src, *dst;
   int* scratch;  // three reductions of WARPS ints
-  double2 *Tu, *Tv;
+  double2 *Tu, *Tv;  // adjoint column passes only
   __device__ __forceinline__ explicit FxThread(void* base) {
     f = threadIdx.x / P::TPS;
     t = threadIdx.x - f * P::TPS;
     q2* a = static_cast<q2*>(base);
-    src = a + f * 2 * P::SEQ;
-    dst = src + P::SEQ;
-    Tu = reinterpret_cast<double2*>(a + 4 * P::SEQ);
+    src = a + f * OTHER;
+    dst = P::PING ? src + P::SEQ : src;
+    int* s = reinterpret_cast<int*>(a + 2 * OTHER);
+    scratch = s + f * 3 * P::WARPS;
+    Tu = reinterpret_cast<double2*>(s + Geo<N, V>::SCRATCH);
     Tv = Tu + Geo<N, V>::PMAX;
-    scratch = reinterpret_cast<int*>(Tv + Geo<N, V>::PMAX) + f * 3 * P::WARPS;
   }
-  // the other sequence's buffer at the same place as p (of this sequence)
-  __device__ __forceinline__ q2* other(q2* p) const { return f ? p - 2 * P::SEQ : p + 2 * P::SEQ; }
+  // sequence 1's buffers lie this far behind sequence 0's
+  static constexpr int OTHER = P::BUFS * P::SEQ;
+  __device__ __forceinline__ q2* first(q2* p) const { return f ? p - OTHER : p; }
 };
 
 // A column under construction: the doubles a thread puts at its retained rows
@@ -381,7 +390,7 @@ struct ColumnPut {
 // The two column values u = i ky/k^2 Yv, v = -i kx/k^2 Yv (scaled by 1/N^2;
 // f = symF entry of the mode) as entry j.
 template <int N, int V>
-__device__ __forceinline__ void put_stage_columns(ColumnPut<N, V>& c, int j, const Sym4& f, double2 Yv) {
+__device__ __forceinline__ void put_stage_columns(ColumnPut<N, V>& c, int j, const Sym2& f, double2 Yv) {
   c.put(j, make_double2(-f.a * Yv.y, f.a * Yv.x),  // u:  i ky / k^2
         make_double2(f.b * Yv.y, -f.b * Yv.x));    // v: -i kx / k^2
 }
@@ -390,8 +399,8 @@ __device__ __forceinline__ void put_stage_columns(ColumnPut<N, V>& c, int j, con
 // 2a = 2 d_xy kb = -2 kx ky kb and b = (d_xx - d_yy) kb = (ky^2 - kx^2) kb,
 // scaled by 1/N^2 (g = symA entry of the mode).
 template <int N, int V>
-__device__ __forceinline__ void put_adjoint_columns(ColumnPut<N, V>& c, int j, const Sym4& g, double2 kb) {
-  c.put(j, cscale(kb, g.c), cscale(kb, g.d));
+__device__ __forceinline__ void put_adjoint_columns(ColumnPut<N, V>& c, int j, const Sym2& g, double2 kb) {
+  c.put(j, cscale(kb, g.a), cscale(kb, g.b));
 }
 
 // Two reductions over the whole CTA at once, (a, b) -> (A, B): `scratch` has
@@ -425,9 +434,8 @@ __device__ __forceinline__ int2 cta_reduce2(int a, int b, int* scratch) {
   return make_int2(a, b);
 }
 
-// Both columns put in c: to integers in x's src buffers, inverse transform
-// along y, into column kx of both fields of Mx.  buf0: sequence 0's buffer to
-// start from, free to write (sequence 1's lies 2 SEQ further).
+// Both columns put in c: to integers in x's src buffers (free to write after
+// a barrier), inverse transform along y, into column kx of both fields of Mx.
 template <int N, int V>
 __device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, V>& c, FxThread<N, V> x, int bm, int kx) {
   using G = Geo<N, V>;
@@ -436,7 +444,7 @@ __device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, 
   int* scratch = x.scratch + (2 - x.f) * 3 * P::WARPS;  // after the two sequences' own
   const int2 f = cta_reduce2<T, false>(c.f0, c.f1, scratch);
   const int e0 = exp_for<kInvBits>(f.x), e1 = exp_for<kInvBits>(f.y);
-  q2 *a0 = x.f ? x.other(x.src) : x.src, *a1 = a0 + 2 * P::SEQ;
+  q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
   unsigned s0 = 0, s1 = 0;
 #pragma unroll
   for (int j = 0; j < ColumnPut<N, V>::MT; ++j) {
@@ -469,17 +477,18 @@ __device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, 
 
 // Column kx of both fields of the column-major Mn (M points at the column,
 // eN at the member's row exponents), forward transform along y, left in the
-// src buffers, synchronised over the CTA.  `between` runs after the loads are
-// issued.  Returns the exponents of the two results.
+// src buffers with one exponent for both, which is returned, and one bit to
+// spare; synchronised over the CTA.  `between` runs after the loads are
+// issued.
 template <int N, int V, typename Between>
-__device__ __forceinline__ int2 forward_columns(const q2* __restrict__ M, const int* __restrict__ eN,
-                                                FxThread<N, V>& x, const int4* tw, Between between) {
+__device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const int* __restrict__ eN,
+                                               FxThread<N, V>& x, const int4* tw, Between between) {
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
   constexpr int R = FirstRadix<typename P::fwd>::value;
   // the first stage only must leave room where that gives two bits more
-  constexpr bool MEASURE = P::GROWTH >= P::GROWTH1 + 2;
-  constexpr int BITS = MEASURE ? 62 - P::GROWTH1 : P::BITS_FWD;
+  constexpr bool MEASURE = P::GROWTH >= P::GROWTH1 + 1;
+  constexpr int BITS = MEASURE ? 62 - P::GROWTH1 : P::BITS_FWD - 1;
   using B = Bfly<P, R>;
   q2 v[B::POINTS];
   int e[B::POINTS], key = kZeroExp;
@@ -496,34 +505,30 @@ __device__ __forceinline__ int2 forward_columns(const q2* __restrict__ M, const 
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) key = max(key, bits32(max(mag32(v[j].x), mag32(v[j].y))) + 32 + e[j]);
   }
-  key = seq_max_put<P::TPS>(key, x.t, x.scratch);
-  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
-  key = seq_max_get<P::TPS>(key, x.scratch);
+  int* cta = x.scratch + (2 - x.f) * 3 * P::WARPS;  // after the two sequences' own
+  key = cta_reduce2<G::THREADS, false>(key, key, cta).x;
   const int e0 = key - BITS;
   if (B::active(x.t)) {
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) v[j] = Shift(e[j] - e0)(v[j]);
   }
-  const int r = fx_forward<P, G::K, MEASURE, 0>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
-  // both sequences' results and exponents, to the whole CTA
-  const int out = clamp_exp(e0 + r + P::SHIFT);
-  if (x.t == 0) x.scratch[0] = out;
+  const int r = fx_forward<P, G::K, MEASURE, 1>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
+  // results of two shifts: bring both to the larger one
+  if (x.t == 0) x.scratch[0] = r;
   __syncthreads();
   const int* s0 = x.scratch - x.f * 3 * P::WARPS;
-  return make_int2(s0[0], s0[3 * P::WARPS]);
-}
-
-// Integers of one exponent to doubles, with the power of two folded into the
-// caller's coefficients where it is an ordinary double: value = s (*this)(v).
-struct FxScale {
-  int e;
-  bool plain;
-  double s;
-  __device__ __forceinline__ explicit FxScale(int e_) : e(e_), plain(e_ >= -960 && e_ <= 960) {
-    s = plain ? pow2_double(e) : 1.0;
+  const int r0 = s0[0], r1 = s0[3 * P::WARPS], rm = max(r0, r1);
+  if constexpr (MEASURE) {
+    if (r < rm) {
+      for (int q = x.t; q < N; q += P::TPS) {
+        const q2 z = x.src[pad(q)];
+        x.src[pad(q)] = mkq(shr_round(z.x, rm - r), shr_round(z.y, rm - r));
+      }
+    }
+    if (r0 != r1) __syncthreads();
   }
-  __device__ __forceinline__ double operator()(i64 v) const { return plain ? (double)v : fx_to_double(v, e); }
-};
+  return clamp_exp(e0 + rm + P::SHIFT);
+}
 
 // s_hat = forward transform along y of the mixed rows in Mn (doubles here,
 // from k_r2c_rows); w0 = mult s_hat into W (and Y); then, unless F_NO_NEXT,
@@ -652,14 +657,14 @@ __device__ __forceinline__ void store_row_pair(const Dev& d, int bm, int y0, con
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
   __syncthreads();  // both rows are in
-  const q2* a = x.f ? x.other(x.src) : x.src;
+  const q2* a = x.first(x.src);
   q2* O = d.Mn + (size_t)bm * G::Kc * 2 * N;
 #pragma unroll
   for (int j = 0; j < (2 * G::Kc + G::THREADS - 1) / G::THREADS; ++j) {
     const int u = threadIdx.x + j * G::THREADS;
     if (u < 2 * G::Kc) {
       const int rr = u & 1, kx = u >> 1;
-      const q2 zk = a[rr * 2 * P::SEQ + pad(kx)], zm = a[rr * 2 * P::SEQ + pad((N - kx) & (N - 1))];
+      const q2 zk = a[rr * x.OTHER + pad(kx)], zm = a[rr * x.OTHER + pad((N - kx) & (N - 1))];
       q2* o = O + (size_t)kx * 2 * N + y0 + rr;
       o[0] = mkq(zk.x + zm.x, zk.y - zm.y);
       o[N] = mkq(zk.y + zm.y, zm.x - zk.x);
@@ -759,7 +764,9 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
   // column transforms
   constexpr int MT = (G::Kr + G::THREADS - 1) / G::THREADS;
   double2 yv[MT], wv[MT], accv[MT];
-  Sym4 f[MT];
+  Sym2 f[MT];
+  FxPair cf[MT];
+  int ce[MT];
   double nk2[MT];
   auto load_inputs = [&](int t) {
     const int rr = threadIdx.x + t * G::THREADS;
@@ -769,17 +776,18 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
       wv[t] = d.W[idx];
       accv[t] = stage > 1 ? d.Acc[idx] : make_double2(0.0, 0.0);
       f[t] = d.symF[kx * G::Kr + rr];
+      cf[t] = d.fxF[kx * G::Kr + rr];
+      ce[t] = d.fxFe[kx * G::Kr + rr];
       nk2[t] = mw.nu * d.k2[kx * G::Kr + rr];
     }
   };
-  const int2 e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
+  const int e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
     if constexpr (G::PREFETCH) {
 #pragma unroll
       for (int t = 0; t < MT; ++t) load_inputs(t);
     }
   });
-  const q2 *a0 = x.f ? x.other(x.src) : x.src, *a1 = a0 + 2 * FxPlan<N, V>::SEQ;
-  const FxScale s0(e.x), s1(e.y);
+  const q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
   const double dt = d.dt;
   const double fval = -d.amp * d.nf * (double)N * N / 2.0;
   ColumnPut<N, V> put;
@@ -792,11 +800,11 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
     const int qi = ky & (N - 1);
     const size_t idx = cidx<N>(bm, rr, kx);
     const q2 pq = a0[pad(qi)], qq = a1[pad(qi)];
-    const double2 ph = make_double2(s0(pq.x), s0(pq.y)), qh = make_double2(s1(qq.x), s1(qq.y));
-    const double cp = f[t].c * s0.s, cq = f[t].d * s1.s;
     // F = -(cp P + cq Q) - nu k^2 y
-    double2 F = make_double2(-fma(cp, ph.x, fma(cq, qh.x, nk2[t] * yv[t].x)),
-                             -fma(cp, ph.y, fma(cq, qh.y, nk2[t] * yv[t].y)));
+    const int eF = e + 64 + ce[t];
+    const double ax = fx_to_double(fx_pair_sum<1>(cf[t], pq.x, qq.x), eF);
+    const double ay = fx_to_double(fx_pair_sum<1>(cf[t], pq.y, qq.y), eF);
+    double2 F = make_double2(-fma(nk2[t], yv[t].x, ax), -fma(nk2[t], yv[t].y, ay));
     if (mw.forced && kx == 0 && (ky == d.nf || ky == -d.nf)) F.x += fval;
     const double2 w = wv[t], acc = accv[t];
     double2 ynext;
@@ -817,7 +825,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, i
     put_stage_columns<N, V>(put, t, f[t], ynext);
   }
   if (flags & F_NO_NEXT) return;
-  swap_bufs(x.src, x.dst);
+  swap_bufs<FxPlan<N, V>>(x.src, x.dst);
   finish_columns<N, V>(d, put, x, bm, kx);
 }
 
@@ -969,9 +977,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) {
       const i64 aa = z[j].x << sh, bb = z[j].y << sh;
-      const int uh = hi_word(uv[j].x), ul = lo_word(uv[j].x), vh = hi_word(uv[j].y), vl = lo_word(uv[j].y);
-      const int ah = hi_word(aa), al = lo_word(aa), bh = hi_word(bb), bl = lo_word(bb);
-      z[j] = mkq(mul_hi2<-1>(vh, vl, bh, bl, uh, ul, ah, al), mul_hi2<+1>(uh, ul, bh, bl, vh, vl, ah, al));
+      const Words u(uv[j].x), v(uv[j].y), a(aa), b(bb), na(-aa);
+      z[j] = mkq(mul_hi2(v, b, u, na), mul_hi2(u, b, v, a));
     }
   }
   const int eT = d.eT[trow];
@@ -997,7 +1004,9 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
   // transforms where registers allow, as in k_fwd_cols)
   constexpr int MT = (G::Kr + G::THREADS - 1) / G::THREADS;
   double2 kbv[MT], lbv[MT], sumv[MT];
-  Sym4 g[MT];
+  Sym2 g[MT];
+  FxPair cf[MT];
+  int ce[MT];
   double nk2[MT];
   auto load_inputs = [&](int t) {
     const int rr = threadIdx.x + t * G::THREADS;
@@ -1007,19 +1016,20 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
       lbv[t] = d.LamBar[idx];
       sumv[t] = stage < 4 ? d.Sum[idx] : make_double2(0.0, 0.0);
       g[t] = d.symA[kx * G::Kr + rr];
+      cf[t] = d.fxA[kx * G::Kr + rr];
+      ce[t] = d.fxAe[kx * G::Kr + rr];
       nk2[t] = mw.nu * d.k2[kx * G::Kr + rr];
     }
   };
   const int slot = (flags & F_SRC) ? obs_slot(d, n - mw.start) : -1;
-  const int2 e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
+  const int e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
     if constexpr (G::PREFETCH) {
 #pragma unroll
       for (int t = 0; t < MT; ++t) load_inputs(t);
     }
     if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, Tu, Tv);
   });
-  const q2 *a0 = x.f ? x.other(x.src) : x.src, *a1 = a0 + 2 * FxPlan<N, V>::SEQ;
-  const FxScale s0(e.x), s1(e.y);
+  const q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
   const double dt = d.dt;
   ColumnPut<N, V> put;
 #pragma unroll
@@ -1031,10 +1041,10 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
     const int qi = ky & (N - 1);
     const size_t idx = cidx<N>(bm, rr, kx);
     const q2 qu = a0[pad(qi)], qv = a1[pad(qi)];
-    const double2 Ru = make_double2(s0(qu.x), s0(qu.y)), Rv = make_double2(s1(qv.x), s1(qv.y));
-    const double a1 = g[t].a * s0.s, c1 = g[t].b * s1.s;
     // t = (-i ky/k^2) Ru + (i kx/k^2) Rv (the 1/2 of the row unpack in a1, c1)
-    const double2 tt = make_double2(fma(a1, Ru.y, -c1 * Rv.y), fma(-a1, Ru.x, c1 * Rv.x));
+    const int eR = e + 64 + ce[t];
+    const double2 tt = make_double2(fx_to_double(fx_pair_sum<-1>(cf[t], qu.y, qv.y), eR),
+                                    -fx_to_double(fx_pair_sum<-1>(cf[t], qu.x, qv.x), eR));
     const double2 kb = kbv[t], lb = lbv[t];
     double2 yb;
     yb.x = -fma(nk2[t], kb.x, tt.x);
@@ -1060,7 +1070,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, i
     put_adjoint_columns<N, V>(put, t, g[t], nk);
   }
   if (stage == 1 && n == mw.start) return;  // the member's first step: lambda_0 stays in LamBar
-  swap_bufs(x.src, x.dst);
+  swap_bufs<FxPlan<N, V>>(x.src, x.dst);
   finish_columns<N, V>(d, put, x, bm, kx);
 }
 

@@ -32,9 +32,9 @@ Ops make_ops() {
     set((const void*)k_fwd_rows<N, V>);
     set((const void*)k_fwd_cols<N, V>);
     set((const void*)k_state_cols<N, V>);
-    set((const void*)k_adj_init<N, V>);
+    set((const void*)k_adj_init<N, V>, G::SMEM_FXP);
     set((const void*)k_adj_rows<N, V>);
-    set((const void*)k_adj_cols<N, V>);
+    set((const void*)k_adj_cols<N, V>, G::SMEM_FXP);
     return e;
   };
   o.r2c_rows = [](const Dev& d, const double* in, cudaStream_t st) {
@@ -65,13 +65,13 @@ Ops make_ops() {
     k_state_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d);
   };
   o.adj_init = [](const Dev& d, int mode, cudaStream_t st) {
-    k_adj_init<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, mode);
+    k_adj_init<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, mode);
   };
   o.adj_rows = [](const Dev& d, int n, int stage, cudaStream_t st) {
     k_adj_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
   };
   o.adj_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_adj_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
+    k_adj_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage, flags);
   };
   o.make_mult = [](const Dev& d, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                    cudaStream_t st) {
