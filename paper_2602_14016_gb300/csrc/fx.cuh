@@ -340,25 +340,29 @@ constexpr int kZeroExp = -100000, kBadExp = 100000;
 
 __device__ __forceinline__ int clamp_exp(int e) { return e < kZeroExp / 2 ? kZeroExp : e > kBadExp / 2 ? kBadExp : e; }
 
-// Magnitude bits of an integer's high word: |v| < 2^(32 + bits).
-__device__ __forceinline__ int mag32(i64 v) {
-  const int h = (int)(v >> 32);
-  return h ^ (h >> 31);
-}
+// Magnitude of an integer's high word: |v| < 2^32 (mag32(v) + 1).
+__device__ __forceinline__ int mag32(i64 v) { return abs((int)(v >> 32)); }
+__device__ __forceinline__ int max_mag(int m, q2 v) { return max(m, max(mag32(v.x), mag32(v.y))); }
 __device__ __forceinline__ int bits32(int m) { return 32 - __clz(m); }
+// Bits of a value whose high word has magnitude at most m: |v| < 2^bits64(m).
+__device__ __forceinline__ int bits64(int m) { return 32 + bits32(m + 1); }
+
+// v / 2^r, rounded, r >= 0 (62 where r is larger).
+struct ShiftRight {
+  int r;
+  i64 half;
+  __device__ __forceinline__ explicit ShiftRight(int r_) : r(min(r_, 62)) { half = (1LL << r) >> 1; }
+  __device__ __forceinline__ i64 operator()(i64 v) const { return (v + half) >> r; }
+  __device__ __forceinline__ q2 operator()(q2 v) const { return mkq((*this)(v.x), (*this)(v.y)); }
+};
 
 // v 2^s: left for s >= 0 (the caller knows that it fits), right with
 // rounding for s < 0.
 struct Shift {
-  int l, r;
-  i64 half;
-  __device__ __forceinline__ explicit Shift(int s) {
-    l = max(s, 0);
-    r = min(max(-s, 0), 62);
-    l = min(l, 62);
-    half = (1LL << r) >> 1;
-  }
-  __device__ __forceinline__ i64 operator()(i64 v) const { return ((v << l) + half) >> r; }
+  int l;
+  ShiftRight right;
+  __device__ __forceinline__ explicit Shift(int s) : l(min(max(s, 0), 62)), right(max(-s, 0)) {}
+  __device__ __forceinline__ i64 operator()(i64 v) const { return right(v << l); }
   __device__ __forceinline__ q2 operator()(q2 v) const { return mkq((*this)(v.x), (*this)(v.y)); }
 };
 
@@ -414,28 +418,31 @@ __device__ __forceinline__ int seq_sum_get(int v, const int* scratch) {
   return v;
 }
 
-// Inputs of an inverse transform are first brought to kInvBits bits, then,
-// as the first stage reads them, shifted right (rounded) until the sum of
-// their magnitudes has 62 bits.  The sum is counted in units of
-// 2^(32 + kSumDrop): mag32 >> kSumDrop, at most 4 x 683 terms of 2^18 each,
-// one unit more a term for the part dropped.
+// Inputs of an inverse transform have at most kInvBits bits; as the first
+// stage reads them, they are shifted (right with rounding, or left) until the
+// sum of their magnitudes has 62 bits, or up to G more (below).  The sum is
+// counted in units of 2^(32 + kSumDrop), one unit more for each group of up to
+// four magnitudes, whose low part is dropped.
 //
 // The second stage scales by 2^-G before it adds, so the sum may have 62 + G
 // bits where the first stage's own sums, at most R sqrt2 times the largest
-// component (61 bits), stay below 2^62.5: from a shift of log2 R - 1 on.
-constexpr int kInvBits = 61, kSumDrop = 12;
+// component, stay below 2^62.5: while the components have 62 - log2 R bits.
 // Nor may it have more than 60 + SHIFT_INV bits: the results then have 60,
 // and the row passes only ever shift them left (RowBits).
+constexpr int kInvBits = 61, kSumDrop = 12;
 template <typename P>
 __device__ __forceinline__ int inv_shift(int sum) {
   using I = typename P::inv;
-  constexpr int first = log2c(FirstRadix<I>::value) - 1;
+  constexpr int first = kInvBits - (62 - log2c(FirstRadix<I>::value));
   constexpr int G0 = stage_shift(FirstRadix<typename TailRadices<I>::type>::value);
   constexpr int G = G0 < P::SHIFT_INV - 2 ? G0 : P::SHIFT_INV - 2;
   const int r = bits32(sum) + 32 + kSumDrop - 62;
-  return max(0, min(r, max(r - G, first)));
+  return min(r, max(r - G, first));
 }
-__device__ __forceinline__ unsigned mag_units(q2 v) { return (unsigned)(((mag32(v.x) + mag32(v.y)) >> kSumDrop) + 1); }
+__device__ __forceinline__ int mag_units(q2 a, q2 b) {
+  const unsigned m = (unsigned)mag32(a.x) + (unsigned)mag32(a.y) + (unsigned)mag32(b.x) + (unsigned)mag32(b.y);
+  return (int)(m >> kSumDrop) + 1;
+}
 
 // v 2^e as a double (one rounding).
 __device__ __forceinline__ double pow2_double(int e) {  // 2^e, -1022 <= e <= 1023
@@ -607,7 +614,8 @@ __device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int
 }
 
 // Inverse transform (S = +1) of the sequence in src, zero outside the band
-// KB: the inputs, of at most kInvBits bits, are shifted right by pre first,
+// KB: the inputs, of at most kInvBits bits, are shifted right by pre (left by
+// -pre) first,
 // and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
 // is left in registers: out[jb R + m] is position t + jb TPS + m N / R for R
 // the last radix.  dst is free afterwards if it is another buffer than src;
@@ -622,14 +630,20 @@ __device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, i
   const int4* T = tw + P::ENTRIES;
   q2 a[B1::POINTS];
   if (B1::active(t)) {
-    const i64 half = (1LL << pre) >> 1;
+    const ShiftRight right(max(pre, 0));
 #pragma unroll
     for (int jb = 0; jb < B1::J; ++jb) {
       q2* b = a + jb * R1;
       fx_load<P, R1, Z>(b, src, t + jb * P::TPS);
+      if (pre > 0) {
 #pragma unroll
-      for (int m = 0; m < R1; ++m)
-        if (!((Z >> m) & 1)) b[m] = mkq((b[m].x + half) >> pre, (b[m].y + half) >> pre);
+        for (int m = 0; m < R1; ++m)
+          if (!((Z >> m) & 1)) b[m] = right(b[m]);
+      } else if (pre < 0) {
+#pragma unroll
+        for (int m = 0; m < R1; ++m)
+          if (!((Z >> m) & 1)) b[m] = mkq(b[m].x << -pre, b[m].y << -pre);
+      }
       qdftR<R1, +1, Z>(b);
     }
   }
@@ -677,7 +691,7 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
       qdftR<R1, -1, 0>(a);
       if constexpr (MEASURE) {
 #pragma unroll
-        for (int m = 0; m < R1; ++m) big = max(big, max(mag32(a[m].x), mag32(a[m].y)));
+        for (int m = 0; m < R1; ++m) big = max_mag(big, a[m]);
       }
       fx_store<P, R1, 1>(a, dst, t + jb * P::TPS);
     }
@@ -685,7 +699,7 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
   if constexpr (MEASURE) big = seq_max_put<P::TPS>(big, t, scratch);
   seq_sync<P::TPS>(id);
   swap_bufs<P>(src, dst);
-  if constexpr (MEASURE) r = max(0, bits32(seq_max_get<P::TPS>(big, scratch)) - (62 - SPARE - P::GROWTH2 - 32));
+  if constexpr (MEASURE) r = max(0, bits64(seq_max_get<P::TPS>(big, scratch)) - (62 - SPARE - P::GROWTH2));
   using Mid = typename InitRadices<Tail>::type;
   constexpr bool MIDDLE = L > R1;  // there are middle stages
   fx_middle<P, -1, R1, MEASURE && MIDDLE>(src, dst, tw, t, id, r, Mid{});

@@ -150,9 +150,13 @@ struct Geo {
   static constexpr size_t SMEM_FXP = SMEM_FX + sizeof(double2) * 2 * PMAX;
   // k_ctrl_cols runs both: the FP64 part first, in the same memory
   static constexpr size_t SMEM_CTRL = SMEM_FOLD > SMEM_FX ? SMEM_FOLD : SMEM_FX;
-  // column passes load their epilogue inputs before the transforms (about
-  // 60 more registers a thread) where a CTA is at most 128 threads
-  static constexpr bool PREFETCH = THREADS <= 128;
+  // Column passes: small grids leave most of the chip idle, so a warp's own
+  // latency counts, and they load their epilogue inputs before the transforms
+  // (about 60 more registers a thread); larger ones hide it behind other
+  // warps, at 768 threads an SM or more (256^2, batch 16: 28.9 us a column
+  // pass with the loads up front at 153 registers, 20.6 us without at 80).
+  static constexpr bool PREFETCH = N <= 128;
+  static constexpr int COL_CTAS = PREFETCH ? 1 : 768 / THREADS;
 };
 
 __device__ __forceinline__ int ky_of_row(int r, int K) { return r <= K ? r : r - (2 * K + 1); }
@@ -453,8 +457,8 @@ __device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, 
     const int q = pad(ky_of_row(rr, G::K) & (N - 1));
     const q2 u = mkq(double_to_fx(c.v0[j].x, e0), double_to_fx(c.v0[j].y, e0));
     const q2 v = mkq(double_to_fx(c.v1[j].x, e1), double_to_fx(c.v1[j].y, e1));
-    s0 += mag_units(u);
-    s1 += mag_units(v);
+    s0 += mag_units(u, mkq(0, 0));
+    s1 += mag_units(v, mkq(0, 0));
     a0[q] = u;
     a1[q] = v;
   }
@@ -491,7 +495,7 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
   constexpr int BITS = MEASURE ? 62 - P::GROWTH1 : P::BITS_FWD - 1;
   using B = Bfly<P, R>;
   q2 v[B::POINTS];
-  int e[B::POINTS], key = kZeroExp;
+  int e[B::POINTS], e0 = 2 * kZeroExp, big = 0;
   if (B::active(x.t)) {
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) {
@@ -501,16 +505,34 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
     }
   }
   between();
+  // to the largest row exponent (the same for both sequences), then left
+  // until the largest component of either has BITS bits
   if (B::active(x.t)) {
 #pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) key = max(key, bits32(max(mag32(v[j].x), mag32(v[j].y))) + 32 + e[j]);
+    for (int j = 0; j < B::POINTS; ++j) e0 = max(e0, e[j]);
+  }
+  e0 = seq_max_put<P::TPS>(e0, x.t, x.scratch);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  e0 = seq_max_get<P::TPS>(e0, x.scratch);
+  if (B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < B::POINTS; ++j) {
+      v[j] = ShiftRight(e0 - e[j])(v[j]);
+      big = max_mag(big, v[j]);
+    }
   }
   int* cta = x.scratch + (2 - x.f) * 3 * P::WARPS;  // after the two sequences' own
-  key = cta_reduce2<G::THREADS, false>(key, key, cta).x;
-  const int e0 = key - BITS;
+  big = cta_reduce2<G::THREADS, false>(big, big, cta).x;
+  const int sh = BITS - bits64(big);
+  e0 -= sh;
   if (B::active(x.t)) {
+    if (sh >= 0) {
 #pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) v[j] = Shift(e[j] - e0)(v[j]);
+      for (int j = 0; j < B::POINTS; ++j) v[j] = mkq(v[j].x << sh, v[j].y << sh);
+    } else {
+#pragma unroll
+      for (int j = 0; j < B::POINTS; ++j) v[j] = ShiftRight(-sh)(v[j]);
+    }
   }
   const int r = fx_forward<P, G::K, MEASURE, 1>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
   // results of two shifts: bring both to the larger one
@@ -593,7 +615,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_state_cols(Dev d) {
 // gap is zeroed.  Into the sequence's src buffer, synchronised.
 struct RowLoad {
   int e;    // exponent of the row as it stands in src
-  int pre;  // right shift its inverse transform starts with
+  int pre;  // shift its inverse transform starts with
 };
 template <int N, int V>
 __device__ __forceinline__ RowLoad load_row(const Dev& d, int bm, int y, const FxThread<N, V>& x) {
@@ -604,7 +626,7 @@ __device__ __forceinline__ RowLoad load_row(const Dev& d, int bm, int y, const F
   const q2* MB = MA + (size_t)N * Kc;
   const int* eX = d.eX + (size_t)bm * 2 * Kc;
   q2 p[J], q[J];
-  int ep[J], eq[J], key = kZeroExp;
+  int ep[J], eq[J], e = 2 * kZeroExp;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     const int kx = x.t + j * P::TPS;
@@ -616,24 +638,26 @@ __device__ __forceinline__ RowLoad load_row(const Dev& d, int bm, int y, const F
     }
   }
   for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(K + 1 + u)] = mkq(0, 0);
+  // one exponent for the row, at which its largest component has kInvBits - 1
+  // bits (sums of two have one more): the columns' own exponents would leave
+  // the small ones to be rounded at the unit of the largest
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     if (x.t + j * P::TPS < Kc) {
-      key = max(key, bits32(max(mag32(p[j].x), mag32(p[j].y))) + 32 + ep[j]);
-      key = max(key, bits32(max(mag32(q[j].x), mag32(q[j].y))) + 32 + eq[j]);
+      e = max(e, bits64(max_mag(0, p[j])) + ep[j]);
+      e = max(e, bits64(max_mag(0, q[j])) + eq[j]);
     }
   }
-  key = seq_max_put<P::TPS>(key, x.t, x.scratch);
+  e = seq_max_put<P::TPS>(e, x.t, x.scratch);
   if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
-  key = seq_max_get<P::TPS>(key, x.scratch);
-  const int e = key - (kInvBits - 1);  // sums of two below kInvBits bits
+  e = seq_max_get<P::TPS>(e, x.scratch) - (kInvBits - 1);
   int sum = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     const int kx = x.t + j * P::TPS;
     if (kx < Kc) {
       const q2 A = Shift(ep[j] - e)(p[j]), B = Shift(eq[j] - e)(q[j]);
-      sum += 2 * (mag_units(A) + mag_units(B));  // of Z(kx) and Z(-kx)
+      sum += 2 * mag_units(A, B);  // of Z(kx) and Z(-kx)
       if (kx == 0) {
         x.src[0] = mkq(A.x, B.x);
       } else {
@@ -684,7 +708,7 @@ struct RowBits {
   static constexpr int UV0 = (64 + F) / 2;  // u v and v^2 - u^2: 2 UV - 64 <= F
   static constexpr int AB0 = 63 + F - UV0;  // sums of two products: UV + AB - 63 <= F
   static constexpr int UV1 = 61, AB1 = P::GROWTH1 <= 3 ? 61 : 60;
-  static constexpr bool MEASURE = UV1 + AB1 >= UV0 + AB0 + 2;
+  static constexpr bool MEASURE = UV1 + AB1 >= UV0 + AB0 + (N >= 1024 ? 1 : 2);
   static constexpr int UV = MEASURE ? UV1 : UV0, AB = MEASURE ? AB1 : AB0;
 };
 
@@ -712,12 +736,12 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
   int m = 0;
   if (B::active(x.t)) {
 #pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) m = max(m, max(mag32(z[j].x), mag32(z[j].y)));
+    for (int j = 0; j < B::POINTS; ++j) m = max_mag(m, z[j]);
   }
   m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
   if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
   m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
-  const int sh = m == 0 ? 0 : RowBits<N, V>::UV - 32 - bits32(m);
+  const int sh = max(0, RowBits<N, V>::UV - bits64(m));  // at most 60 bits: never right
   const int ex = clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
   const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y;
   const bool store = (flags & F_STORE) != 0;
@@ -752,7 +776,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
 // transforms of u and v of the next stage state.  Acc holds k1 + 2 k2 +
 // 2 k3 (+ k4).  grid (Kc, B).
 template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_cols(Dev d, int n, int stage, int flags) {
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd_cols(Dev d, int n, int stage, int flags) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
   FxThread<N, V> x(sm);
@@ -965,12 +989,12 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) uv[j] = d.traj[trow * N + x.t + (j / R) * P::TPS + (j % R) * B::NB];
 #pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) m = max(m, max(mag32(z[j].x), mag32(z[j].y)));
+    for (int j = 0; j < B::POINTS; ++j) m = max_mag(m, z[j]);
   }
   m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
   if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
   m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
-  const int sh = m == 0 ? 0 : RowBits<N, V>::AB - 32 - bits32(m);
+  const int sh = max(0, RowBits<N, V>::AB - bits64(m));
   const int ex = clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
   // rho_u = v b - u 2a, rho_v = u b + v 2a with the stored u, v
   if (B::active(x.t)) {
@@ -992,7 +1016,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
 // stage 1), and the inverse column transforms of a, b of the next kbar.
 // grid (Kc, B).
 template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_cols(Dev d, int n, int stage, int flags) {
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj_cols(Dev d, int n, int stage, int flags) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
   FxThread<N, V> x(sm);
