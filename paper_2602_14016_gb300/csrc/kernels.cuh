@@ -143,8 +143,7 @@ struct Geo {
   static constexpr size_t SMEM = sizeof(double2) * 2 * N;  // static_ctrl.cu: plain table and one sequence
   static constexpr size_t SMEM_FOLD = sizeof(double) * FoldInfo<N, V>::PADDED + sizeof(double2) * (N + 2);
   // passes that run the integer transforms: the buffers of two sequences,
-  // scratch of the reductions (three of WARPS ints for each sequence, two of a
-  // pair per warp for the CTA), and probe sums (adjoint column passes)
+  // scratch of the reductions (Place), and probe sums (adjoint column passes)
   static constexpr int SCRATCH = ((3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS + 3) / 4 * 4;
   static constexpr size_t SMEM_FX = sizeof(q2) * (2 * FxPlan<N, V>::BUFS * FxPlan<N, V>::SEQ) + sizeof(int) * SCRATCH;
   static constexpr size_t SMEM_FXP = SMEM_FX + sizeof(double2) * 2 * PMAX;
@@ -350,37 +349,81 @@ __global__ void k_half_to_compact(const double2* __restrict__ in, double2* __res
 // Control map and the inverse column transforms of a stage state
 // ---------------------------------------------------------------------------
 
-// A thread's place in a pass kernel's CTA of two sequences: sequence f,
-// thread t of it; the sequence's two buffers and its scratch; the probe sums.
-template <int N, int V>
-struct FxThread {
-  using P = FxPlan<N, V>;
-  int t, f;
-  q2 *src, *dst;
-  int* scratch;  // three reductions of WARPS ints
-  double2 *Tu, *Tv;  // adjoint column passes only
-  __device__ __forceinline__ explicit FxThread(void* base) {
-    f = threadIdx.x / P::TPS;
-    t = threadIdx.x - f * P::TPS;
-    q2* a = static_cast<q2*>(base);
-    src = a + f * OTHER;
-    dst = P::PING ? src + P::SEQ : src;
-    int* s = reinterpret_cast<int*>(a + 2 * OTHER);
-    scratch = s + f * 3 * P::WARPS;
-    Tu = reinterpret_cast<double2*>(s + Geo<N, V>::SCRATCH);
-    Tv = Tu + Geo<N, V>::PMAX;
-  }
-  // sequence 1's buffers lie this far behind sequence 0's
+// A thread's place in a column pass: sequence f of its column, thread t of
+// the sequence and pt of the column's PT threads; the buffers of its sequence
+// and of the column's first sequence (the other's lie OTHER further); scratch of
+// the sequence's reductions (three of WARPS ints) and of the column's (two of
+// PAIR ints).  In a row pass the two sequences are rows.
+template <typename P_>
+struct Place {
+  using P = P_;
+  static constexpr int PT = 2 * P::TPS;
   static constexpr int OTHER = P::BUFS * P::SEQ;
+  static constexpr int PAIR = PT > 32 ? 2 * (PT / 32) : 0;
+  static constexpr int SCRATCH = 2 * 3 * P::WARPS + 2 * PAIR;  // ints of the pair
+  int t, f, pt;
+  q2 *src, *dst;
+  int *scratch, *pscratch;
+  // pair: index of the pair of sequences in the CTA; thread: index in the pair
+  __device__ __forceinline__ Place(q2* bufs, int* ints, int pair, int thread) : pt(thread) {
+    f = thread / P::TPS;
+    t = thread - f * P::TPS;
+    src = bufs + (pair * 2 + f) * OTHER;
+    dst = P::PING ? src + P::SEQ : src;
+    int* s = ints + pair * SCRATCH;
+    scratch = s + f * 3 * P::WARPS;
+    pscratch = s + 2 * 3 * P::WARPS;
+  }
   __device__ __forceinline__ q2* first(q2* p) const { return f ? p - OTHER : p; }
+  // scratch of the pair's sequence g
+  __device__ __forceinline__ int* seq_scratch(int g) const { return scratch + (g - f) * 3 * P::WARPS; }
 };
 
+// Barrier of a pair: its warp, or the CTA.
+template <typename P>
+__device__ __forceinline__ void pair_sync() {
+  if constexpr (Place<P>::PT <= 32) __syncwarp();
+  else __syncthreads();
+}
+
+// Two reductions over a pair at once.  scratch: PAIR ints, not in use since
+// the barrier before last.  Ends with the pair's barrier.
+template <typename P, bool SUM>
+__device__ __forceinline__ int2 pair_reduce2(int a, int b, int pt, int* scratch) {
+  constexpr int PT = Place<P>::PT;
+  const unsigned mask = seq_mask<(PT < 32 ? PT : 32)>(PT < 32 ? pt : 0);
+  if constexpr (SUM) {
+    a = (int)__reduce_add_sync(mask, (unsigned)a);
+    b = (int)__reduce_add_sync(mask, (unsigned)b);
+  } else {
+    a = __reduce_max_sync(mask, a);
+    b = __reduce_max_sync(mask, b);
+  }
+  if constexpr (PT > 32) {
+    if ((pt & 31) == 0) {
+      scratch[(pt >> 5) * 2] = a;
+      scratch[(pt >> 5) * 2 + 1] = b;
+    }
+    pair_sync<P>();
+    a = scratch[0];
+    b = scratch[1];
+#pragma unroll
+    for (int w = 1; w < PT / 32; ++w) {
+      a = SUM ? a + scratch[2 * w] : max(a, scratch[2 * w]);
+      b = SUM ? b + scratch[2 * w + 1] : max(b, scratch[2 * w + 1]);
+    }
+  } else {
+    pair_sync<P>();
+  }
+  return make_int2(a, b);
+}
+
 // A column under construction: the doubles a thread puts at its retained rows
-// rr = threadIdx.x + j THREADS of the two fields, and the largest exponent
-// fields.
-template <int N, int V>
+// rr = pt + j PT of the two fields, and the largest exponent fields.
+template <typename P>
 struct ColumnPut {
-  static constexpr int MT = (Geo<N, V>::Kr + Geo<N, V>::THREADS - 1) / Geo<N, V>::THREADS;
+  static constexpr int PT = Place<P>::PT;
+  static constexpr int MT = (Geo<P::N>::Kr + PT - 1) / PT;
   double2 v0[MT], v1[MT];
   int f0 = 0, f1 = 0;
   __device__ __forceinline__ void put(int j, double2 a, double2 b) {
@@ -393,8 +436,8 @@ struct ColumnPut {
 
 // The two column values u = i ky/k^2 Yv, v = -i kx/k^2 Yv (scaled by 1/N^2;
 // f = symF entry of the mode) as entry j.
-template <int N, int V>
-__device__ __forceinline__ void put_stage_columns(ColumnPut<N, V>& c, int j, const Sym2& f, double2 Yv) {
+template <typename P>
+__device__ __forceinline__ void put_stage_columns(ColumnPut<P>& c, int j, const Sym2& f, double2 Yv) {
   c.put(j, make_double2(-f.a * Yv.y, f.a * Yv.x),  // u:  i ky / k^2
         make_double2(f.b * Yv.y, -f.b * Yv.x));    // v: -i kx / k^2
 }
@@ -402,57 +445,25 @@ __device__ __forceinline__ void put_stage_columns(ColumnPut<N, V>& c, int j, con
 // The two column values of the adjoint fields of an adjoint stage value kb:
 // 2a = 2 d_xy kb = -2 kx ky kb and b = (d_xx - d_yy) kb = (ky^2 - kx^2) kb,
 // scaled by 1/N^2 (g = symA entry of the mode).
-template <int N, int V>
-__device__ __forceinline__ void put_adjoint_columns(ColumnPut<N, V>& c, int j, const Sym2& g, double2 kb) {
+template <typename P>
+__device__ __forceinline__ void put_adjoint_columns(ColumnPut<P>& c, int j, const Sym2& g, double2 kb) {
   c.put(j, cscale(kb, g.a), cscale(kb, g.b));
 }
 
-// Two reductions over the whole CTA at once, (a, b) -> (A, B): `scratch` has
-// a pair per warp, not in use since the barrier before last.  Ends with a
-// barrier.
-template <int T, bool SUM>
-__device__ __forceinline__ int2 cta_reduce2(int a, int b, int* scratch) {
-  if constexpr (SUM) {
-    a = (int)__reduce_add_sync(0xffffffffu, (unsigned)a);
-    b = (int)__reduce_add_sync(0xffffffffu, (unsigned)b);
-  } else {
-    a = __reduce_max_sync(0xffffffffu, a);
-    b = __reduce_max_sync(0xffffffffu, b);
-  }
-  if constexpr (T > 32) {
-    if ((threadIdx.x & 31) == 0) {
-      scratch[(threadIdx.x >> 5) * 2] = a;
-      scratch[(threadIdx.x >> 5) * 2 + 1] = b;
-    }
-    __syncthreads();
-    a = scratch[0];
-    b = scratch[1];
-#pragma unroll
-    for (int w = 1; w < T / 32; ++w) {
-      a = SUM ? a + scratch[2 * w] : max(a, scratch[2 * w]);
-      b = SUM ? b + scratch[2 * w + 1] : max(b, scratch[2 * w + 1]);
-    }
-  } else {
-    __syncthreads();
-  }
-  return make_int2(a, b);
-}
-
-// Both columns put in c: to integers in x's src buffers (free to write after
-// a barrier), inverse transform along y, into column kx of both fields of Mx.
-template <int N, int V>
-__device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, V>& c, FxThread<N, V> x, int bm, int kx) {
-  using G = Geo<N, V>;
-  using P = FxPlan<N, V>;
-  constexpr int T = G::THREADS, GAP = N - 2 * G::K - 1;
-  int* scratch = x.scratch + (2 - x.f) * 3 * P::WARPS;  // after the two sequences' own
-  const int2 f = cta_reduce2<T, false>(c.f0, c.f1, scratch);
+// Both columns put in c: to integers in the pair's src buffers (free to write
+// after a barrier), inverse transform along y; store(y, value) gets this
+// thread's results of its own sequence.  Returns the sequence's exponent.
+template <typename P, typename Store>
+__device__ __forceinline__ int finish_columns(const ColumnPut<P>& c, Place<P>& x, const int4* tw, Store store) {
+  using G = Geo<P::N>;
+  constexpr int N = P::N, PT = Place<P>::PT, GAP = N - 2 * G::K - 1;
+  const int2 f = pair_reduce2<P, false>(c.f0, c.f1, x.pt, x.pscratch);
   const int e0 = exp_for<kInvBits>(f.x), e1 = exp_for<kInvBits>(f.y);
   q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
   unsigned s0 = 0, s1 = 0;
 #pragma unroll
-  for (int j = 0; j < ColumnPut<N, V>::MT; ++j) {
-    const int rr = threadIdx.x + j * T;
+  for (int j = 0; j < c.MT; ++j) {
+    const int rr = x.pt + j * PT;
     if (rr >= G::Kr) break;
     const int q = pad(ky_of_row(rr, G::K) & (N - 1));
     const q2 u = mkq(double_to_fx(c.v0[j].x, e0), double_to_fx(c.v0[j].y, e0));
@@ -463,34 +474,40 @@ __device__ __forceinline__ void finish_columns(const Dev& d, const ColumnPut<N, 
     a1[q] = v;
   }
   for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(G::K + 1 + u)] = mkq(0, 0);
-  const int2 sum = cta_reduce2<T, true>(s0, s1, scratch + 4 * P::WARPS);
+  const int2 sum = pair_reduce2<P, true>(s0, s1, x.pt, x.pscratch + x.PAIR);
   const int pre = inv_shift<P>(x.f ? sum.y : sum.x);
   constexpr int R = LastRadix<typename P::inv>::value;
   using B = Bfly<P, R>;
   q2 out[B::POINTS];
-  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, pre, out);
+  fx_inverse<P, G::K>(x.src, x.dst, tw, x.t, x.f, pre, out);
   if (B::active(x.t)) {
-    q2* M = d.Mx + (size_t)bm * 2 * N * G::Kc + (size_t)(x.f * N + x.t) * G::Kc + kx;
 #pragma unroll
     for (int jb = 0; jb < B::J; ++jb)
 #pragma unroll
-      for (int m = 0; m < R; ++m) M[(size_t)(jb * P::TPS + m * B::NB) * G::Kc] = out[jb * R + m];
+      for (int m = 0; m < R; ++m) store(x.t + jb * P::TPS + m * B::NB, out[jb * R + m]);
   }
-  if (x.t == 0) d.eX[(bm * 2 + x.f) * G::Kc + kx] = clamp_exp((x.f ? e1 : e0) + pre + P::SHIFT_INV);
+  return clamp_exp((x.f ? e1 : e0) + pre + P::SHIFT_INV);
 }
 
-// Column kx of both fields of the column-major Mn (M points at the column,
-// eN at the member's row exponents), forward transform along y, left in the
-// src buffers with one exponent for both, which is returned, and one bit to
-// spare; synchronised over the CTA.  `between` runs after the loads are
-// issued.
-template <int N, int V, typename Between>
-__device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const int* __restrict__ eN,
-                                               FxThread<N, V>& x, const int4* tw, Between between) {
-  using G = Geo<N, V>;
-  using P = FxPlan<N, V>;
-  constexpr int R = FirstRadix<typename P::fwd>::value;
-  // the first stage only must leave room where that gives two bits more
+// finish_columns into column kx of both fields of Mx.
+template <typename P>
+__device__ __forceinline__ void finish_to_mixed(const Dev& d, const ColumnPut<P>& c, Place<P>& x, int bm, int kx) {
+  constexpr int N = P::N, Kc = Geo<N>::Kc;
+  q2* M = d.Mx + ((size_t)bm * 2 + x.f) * N * Kc + kx;
+  const int e = finish_columns<P>(c, x, d.fxtw, [&](int y, q2 z) { M[(size_t)y * Kc] = z; });
+  if (x.t == 0) d.eX[(bm * 2 + x.f) * Kc + kx] = e;
+}
+
+// Forward transform along y of a sequence of the pair (M: its N values; eN:
+// the exponents of the N rows), left in the src buffers with one exponent for
+// both sequences, which is returned, and one bit to spare; synchronised over
+// the pair.  `between` runs after the loads are issued.
+template <typename P, typename Between>
+__device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const int* __restrict__ eN, Place<P>& x,
+                                               const int4* __restrict__ tw, Between between) {
+  using G = Geo<P::N>;
+  constexpr int N = P::N, R = FirstRadix<typename P::fwd>::value;
+  // the first stage only must leave room where that gives a bit more
   constexpr bool MEASURE = P::GROWTH >= P::GROWTH1 + 1;
   constexpr int BITS = MEASURE ? 62 - P::GROWTH1 : P::BITS_FWD - 1;
   using B = Bfly<P, R>;
@@ -500,7 +517,7 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) {
       const int y = x.t + (j / R) * P::TPS + (j % R) * B::NB;
-      v[j] = M[x.f * N + y];
+      v[j] = M[y];
       e[j] = eN[y];
     }
   }
@@ -521,8 +538,7 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
       big = max_mag(big, v[j]);
     }
   }
-  int* cta = x.scratch + (2 - x.f) * 3 * P::WARPS;  // after the two sequences' own
-  big = cta_reduce2<G::THREADS, false>(big, big, cta).x;
+  big = pair_reduce2<P, false>(big, big, x.pt, x.pscratch).x;
   const int sh = BITS - bits64(big);
   e0 -= sh;
   if (B::active(x.t)) {
@@ -535,21 +551,114 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
     }
   }
   const int r = fx_forward<P, G::K, MEASURE, 1>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
-  // results of two shifts: bring both to the larger one
-  if (x.t == 0) x.scratch[0] = r;
-  __syncthreads();
-  const int* s0 = x.scratch - x.f * 3 * P::WARPS;
-  const int r0 = s0[0], r1 = s0[3 * P::WARPS], rm = max(r0, r1);
-  if constexpr (MEASURE) {
+  if constexpr (MEASURE) {  // results of two shifts: bring both to the larger one
+    if (x.t == 0) x.scratch[0] = r;
+    pair_sync<P>();
+    const int rm = max(x.seq_scratch(0)[0], x.seq_scratch(1)[0]);
     if (r < rm) {
       for (int q = x.t; q < N; q += P::TPS) {
         const q2 z = x.src[pad(q)];
         x.src[pad(q)] = mkq(shr_round(z.x, rm - r), shr_round(z.y, rm - r));
       }
     }
-    if (r0 != r1) __syncthreads();
+    pair_sync<P>();
+    return clamp_exp(e0 + rm + P::SHIFT);
+  } else {
+    pair_sync<P>();
+    return clamp_exp(e0 + P::SHIFT);
   }
-  return clamp_exp(e0 + rm + P::SHIFT);
+}
+
+// The constants of one mode in a column pass (see Sym2).
+struct ModeConst {
+  Sym2 s;
+  FxPair c;
+  int ce;
+  double k2;
+};
+__device__ __forceinline__ ModeConst mode_fwd(const Dev& d, int i) {
+  return {d.symF[i], d.fxF[i], d.fxFe[i], d.k2[i]};
+}
+__device__ __forceinline__ ModeConst mode_adj(const Dev& d, int i) {
+  return {d.symA[i], d.fxA[i], d.fxAe[i], d.k2[i]};
+}
+
+// One mode of the forward column pass: p, q the transforms of u v and v^2 -
+// u^2 at exponent e; w the state at the step's start, y the stage value, acc
+// the RK sum.  Updates w (stage 4), y and acc.  forced: the mode carries the
+// force's coefficient fval.
+__device__ __forceinline__ void rk_mode(const Dev& d, int stage, const ModeConst& m, double nk2, q2 p, q2 q, int e,
+                                        bool forced, double fval, double2& w, double2& y, double2& acc) {
+  // F = -(cp P + cq Q) - nu k^2 y
+  const int eF = e + 64 + m.ce;
+  const double ax = fx_to_double(fx_pair_sum<1>(m.c, p.x, q.x), eF);
+  const double ay = fx_to_double(fx_pair_sum<1>(m.c, p.y, q.y), eF);
+  double2 F = make_double2(-fma(nk2, y.x, ax), -fma(nk2, y.y, ay));
+  if (forced) F.x += fval;
+  if (stage == 1) {
+    acc = F;
+    y = make_double2(fma(d.dt2, F.x, w.x), fma(d.dt2, F.y, w.y));
+  } else if (stage == 2) {
+    acc = make_double2(fma(2.0, F.x, acc.x), fma(2.0, F.y, acc.y));
+    y = make_double2(fma(d.dt2, F.x, w.x), fma(d.dt2, F.y, w.y));
+  } else if (stage == 3) {
+    acc = make_double2(fma(2.0, F.x, acc.x), fma(2.0, F.y, acc.y));
+    y = make_double2(fma(d.dt, F.x, w.x), fma(d.dt, F.y, w.y));
+  } else {
+    y = make_double2(fma(d.dt6, acc.x + F.x, w.x), fma(d.dt6, acc.y + F.y, w.y));
+    w = y;
+  }
+}
+
+// One mode of the adjoint column pass of stage 4..1: ru, rv the transforms of
+// rho_u, rho_v at exponent e; kb the stage value, lb lambda at the step's end,
+// sum the stages' sum.  Updates sum, kb (the next stage's) and, on stage 1, lb
+// (lambda at the step's start; src: the observation source there).
+__device__ __forceinline__ void adj_mode(const Dev& d, int stage, const ModeConst& m, double nk2, q2 ru, q2 rv, int e,
+                                         bool has_src, double2 src, double2& kb, double2& lb, double2& sum) {
+  // t = (-i ky/k^2) Ru + (i kx/k^2) Rv (the 1/2 of the row unpack in a1, c1)
+  const int eR = e + 64 + m.ce;
+  const double2 tt = make_double2(fx_to_double(fx_pair_sum<-1>(m.c, ru.y, rv.y), eR),
+                                  -fx_to_double(fx_pair_sum<-1>(m.c, ru.x, rv.x), eR));
+  double2 yb;
+  yb.x = -fma(nk2, kb.x, tt.x);
+  yb.y = -fma(nk2, kb.y, tt.y);
+  if (stage == 4) {
+    sum = yb;
+    kb = make_double2(fma(d.dt3, lb.x, d.dt * yb.x), fma(d.dt3, lb.y, d.dt * yb.y));
+  } else if (stage == 3) {
+    sum = cadd(sum, yb);
+    kb = make_double2(fma(d.dt3, lb.x, d.dt2 * yb.x), fma(d.dt3, lb.y, d.dt2 * yb.y));
+  } else if (stage == 2) {
+    sum = cadd(sum, yb);
+    kb = make_double2(fma(d.dt6, lb.x, d.dt2 * yb.x), fma(d.dt6, lb.y, d.dt2 * yb.y));
+  } else {
+    lb = cadd(lb, cadd(sum, yb));
+    if (has_src) lb = cadd(lb, src);
+    kb = cscale(lb, d.dt6);
+  }
+}
+
+// Whether mode (kx, ky) carries the Kolmogorov force, and its coefficient.
+__device__ __forceinline__ bool forced_mode(const Dev& d, const MemberWindow& mw, int kx, int ky) {
+  return mw.forced && kx == 0 && (ky == d.nf || ky == -d.nf);
+}
+template <int N>
+__device__ __forceinline__ double force_value(const Dev& d) {
+  return -d.amp * d.nf * (double)N * N / 2.0;
+}
+
+// The place of a thread of a pass kernel, whose CTA is one pair, in its
+// dynamic shared memory; the probe sums after it (adjoint column passes).
+template <int N, int V>
+__device__ __forceinline__ Place<FxPlan<N, V>> pass_place(void* base) {
+  using X = Place<FxPlan<N, V>>;
+  q2* a = static_cast<q2*>(base);
+  return X(a, reinterpret_cast<int*>(a + 2 * X::OTHER), 0, threadIdx.x);
+}
+template <int N, int V>
+__device__ __forceinline__ double2* pass_probe_sums(void* base) {
+  return reinterpret_cast<double2*>(static_cast<char*>(base) + Geo<N, V>::SMEM_FX);
 }
 
 // s_hat = forward transform along y of the mixed rows in Mn (doubles here,
@@ -568,7 +677,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d, int fla
   for (int y = threadIdx.x; y < N; y += G::THREADS) a[y] = M[y];
   __syncthreads();
   fft_folded<N, V, -1, 1, -1, G::K>(a, T);
-  ColumnPut<N, V> put;
+  ColumnPut<FxPlan<N, V>> put;
 #pragma unroll
   for (int j = 0; j < put.MT; ++j) {
     const int rr = threadIdx.x + j * G::THREADS;
@@ -578,11 +687,12 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d, int fla
     const double2 w0 = cscale(a[ky & (N - 1)], d.mult[idx]);
     d.W[idx] = w0;
     d.Y[idx] = w0;
-    put_stage_columns<N, V>(put, j, d.symF[kx * G::Kr + rr], w0);
+    put_stage_columns(put, j, d.symF[kx * G::Kr + rr], w0);
   }
   if (flags & F_NO_NEXT) return;
   __syncthreads();  // the FP64 part's memory is read no more
-  finish_columns<N, V>(d, put, FxThread<N, V>(sm), bm, kx);
+  Place<FxPlan<N, V>> x = pass_place<N, V>(sm);
+  finish_to_mixed(d, put, x, bm, kx);
 }
 
 // Restart from the compact state in W (a checkpoint): Y = W and the inverse
@@ -592,7 +702,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_state_cols(Dev d) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
   const int kx = blockIdx.x, bm = blockIdx.y;
-  ColumnPut<N, V> put;
+  ColumnPut<FxPlan<N, V>> put;
 #pragma unroll
   for (int j = 0; j < put.MT; ++j) {
     const int rr = threadIdx.x + j * G::THREADS;
@@ -600,31 +710,30 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_state_cols(Dev d) {
     const size_t idx = cidx<N>(bm, rr, kx);
     const double2 w = d.W[idx];
     d.Y[idx] = w;
-    put_stage_columns<N, V>(put, j, d.symF[kx * G::Kr + rr], w);
+    put_stage_columns(put, j, d.symF[kx * G::Kr + rr], w);
   }
-  finish_columns<N, V>(d, put, FxThread<N, V>(sm), bm, kx);
+  Place<FxPlan<N, V>> x = pass_place<N, V>(sm);
+  finish_to_mixed(d, put, x, bm, kx);
 }
 
 // ---------------------------------------------------------------------------
 // Row passes
 // ---------------------------------------------------------------------------
 
-// Row y of the two fields of Mx, packed for the inverse transform along x as
-// field 0 + i field 1: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B) for the
+// A row of the two mixed fields (MA, MB: its Kc values each; eX: the exponents
+// of the Kc columns, field 0 then field 1), packed for the inverse transform
+// along x as field 0 + i field 1: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B) for the
 // mixed half spectra A, B (kx = 0..K); the DC bin keeps real parts only; the
 // gap is zeroed.  Into the sequence's src buffer, synchronised.
 struct RowLoad {
   int e;    // exponent of the row as it stands in src
   int pre;  // shift its inverse transform starts with
 };
-template <int N, int V>
-__device__ __forceinline__ RowLoad load_row(const Dev& d, int bm, int y, const FxThread<N, V>& x) {
-  using G = Geo<N, V>;
-  using P = FxPlan<N, V>;
-  constexpr int K = G::K, Kc = G::Kc, GAP = N - 2 * K - 1, J = (Kc + P::TPS - 1) / P::TPS;
-  const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
-  const q2* MB = MA + (size_t)N * Kc;
-  const int* eX = d.eX + (size_t)bm * 2 * Kc;
+template <typename P>
+__device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2* __restrict__ MB, const int* __restrict__ eX,
+                                            Place<P>& x) {
+  using G = Geo<P::N>;
+  constexpr int N = P::N, K = G::K, Kc = G::Kc, GAP = N - 2 * K - 1, J = (Kc + P::TPS - 1) / P::TPS;
   q2 p[J], q[J];
   int ep[J], eq[J], e = 2 * kZeroExp;
 #pragma unroll
@@ -677,9 +786,8 @@ __device__ __forceinline__ RowLoad load_row(const Dev& d, int bm, int y, const F
 // symbols carry the 1/2) in the column-major Mn of the member: entry
 // (kx, f, y) at (kx * 2 + f) * N + y; e: this sequence's exponent.
 template <int N, int V>
-__device__ __forceinline__ void store_row_pair(const Dev& d, int bm, int y0, const FxThread<N, V>& x, int e) {
+__device__ __forceinline__ void store_row_pair(const Dev& d, int bm, int y0, const Place<FxPlan<N, V>>& x, int e) {
   using G = Geo<N, V>;
-  using P = FxPlan<N, V>;
   __syncthreads();  // both rows are in
   const q2* a = x.first(x.src);
   q2* O = d.Mn + (size_t)bm * G::Kc * 2 * N;
@@ -701,16 +809,71 @@ __device__ __forceinline__ void store_row_pair(const Dev& d, int bm, int y0, con
 // the 64 bits dropped, enter the forward transform with one bit to spare for
 // the sums of store_row_pair: room for all its stages, or (MEASURE, where it
 // gives the products at least two bits more) for the first one.
-template <int N, int V>
+template <typename P>
 struct RowBits {
-  using P = FxPlan<N, V>;
   static constexpr int F = P::BITS_FWD - 1;
   static constexpr int UV0 = (64 + F) / 2;  // u v and v^2 - u^2: 2 UV - 64 <= F
   static constexpr int AB0 = 63 + F - UV0;  // sums of two products: UV + AB - 63 <= F
   static constexpr int UV1 = 61, AB1 = P::GROWTH1 <= 3 ? 61 : 60;
-  static constexpr bool MEASURE = UV1 + AB1 >= UV0 + AB0 + (N >= 1024 ? 1 : 2);
+  static constexpr bool MEASURE = UV1 + AB1 >= UV0 + AB0 + (P::N >= 1024 ? 1 : 2);
   static constexpr int UV = MEASURE ? UV1 : UV0, AB = MEASURE ? AB1 : AB0;
 };
+
+// Inverse transform along x of a loaded row, brought to BITS bits: z[j] at x =
+// row_x(j).  between runs before the results are measured.  Returns the row's
+// exponent.
+template <typename P>
+struct RowPoints {
+  static constexpr int R = LastRadix<typename P::inv>::value;
+  using B = Bfly<P, R>;
+  static constexpr int POINTS = B::POINTS;
+  __device__ static __forceinline__ int x(int t, int j) { return t + (j / R) * P::TPS + (j % R) * B::NB; }
+};
+template <typename P, int BITS, typename Between>
+__device__ __forceinline__ int row_fields(const RowLoad& in, Place<P>& x, const int4* tw, q2* z, Between between) {
+  using RP = RowPoints<P>;
+  fx_inverse<P, Geo<P::N>::K>(x.src, x.dst, tw, x.t, x.f, in.pre, z);
+  between();
+  int m = 0;
+  if (RP::B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < RP::POINTS; ++j) m = max_mag(m, z[j]);
+  }
+  m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
+  const int sh = max(0, BITS - bits64(m));  // at most 60 bits: never right
+  if (RP::B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < RP::POINTS; ++j) z[j] = mkq(z[j].x << sh, z[j].y << sh);
+  }
+  return clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
+}
+
+// (u, v) -> P + i Q, P = u v, Q = v^2 - u^2 (less 64 bits).
+__device__ __forceinline__ q2 uv_products(q2 z) {
+  return mkq(mul_hi(z.x, z.y), mul_hi(z.y - z.x, z.y + z.x));
+}
+// (2a, b) with the stored u, v -> rho_u + i rho_v, rho_u = v b - u 2a, rho_v =
+// u b + v 2a (less 64 bits).
+__device__ __forceinline__ q2 rho_products(q2 uv, q2 ab) {
+  const Words u(uv.x), v(uv.y), a(ab.x), b(ab.y), na(-ab.x);
+  return mkq(mul_hi2(v, b, u, na), mul_hi2(u, b, v, a));
+}
+
+// Velocity at a probe of row y, column xx into its slot of the observations.
+__device__ __forceinline__ void put_probe(const Dev& d, int bm, int slot, int P, int st, int y, int xx, q2 uv, int e) {
+  double* o = d.obs + bm * d.obs_stride + ((size_t)slot * P * P + (y / st) * P + xx / st) * 2;
+  o[0] = fx_to_double(uv.x, e);
+  o[1] = fx_to_double(uv.y, e);
+}
+
+// First value of the stored stage fields of stage `stage` of step n, row y of
+// member bm, over N: index of the row (times N: of its values).
+template <int N>
+__device__ __forceinline__ size_t stored_row(const Dev& d, int bm, int n, int stage, int y) {
+  return (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y;
+}
 
 // Row pass of stage `stage` (1..4) of step n: u, v of rows y0, y0+1; the
 // stage-field store and probe gather; the products u v and v^2 - u^2 of
@@ -718,51 +881,35 @@ struct RowBits {
 // Mn.  grid (N/2, B).
 template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, int stage, int flags) {
-  using G = Geo<N, V>;
   using P = FxPlan<N, V>;
+  using RP = RowPoints<P>;
   extern __shared__ double2 sm[];
-  FxThread<N, V> x(sm);
+  Place<P> x = pass_place<N, V>(sm);
   const int bm = blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;  // the member's window has not begun
-  constexpr int R = LastRadix<typename P::inv>::value;
-  using B = Bfly<P, R>;
-  const RowLoad in = load_row<N, V>(d, bm, y, x);
+  constexpr int Kc = Geo<N>::Kc;
+  const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
+  const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, d.eX + (size_t)bm * 2 * Kc, x);
   const int Pp = mw.P, st = N / Pp;
   const int slot = (flags & (F_OBS | F_OBS_ONLY)) ? obs_slot(d, n - mw.start) : -1;
-  q2 z[B::POINTS];
-  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, in.pre, z);
-  // u, v to UV bits
-  int m = 0;
-  if (B::active(x.t)) {
-#pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) m = max_mag(m, z[j]);
-  }
-  m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
-  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
-  m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
-  const int sh = max(0, RowBits<N, V>::UV - bits64(m));  // at most 60 bits: never right
-  const int ex = clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
-  const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y;
+  q2 z[RP::POINTS];
+  const int ex = row_fields<P, RowBits<P>::UV>(in, x, d.fxtw, z, [] {});
+  const size_t trow = stored_row<N>(d, bm, n, stage, y);
   const bool store = (flags & F_STORE) != 0;
   if (store && x.t == 0) d.eT[trow] = ex;
   const bool probes = slot >= 0 && (y % st) == 0;
-  if (B::active(x.t)) {
+  if (RP::B::active(x.t)) {
 #pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) {
-      const int xx = x.t + (j / R) * P::TPS + (j % R) * B::NB;
-      const i64 u = z[j].x << sh, v = z[j].y << sh;
-      if (store) d.traj[trow * N + xx] = mkq(u, v);
-      if (probes && (xx % st) == 0) {
-        double* o = d.obs + bm * d.obs_stride + ((size_t)slot * Pp * Pp + (y / st) * Pp + xx / st) * 2;
-        o[0] = fx_to_double(u, ex);
-        o[1] = fx_to_double(v, ex);
-      }
-      z[j] = mkq(mul_hi(u, v), mul_hi(v - u, v + u));
+    for (int j = 0; j < RP::POINTS; ++j) {
+      const int xx = RP::x(x.t, j);
+      if (store) d.traj[trow * N + xx] = z[j];
+      if (probes && (xx % st) == 0) put_probe(d, bm, slot, Pp, st, y, xx, z[j], ex);
+      z[j] = uv_products(z[j]);
     }
   }
   if (flags & F_OBS_ONLY) return;  // the final state: probes only
-  const int r = fx_forward<P, G::K, RowBits<N, V>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+  const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
   store_row_pair<N, V>(d, bm, y0, x, 2 * ex + 64 + P::SHIFT + r);
 }
 
@@ -778,20 +925,16 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
 template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd_cols(Dev d, int n, int stage, int flags) {
   using G = Geo<N, V>;
+  using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
-  FxThread<N, V> x(sm);
+  Place<P> x = pass_place<N, V>(sm);
   const int kx = blockIdx.x, bm = blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
-  // the epilogue's inputs for this thread's modes; where registers allow
-  // (G::PREFETCH), loaded early so that their latency hides behind the
-  // column transforms
-  constexpr int MT = (G::Kr + G::THREADS - 1) / G::THREADS;
-  double2 yv[MT], wv[MT], accv[MT];
-  Sym2 f[MT];
-  FxPair cf[MT];
-  int ce[MT];
-  double nk2[MT];
+  // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
+  ColumnPut<P> put;
+  double2 yv[put.MT], wv[put.MT], accv[put.MT];
+  ModeConst mc[put.MT];
   auto load_inputs = [&](int t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr < G::Kr) {
@@ -799,58 +942,35 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
       yv[t] = d.Y[idx];
       wv[t] = d.W[idx];
       accv[t] = stage > 1 ? d.Acc[idx] : make_double2(0.0, 0.0);
-      f[t] = d.symF[kx * G::Kr + rr];
-      cf[t] = d.fxF[kx * G::Kr + rr];
-      ce[t] = d.fxFe[kx * G::Kr + rr];
-      nk2[t] = mw.nu * d.k2[kx * G::Kr + rr];
+      mc[t] = mode_fwd(d, kx * G::Kr + rr);
     }
   };
-  const int e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
+  const int e = forward_columns<P>(d.Mn + (((size_t)bm * G::Kc + kx) * 2 + x.f) * N, d.eN + bm * N, x, d.fxtw, [&] {
     if constexpr (G::PREFETCH) {
 #pragma unroll
-      for (int t = 0; t < MT; ++t) load_inputs(t);
+      for (int t = 0; t < put.MT; ++t) load_inputs(t);
     }
   });
   const q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
-  const double dt = d.dt;
-  const double fval = -d.amp * d.nf * (double)N * N / 2.0;
-  ColumnPut<N, V> put;
+  const double fval = force_value<N>(d);
 #pragma unroll
-  for (int t = 0; t < MT; ++t) {
+  for (int t = 0; t < put.MT; ++t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr >= G::Kr) break;
     if constexpr (!G::PREFETCH) load_inputs(t);
     const int ky = ky_of_row(rr, G::K);
-    const int qi = ky & (N - 1);
+    const int qi = pad(ky & (N - 1));
     const size_t idx = cidx<N>(bm, rr, kx);
-    const q2 pq = a0[pad(qi)], qq = a1[pad(qi)];
-    // F = -(cp P + cq Q) - nu k^2 y
-    const int eF = e + 64 + ce[t];
-    const double ax = fx_to_double(fx_pair_sum<1>(cf[t], pq.x, qq.x), eF);
-    const double ay = fx_to_double(fx_pair_sum<1>(cf[t], pq.y, qq.y), eF);
-    double2 F = make_double2(-fma(nk2[t], yv[t].x, ax), -fma(nk2[t], yv[t].y, ay));
-    if (mw.forced && kx == 0 && (ky == d.nf || ky == -d.nf)) F.x += fval;
-    const double2 w = wv[t], acc = accv[t];
-    double2 ynext;
-    if (stage == 1) {
-      d.Acc[idx] = F;
-      ynext = make_double2(fma(d.dt2, F.x, w.x), fma(d.dt2, F.y, w.y));
-    } else if (stage == 2) {
-      d.Acc[idx] = make_double2(fma(2.0, F.x, acc.x), fma(2.0, F.y, acc.y));
-      ynext = make_double2(fma(d.dt2, F.x, w.x), fma(d.dt2, F.y, w.y));
-    } else if (stage == 3) {
-      d.Acc[idx] = make_double2(fma(2.0, F.x, acc.x), fma(2.0, F.y, acc.y));
-      ynext = make_double2(fma(dt, F.x, w.x), fma(dt, F.y, w.y));
-    } else {
-      ynext = make_double2(fma(d.dt6, acc.x + F.x, w.x), fma(d.dt6, acc.y + F.y, w.y));
-      d.W[idx] = ynext;
-    }
-    d.Y[idx] = ynext;
-    put_stage_columns<N, V>(put, t, f[t], ynext);
+    rk_mode(d, stage, mc[t], mw.nu * mc[t].k2, a0[qi], a1[qi], e, forced_mode(d, mw, kx, ky), fval, wv[t], yv[t],
+            accv[t]);
+    if (stage < 4) d.Acc[idx] = accv[t];
+    else d.W[idx] = wv[t];
+    d.Y[idx] = yv[t];
+    put_stage_columns(put, t, mc[t].s, yv[t]);
   }
   if (flags & F_NO_NEXT) return;
-  swap_bufs<FxPlan<N, V>>(x.src, x.dst);
-  finish_columns<N, V>(d, put, x, bm, kx);
+  swap_bufs<P>(x.src, x.dst);
+  finish_to_mixed(d, put, x, bm, kx);
 }
 
 // r = model observations - data and J = 1/2 sum r^2 per member, in a fixed
@@ -887,11 +1007,11 @@ __global__ void k_sobolev_grad(double2* lam, const double2* w0, double lambda, i
 // Separable DFT of the residual at observation slot `slot` on the probe
 // lattice: for each lattice row, T(kx) = sum_q r[row][q] W_P^{kx q}; the
 // column pass then sums over rows with W_P^{ky row}.  Fills Tu, Tv [P].
-__device__ __forceinline__ void probe_row_sums(const Dev& d, int bm, int P, int slot, int kx, double2* Tu,
-                                               double2* Tv) {
+__device__ __forceinline__ void probe_row_sums(const Dev& d, int bm, int P, int slot, int kx, int thread, int threads,
+                                               double2* Tu, double2* Tv) {
   const double* r = d.res + bm * d.obs_stride + (size_t)slot * P * P * 2;
   const int tws = 64 / P;
-  for (int row = threadIdx.x; row < P; row += blockDim.x) {
+  for (int row = thread; row < P; row += threads) {
     double2 su = make_double2(0.0, 0.0), sv = make_double2(0.0, 0.0);
     for (int qq = 0; qq < P; ++qq) {
       const double2 w = d.twP[((kx * qq) % P) * tws];
@@ -932,17 +1052,17 @@ template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode) {
   using G = Geo<N, V>;
   extern __shared__ double2 sm[];
-  const FxThread<N, V> x(sm);
-  double2 *Tu = x.Tu, *Tv = x.Tv;
+  Place<FxPlan<N, V>> x = pass_place<N, V>(sm);
+  double2 *Tu = pass_probe_sums<N, V>(sm), *Tv = Tu + G::PMAX;
   const int kx = blockIdx.x, bm = blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   // an idle member starts (and stays) at lambda = 0
   if (mw.start > d.nsteps) mode = 0;
   const bool resume = (mode & INIT_RESUME) != 0;
   const int slot = (!resume && (mode & INIT_SRC)) ? obs_slot(d, d.nsteps - mw.start) : -1;
-  if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, Tu, Tv);
+  if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, threadIdx.x, G::THREADS, Tu, Tv);
   __syncthreads();
-  ColumnPut<N, V> put;
+  ColumnPut<FxPlan<N, V>> put;
 #pragma unroll
   for (int j = 0; j < put.MT; ++j) {
     const int rr = threadIdx.x + j * G::THREADS;
@@ -959,9 +1079,9 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode
       kb = cscale(lam, d.dt6);
       d.KB[idx] = kb;
     }
-    put_adjoint_columns<N, V>(put, j, d.symA[kx * G::Kr + rr], kb);
+    put_adjoint_columns(put, j, d.symA[kx * G::Kr + rr], kb);
   }
-  finish_columns<N, V>(d, put, x, bm, kx);
+  finish_to_mixed(d, put, x, bm, kx);
 }
 
 // Adjoint row pass of stage `stage` of step n: 2a, b of rows y0, y0+1
@@ -971,42 +1091,28 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode
 template <int N, int V = 0>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, int stage) {
   using P = FxPlan<N, V>;
-  using G = Geo<N, V>;
+  using RP = RowPoints<P>;
   extern __shared__ double2 sm[];
-  FxThread<N, V> x(sm);
+  Place<P> x = pass_place<N, V>(sm);
   const int bm = blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
   if (d.ragged && n < d.mstart[bm]) return;
-  constexpr int R = LastRadix<typename P::inv>::value;
-  using B = Bfly<P, R>;
-  const RowLoad in = load_row<N, V>(d, bm, y, x);
-  const size_t trow = (((size_t)bm * d.traj_steps + (n - d.seg0)) * 4 + (stage - 1)) * N + y;
-  q2 z[B::POINTS];
-  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, in.pre, z);
-  // 2a, b to AB bits
-  int m = 0;
-  q2 uv[B::POINTS];
-  if (B::active(x.t)) {
+  constexpr int Kc = Geo<N>::Kc;
+  const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
+  const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, d.eX + (size_t)bm * 2 * Kc, x);
+  const size_t trow = stored_row<N>(d, bm, n, stage, y);
+  q2 z[RP::POINTS], uv[RP::POINTS];
+  const int ex = row_fields<P, RowBits<P>::AB>(in, x, d.fxtw, z, [&] {
+    if (RP::B::active(x.t)) {
 #pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) uv[j] = d.traj[trow * N + x.t + (j / R) * P::TPS + (j % R) * B::NB];
-#pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) m = max_mag(m, z[j]);
-  }
-  m = seq_max_put<P::TPS>(m, x.t, x.scratch + 2 * P::WARPS);
-  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
-  m = seq_max_get<P::TPS>(m, x.scratch + 2 * P::WARPS);
-  const int sh = max(0, RowBits<N, V>::AB - bits64(m));
-  const int ex = clamp_exp(in.e + in.pre + P::SHIFT_INV - sh);
-  // rho_u = v b - u 2a, rho_v = u b + v 2a with the stored u, v
-  if (B::active(x.t)) {
-#pragma unroll
-    for (int j = 0; j < B::POINTS; ++j) {
-      const i64 aa = z[j].x << sh, bb = z[j].y << sh;
-      const Words u(uv[j].x), v(uv[j].y), a(aa), b(bb), na(-aa);
-      z[j] = mkq(mul_hi2(v, b, u, na), mul_hi2(u, b, v, a));
+      for (int j = 0; j < RP::POINTS; ++j) uv[j] = d.traj[trow * N + RP::x(x.t, j)];
     }
+  });
+  if (RP::B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < RP::POINTS; ++j) z[j] = rho_products(uv[j], z[j]);
   }
   const int eT = d.eT[trow];
-  const int r = fx_forward<P, G::K, RowBits<N, V>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+  const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
   store_row_pair<N, V>(d, bm, y0, x, clamp_exp(ex + eT) + 64 + P::SHIFT + r);
 }
 
@@ -1014,24 +1120,22 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
 //   ybar_j = -P[(-i ky/k^2) DFT(rho_u) + (i kx/k^2) DFT(rho_v)] - nu k^2 kbar_j,
 // the transposed RK4 combination, the observation source at step n (on
 // stage 1), and the inverse column transforms of a, b of the next kbar.
-// grid (Kc, B).
-template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj_cols(Dev d, int n, int stage, int flags) {
+// SRC: with the observation source, which few steps have and whose code would
+// double the kernel.  grid (Kc, B).
+template <int N, int V, bool SRC>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj_cols(Dev d, int n, int stage) {
   using G = Geo<N, V>;
+  using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
-  FxThread<N, V> x(sm);
-  double2 *Tu = x.Tu, *Tv = x.Tv;
+  Place<P> x = pass_place<N, V>(sm);
+  double2 *Tu = pass_probe_sums<N, V>(sm), *Tv = Tu + G::PMAX;
   const int kx = blockIdx.x, bm = blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
-  // the epilogue's inputs for this thread's modes (before the column
-  // transforms where registers allow, as in k_fwd_cols)
-  constexpr int MT = (G::Kr + G::THREADS - 1) / G::THREADS;
-  double2 kbv[MT], lbv[MT], sumv[MT];
-  Sym2 g[MT];
-  FxPair cf[MT];
-  int ce[MT];
-  double nk2[MT];
+  // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
+  ColumnPut<P> put;
+  double2 kbv[put.MT], lbv[put.MT], sumv[put.MT];
+  ModeConst mc[put.MT];
   auto load_inputs = [&](int t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr < G::Kr) {
@@ -1039,63 +1143,41 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
       kbv[t] = d.KB[idx];
       lbv[t] = d.LamBar[idx];
       sumv[t] = stage < 4 ? d.Sum[idx] : make_double2(0.0, 0.0);
-      g[t] = d.symA[kx * G::Kr + rr];
-      cf[t] = d.fxA[kx * G::Kr + rr];
-      ce[t] = d.fxAe[kx * G::Kr + rr];
-      nk2[t] = mw.nu * d.k2[kx * G::Kr + rr];
+      mc[t] = mode_adj(d, kx * G::Kr + rr);
     }
   };
-  const int slot = (flags & F_SRC) ? obs_slot(d, n - mw.start) : -1;
-  const int e = forward_columns<N, V>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [&] {
+  const int slot = SRC ? obs_slot(d, n - mw.start) : -1;
+  const int e = forward_columns<P>(d.Mn + (((size_t)bm * G::Kc + kx) * 2 + x.f) * N, d.eN + bm * N, x, d.fxtw, [&] {
     if constexpr (G::PREFETCH) {
 #pragma unroll
-      for (int t = 0; t < MT; ++t) load_inputs(t);
+      for (int t = 0; t < put.MT; ++t) load_inputs(t);
     }
-    if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, Tu, Tv);
+    if constexpr (SRC) {
+      if (slot >= 0) probe_row_sums(d, bm, mw.P, slot, kx, threadIdx.x, G::THREADS, Tu, Tv);
+    }
   });
   const q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
-  const double dt = d.dt;
-  ColumnPut<N, V> put;
 #pragma unroll
-  for (int t = 0; t < MT; ++t) {
+  for (int t = 0; t < put.MT; ++t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr >= G::Kr) break;
     if constexpr (!G::PREFETCH) load_inputs(t);
     const int ky = ky_of_row(rr, G::K);
-    const int qi = ky & (N - 1);
+    const int qi = pad(ky & (N - 1));
     const size_t idx = cidx<N>(bm, rr, kx);
-    const q2 qu = a0[pad(qi)], qv = a1[pad(qi)];
-    // t = (-i ky/k^2) Ru + (i kx/k^2) Rv (the 1/2 of the row unpack in a1, c1)
-    const int eR = e + 64 + ce[t];
-    const double2 tt = make_double2(fx_to_double(fx_pair_sum<-1>(cf[t], qu.y, qv.y), eR),
-                                    -fx_to_double(fx_pair_sum<-1>(cf[t], qu.x, qv.x), eR));
-    const double2 kb = kbv[t], lb = lbv[t];
-    double2 yb;
-    yb.x = -fma(nk2[t], kb.x, tt.x);
-    yb.y = -fma(nk2[t], kb.y, tt.y);
-    double2 nk;
-    if (stage == 4) {
-      d.Sum[idx] = yb;
-      nk = make_double2(fma(d.dt3, lb.x, dt * yb.x), fma(d.dt3, lb.y, dt * yb.y));
-    } else if (stage == 3) {
-      d.Sum[idx] = cadd(sumv[t], yb);
-      nk = make_double2(fma(d.dt3, lb.x, d.dt2 * yb.x), fma(d.dt3, lb.y, d.dt2 * yb.y));
-    } else if (stage == 2) {
-      d.Sum[idx] = cadd(sumv[t], yb);
-      nk = make_double2(fma(d.dt6, lb.x, d.dt2 * yb.x), fma(d.dt6, lb.y, d.dt2 * yb.y));
-    } else {
-      const double2 sum = cadd(sumv[t], yb);
-      double2 lam = cadd(lb, sum);
-      if (slot >= 0) lam = cadd(lam, probe_source(d, mw.P, kx, ky, Tu, Tv));
-      d.LamBar[idx] = lam;
-      nk = cscale(lam, d.dt6);
+    double2 src = make_double2(0.0, 0.0);
+    if constexpr (SRC) {
+      if (slot >= 0) src = probe_source(d, mw.P, kx, ky, Tu, Tv);
     }
-    d.KB[idx] = nk;
-    put_adjoint_columns<N, V>(put, t, g[t], nk);
+    adj_mode(d, stage, mc[t], mw.nu * mc[t].k2, a0[qi], a1[qi], e, slot >= 0, src, kbv[t], lbv[t], sumv[t]);
+    if (stage > 1) d.Sum[idx] = sumv[t];
+    else d.LamBar[idx] = lbv[t];
+    d.KB[idx] = kbv[t];
+    put_adjoint_columns(put, t, mc[t].s, kbv[t]);
   }
   if (stage == 1 && n == mw.start) return;  // the member's first step: lambda_0 stays in LamBar
-  swap_bufs<FxPlan<N, V>>(x.src, x.dst);
-  finish_columns<N, V>(d, put, x, bm, kx);
+  swap_bufs<P>(x.src, x.dst);
+  finish_to_mixed(d, put, x, bm, kx);
 }
 
 // Control multipliers m(k) = |k| W(k)^{1/2} on the retained set (0 at k = 0),

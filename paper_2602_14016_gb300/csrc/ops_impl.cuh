@@ -34,7 +34,8 @@ Ops make_ops() {
     set((const void*)k_state_cols<N, V>);
     set((const void*)k_adj_init<N, V>, G::SMEM_FXP);
     set((const void*)k_adj_rows<N, V>);
-    set((const void*)k_adj_cols<N, V>, G::SMEM_FXP);
+    set((const void*)k_adj_cols<N, V, false>, G::SMEM_FXP);
+    set((const void*)k_adj_cols<N, V, true>, G::SMEM_FXP);
     return e;
   };
   o.r2c_rows = [](const Dev& d, const double* in, cudaStream_t st) {
@@ -71,7 +72,8 @@ Ops make_ops() {
     k_adj_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
   };
   o.adj_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_adj_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage, flags);
+    if (flags & F_SRC) k_adj_cols<N, V, true><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
+    else k_adj_cols<N, V, false><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
   };
   o.make_mult = [](const Dev& d, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                    cudaStream_t st) {
