@@ -178,6 +178,12 @@ da_status dalloc(da_ctx* c, T** p, size_t count) {
 // multiples of obs.every; the kernels find each member's slot).
 inline bool obs_step_host(const da_ctx* c, int k) { return k % c->obs.every == 0; }
 
+// Whether this context's windows run as single kernels (window.cuh): small
+// grids and batches, unless a class of pass kernels is being timed.
+inline bool whole_windows(const da_ctx* c) {
+  return c->ops->window_fwd && c->B <= c->ops->window_batch && c->timed_class == 0;
+}
+
 // Sets the evaluation window for the members marked in `live` (all members
 // with a non-empty window if live is NULL): eval_steps = the longest live
 // window, each live member end-aligned in it, the others idle; uploads the

@@ -329,13 +329,28 @@ static da_status run_forward(da_ctx* c, const double* s, bool gather, cudaStream
   const int last0 = ((E - 1) / K) * K;  // first step of the last segment
   const size_t comp = (size_t)c->B * o->Kr * o->Kc;
   c->have_fwd = false;
+  const bool whole = whole_windows(c);
   o->r2c_rows(d, s, st);
-  o->ctrl_cols(d, 0, st);
+  o->ctrl_cols(d, whole ? da::F_NO_NEXT : 0, st);
   da_status r = check_launch(c, 2);
   if (r) return r;
   if (c->w0) DA_TRY_CUDA(c, cudaMemcpyAsync(c->w0, d.W, comp * sizeof(double2), cudaMemcpyDeviceToDevice, st));
   d.seg0 = last0;
   if (c->ckpt == 0) d.seg0 = 0;
+  if (whole) {
+    for (int k0 = 0; k0 < E; k0 += K) {
+      const int k1 = std::min(k0 + K, E);
+      if (c->ckpt > 0 && store)
+        DA_TRY_CUDA(c, cudaMemcpyAsync(c->ckpt_buf + (size_t)(k0 / K) * comp, d.W, comp * sizeof(double2),
+                                       cudaMemcpyDeviceToDevice, st));
+      const int flags = (gather ? da::W_OBS : 0) | (store && k0 >= d.seg0 ? da::W_STORE : 0) |
+                        (gather && k1 == E ? da::W_FINAL : 0);
+      o->window_fwd(d, k0, k1, flags, st);
+      if ((r = check_launch(c))) return r;
+    }
+    c->have_fwd = store;
+    return DA_OK;
+  }
   for (int k = 0; k < E; ++k) {
     if (c->ckpt > 0 && store && k % K == 0)
       DA_TRY_CUDA(c, cudaMemcpyAsync(c->ckpt_buf + (size_t)(k / K) * comp, d.W, comp * sizeof(double2),
@@ -405,9 +420,29 @@ static da_status run_adjoint(da_ctx* c, bool sources, cudaStream_t st, const Spe
   const int K = c->ckpt > 0 ? c->ckpt : E;
   const int nseg = (E + K - 1) / K;
   const size_t comp = (size_t)c->B * o->Kr * o->Kc;
+  const bool whole = whole_windows(c);
   da_status r;
   for (int seg = nseg - 1; seg >= 0; --seg) {
     const int k0 = seg * K, k1 = std::min(k0 + K, E);
+    if (whole) {
+      if (seg != nseg - 1) {
+        DA_TRY_CUDA(c, cudaMemcpyAsync(d.W, c->ckpt_buf + (size_t)seg * comp, comp * sizeof(double2),
+                                       cudaMemcpyDeviceToDevice, st));
+        d.seg0 = k0;
+        o->window_fwd(d, k0, k1, da::W_STORE, st);
+        if ((r = check_launch(c))) return r;
+      }
+      d.seg0 = k0;
+      for (int k = k1; k > k0;) {  // to the next step whose spectra are recorded
+        int to = k0;
+        if (sp && sp->every > 0) to = std::max(k0, c->nsteps - ((c->nsteps - k) / sp->every + 1) * sp->every);
+        o->window_adj(d, k, to, sources, st);
+        if ((r = check_launch(c))) return r;
+        if ((r = record_spectra(c, sp, to, st))) return r;
+        k = to;
+      }
+      continue;
+    }
     if (seg != nseg - 1) {
       DA_TRY_CUDA(c, cudaMemcpyAsync(d.W, c->ckpt_buf + (size_t)seg * comp, comp * sizeof(double2),
                                      cudaMemcpyDeviceToDevice, st));

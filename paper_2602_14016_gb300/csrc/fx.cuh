@@ -448,20 +448,23 @@ __device__ __forceinline__ int mag_units(q2 a, q2 b) {
 __device__ __forceinline__ double pow2_double(int e) {  // 2^e, -1022 <= e <= 1023
   return __hiloint2double((e + 1023) << 20, 0);
 }
-__device__ __forceinline__ double fx_to_double(i64 v, int e) {
+// The scaling where 2^e is not an ordinary double: in steps, each within a
+// double's range.  Out of line: states in the ordinary range never come here.
+static __device__ __noinline__ double fx_scale_far(double d, int e) {
   if (e >= kBadExp) return __hiloint2double(0x7ff80000, 0);
-  const double d = (double)v;
-  if (e >= -960 && e <= 960) return d * pow2_double(e);
-  if (v == 0) return 0.0;
-  // outside that range the scaling goes in steps, each within a double's
+  if (d == 0.0) return 0.0;
   int left = max(min(e, 2200), -2200);
-  double r = d;
   while (left != 0) {
     const int s = max(min(left, 900), -900);
-    r *= pow2_double(s);
+    d *= pow2_double(s);
     left -= s;
   }
-  return r;
+  return d;
+}
+__device__ __forceinline__ double fx_to_double(i64 v, int e) {
+  const double d = (double)v;
+  if (e < -960 || e > 960) return fx_scale_far(d, e);
+  return d * pow2_double(e);
 }
 
 // Two real coefficients of a mode, a and b, as integers of one exponent: the

@@ -59,6 +59,13 @@ enum : int {
   F_SRC = 16       // adjoint column pass: add the observation source at this step
 };
 
+// Whole windows in one kernel (window.cuh).
+enum : int {
+  W_OBS = 1,    // forward: gather probes at the observation steps
+  W_STORE = 2,  // forward: write stage fields of the steps from seg0 on
+  W_FINAL = 4   // forward: gather the probes of the state after the last step
+};
+
 // Start of the adjoint sweep (k_adj_init): add the observation source of
 // the last step, and/or start from the terminal field already in LamBar; or
 // resume from the adjoint stage value in KB after a checkpoint recompute.
@@ -861,11 +868,16 @@ __device__ __forceinline__ q2 rho_products(q2 uv, q2 ab) {
   return mkq(mul_hi2(v, b, u, na), mul_hi2(u, b, v, a));
 }
 
-// Velocity at a probe of row y, column xx into its slot of the observations.
-__device__ __forceinline__ void put_probe(const Dev& d, int bm, int slot, int P, int st, int y, int xx, q2 uv, int e) {
-  double* o = d.obs + bm * d.obs_stride + ((size_t)slot * P * P + (y / st) * P + xx / st) * 2;
-  o[0] = fx_to_double(uv.x, e);
-  o[1] = fx_to_double(uv.y, e);
+// Velocity at a probe into its place o of the observations.  Out of line: few
+// steps have probes, and few threads one.
+static __device__ __noinline__ void put_probe(double* o, i64 u, i64 v, int e) {
+  o[0] = fx_to_double(u, e);
+  o[1] = fx_to_double(v, e);
+}
+// Place of the probe of row y, column xx of a member's slot (P probes a side,
+// st points apart).
+__device__ __forceinline__ double* probe_place(const Dev& d, int bm, int slot, int P, int st, int y, int xx) {
+  return d.obs + bm * d.obs_stride + ((size_t)slot * P * P + (y / st) * P + xx / st) * 2;
 }
 
 // First value of the stored stage fields of stage `stage` of step n, row y of
@@ -878,8 +890,8 @@ __device__ __forceinline__ size_t stored_row(const Dev& d, int bm, int n, int st
 // Row pass of stage `stage` (1..4) of step n: u, v of rows y0, y0+1; the
 // stage-field store and probe gather; the products u v and v^2 - u^2 of
 // each row (packed as P + i Q) and their forward transforms along x into
-// Mn.  grid (N/2, B).
-template <int N, int V = 0>
+// Mn.  OBS: with the probe gather.  grid (N/2, B).
+template <int N, int V, bool OBS>
 __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, int stage, int flags) {
   using P = FxPlan<N, V>;
   using RP = RowPoints<P>;
@@ -891,24 +903,31 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
   constexpr int Kc = Geo<N>::Kc;
   const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
   const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, d.eX + (size_t)bm * 2 * Kc, x);
-  const int Pp = mw.P, st = N / Pp;
-  const int slot = (flags & (F_OBS | F_OBS_ONLY)) ? obs_slot(d, n - mw.start) : -1;
   q2 z[RP::POINTS];
   const int ex = row_fields<P, RowBits<P>::UV>(in, x, d.fxtw, z, [] {});
   const size_t trow = stored_row<N>(d, bm, n, stage, y);
   const bool store = (flags & F_STORE) != 0;
   if (store && x.t == 0) d.eT[trow] = ex;
-  const bool probes = slot >= 0 && (y % st) == 0;
   if (RP::B::active(x.t)) {
+    if constexpr (OBS) {
+      const int st = N / mw.P, slot = obs_slot(d, n - mw.start);
+      if (slot >= 0 && (y % st) == 0) {
+#pragma unroll
+        for (int j = 0; j < RP::POINTS; ++j) {
+          const int xx = RP::x(x.t, j);
+          if ((xx % st) == 0) put_probe(probe_place(d, bm, slot, mw.P, st, y, xx), z[j].x, z[j].y, ex);
+        }
+      }
+    }
 #pragma unroll
     for (int j = 0; j < RP::POINTS; ++j) {
-      const int xx = RP::x(x.t, j);
-      if (store) d.traj[trow * N + xx] = z[j];
-      if (probes && (xx % st) == 0) put_probe(d, bm, slot, Pp, st, y, xx, z[j], ex);
+      if (store) d.traj[trow * N + RP::x(x.t, j)] = z[j];
       z[j] = uv_products(z[j]);
     }
   }
-  if (flags & F_OBS_ONLY) return;  // the final state: probes only
+  if constexpr (OBS) {
+    if (flags & F_OBS_ONLY) return;  // the final state: probes only
+  }
   const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
   store_row_pair<N, V>(d, bm, y0, x, 2 * ex + 64 + P::SHIFT + r);
 }

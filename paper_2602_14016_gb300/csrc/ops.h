@@ -30,6 +30,11 @@ struct Ops {
   void (*adj_init)(const Dev&, int mode, cudaStream_t);
   void (*adj_rows)(const Dev&, int n, int stage, cudaStream_t);
   void (*adj_cols)(const Dev&, int n, int stage, int flags, cudaStream_t);
+  // whole windows in one launch (window.cuh), for batches of at most
+  // window_batch members; 0: not for this grid
+  int window_batch;
+  void (*window_fwd)(const Dev&, int k0, int k1, int flags, cudaStream_t);
+  void (*window_adj)(const Dev&, int k1, int k0, int sources, cudaStream_t);
   void (*make_mult)(const Dev&, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                     cudaStream_t);
 };

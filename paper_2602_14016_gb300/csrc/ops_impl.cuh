@@ -1,8 +1,26 @@
 // ops_impl.cuh -- launch configurations of the pass kernels for one N.
 #pragma once
 #include "ops.h"
+#include "window.cuh"
 
 namespace da {
+
+// One cluster of C CTAs per member.
+template <int C, typename... A>
+inline void launch_clusters(void (*f)(A...), int members, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = C;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(members * C);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, f, args...);
+}
 
 template <int N, int V>
 Ops make_ops() {
@@ -29,13 +47,20 @@ Ops make_ops() {
     set((const void*)k_c2r_rows<N, V>, G::SMEM_FOLD);
     set((const void*)k_spec_to_mixed<N, V>, G::SMEM_FOLD);
     set((const void*)k_ctrl_cols<N, V>, G::SMEM_CTRL);
-    set((const void*)k_fwd_rows<N, V>);
+    set((const void*)k_fwd_rows<N, V, false>);
+    set((const void*)k_fwd_rows<N, V, true>);
     set((const void*)k_fwd_cols<N, V>);
     set((const void*)k_state_cols<N, V>);
     set((const void*)k_adj_init<N, V>, G::SMEM_FXP);
     set((const void*)k_adj_rows<N, V>);
     set((const void*)k_adj_cols<N, V, false>, G::SMEM_FXP);
     set((const void*)k_adj_cols<N, V, true>, G::SMEM_FXP);
+    if constexpr (WinGeo<N, V>::SUPPORTED) {
+      for (const void* f : {(const void*)k_window_fwd<N, V>, (const void*)k_window_adj<N, V>}) {
+        set(f, WinGeo<N, V>::SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      }
+    }
     return e;
   };
   o.r2c_rows = [](const Dev& d, const double* in, cudaStream_t st) {
@@ -57,7 +82,10 @@ Ops make_ops() {
     k_ctrl_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_CTRL, st>>>(d, flags);
   };
   o.fwd_rows = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_fwd_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
+    if (flags & (F_OBS | F_OBS_ONLY))
+      k_fwd_rows<N, V, true><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
+    else
+      k_fwd_rows<N, V, false><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
   };
   o.fwd_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
     k_fwd_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
@@ -75,6 +103,19 @@ Ops make_ops() {
     if (flags & F_SRC) k_adj_cols<N, V, true><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
     else k_adj_cols<N, V, false><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
   };
+  o.window_batch = 0;
+  o.window_fwd = nullptr;
+  o.window_adj = nullptr;
+  if constexpr (WinGeo<N, V>::SUPPORTED) {
+    using W = WinGeo<N, V>;
+    o.window_batch = 1 << 30;
+    o.window_fwd = [](const Dev& d, int k0, int k1, int flags, cudaStream_t st) {
+      launch_clusters<W::C>(k_window_fwd<N, V>, d.B, W::THREADS, W::SMEM, st, d, k0, k1, flags);
+    };
+    o.window_adj = [](const Dev& d, int k1, int k0, int sources, cudaStream_t st) {
+      launch_clusters<W::C>(k_window_adj<N, V>, d.B, W::THREADS, W::SMEM, st, d, k1, k0, sources);
+    };
+  }
   o.make_mult = [](const Dev& d, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                    cudaStream_t st) {
     k_make_mult<N, V><<<dim3((G::Kr * G::Kc + 255) / 256, d.B), 256, 0, st>>>(mult, kind, param, table, nu);

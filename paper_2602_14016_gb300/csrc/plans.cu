@@ -1,5 +1,6 @@
 // plans.cu -- FFT plan variants of the pass kernels and the autotuner
 // (da_plan_count, da_get_plan, da_set_plan, da_autotune of include/da.h).
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -84,6 +85,17 @@ static da_status tuning_steps(da_ctx* c, int steps, cudaStream_t st) {
   Dev d = c->dev;
   d.ragged = 0;  // every member works, whatever windows a ragged batch holds
   const bool store = d.traj != nullptr;
+  if (whole_windows(c)) {
+    const int most = store ? d.traj_steps : steps;
+    for (int i = 0; i < steps; i += most) {
+      const int k = std::min(most, steps - i);
+      o->window_fwd(d, 0, k, store ? da::W_STORE : 0, st);
+      if (store) o->window_adj(d, k, 0, 0, st);
+      da_status r = check_launch(c, store ? 2 : 1);
+      if (r) return r;
+    }
+    return DA_OK;
+  }
   for (int i = 0; i < steps; ++i) {
     const int k = store ? i % d.traj_steps : 0;
     for (int j = 1; j <= 4; ++j) {
