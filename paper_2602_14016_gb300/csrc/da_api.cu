@@ -117,12 +117,9 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   A(dalloc(c, (double**)&d.fold, fold_max));
   A(dalloc(c, (int4**)&d.fxtw, fx_max));
   A(dalloc(c, (double2**)&d.twP, (size_t)64));
-  A(dalloc(c, (da::Sym2**)&d.symF, comp / B));
-  A(dalloc(c, (da::Sym2**)&d.symA, comp / B));
-  A(dalloc(c, (da::FxPair**)&d.fxF, comp / B));
-  A(dalloc(c, (da::FxPair**)&d.fxA, comp / B));
-  A(dalloc(c, (int**)&d.fxFe, comp / B));
-  A(dalloc(c, (int**)&d.fxAe, comp / B));
+  A(dalloc(c, (da::ModeSym**)&d.symF, comp / B));
+  A(dalloc(c, (da::ModeSym**)&d.symA, comp / B));
+  A(dalloc(c, (double**)&d.nuk2, comp / B));
   A(dalloc(c, (double**)&d.k2, comp / B));
   A(dalloc(c, &c->d_mstart, B));
   A(dalloc(c, &c->d_mnt, B));
@@ -179,10 +176,8 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   // per-mode symbols of the column passes, column-major [Kc][Kr]
   const int K = ops->K, Kr = ops->Kr, Kc = ops->Kc;
   const size_t modes = (size_t)Kr * Kc;
-  std::vector<da::Sym2> symF(modes), symA(modes);
-  std::vector<da::FxPair> fxF(modes), fxA(modes);
-  std::vector<int> fxFe(modes), fxAe(modes);
-  std::vector<double> k2tab(modes);
+  std::vector<da::ModeSym> symF(modes), symA(modes);
+  std::vector<double> k2tab(modes), nuk2(modes);
   const double s2 = 1.0 / ((double)n * n);
   for (int kx = 0; kx < Kc; ++kx)
     for (int r = 0; r < Kr; ++r) {
@@ -190,21 +185,20 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
       const double k2 = (double)(kx * kx + ky * ky);
       const double ik2 = k2 > 0.0 ? 1.0 / k2 : 0.0;
       const size_t i = (size_t)kx * Kr + r;
-      symF[i] = {ky * ik2 * s2, kx * ik2 * s2};
-      symA[i] = {-2.0 * kx * ky * s2, (double)(ky * ky - kx * kx) * s2};
-      fxF[i] = da::fx_pair(0.5 * (ky * ky - kx * kx), -0.5 * kx * ky, &fxFe[i]);
-      fxA[i] = da::fx_pair(0.5 * ky * ik2, 0.5 * kx * ik2, &fxAe[i]);
+      // (a mode whose symbols vanish must not set its column's exponent)
+      symF[i].put = da::fx_pair(ky * ik2 * s2, kx * ik2 * s2, da::kZeroExp, &symF[i].put_e);
+      symF[i].get = da::fx_pair(0.5 * (ky * ky - kx * kx), -0.5 * kx * ky, 0, &symF[i].get_e);
+      symA[i].put = da::fx_pair(-2.0 * kx * ky * s2, (double)(ky * ky - kx * kx) * s2, da::kZeroExp, &symA[i].put_e);
+      symA[i].get = da::fx_pair(0.5 * ky * ik2, 0.5 * kx * ik2, 0, &symA[i].get_e);
+      nuk2[i] = nu * k2;
       k2tab[i] = k2;
     }
   auto upload = [&](const void* dst, const void* src, size_t bytes) {
     if (e == cudaSuccess) e = cudaMemcpy((void*)dst, src, bytes, cudaMemcpyHostToDevice);
   };
-  upload(d.symF, symF.data(), modes * sizeof(da::Sym2));
-  upload(d.symA, symA.data(), modes * sizeof(da::Sym2));
-  upload(d.fxF, fxF.data(), modes * sizeof(da::FxPair));
-  upload(d.fxA, fxA.data(), modes * sizeof(da::FxPair));
-  upload(d.fxFe, fxFe.data(), modes * sizeof(int));
-  upload(d.fxAe, fxAe.data(), modes * sizeof(int));
+  upload(d.symF, symF.data(), modes * sizeof(da::ModeSym));
+  upload(d.symA, symA.data(), modes * sizeof(da::ModeSym));
+  upload(d.nuk2, nuk2.data(), modes * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpy((void*)d.k2, k2tab.data(), k2tab.size() * sizeof(double), cudaMemcpyHostToDevice);
   {
     const std::vector<int> zeros(B, 0), nts(B, c->nt), pxs(B, c->P), forces(B, d.force);

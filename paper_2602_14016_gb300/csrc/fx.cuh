@@ -418,7 +418,7 @@ __device__ __forceinline__ int seq_sum_get(int v, const int* scratch) {
   return v;
 }
 
-// Inputs of an inverse transform have at most kInvBits bits; as the first
+// Inputs of an inverse transform have at most BITS bits (columns 60, rows 61); as the first
 // stage reads them, they are shifted (right with rounding, or left) until the
 // sum of their magnitudes has 62 bits, or up to G more (below).  The sum is
 // counted in units of 2^(32 + kSumDrop), one unit more for each group of up to
@@ -429,11 +429,11 @@ __device__ __forceinline__ int seq_sum_get(int v, const int* scratch) {
 // component, stay below 2^62.5: while the components have 62 - log2 R bits.
 // Nor may it have more than 60 + SHIFT_INV bits: the results then have 60,
 // and the row passes only ever shift them left (RowBits).
-constexpr int kInvBits = 61, kSumDrop = 12;
-template <typename P>
+constexpr int kSumDrop = 12;
+template <typename P, int BITS>
 __device__ __forceinline__ int inv_shift(int sum) {
   using I = typename P::inv;
-  constexpr int first = kInvBits - (62 - log2c(FirstRadix<I>::value));
+  constexpr int first = BITS - (62 - log2c(FirstRadix<I>::value));
   constexpr int G0 = stage_shift(FirstRadix<typename TailRadices<I>::type>::value);
   constexpr int G = G0 < P::SHIFT_INV - 2 ? G0 : P::SHIFT_INV - 2;
   const int r = bits32(sum) + 32 + kSumDrop - 62;
@@ -464,7 +464,8 @@ static __device__ __noinline__ double fx_scale_far(double d, int e) {
 __device__ __forceinline__ double fx_to_double(i64 v, int e) {
   const double d = (double)v;
   if (e < -960 || e > 960) return fx_scale_far(d, e);
-  return d * pow2_double(e);
+  // times 2^e by the exponent field: an FP64 product would cost a warp 64 clocks
+  return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
 }
 
 // Two real coefficients of a mode, a and b, as integers of one exponent: the
@@ -472,15 +473,21 @@ __device__ __forceinline__ double fx_to_double(i64 v, int e) {
 struct __align__(16) FxPair {
   int ah, al, bh, bl;
 };
-inline FxPair fx_pair(double a, double b, int* e) {
+// A pair of zeros gets the exponent zero_e.
+inline FxPair fx_pair(double a, double b, int zero_e, int* e) {
   const double big = std::fmax(std::fabs(a), std::fabs(b));
-  *e = 0;
+  *e = zero_e;
   if (big == 0.0) return {0, 0, 0, 0};
   std::frexp(big, e);
   *e -= 62;
   const i64 x = (i64)std::ldexp(a, -*e), y = (i64)std::ldexp(b, -*e);  // the smaller may lose what lies below a unit
   const int2 a2 = fx_words(x), b2 = fx_words(y);
   return {a2.x, a2.y, b2.x, b2.y};
+}
+// a b / 2^64 of two factors in words.
+__device__ __forceinline__ i64 mul_hi(Words a, Words b) {
+  const i64 mid = madw(a.h, b.l, madw(a.l, b.h, kHalfWord));
+  return madw(a.h, b.h, (i64)(int)(mid >> 32));
 }
 // (a p + SG b q) / 2^64, |p|, |q| < 2^61.5.
 template <int SG>
@@ -505,7 +512,7 @@ __device__ __forceinline__ i64 double_to_fx(double d, int e) {
   const int f = (hi >> 20) & 0x7ff;
   // 53-bit significand m, value m 2^(f - 1075): m 2^9 >> r
   const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
-  const int r = min(9 - (f - 1075 - e), 63);
+  const int r = (int)min((unsigned)(9 - (f - 1075 - e)), 63u);
   const i64 q = f == 0 ? 0 : (m << 9) >> r;
   return hi < 0 ? -q : q;
 }
@@ -617,7 +624,7 @@ __device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int
 }
 
 // Inverse transform (S = +1) of the sequence in src, zero outside the band
-// KB: the inputs, of at most kInvBits bits, are shifted right by pre (left by
+// KB: the inputs are shifted right by pre (left by
 // -pre) first,
 // and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
 // is left in registers: out[jb R + m] is position t + jb TPS + m N / R for R

@@ -75,20 +75,19 @@ enum : int { INIT_SRC = 1, INIT_LAMBAR = 2, INIT_RESUME = 4 };
 enum : int { M_ONE = 0, M_CTRL = 1, M_FILTERED = 2, M_INV_CTRL = 3 };
 
 // Per-mode constants of the column passes, column-major [Kc][Kr] (entry
-// kx * Kr + r), computed once on the host so that no column pass divides or
-// converts integers in FP64:
-//   fwd: symF = su = ky/k^2/N^2, sv = kx/k^2/N^2 (u, v columns of a state
-//        value); fxF = cp = (ky^2 - kx^2)/2, cq = -kx ky/2 (advection symbols;
+// kx * Kr + r), computed once on the host: pairs of real symbols as integers
+// of one exponent (fx_pair), since an FP64 product costs a warp 64 clocks of
+// its SM's quarter and the integer one a fifth of that:
+//   fwd: put = su = ky/k^2/N^2, sv = kx/k^2/N^2 (u, v columns of a state
+//        value); get = cp = (ky^2 - kx^2)/2, cq = -kx ky/2 (advection symbols;
 //        the 1/2 is the one the row pass leaves out when it unpacks two real
 //        rows);
-//   adj: symA = ca = -2 kx ky/N^2, cb = (ky^2 - kx^2)/N^2 (adjoint-field
-//        columns; ca carries the 2 of rho_u, rho_v); fxA = a1 = ky/k^2/2, c1 =
-//        kx/k^2/2 (transposed velocity symbols, same 1/2);
-//   k2 = k^2 (the column passes multiply it by the member's viscosity).
-// fxF and fxA multiply integer transforms before the conversion to doubles:
-// one conversion per component instead of two, and no FP64 products.
-struct __align__(16) Sym2 {
-  double a, b;
+//   adj: put = ca = -2 kx ky/N^2, cb = (ky^2 - kx^2)/N^2 (adjoint-field
+//        columns; ca carries the 2 of rho_u, rho_v); get = a1 = ky/k^2/2, c1 =
+//        kx/k^2/2 (transposed velocity symbols, same 1/2).
+struct __align__(16) ModeSym {
+  FxPair get, put;
+  int get_e, put_e, pad0, pad1;
 };
 
 // Everything a kernel needs, passed by value.
@@ -127,13 +126,10 @@ struct Dev {
   const double* fold;                        // folded twiddles of Plan<N> (fft.cuh)
   const int4* fxtw;                          // integer twiddles of FxPlan<N> (fx.cuh)
   const double2* twP;                        // W_64^t, t < 64 (W_P^t = W_64^{t 64/P})
-  const Sym2* symF;                          // [Kc][Kr] su, sv
-  const Sym2* symA;                          // [Kc][Kr] ca, cb
-  const FxPair* fxF;                         // [Kc][Kr] cp, cq
-  const FxPair* fxA;                         // [Kc][Kr] a1, c1
-  const int* fxFe;                           // [Kc][Kr] exponents of fxF
-  const int* fxAe;                           // [Kc][Kr] exponents of fxA
-  const double* k2;                          // [Kc][Kr] k^2 (times nu of the member)
+  const ModeSym* symF;                       // [Kc][Kr] forward
+  const ModeSym* symA;                       // [Kc][Kr] adjoint
+  const double* k2;                          // [Kc][Kr] k^2
+  const double* nuk2;                        // [Kc][Kr] nu k^2, the context's nu
   double dt2, dt3, dt6;                      // dt/2, dt/3, dt/6
 };
 
@@ -425,47 +421,57 @@ __device__ __forceinline__ int2 pair_reduce2(int a, int b, int pt, int* scratch)
   return make_int2(a, b);
 }
 
-// A column under construction: the doubles a thread puts at its retained rows
-// rr = pt + j PT of the two fields, and the largest exponent fields.
+// A column under construction: the integers a thread puts at its retained rows
+// rr = pt + j PT of the two fields, each mode at its own exponent, and the
+// largest of those.
 template <typename P>
 struct ColumnPut {
   static constexpr int PT = Place<P>::PT;
   static constexpr int MT = (Geo<P::N>::Kr + PT - 1) / PT;
-  double2 v0[MT], v1[MT];
-  int f0 = 0, f1 = 0;
-  __device__ __forceinline__ void put(int j, double2 a, double2 b) {
-    v0[j] = a;
-    v1[j] = b;
-    f0 = max(f0, max(exp_field(a.x), exp_field(a.y)));
-    f1 = max(f1, max(exp_field(b.x), exp_field(b.y)));
+  q2 v0[MT], v1[MT];
+  int e[MT];
+  int top = 2 * kZeroExp;
+  __device__ __forceinline__ void zero(int j) {
+    v0[j] = v1[j] = mkq(0, 0);
+    e[j] = 2 * kZeroExp;
+  }
+  // the pair c times the value y: (a y.x, a y.y), (b y.x, b y.y), of at most
+  // 60 bits
+  __device__ __forceinline__ void times(int j, const FxPair& c, int ce, double2 y) {
+    const int em = exp_for<62>(max(exp_field(y.x), exp_field(y.y)));
+    const Words yx(double_to_fx(y.x, em)), yy(double_to_fx(y.y, em)), a(c.ah, c.al), b(c.bh, c.bl);
+    v0[j] = mkq(mul_hi(yx, a), mul_hi(yy, a));
+    v1[j] = mkq(mul_hi(yx, b), mul_hi(yy, b));
+    e[j] = em + 64 + ce;
+    top = max(top, e[j]);
   }
 };
 
-// The two column values u = i ky/k^2 Yv, v = -i kx/k^2 Yv (scaled by 1/N^2;
-// f = symF entry of the mode) as entry j.
+// The two column values u = i ky/k^2 y, v = -i kx/k^2 y of a state value y
+// (scaled by 1/N^2) as entry j.
 template <typename P>
-__device__ __forceinline__ void put_stage_columns(ColumnPut<P>& c, int j, const Sym2& f, double2 Yv) {
-  c.put(j, make_double2(-f.a * Yv.y, f.a * Yv.x),  // u:  i ky / k^2
-        make_double2(f.b * Yv.y, -f.b * Yv.x));    // v: -i kx / k^2
+__device__ __forceinline__ void put_stage_columns(ColumnPut<P>& c, int j, const ModeSym& s, double2 y) {
+  c.times(j, s.put, s.put_e, y);
+  c.v0[j] = mkq(-c.v0[j].y, c.v0[j].x);  // i a y
+  c.v1[j] = mkq(c.v1[j].y, -c.v1[j].x);  // -i b y
 }
 
 // The two column values of the adjoint fields of an adjoint stage value kb:
 // 2a = 2 d_xy kb = -2 kx ky kb and b = (d_xx - d_yy) kb = (ky^2 - kx^2) kb,
-// scaled by 1/N^2 (g = symA entry of the mode).
+// scaled by 1/N^2.
 template <typename P>
-__device__ __forceinline__ void put_adjoint_columns(ColumnPut<P>& c, int j, const Sym2& g, double2 kb) {
-  c.put(j, cscale(kb, g.a), cscale(kb, g.b));
+__device__ __forceinline__ void put_adjoint_columns(ColumnPut<P>& c, int j, const ModeSym& s, double2 kb) {
+  c.times(j, s.put, s.put_e, kb);
 }
 
-// Both columns put in c: to integers in the pair's src buffers (free to write
-// after a barrier), inverse transform along y; store(y, value) gets this
+// Both columns put in c: at one exponent into the pair's src buffers (free to
+// write after a barrier), inverse transform along y; store(y, value) gets this
 // thread's results of its own sequence.  Returns the sequence's exponent.
 template <typename P, typename Store>
 __device__ __forceinline__ int finish_columns(const ColumnPut<P>& c, Place<P>& x, const int4* tw, Store store) {
   using G = Geo<P::N>;
   constexpr int N = P::N, PT = Place<P>::PT, GAP = N - 2 * G::K - 1;
-  const int2 f = pair_reduce2<P, false>(c.f0, c.f1, x.pt, x.pscratch);
-  const int e0 = exp_for<kInvBits>(f.x), e1 = exp_for<kInvBits>(f.y);
+  const int e0 = pair_reduce2<P, false>(c.top, c.top, x.pt, x.pscratch).x;
   q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
   unsigned s0 = 0, s1 = 0;
 #pragma unroll
@@ -473,8 +479,8 @@ __device__ __forceinline__ int finish_columns(const ColumnPut<P>& c, Place<P>& x
     const int rr = x.pt + j * PT;
     if (rr >= G::Kr) break;
     const int q = pad(ky_of_row(rr, G::K) & (N - 1));
-    const q2 u = mkq(double_to_fx(c.v0[j].x, e0), double_to_fx(c.v0[j].y, e0));
-    const q2 v = mkq(double_to_fx(c.v1[j].x, e1), double_to_fx(c.v1[j].y, e1));
+    const ShiftRight down(e0 - c.e[j]);
+    const q2 u = down(c.v0[j]), v = down(c.v1[j]);
     s0 += mag_units(u, mkq(0, 0));
     s1 += mag_units(v, mkq(0, 0));
     a0[q] = u;
@@ -482,7 +488,7 @@ __device__ __forceinline__ int finish_columns(const ColumnPut<P>& c, Place<P>& x
   }
   for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(G::K + 1 + u)] = mkq(0, 0);
   const int2 sum = pair_reduce2<P, true>(s0, s1, x.pt, x.pscratch + x.PAIR);
-  const int pre = inv_shift<P>(x.f ? sum.y : sum.x);
+  const int pre = inv_shift<P, 60>(x.f ? sum.y : sum.x);
   constexpr int R = LastRadix<typename P::inv>::value;
   using B = Bfly<P, R>;
   q2 out[B::POINTS];
@@ -493,7 +499,7 @@ __device__ __forceinline__ int finish_columns(const ColumnPut<P>& c, Place<P>& x
 #pragma unroll
       for (int m = 0; m < R; ++m) store(x.t + jb * P::TPS + m * B::NB, out[jb * R + m]);
   }
-  return clamp_exp((x.f ? e1 : e0) + pre + P::SHIFT_INV);
+  return clamp_exp(e0 + pre + P::SHIFT_INV);
 }
 
 // finish_columns into column kx of both fields of Mx.
@@ -576,30 +582,21 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
   }
 }
 
-// The constants of one mode in a column pass (see Sym2).
-struct ModeConst {
-  Sym2 s;
-  FxPair c;
-  int ce;
-  double k2;
-};
-__device__ __forceinline__ ModeConst mode_fwd(const Dev& d, int i) {
-  return {d.symF[i], d.fxF[i], d.fxFe[i], d.k2[i]};
-}
-__device__ __forceinline__ ModeConst mode_adj(const Dev& d, int i) {
-  return {d.symA[i], d.fxA[i], d.fxAe[i], d.k2[i]};
+// nu k^2 of mode i for a member.
+__device__ __forceinline__ double mode_nuk2(const Dev& d, const MemberWindow& mw, int i) {
+  return d.ragged ? mw.nu * d.k2[i] : d.nuk2[i];
 }
 
 // One mode of the forward column pass: p, q the transforms of u v and v^2 -
 // u^2 at exponent e; w the state at the step's start, y the stage value, acc
 // the RK sum.  Updates w (stage 4), y and acc.  forced: the mode carries the
 // force's coefficient fval.
-__device__ __forceinline__ void rk_mode(const Dev& d, int stage, const ModeConst& m, double nk2, q2 p, q2 q, int e,
+__device__ __forceinline__ void rk_mode(const Dev& d, int stage, const ModeSym& m, double nk2, q2 p, q2 q, int e,
                                         bool forced, double fval, double2& w, double2& y, double2& acc) {
   // F = -(cp P + cq Q) - nu k^2 y
-  const int eF = e + 64 + m.ce;
-  const double ax = fx_to_double(fx_pair_sum<1>(m.c, p.x, q.x), eF);
-  const double ay = fx_to_double(fx_pair_sum<1>(m.c, p.y, q.y), eF);
+  const int eF = e + 64 + m.get_e;
+  const double ax = fx_to_double(fx_pair_sum<1>(m.get, p.x, q.x), eF);
+  const double ay = fx_to_double(fx_pair_sum<1>(m.get, p.y, q.y), eF);
   double2 F = make_double2(-fma(nk2, y.x, ax), -fma(nk2, y.y, ay));
   if (forced) F.x += fval;
   if (stage == 1) {
@@ -621,12 +618,12 @@ __device__ __forceinline__ void rk_mode(const Dev& d, int stage, const ModeConst
 // rho_u, rho_v at exponent e; kb the stage value, lb lambda at the step's end,
 // sum the stages' sum.  Updates sum, kb (the next stage's) and, on stage 1, lb
 // (lambda at the step's start; src: the observation source there).
-__device__ __forceinline__ void adj_mode(const Dev& d, int stage, const ModeConst& m, double nk2, q2 ru, q2 rv, int e,
+__device__ __forceinline__ void adj_mode(const Dev& d, int stage, const ModeSym& m, double nk2, q2 ru, q2 rv, int e,
                                          bool has_src, double2 src, double2& kb, double2& lb, double2& sum) {
   // t = (-i ky/k^2) Ru + (i kx/k^2) Rv (the 1/2 of the row unpack in a1, c1)
-  const int eR = e + 64 + m.ce;
-  const double2 tt = make_double2(fx_to_double(fx_pair_sum<-1>(m.c, ru.y, rv.y), eR),
-                                  -fx_to_double(fx_pair_sum<-1>(m.c, ru.x, rv.x), eR));
+  const int eR = e + 64 + m.get_e;
+  const double2 tt = make_double2(fx_to_double(fx_pair_sum<-1>(m.get, ru.y, rv.y), eR),
+                                  -fx_to_double(fx_pair_sum<-1>(m.get, ru.x, rv.x), eR));
   double2 yb;
   yb.x = -fma(nk2, kb.x, tt.x);
   yb.y = -fma(nk2, kb.y, tt.y);
@@ -732,6 +729,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_state_cols(Dev d) {
 // along x as field 0 + i field 1: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B) for the
 // mixed half spectra A, B (kx = 0..K); the DC bin keeps real parts only; the
 // gap is zeroed.  Into the sequence's src buffer, synchronised.
+constexpr int kRowBits = 61;
 struct RowLoad {
   int e;    // exponent of the row as it stands in src
   int pre;  // shift its inverse transform starts with
@@ -754,7 +752,7 @@ __device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2*
     }
   }
   for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(K + 1 + u)] = mkq(0, 0);
-  // one exponent for the row, at which its largest component has kInvBits - 1
+  // one exponent for the row, at which its largest component has kRowBits - 1
   // bits (sums of two have one more): the columns' own exponents would leave
   // the small ones to be rounded at the unit of the largest
 #pragma unroll
@@ -766,7 +764,7 @@ __device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2*
   }
   e = seq_max_put<P::TPS>(e, x.t, x.scratch);
   if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
-  e = seq_max_get<P::TPS>(e, x.scratch) - (kInvBits - 1);
+  e = seq_max_get<P::TPS>(e, x.scratch) - (kRowBits - 1);
   int sum = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
@@ -784,7 +782,7 @@ __device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2*
   }
   sum = seq_sum_put<P::TPS>(sum, x.t, x.scratch + P::WARPS);
   seq_sync<P::TPS>(x.f);
-  return {e, inv_shift<P>(seq_sum_get<P::TPS>(sum, x.scratch + P::WARPS))};
+  return {e, inv_shift<P, kRowBits>(seq_sum_get<P::TPS>(sum, x.scratch + P::WARPS))};
 }
 
 // Forward transforms along x of rows y0, y0+1, sequence f packed as (field 0
@@ -953,7 +951,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
   // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
   ColumnPut<P> put;
   double2 yv[put.MT], wv[put.MT], accv[put.MT];
-  ModeConst mc[put.MT];
+  ModeSym mc[put.MT];
+  double nk2[put.MT];
   auto load_inputs = [&](int t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr < G::Kr) {
@@ -961,7 +960,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
       yv[t] = d.Y[idx];
       wv[t] = d.W[idx];
       accv[t] = stage > 1 ? d.Acc[idx] : make_double2(0.0, 0.0);
-      mc[t] = mode_fwd(d, kx * G::Kr + rr);
+      mc[t] = d.symF[kx * G::Kr + rr];
+      nk2[t] = mode_nuk2(d, mw, kx * G::Kr + rr);
     }
   };
   const int e = forward_columns<P>(d.Mn + (((size_t)bm * G::Kc + kx) * 2 + x.f) * N, d.eN + bm * N, x, d.fxtw, [&] {
@@ -980,12 +980,12 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
     const int ky = ky_of_row(rr, G::K);
     const int qi = pad(ky & (N - 1));
     const size_t idx = cidx<N>(bm, rr, kx);
-    rk_mode(d, stage, mc[t], mw.nu * mc[t].k2, a0[qi], a1[qi], e, forced_mode(d, mw, kx, ky), fval, wv[t], yv[t],
+    rk_mode(d, stage, mc[t], nk2[t], a0[qi], a1[qi], e, forced_mode(d, mw, kx, ky), fval, wv[t], yv[t],
             accv[t]);
     if (stage < 4) d.Acc[idx] = accv[t];
     else d.W[idx] = wv[t];
     d.Y[idx] = yv[t];
-    put_stage_columns(put, t, mc[t].s, yv[t]);
+    put_stage_columns(put, t, mc[t], yv[t]);
   }
   if (flags & F_NO_NEXT) return;
   swap_bufs<P>(x.src, x.dst);
@@ -1154,7 +1154,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
   // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
   ColumnPut<P> put;
   double2 kbv[put.MT], lbv[put.MT], sumv[put.MT];
-  ModeConst mc[put.MT];
+  ModeSym mc[put.MT];
+  double nk2[put.MT];
   auto load_inputs = [&](int t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr < G::Kr) {
@@ -1162,7 +1163,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
       kbv[t] = d.KB[idx];
       lbv[t] = d.LamBar[idx];
       sumv[t] = stage < 4 ? d.Sum[idx] : make_double2(0.0, 0.0);
-      mc[t] = mode_adj(d, kx * G::Kr + rr);
+      mc[t] = d.symA[kx * G::Kr + rr];
+      nk2[t] = mode_nuk2(d, mw, kx * G::Kr + rr);
     }
   };
   const int slot = SRC ? obs_slot(d, n - mw.start) : -1;
@@ -1188,11 +1190,11 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
     if constexpr (SRC) {
       if (slot >= 0) src = probe_source(d, mw.P, kx, ky, Tu, Tv);
     }
-    adj_mode(d, stage, mc[t], mw.nu * mc[t].k2, a0[qi], a1[qi], e, slot >= 0, src, kbv[t], lbv[t], sumv[t]);
+    adj_mode(d, stage, mc[t], nk2[t], a0[qi], a1[qi], e, slot >= 0, src, kbv[t], lbv[t], sumv[t]);
     if (stage > 1) d.Sum[idx] = sumv[t];
     else d.LamBar[idx] = lbv[t];
     d.KB[idx] = kbv[t];
-    put_adjoint_columns(put, t, mc[t].s, kbv[t]);
+    put_adjoint_columns(put, t, mc[t], kbv[t]);
   }
   if (stage == 1 && n == mw.start) return;  // the member's first step: lambda_0 stays in LamBar
   swap_bufs<P>(x.src, x.dst);

@@ -135,16 +135,18 @@ __global__ void __launch_bounds__(WinGeo<N, V>::THREADS) k_window_fwd(Dev d, int
   const bool final_probes = (flags & W_FINAL) != 0;
   if (first > k1 || (first == k1 && !final_probes)) return;  // nothing of the member's window here
   double2 ws[Wn::MT], ys[Wn::MT], acc[Wn::MT];
-  ModeConst mc[Wn::MT];
+  ModeSym mc[Wn::MT];
+  double nk2[Wn::MT];
   ColumnPut<P> put;
 #pragma unroll
   for (int j = 0; j < Wn::MT; ++j) {
     const int rr = w.has(j) ? w.mode(j) : 0;
-    mc[j] = mode_fwd(d, w.kxs * G::Kr + rr);
+    mc[j] = d.symF[w.kxs * G::Kr + rr];
+    nk2[j] = mode_nuk2(d, mw, w.kxs * G::Kr + rr);
     ws[j] = w.has(j) ? d.W[cidx<N>(bm, rr, w.kx)] : make_double2(0.0, 0.0);
     ys[j] = ws[j];
     acc[j] = make_double2(0.0, 0.0);
-    put_stage_columns(put, j, mc[j].s, ys[j]);
+    put_stage_columns(put, j, mc[j], ys[j]);
   }
   Wn::sync();  // every CTA of the cluster runs
   w.send_columns(put, d.fxtw);
@@ -180,18 +182,18 @@ __global__ void __launch_bounds__(WinGeo<N, V>::THREADS) k_window_fwd(Dev d, int
       // column pass
       const int e = w.take_columns(d.fxtw);
       const q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
-      put.f0 = put.f1 = 0;
+      put.top = 2 * kZeroExp;
 #pragma unroll
       for (int j = 0; j < Wn::MT; ++j) {
         if (!w.has(j)) {
-          put.v0[j] = put.v1[j] = make_double2(0.0, 0.0);
+          put.zero(j);
           continue;
         }
         const int ky = ky_of_row(w.mode(j), G::K);
         const int qi = pad(ky & (N - 1));
-        rk_mode(d, stage, mc[j], mw.nu * mc[j].k2, a0[qi], a1[qi], e, forced_mode(d, mw, w.kx, ky), fval, ws[j], ys[j],
+        rk_mode(d, stage, mc[j], nk2[j], a0[qi], a1[qi], e, forced_mode(d, mw, w.kx, ky), fval, ws[j], ys[j],
                 acc[j]);
-        put_stage_columns(put, j, mc[j].s, ys[j]);
+        put_stage_columns(put, j, mc[j], ys[j]);
       }
       if (stage == 4 && n == k1 - 1 && !final_probes) break;  // nothing reads the columns
       w.send_columns(put, d.fxtw);
@@ -220,17 +222,19 @@ __global__ void __launch_bounds__(WinGeo<N, V>::THREADS) k_window_adj(Dev d, int
   const int last = max(k0, mw.start);
   if (last >= k1) return;  // nothing of the member's window here
   double2 kb[Wn::MT], lb[Wn::MT], sum[Wn::MT];
-  ModeConst mc[Wn::MT];
+  ModeSym mc[Wn::MT];
+  double nk2[Wn::MT];
   ColumnPut<P> put;
 #pragma unroll
   for (int j = 0; j < Wn::MT; ++j) {
     const int rr = w.has(j) ? w.mode(j) : 0;
-    mc[j] = mode_adj(d, w.kxs * G::Kr + rr);
+    mc[j] = d.symA[w.kxs * G::Kr + rr];
+    nk2[j] = mode_nuk2(d, mw, w.kxs * G::Kr + rr);
     const size_t idx = cidx<N>(bm, rr, w.kxs);
     kb[j] = w.has(j) ? d.KB[idx] : make_double2(0.0, 0.0);
     lb[j] = w.has(j) ? d.LamBar[idx] : make_double2(0.0, 0.0);
     sum[j] = make_double2(0.0, 0.0);
-    put_adjoint_columns(put, j, mc[j].s, kb[j]);
+    put_adjoint_columns(put, j, mc[j], kb[j]);
   }
   Wn::sync();  // every CTA of the cluster runs
   w.send_columns(put, d.fxtw);
@@ -263,19 +267,19 @@ __global__ void __launch_bounds__(WinGeo<N, V>::THREADS) k_window_adj(Dev d, int
       if (slot >= 0 && w.column) probe_row_sums(d, bm, mw.P, slot, w.kx, x.pt, Place<P>::PT, Tu, Tv);
       const int e = w.take_columns(d.fxtw);  // ends with the pair's barrier
       const q2 *a0 = x.first(x.src), *a1 = a0 + x.OTHER;
-      put.f0 = put.f1 = 0;
+      put.top = 2 * kZeroExp;
 #pragma unroll
       for (int j = 0; j < Wn::MT; ++j) {
         if (!w.has(j)) {
-          put.v0[j] = put.v1[j] = make_double2(0.0, 0.0);
+          put.zero(j);
           continue;
         }
         const int ky = ky_of_row(w.mode(j), G::K);
         const int qi = pad(ky & (N - 1));
         double2 src = make_double2(0.0, 0.0);
         if (slot >= 0) src = probe_source(d, mw.P, w.kx, ky, Tu, Tv);
-        adj_mode(d, stage, mc[j], mw.nu * mc[j].k2, a0[qi], a1[qi], e, slot >= 0, src, kb[j], lb[j], sum[j]);
-        put_adjoint_columns(put, j, mc[j].s, kb[j]);
+        adj_mode(d, stage, mc[j], nk2[j], a0[qi], a1[qi], e, slot >= 0, src, kb[j], lb[j], sum[j]);
+        put_adjoint_columns(put, j, mc[j], kb[j]);
       }
       if (stage == 1 && n == last) break;  // nothing reads the columns
       w.send_columns(put, d.fxtw);
