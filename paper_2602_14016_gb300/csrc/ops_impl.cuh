@@ -108,7 +108,7 @@ Ops make_ops() {
   o.window_adj = nullptr;
   if constexpr (WinGeo<N, V>::SUPPORTED) {
     using W = WinGeo<N, V>;
-    o.window_batch = 1 << 30;
+    o.window_batch = W::BATCH;
     o.window_fwd = [](const Dev& d, int k0, int k1, int flags, cudaStream_t st) {
       launch_clusters<W::C>(k_window_fwd<N, V>, d.B, W::THREADS, W::SMEM, st, d, k0, k1, flags);
     };

@@ -27,6 +27,14 @@ struct WinGeo {
   using G = Geo<N>;
   static constexpr bool SUPPORTED = N <= 64;
   static constexpr int C = N == 16 ? 1 : N == 32 ? 4 : 16;
+  // Largest batch that runs this way: beyond it the pass kernels, which spread
+  // a batch over the whole chip, are the faster ones.  us a pass by captured
+  // graphs, this way / pass kernels: 64^2 plans 0, 1, 2 at 13 members 4.4/5.3,
+  // 6.6/6.6, 3.8/4.5, at 24 members 5.4/5.5, 7.9/6.8, 6.4/5.2; 32^2 plans 0, 1
+  // at 64 members 5.6/5.2, 3.6/4.4, at 256 members 12.5/10.7, 8.1/7.8; 16^2 at
+  // 1 member 3.9/3.8, at 256 members 4.1/5.2.  Launched directly, a pass
+  // kernel costs the host 6 us, which decides for this way at 16^2 and 32^2.
+  static constexpr int BATCH = N == 16 ? 1 << 30 : N == 32 ? 128 : V == 1 ? 4 : 16;
   static constexpr int ROWS = N / C, COLS = (G::Kc + C - 1) / C;
   static constexpr int RMAX = FirstRadix<typename Plan<N, V>::two>::value;
   static constexpr int TPS = N / (RMAX < 4 ? 2 : 4) < 32 ? N / (RMAX < 4 ? 2 : 4) : 32;
