@@ -109,12 +109,8 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   A(dalloc(c, &d.res, B * c->nt * P2 * 2));
   A(dalloc(c, &d.J, B));
   A(dalloc(c, (double**)&d.mult, comp));
-  size_t fold_max = 0, fx_max = 0;  // room for the twiddle tables of any plan variant
-  for (int v = 0; v < da::plan_count(n); ++v) {
-    fold_max = std::max(fold_max, (size_t)da::ops_for(n, v)->fold_doubles);
-    fx_max = std::max(fx_max, (size_t)da::ops_for(n, v)->fx_entries);
-  }
-  A(dalloc(c, (double**)&d.fold, fold_max));
+  size_t fx_max = 0;  // room for the twiddle tables of any plan variant
+  for (int v = 0; v < da::plan_count(n); ++v) fx_max = std::max(fx_max, (size_t)da::ops_for(n, v)->fx_entries);
   A(dalloc(c, (int4**)&d.fxtw, fx_max));
   A(dalloc(c, (double2**)&d.twP, (size_t)64));
   A(dalloc(c, (da::ModeSym**)&d.symF, comp / B));
@@ -155,12 +151,8 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
     da_destroy(c);
     return s;
   }
-  // constant tables: folded twiddles of the FFT plan, twiddles of the probe
-  // lattice
-  std::vector<double> fold(ops->fold_doubles);
-  ops->fold_table(fold.data());
-  std::vector<int4> fxtw(ops->fx_entries);
-  ops->fx_table(fxtw.data());
+  // constant tables: twiddles of the FFT plan and of the probe lattice
+  const std::vector<int4>& fxtw = ops->fx_table();
   std::vector<double2> twP = roots_of_unity(64);
   std::vector<int>& kind = c->h_kind;
   std::vector<double>& param = c->h_param;
@@ -170,36 +162,8 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
     kind[b] = kernels[b].kind;
     param[b] = kernels[b].param;
   }
-  cudaError_t e = cudaMemcpy((void*)d.fold, fold.data(), fold.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy((void*)d.fxtw, fxtw.data(), fxtw.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpy((void*)d.fxtw, fxtw.data(), fxtw.size() * sizeof(int4), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy((void*)d.twP, twP.data(), 64 * sizeof(double2), cudaMemcpyHostToDevice);
-  // per-mode symbols of the column passes, column-major [Kc][Kr]
-  const int K = ops->K, Kr = ops->Kr, Kc = ops->Kc;
-  const size_t modes = (size_t)Kr * Kc;
-  std::vector<da::ModeSym> symF(modes), symA(modes);
-  std::vector<double> k2tab(modes), nuk2(modes);
-  const double s2 = 1.0 / ((double)n * n);
-  for (int kx = 0; kx < Kc; ++kx)
-    for (int r = 0; r < Kr; ++r) {
-      const int ky = r <= K ? r : r - Kr;
-      const double k2 = (double)(kx * kx + ky * ky);
-      const double ik2 = k2 > 0.0 ? 1.0 / k2 : 0.0;
-      const size_t i = (size_t)kx * Kr + r;
-      // (a mode whose symbols vanish must not set its column's exponent)
-      symF[i].put = da::fx_pair(ky * ik2 * s2, kx * ik2 * s2, da::kZeroExp, &symF[i].put_e);
-      symF[i].get = da::fx_pair(0.5 * (ky * ky - kx * kx), -0.5 * kx * ky, 0, &symF[i].get_e);
-      symA[i].put = da::fx_pair(-2.0 * kx * ky * s2, (double)(ky * ky - kx * kx) * s2, da::kZeroExp, &symA[i].put_e);
-      symA[i].get = da::fx_pair(0.5 * ky * ik2, 0.5 * kx * ik2, 0, &symA[i].get_e);
-      nuk2[i] = nu * k2;
-      k2tab[i] = k2;
-    }
-  auto upload = [&](const void* dst, const void* src, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMemcpy((void*)dst, src, bytes, cudaMemcpyHostToDevice);
-  };
-  upload(d.symF, symF.data(), modes * sizeof(da::ModeSym));
-  upload(d.symA, symA.data(), modes * sizeof(da::ModeSym));
-  upload(d.nuk2, nuk2.data(), modes * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemcpy((void*)d.k2, k2tab.data(), k2tab.size() * sizeof(double), cudaMemcpyHostToDevice);
   {
     const std::vector<int> zeros(B, 0), nts(B, c->nt), pxs(B, c->P), forces(B, d.force);
     const std::vector<double> nus(B, nu);
@@ -222,13 +186,14 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
     da_destroy(c);
     return DA_ECUDA;
   }
-  // the multiplier on a stream of its own, waited for alone (a device-wide
+  // the per-mode tables and the multiplier on a stream of its own, waited for alone (a device-wide
   // wait would also disturb other threads' work, e.g. a graph capture)
   cudaStream_t mk = nullptr;
   e = cudaStreamCreateWithFlags(&mk, cudaStreamNonBlocking);
   if (e == cudaSuccess) {
+    ops->make_symbols(d, nu, mk);
     ops->make_mult(d, (double*)d.mult, d_kind, d_param, d_table, c->d_mnu, mk);
-    c->launches++;
+    c->launches += 2;
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(mk);
     cudaStreamDestroy(mk);
@@ -325,7 +290,7 @@ static da_status run_forward(da_ctx* c, const double* s, bool gather, cudaStream
   c->have_fwd = false;
   const bool whole = whole_windows(c);
   o->r2c_rows(d, s, st);
-  o->ctrl_cols(d, whole ? da::F_NO_NEXT : 0, st);
+  o->ctrl_cols(d, !whole, st);
   da_status r = check_launch(c, 2);
   if (r) return r;
   if (c->w0) DA_TRY_CUDA(c, cudaMemcpyAsync(c->w0, d.W, comp * sizeof(double2), cudaMemcpyDeviceToDevice, st));
@@ -357,7 +322,7 @@ static da_status run_forward(da_ctx* c, const double* s, bool gather, cudaStream
         o->fwd_rows(d, k, j, store_flag | (j == 1 ? obs_flag : 0), st);
       }
       Timed t(c, 2, st);
-      o->fwd_cols(d, k, j, 0, st);
+      o->fwd_cols(d, k, j, st);
     }
     if ((r = check_launch(c, 8))) return r;
   }
@@ -450,7 +415,7 @@ static da_status run_adjoint(da_ctx* c, bool sources, cudaStream_t st, const Spe
             o->fwd_rows(d, k, j, da::F_STORE, st);
           }
           Timed t(c, 2, st);
-          o->fwd_cols(d, k, j, 0, st);
+          o->fwd_cols(d, k, j, st);
         }
         if ((r = check_launch(c, 8))) return r;
       }
@@ -906,7 +871,7 @@ extern "C" da_status da_omega_from_control(da_ctx* c, const double* s, double* o
   if (!c || !s || !omega0) return fail(c, DA_EINVAL, "arguments must not be NULL");
   cudaStream_t st = (cudaStream_t)stream;
   c->ops->r2c_rows(c->dev, s, st);
-  c->ops->ctrl_cols(c->dev, da::F_NO_NEXT, st);
+  c->ops->ctrl_cols(c->dev, false, st);
   c->ops->compact_to_half(c->dev, c->dev.W, (double2*)omega0, st);
   return check_launch(c, 3);
 }

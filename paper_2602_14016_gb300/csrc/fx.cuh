@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <vector>
 
 #include "fft.cuh"
 
@@ -296,7 +297,7 @@ using FxPlan = FxPlanOf<N, PlanInfo<N, V>::THREADS / 2, typename Plan<N, V>::two
 
 // Signed words (hi, lo) of a coefficient; a low word of -2^31, which could
 // not be negated, is moved by one unit (2^-62).
-inline int2 fx_words(i64 v) {
+__host__ __device__ inline int2 fx_words(i64 v) {
   if ((unsigned)v == 0x80000000u) ++v;
   const int lo = (int)(unsigned)v;
   return make_int2((int)((v - lo) >> 32), lo);
@@ -324,10 +325,17 @@ inline void fx_fill(int4* out, Radices<R, Rs...>) {
   fx_fill<L * R>(out, Radices<Rs...>{});
 }
 
+// The two tables of a plan, computed on first use (a long double cosine is
+// software on some hosts: 6 ms for 1024 points).
 template <typename P>
-inline void fx_table(int4* out) {
-  fx_fill<1>(out, typename P::fwd{});
-  fx_fill<1>(out + P::ENTRIES, typename P::inv{});
+inline const std::vector<int4>& fx_table() {
+  static const std::vector<int4> table = [] {
+    std::vector<int4> t(P::TABLE);
+    fx_fill<1>(t.data(), typename P::fwd{});
+    fx_fill<1>(t.data() + P::ENTRIES, typename P::inv{});
+    return t;
+  }();
+  return table;
 }
 
 // ---------------------------------------------------------------------------
@@ -469,21 +477,12 @@ __device__ __forceinline__ double fx_to_double(i64 v, int e) {
 }
 
 // Two real coefficients of a mode, a and b, as integers of one exponent: the
-// larger of |a|, |b| has 62 bits; words (a_hi, a_lo, b_hi, b_lo).
+// larger of |a|, |b| has 62 bits (the smaller may lose what lies below a
+// unit); words (a_hi, a_lo, b_hi, b_lo).
 struct __align__(16) FxPair {
   int ah, al, bh, bl;
 };
-// A pair of zeros gets the exponent zero_e.
-inline FxPair fx_pair(double a, double b, int zero_e, int* e) {
-  const double big = std::fmax(std::fabs(a), std::fabs(b));
-  *e = zero_e;
-  if (big == 0.0) return {0, 0, 0, 0};
-  std::frexp(big, e);
-  *e -= 62;
-  const i64 x = (i64)std::ldexp(a, -*e), y = (i64)std::ldexp(b, -*e);  // the smaller may lose what lies below a unit
-  const int2 a2 = fx_words(x), b2 = fx_words(y);
-  return {a2.x, a2.y, b2.x, b2.y};
-}
+
 // a b / 2^64 of two factors in words.
 __device__ __forceinline__ i64 mul_hi(Words a, Words b) {
   const i64 mid = madw(a.h, b.l, madw(a.l, b.h, kHalfWord));
@@ -515,6 +514,15 @@ __device__ __forceinline__ i64 double_to_fx(double d, int e) {
   const int r = (int)min((unsigned)(9 - (f - 1075 - e)), 63u);
   const i64 q = f == 0 ? 0 : (m << 9) >> r;
   return hi < 0 ? -q : q;
+}
+
+// The pair of coefficients a, b and its exponent; a pair of zeros gets zero_e.
+__device__ __forceinline__ FxPair fx_pair(double a, double b, int zero_e, int* e) {
+  const int f = max(exp_field(a), exp_field(b));
+  *e = f == 0 ? zero_e : exp_for<62>(f);
+  if (f == 0) return {0, 0, 0, 0};
+  const int2 x = fx_words(double_to_fx(a, *e)), y = fx_words(double_to_fx(b, *e));
+  return {x.x, x.y, y.x, y.y};
 }
 
 // ---------------------------------------------------------------------------

@@ -16,8 +16,7 @@
 //                    the adjoint row pass.
 // Mixed and stage fields are 64-bit integers (fx.cuh) with one exponent per
 // column and field (Mx) or per row (Mn, stage fields) beside them; compact
-// spectra, observations, controls and gradients are doubles.  (The control
-// maps use Mn as a field of doubles.)
+// spectra, observations, controls and gradients are doubles.
 //
 // The advection term is evaluated in the divergence form of Basdevant
 // (1983): for a divergence-free band-limited velocity,
@@ -35,9 +34,8 @@
 // pass (forward transforms along y of the two products, the advection term,
 // RK epilogue with viscosity, forcing and the stage update, then the
 // inverse column transforms of the next stage's u and v).  The adjoint
-// mirrors this with the transposed operators.  Every transform between the
-// control and its gradient is an integer FFT from fx.cuh; those of the control
-// maps are FP64 FFTs from fft.cuh.  The 1/N^2 of the inverse 2D transform is
+// mirrors this with the transposed operators.  Every transform is an integer
+// FFT from fx.cuh.  The 1/N^2 of the inverse 2D transform is
 // applied once, to the spectral coefficients before the column transform.
 // Every inverse transform here reads a sequence that is zero in the gap
 // K < q < N - K, and every forward transform is read back only on the band
@@ -55,8 +53,7 @@ enum : int {
   F_STORE = 1,     // forward row pass: write stage fields
   F_OBS = 2,       // forward row pass: gather probes into the observation slot
   F_OBS_ONLY = 4,  // forward row pass: only gather probes (final state)
-  F_NO_NEXT = 8,   // column pass: skip the inverse transforms of the next stage
-  F_SRC = 16       // adjoint column pass: add the observation source at this step
+  F_SRC = 8       // adjoint column pass: add the observation source at this step
 };
 
 // Whole windows in one kernel (window.cuh).
@@ -75,7 +72,7 @@ enum : int { INIT_SRC = 1, INIT_LAMBAR = 2, INIT_RESUME = 4 };
 enum : int { M_ONE = 0, M_CTRL = 1, M_FILTERED = 2, M_INV_CTRL = 3 };
 
 // Per-mode constants of the column passes, column-major [Kc][Kr] (entry
-// kx * Kr + r), computed once on the host: pairs of real symbols as integers
+// kx * Kr + r), computed once (k_make_symbols): pairs of real symbols as integers
 // of one exponent (fx_pair), since an FP64 product costs a warp 64 clocks of
 // its SM's quarter and the integer one a fifth of that:
 //   fwd: put = su = ky/k^2/N^2, sv = kx/k^2/N^2 (u, v columns of a state
@@ -123,7 +120,6 @@ struct Dev {
   double* res;                               // residuals [B][nt][P2][2]
   double* J;                                 // [B]
   const double* mult;                        // control multiplier |k| W^1/2, compact [B][Kc][Kr]
-  const double* fold;                        // folded twiddles of Plan<N> (fft.cuh)
   const int4* fxtw;                          // integer twiddles of FxPlan<N> (fx.cuh)
   const double2* twP;                        // W_64^t, t < 64 (W_P^t = W_64^{t 64/P})
   const ModeSym* symF;                       // [Kc][Kr] forward
@@ -142,16 +138,12 @@ struct Geo {
   // threads: two transforms at a time (fft.cuh)
   static constexpr int THREADS = PlanInfo<N, V>::THREADS;
   static constexpr int PMAX = 64;
-  // shared memory of the control maps: folded twiddle table + one sequence
   static constexpr size_t SMEM = sizeof(double2) * 2 * N;  // static_ctrl.cu: plain table and one sequence
-  static constexpr size_t SMEM_FOLD = sizeof(double) * FoldInfo<N, V>::PADDED + sizeof(double2) * (N + 2);
   // passes that run the integer transforms: the buffers of two sequences,
   // scratch of the reductions (Place), and probe sums (adjoint column passes)
   static constexpr int SCRATCH = ((3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS + 3) / 4 * 4;
   static constexpr size_t SMEM_FX = sizeof(q2) * (2 * FxPlan<N, V>::BUFS * FxPlan<N, V>::SEQ) + sizeof(int) * SCRATCH;
   static constexpr size_t SMEM_FXP = SMEM_FX + sizeof(double2) * 2 * PMAX;
-  // k_ctrl_cols runs both: the FP64 part first, in the same memory
-  static constexpr size_t SMEM_CTRL = SMEM_FOLD > SMEM_FX ? SMEM_FOLD : SMEM_FX;
   // Column passes: small grids leave most of the chip idle, so a warp's own
   // latency counts, and they load their epilogue inputs before the transforms
   // (about 60 more registers a thread); larger ones hide it behind other
@@ -167,11 +159,6 @@ __device__ __forceinline__ int ky_of_row(int r, int K) { return r <= K ? r : r -
 template <int N>
 __host__ __device__ __forceinline__ size_t cidx(int bm, int r, int kx) {
   return ((size_t)bm * Geo<N>::Kc + kx) * Geo<N>::Kr + r;
-}
-
-template <int N, int V = 0>
-__device__ __forceinline__ void load_fold(double* T, const double* __restrict__ g) {
-  for (int i = threadIdx.x; i < FoldInfo<N, V>::DOUBLES; i += blockDim.x) T[i] = g[i];
 }
 
 // The window of member bm in this evaluation (see Dev).
@@ -193,36 +180,6 @@ __device__ __forceinline__ int obs_slot(const Dev& d, int k) {
   return k / d.every - 1 + (d.include_t0 ? 1 : 0);
 }
 
-// Full-length sequence whose inverse transform is a + i b, for two real rows
-// a, b given by their mixed half spectra A, B (kx = 0..K): Z(kx) = A + iB,
-// Z(-kx) = conj(A) + i conj(B); the DC bin keeps real parts only.  Every
-// coefficient is loaded once and written to kx and -kx; the gap
-// K < kx < N-K is zeroed.  Coefficient kx of A and Bv is at [kx * STRIDE].
-// Loops run over compile-time trip counts so that a thread's loads are
-// issued together.
-template <int N, int T, int STRIDE = 1>
-__device__ __forceinline__ void pack_rows(double2* seq, const double2* __restrict__ A, const double2* __restrict__ Bv) {
-  constexpr int K = Geo<N>::K, GAP = N - 2 * K - 1;
-#pragma unroll
-  for (int t = 0; t < (GAP + T - 1) / T; ++t) {
-    const int u = threadIdx.x + t * T;
-    if (u < GAP) seq[K + 1 + u] = make_double2(0.0, 0.0);
-  }
-#pragma unroll
-  for (int t = 0; t < (K + 1 + T - 1) / T; ++t) {
-    const int kx = threadIdx.x + t * T;
-    if (kx <= K) {
-      const double2 p = A[(size_t)kx * STRIDE], q = Bv[(size_t)kx * STRIDE];
-      if (kx == 0) {
-        seq[0] = make_double2(p.x, q.x);
-      } else {
-        seq[kx] = make_double2(p.x - q.y, p.y + q.x);
-        seq[N - kx] = make_double2(p.x + q.y, q.x - p.y);
-      }
-    }
-  }
-}
-
 // The two half spectra packed in a forward transform Z of a + i b:
 // A(k) = (Z(k) + conj Z(-k))/2, B(k) = -i (Z(k) - conj Z(-k))/2.
 template <int N, int V = 0>
@@ -232,92 +189,6 @@ __device__ __forceinline__ void unpack_pair(const double2* Z, int kx, double2& A
   const double tx = zk.x - zm.x, ty = zk.y + zm.y;
   A = make_double2(0.5 * sx, 0.5 * sy);
   Bv = make_double2(0.5 * ty, -0.5 * tx);
-}
-
-// ---------------------------------------------------------------------------
-// Generic row transforms (control map, gradient map)
-// ---------------------------------------------------------------------------
-
-// Real rows in[b][y][x] -> mixed half rows Mn[b][y][kx], kx <= K (forward,
-// unnormalised), two rows per complex transform.  grid (N/2, B).
-template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_r2c_rows(Dev d, const double* __restrict__ in) {
-  using G = Geo<N, V>;
-  extern __shared__ double2 sm[];
-  double* T = reinterpret_cast<double*>(sm);
-  double2* a = sm + FoldInfo<N, V>::PADDED / 2;
-  const int bm = blockIdx.y, y0 = 2 * blockIdx.x;
-  load_fold<N, V>(T, d.fold);
-  const double* r0 = in + ((size_t)bm * N + y0) * N;
-  #pragma unroll
-  for (int x = threadIdx.x; x < N; x += G::THREADS) a[x] = make_double2(r0[x], r0[N + x]);
-  __syncthreads();
-  fft_folded<N, V, -1, 1, -1, G::K>(a, T);
-  double2* M = reinterpret_cast<double2*>(d.Mn) + (size_t)bm * G::Kc * 2 * N + y0;  // field 0, rows y0 and y0 + 1
-  #pragma unroll
-  for (int kx = threadIdx.x; kx < G::Kc; kx += G::THREADS) {
-    double2 A, Bv;
-    unpack_pair<N>(a, kx, A, Bv);
-    M[(size_t)kx * 2 * N] = A;
-    M[(size_t)kx * 2 * N + 1] = Bv;
-  }
-}
-
-// Mixed half rows Mn[b][y][kx] -> real rows out[b][y][x] (the inverse along
-// x; the 1/N^2 is already in Mn), two rows per complex transform.
-template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_c2r_rows(Dev d, double* __restrict__ out) {
-  using G = Geo<N, V>;
-  extern __shared__ double2 sm[];
-  double* T = reinterpret_cast<double*>(sm);
-  double2* a = sm + FoldInfo<N, V>::PADDED / 2;
-  const int bm = blockIdx.y, y0 = 2 * blockIdx.x;
-  load_fold<N, V>(T, d.fold);
-  const double2* M = reinterpret_cast<const double2*>(d.Mn) + (size_t)bm * G::Kc * 2 * N + y0;  // field 0, rows y0 and y0 + 1
-  pack_rows<N, G::THREADS, 2 * N>(a, M, M + 1);
-  __syncthreads();
-  fft_folded<N, V, +1, 1, G::K>(a, T);
-  double* r0 = out + ((size_t)bm * N + y0) * N;
-  #pragma unroll
-  for (int x = threadIdx.x; x < N; x += G::THREADS) {
-    r0[x] = a[x].x;
-    r0[N + x] = a[x].y;
-  }
-}
-
-// Compact spectrum src[b] times a multiplier (and 1/N^2), transformed along
-// y -> mixed Mn[b] (first field).  grid (Kc, B).
-template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_spec_to_mixed(Dev d, const double2* __restrict__ src, int mode) {
-  using G = Geo<N, V>;
-  extern __shared__ double2 sm[];
-  double* T = reinterpret_cast<double*>(sm);
-  double2* a = sm + FoldInfo<N, V>::PADDED / 2;
-  const int kx = blockIdx.x, bm = blockIdx.y;
-  load_fold<N, V>(T, d.fold);
-  const double s = 1.0 / ((double)N * N);
-  #pragma unroll
-  for (int q = threadIdx.x; q < N; q += G::THREADS) {
-    const int ky = q < N / 2 ? q : q - N;
-    double2 v = make_double2(0.0, 0.0);
-    if (ky >= -G::K && ky <= G::K) {
-      const int r = ky >= 0 ? ky : ky + G::Kr;
-      const size_t idx = cidx<N>(bm, r, kx);
-      const double m = d.mult[idx];
-      double f;
-      if (mode == M_ONE) f = 1.0;
-      else if (mode == M_CTRL) f = m;
-      else if (mode == M_FILTERED) f = (kx == 0 && ky == 0) ? 0.0 : m * m / sqrt((double)(kx * kx + ky * ky));
-      else f = m != 0.0 ? 1.0 / m : 0.0;
-      v = cscale(src[idx], f * s);
-    }
-    a[q] = v;
-  }
-  __syncthreads();
-  fft_folded<N, V, +1, 1, G::K>(a, T);
-  double2* M = reinterpret_cast<double2*>(d.Mn) + ((size_t)bm * G::Kc + kx) * 2 * N;  // field 0 of column kx
-  #pragma unroll
-  for (int y = threadIdx.x; y < N; y += G::THREADS) M[y] = a[y];
 }
 
 // Compact <-> half-spectrum copies.  grid (ceil(N*NH/256), B), block 256.
@@ -349,7 +220,7 @@ __global__ void k_half_to_compact(const double2* __restrict__ in, double2* __res
 }
 
 // ---------------------------------------------------------------------------
-// Control map and the inverse column transforms of a stage state
+// Column passes: parts, and the inverse column transforms of a stage state
 // ---------------------------------------------------------------------------
 
 // A thread's place in a column pass: sequence f of its column, thread t of
@@ -513,9 +384,10 @@ __device__ __forceinline__ void finish_to_mixed(const Dev& d, const ColumnPut<P>
 
 // Forward transform along y of a sequence of the pair (M: its N values; eN:
 // the exponents of the N rows), left in the src buffers with one exponent for
-// both sequences, which is returned, and one bit to spare; synchronised over
-// the pair.  `between` runs after the loads are issued.
-template <typename P, typename Between>
+// both sequences (COMMON; else one each), which is returned, and one bit to
+// spare; synchronised over the pair.  `between` runs after the loads are
+// issued.
+template <typename P, bool COMMON = true, typename Between>
 __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const int* __restrict__ eN, Place<P>& x,
                                                const int4* __restrict__ tw, Between between) {
   using G = Geo<P::N>;
@@ -551,7 +423,13 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
       big = max_mag(big, v[j]);
     }
   }
-  big = pair_reduce2<P, false>(big, big, x.pt, x.pscratch).x;
+  if constexpr (COMMON) {
+    big = pair_reduce2<P, false>(big, big, x.pt, x.pscratch).x;
+  } else {
+    big = seq_max_put<P::TPS>(big, x.t, x.scratch + 2 * P::WARPS);
+    if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+    big = seq_max_get<P::TPS>(big, x.scratch + 2 * P::WARPS);
+  }
   const int sh = BITS - bits64(big);
   e0 -= sh;
   if (B::active(x.t)) {
@@ -564,7 +442,7 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
     }
   }
   const int r = fx_forward<P, G::K, MEASURE, 1>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
-  if constexpr (MEASURE) {  // results of two shifts: bring both to the larger one
+  if constexpr (MEASURE && COMMON) {  // results of two shifts: bring both to the larger one
     if (x.t == 0) x.scratch[0] = r;
     pair_sync<P>();
     const int rm = max(x.seq_scratch(0)[0], x.seq_scratch(1)[0]);
@@ -578,7 +456,7 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
     return clamp_exp(e0 + rm + P::SHIFT);
   } else {
     pair_sync<P>();
-    return clamp_exp(e0 + P::SHIFT);
+    return clamp_exp(e0 + r + P::SHIFT);
   }
 }
 
@@ -665,40 +543,6 @@ __device__ __forceinline__ double2* pass_probe_sums(void* base) {
   return reinterpret_cast<double2*>(static_cast<char*>(base) + Geo<N, V>::SMEM_FX);
 }
 
-// s_hat = forward transform along y of the mixed rows in Mn (doubles here,
-// from k_r2c_rows); w0 = mult s_hat into W (and Y); then, unless F_NO_NEXT,
-// the inverse column transforms of u and v of stage 1.  grid (Kc, B).
-template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d, int flags) {
-  using G = Geo<N, V>;
-  extern __shared__ double2 sm[];
-  double* T = reinterpret_cast<double*>(sm);
-  double2* a = sm + FoldInfo<N, V>::PADDED / 2;
-  const int kx = blockIdx.x, bm = blockIdx.y;
-  load_fold<N, V>(T, d.fold);
-  const double2* M = reinterpret_cast<const double2*>(d.Mn) + ((size_t)bm * G::Kc + kx) * 2 * N;
-#pragma unroll
-  for (int y = threadIdx.x; y < N; y += G::THREADS) a[y] = M[y];
-  __syncthreads();
-  fft_folded<N, V, -1, 1, -1, G::K>(a, T);
-  ColumnPut<FxPlan<N, V>> put;
-#pragma unroll
-  for (int j = 0; j < put.MT; ++j) {
-    const int rr = threadIdx.x + j * G::THREADS;
-    if (rr >= G::Kr) break;
-    const int ky = ky_of_row(rr, G::K);
-    const size_t idx = cidx<N>(bm, rr, kx);
-    const double2 w0 = cscale(a[ky & (N - 1)], d.mult[idx]);
-    d.W[idx] = w0;
-    d.Y[idx] = w0;
-    put_stage_columns(put, j, d.symF[kx * G::Kr + rr], w0);
-  }
-  if (flags & F_NO_NEXT) return;
-  __syncthreads();  // the FP64 part's memory is read no more
-  Place<FxPlan<N, V>> x = pass_place<N, V>(sm);
-  finish_to_mixed(d, put, x, bm, kx);
-}
-
 // Restart from the compact state in W (a checkpoint): Y = W and the inverse
 // column transforms of u and v of stage 1.  grid (Kc, B).
 template <int N, int V = 0>
@@ -724,9 +568,9 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_state_cols(Dev d) {
 // Row passes
 // ---------------------------------------------------------------------------
 
-// A row of the two mixed fields (MA, MB: its Kc values each; eX: the exponents
-// of the Kc columns, field 0 then field 1), packed for the inverse transform
-// along x as field 0 + i field 1: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B) for the
+// A row of each of two mixed fields (MA, MB: Kc values each; eA, eB: the
+// exponents of the Kc columns), packed for the inverse transform along x as
+// the first + i the second: Z(kx) = A + iB, Z(-kx) = conj(A) + i conj(B) for the
 // mixed half spectra A, B (kx = 0..K); the DC bin keeps real parts only; the
 // gap is zeroed.  Into the sequence's src buffer, synchronised.
 constexpr int kRowBits = 61;
@@ -735,8 +579,8 @@ struct RowLoad {
   int pre;  // shift its inverse transform starts with
 };
 template <typename P>
-__device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2* __restrict__ MB, const int* __restrict__ eX,
-                                            Place<P>& x) {
+__device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2* __restrict__ MB,
+                                            const int* __restrict__ eA, const int* __restrict__ eB, Place<P>& x) {
   using G = Geo<P::N>;
   constexpr int N = P::N, K = G::K, Kc = G::Kc, GAP = N - 2 * K - 1, J = (Kc + P::TPS - 1) / P::TPS;
   q2 p[J], q[J];
@@ -747,8 +591,8 @@ __device__ __forceinline__ RowLoad load_row(const q2* __restrict__ MA, const q2*
     if (kx < Kc) {
       p[j] = MA[kx];
       q[j] = MB[kx];
-      ep[j] = eX[kx];
-      eq[j] = eX[Kc + kx];
+      ep[j] = eA[kx];
+      eq[j] = eB[kx];
     }
   }
   for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(K + 1 + u)] = mkq(0, 0);
@@ -900,7 +744,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
   if (n < mw.start) return;  // the member's window has not begun
   constexpr int Kc = Geo<N>::Kc;
   const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
-  const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, d.eX + (size_t)bm * 2 * Kc, x);
+  const int* eX = d.eX + (size_t)bm * 2 * Kc;
+  const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, eX, eX + Kc, x);
   q2 z[RP::POINTS];
   const int ex = row_fields<P, RowBits<P>::UV>(in, x, d.fxtw, z, [] {});
   const size_t trow = stored_row<N>(d, bm, n, stage, y);
@@ -931,6 +776,174 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
 }
 
 // ---------------------------------------------------------------------------
+// Control map, its inverse and the gradient map
+// ---------------------------------------------------------------------------
+//
+// One real field: two rows make one complex sequence, and the two sequences of
+// a CTA are two pairs of rows, or two columns (the second of the last pair a
+// copy of the first where Kc is odd).
+
+// Real rows in[b][y][x] -> mixed half rows in field 0 of Mn (forward along x,
+// unnormalised).  grid (N/4, B).
+template <int N, int V = 0>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_r2c_rows(Dev d, const double* __restrict__ in) {
+  using P = FxPlan<N, V>;
+  using G = Geo<N>;
+  extern __shared__ double2 sm[];
+  Place<P> x = pass_place<N, V>(sm);
+  const int bm = blockIdx.y, y0 = 4 * blockIdx.x + 2 * x.f;
+  constexpr int R = FirstRadix<typename P::fwd>::value;
+  constexpr bool MEASURE = P::GROWTH >= P::GROWTH1 + 1;
+  constexpr int BITS = MEASURE ? 62 - P::GROWTH1 : P::BITS_FWD - 1;
+  using B = Bfly<P, R>;
+  const double* r0 = in + ((size_t)bm * N + y0) * N;
+  double2 v[B::POINTS];
+  int f = 0;
+  if (B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < B::POINTS; ++j) {
+      const int xx = x.t + (j / R) * P::TPS + (j % R) * B::NB;
+      v[j] = make_double2(r0[xx], r0[N + xx]);
+      f = max(f, max(exp_field(v[j].x), exp_field(v[j].y)));
+    }
+  }
+  f = seq_max_put<P::TPS>(f, x.t, x.scratch);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  const int e = exp_for<BITS>(seq_max_get<P::TPS>(f, x.scratch));
+  q2 z[B::POINTS];
+  if (B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < B::POINTS; ++j) z[j] = mkq(double_to_fx(v[j].x, e), double_to_fx(v[j].y, e));
+  }
+  const int r = fx_forward<P, G::K, MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch + P::WARPS);
+  q2* M = d.Mn + (size_t)bm * G::Kc * 2 * N + y0;
+  for (int kx = x.t; kx < G::Kc; kx += P::TPS) {
+    const q2 zk = x.src[pad(kx)], zm = x.src[pad((N - kx) & (N - 1))];
+    q2* o = M + (size_t)kx * 2 * N;
+    o[0] = mkq(zk.x + zm.x, zk.y - zm.y);
+    o[1] = mkq(zk.y + zm.y, zm.x - zk.x);
+  }
+  if (x.t < 2) d.eN[bm * N + y0 + x.t] = clamp_exp(e + r + P::SHIFT - 1);  // the sums are twice the spectra
+}
+
+// s_hat = forward transform along y of field 0 of Mn; w0 = mult s_hat into W.
+// NEXT: also into Y, and the inverse column transforms of u and v of stage 1;
+// a CTA then has one column, which both its sequences transform.
+// grid ((Kc + 1) / 2, B), with NEXT (Kc, B).
+template <int N, int V, bool NEXT>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d) {
+  using P = FxPlan<N, V>;
+  using G = Geo<N, V>;
+  extern __shared__ double2 sm[];
+  Place<P> x = pass_place<N, V>(sm);
+  const int bm = blockIdx.y, kx = NEXT ? (int)blockIdx.x : min(2 * (int)blockIdx.x + x.f, G::Kc - 1);
+  const int e =
+      forward_columns<P, false>(d.Mn + ((size_t)bm * G::Kc + kx) * 2 * N, d.eN + bm * N, x, d.fxtw, [] {});
+  auto w0 = [&](int rr, const q2* a) {
+    const size_t idx = cidx<N>(bm, rr, kx);
+    const q2 z = a[pad(ky_of_row(rr, G::K) & (N - 1))];
+    const double2 w = cscale(make_double2(fx_to_double(z.x, e), fx_to_double(z.y, e)), d.mult[idx]);
+    d.W[idx] = w;
+    if constexpr (NEXT) d.Y[idx] = w;
+    return w;
+  };
+  if constexpr (NEXT) {
+    ColumnPut<P> put;
+#pragma unroll
+    for (int j = 0; j < put.MT; ++j) {
+      const int rr = threadIdx.x + j * G::THREADS;
+      if (rr >= G::Kr) break;
+      put_stage_columns(put, j, d.symF[kx * G::Kr + rr], w0(rr, x.first(x.src)));
+    }
+    swap_bufs<P>(x.src, x.dst);
+    finish_to_mixed(d, put, x, bm, kx);
+  } else {
+    for (int rr = x.t; rr < G::Kr; rr += P::TPS) w0(rr, x.src);
+  }
+}
+
+// Compact spectrum src[b] times a multiplier (and 1/N^2), transformed along
+// y -> field 0 of Mx.  grid ((Kc + 1) / 2, B).
+template <int N, int V = 0>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_spec_to_mixed(Dev d, const double2* __restrict__ src, int mode) {
+  using P = FxPlan<N, V>;
+  using G = Geo<N>;
+  extern __shared__ double2 sm[];
+  Place<P> x = pass_place<N, V>(sm);
+  const int bm = blockIdx.y, kx = min(2 * (int)blockIdx.x + x.f, G::Kc - 1);
+  constexpr int MT = (G::Kr + P::TPS - 1) / P::TPS, GAP = N - 2 * G::K - 1;
+  const double s = 1.0 / ((double)N * N);
+  double2 v[MT];
+  int top = 0;
+#pragma unroll
+  for (int j = 0; j < MT; ++j) {
+    const int rr = x.t + j * P::TPS;
+    if (rr >= G::Kr) break;
+    const int ky = ky_of_row(rr, G::K);
+    const size_t idx = cidx<N>(bm, rr, kx);
+    const double m = d.mult[idx];
+    double f;
+    if (mode == M_ONE) f = 1.0;
+    else if (mode == M_CTRL) f = m;
+    else if (mode == M_FILTERED) f = (kx == 0 && ky == 0) ? 0.0 : m * m / sqrt((double)(kx * kx + ky * ky));
+    else f = m != 0.0 ? 1.0 / m : 0.0;
+    v[j] = cscale(src[idx], f * s);
+    top = max(top, max(exp_field(v[j].x), exp_field(v[j].y)));
+  }
+  top = seq_max_put<P::TPS>(top, x.t, x.scratch);
+  if constexpr (P::TPS > 32) seq_sync<P::TPS>(x.f);
+  const int e = exp_for<60>(seq_max_get<P::TPS>(top, x.scratch));
+  int sum = 0;
+#pragma unroll
+  for (int j = 0; j < MT; ++j) {
+    const int rr = x.t + j * P::TPS;
+    if (rr >= G::Kr) break;
+    const q2 z = mkq(double_to_fx(v[j].x, e), double_to_fx(v[j].y, e));
+    sum += mag_units(z, mkq(0, 0));
+    x.src[pad(ky_of_row(rr, G::K) & (N - 1))] = z;
+  }
+  for (int u = x.t; u < GAP; u += P::TPS) x.src[pad(G::K + 1 + u)] = mkq(0, 0);
+  sum = seq_sum_put<P::TPS>(sum, x.t, x.scratch + P::WARPS);
+  seq_sync<P::TPS>(x.f);
+  const int pre = inv_shift<P, 60>(seq_sum_get<P::TPS>(sum, x.scratch + P::WARPS));
+  using RP = RowPoints<P>;
+  q2 z[RP::POINTS];
+  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, pre, z);
+  q2* M = d.Mx + (size_t)bm * 2 * N * G::Kc + kx;
+  if (RP::B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < RP::POINTS; ++j) M[(size_t)RP::x(x.t, j) * G::Kc] = z[j];
+  }
+  if (x.t == 0) d.eX[bm * 2 * G::Kc + kx] = clamp_exp(e + pre + P::SHIFT_INV);
+}
+
+// Mixed half rows of field 0 of Mx -> real rows out[b][y][x] (the inverse
+// along x; the 1/N^2 is already in Mx).  grid (N/4, B).
+template <int N, int V = 0>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_c2r_rows(Dev d, double* __restrict__ out) {
+  using P = FxPlan<N, V>;
+  using G = Geo<N>;
+  using RP = RowPoints<P>;
+  extern __shared__ double2 sm[];
+  Place<P> x = pass_place<N, V>(sm);
+  const int bm = blockIdx.y, y0 = 4 * blockIdx.x + 2 * x.f;
+  const q2* M = d.Mx + ((size_t)bm * 2 * N + y0) * G::Kc;
+  const int* eX = d.eX + (size_t)bm * 2 * G::Kc;
+  const RowLoad in = load_row<P>(M, M + G::Kc, eX, eX, x);
+  q2 z[RP::POINTS];
+  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, in.pre, z);
+  const int e = clamp_exp(in.e + in.pre + P::SHIFT_INV);
+  double* r0 = out + ((size_t)bm * N + y0) * N;
+  if (RP::B::active(x.t)) {
+#pragma unroll
+    for (int j = 0; j < RP::POINTS; ++j) {
+      r0[RP::x(x.t, j)] = fx_to_double(z[j].x, e);
+      r0[N + RP::x(x.t, j)] = fx_to_double(z[j].y, e);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Forward RK stage: column pass
 // ---------------------------------------------------------------------------
 
@@ -940,7 +953,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
 // transforms of u and v of the next stage state.  Acc holds k1 + 2 k2 +
 // 2 k3 (+ k4).  grid (Kc, B).
 template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd_cols(Dev d, int n, int stage, int flags) {
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd_cols(Dev d, int n, int stage) {
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
@@ -987,7 +1000,6 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
     d.Y[idx] = yv[t];
     put_stage_columns(put, t, mc[t], yv[t]);
   }
-  if (flags & F_NO_NEXT) return;
   swap_bufs<P>(x.src, x.dst);
   finish_to_mixed(d, put, x, bm, kx);
 }
@@ -1117,7 +1129,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
   if (d.ragged && n < d.mstart[bm]) return;
   constexpr int Kc = Geo<N>::Kc;
   const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
-  const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, d.eX + (size_t)bm * 2 * Kc, x);
+  const int* eX = d.eX + (size_t)bm * 2 * Kc;
+  const RowLoad in = load_row<P>(MA, MA + (size_t)N * Kc, eX, eX + Kc, x);
   const size_t trow = stored_row<N>(d, bm, n, stage, y);
   q2 z[RP::POINTS], uv[RP::POINTS];
   const int ex = row_fields<P, RowBits<P>::AB>(in, x, d.fxtw, z, [&] {
@@ -1199,6 +1212,31 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
   if (stage == 1 && n == mw.start) return;  // the member's first step: lambda_0 stays in LamBar
   swap_bufs<P>(x.src, x.dst);
   finish_to_mixed(d, put, x, bm, kx);
+}
+
+// Per-mode constants of the column passes (ModeSym), k^2 and nu k^2.
+// grid ceil(Kr*Kc/256), block 256.
+template <int N, int V = 0>
+__global__ void k_make_symbols(ModeSym* __restrict__ F, ModeSym* __restrict__ A, double* __restrict__ k2out,
+                               double* __restrict__ nuk2, double nu) {
+  using G = Geo<N, V>;
+  const double s2 = 1.0 / ((double)N * N);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G::Kr * G::Kc; i += gridDim.x * blockDim.x) {
+    const int kx = i / G::Kr, r = i - kx * G::Kr;
+    const int ky = ky_of_row(r, G::K);
+    const double k2 = (double)(kx * kx + ky * ky);
+    const double ik2 = k2 > 0.0 ? 1.0 / k2 : 0.0;
+    ModeSym f{}, a{};
+    // a mode whose put symbols vanish must not set its column's exponent
+    f.put = fx_pair(ky * ik2 * s2, kx * ik2 * s2, kZeroExp, &f.put_e);
+    f.get = fx_pair(0.5 * (ky * ky - kx * kx), -0.5 * kx * ky, 0, &f.get_e);
+    a.put = fx_pair(-2.0 * kx * ky * s2, (double)(ky * ky - kx * kx) * s2, kZeroExp, &a.put_e);
+    a.get = fx_pair(0.5 * ky * ik2, 0.5 * kx * ik2, 0, &a.get_e);
+    F[i] = f;
+    A[i] = a;
+    k2out[i] = k2;
+    nuk2[i] = nu * k2;
+  }
 }
 
 // Control multipliers m(k) = |k| W(k)^{1/2} on the retained set (0 at k = 0),

@@ -11,21 +11,19 @@ struct Ops {
   int n, K, Kc, Kr;
   int variant;                      // plan variant (fft.cuh)
   int threads;                      // CTA width of the pass kernels
-  int fold_doubles;                 // entries of the folded twiddle table
   double flops_inverse;             // nominal flops of one band-limited inverse transform
   double flops_forward;             // ... and forward transform (band_transform_flops)
-  void (*fold_table)(double* out);  // fills it on the host
   int fx_entries;                   // entries of the integer twiddle tables
-  void (*fx_table)(int4* out);      // fills them on the host
+  const std::vector<int4>& (*fx_table)();
   cudaError_t (*setup)();
   void (*r2c_rows)(const Dev&, const double* in, cudaStream_t);
   void (*c2r_rows)(const Dev&, double* out, cudaStream_t);
   void (*spec_to_mixed)(const Dev&, const double2* src, int mode, cudaStream_t);
   void (*compact_to_half)(const Dev&, const double2* src, double2* out, cudaStream_t);
   void (*half_to_compact)(const Dev&, const double2* in, double2* dst, cudaStream_t);
-  void (*ctrl_cols)(const Dev&, int flags, cudaStream_t);
+  void (*ctrl_cols)(const Dev&, bool next, cudaStream_t);
   void (*fwd_rows)(const Dev&, int n, int stage, int flags, cudaStream_t);
-  void (*fwd_cols)(const Dev&, int n, int stage, int flags, cudaStream_t);
+  void (*fwd_cols)(const Dev&, int n, int stage, cudaStream_t);
   void (*state_cols)(const Dev&, cudaStream_t);
   void (*adj_init)(const Dev&, int mode, cudaStream_t);
   void (*adj_rows)(const Dev&, int n, int stage, cudaStream_t);
@@ -35,6 +33,7 @@ struct Ops {
   int window_batch;
   void (*window_fwd)(const Dev&, int k0, int k1, int flags, cudaStream_t);
   void (*window_adj)(const Dev&, int k1, int k0, int sources, cudaStream_t);
+  void (*make_symbols)(const Dev&, double nu, cudaStream_t);
   void (*make_mult)(const Dev&, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                     cudaStream_t);
 };

@@ -32,21 +32,20 @@ Ops make_ops() {
   o.Kr = G::Kr;
   o.variant = V;
   o.threads = G::THREADS;
-  o.fold_doubles = FoldInfo<N, V>::DOUBLES;
   o.flops_inverse = band_transform_flops<N, V, G::K>(true);
   o.flops_forward = band_transform_flops<N, V, G::K>(false);
-  o.fold_table = [](double* out) { fold_table<N, V>(out); };
   o.fx_entries = FxPlan<N, V>::TABLE;
-  o.fx_table = [](int4* out) { fx_table<FxPlan<N, V>>(out); };
+  o.fx_table = []() -> const std::vector<int4>& { return fx_table<FxPlan<N, V>>(); };
   o.setup = []() -> cudaError_t {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* f, size_t s = G::SMEM_FX) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s);
     };
-    set((const void*)k_r2c_rows<N, V>, G::SMEM_FOLD);
-    set((const void*)k_c2r_rows<N, V>, G::SMEM_FOLD);
-    set((const void*)k_spec_to_mixed<N, V>, G::SMEM_FOLD);
-    set((const void*)k_ctrl_cols<N, V>, G::SMEM_CTRL);
+    set((const void*)k_r2c_rows<N, V>);
+    set((const void*)k_c2r_rows<N, V>);
+    set((const void*)k_spec_to_mixed<N, V>);
+    set((const void*)k_ctrl_cols<N, V, false>);
+    set((const void*)k_ctrl_cols<N, V, true>);
     set((const void*)k_fwd_rows<N, V, false>);
     set((const void*)k_fwd_rows<N, V, true>);
     set((const void*)k_fwd_cols<N, V>);
@@ -64,13 +63,13 @@ Ops make_ops() {
     return e;
   };
   o.r2c_rows = [](const Dev& d, const double* in, cudaStream_t st) {
-    k_r2c_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FOLD, st>>>(d, in);
+    k_r2c_rows<N, V><<<dim3(N / 4, d.B), G::THREADS, G::SMEM_FX, st>>>(d, in);
   };
   o.c2r_rows = [](const Dev& d, double* out, cudaStream_t st) {
-    k_c2r_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FOLD, st>>>(d, out);
+    k_c2r_rows<N, V><<<dim3(N / 4, d.B), G::THREADS, G::SMEM_FX, st>>>(d, out);
   };
   o.spec_to_mixed = [](const Dev& d, const double2* src, int mode, cudaStream_t st) {
-    k_spec_to_mixed<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FOLD, st>>>(d, src, mode);
+    k_spec_to_mixed<N, V><<<dim3((G::Kc + 1) / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, src, mode);
   };
   o.compact_to_half = [](const Dev& d, const double2* src, double2* out, cudaStream_t st) {
     k_compact_to_half<N, V><<<dim3((N * G::NH + 255) / 256, d.B), 256, 0, st>>>(src, out);
@@ -78,8 +77,9 @@ Ops make_ops() {
   o.half_to_compact = [](const Dev& d, const double2* in, double2* dst, cudaStream_t st) {
     k_half_to_compact<N, V><<<dim3((G::Kr * G::Kc + 255) / 256, d.B), 256, 0, st>>>(in, dst);
   };
-  o.ctrl_cols = [](const Dev& d, int flags, cudaStream_t st) {
-    k_ctrl_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_CTRL, st>>>(d, flags);
+  o.ctrl_cols = [](const Dev& d, bool next, cudaStream_t st) {
+    if (next) k_ctrl_cols<N, V, true><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d);
+    else k_ctrl_cols<N, V, false><<<dim3((G::Kc + 1) / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d);
   };
   o.fwd_rows = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
     if (flags & (F_OBS | F_OBS_ONLY))
@@ -87,8 +87,8 @@ Ops make_ops() {
     else
       k_fwd_rows<N, V, false><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
   };
-  o.fwd_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    k_fwd_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
+  o.fwd_cols = [](const Dev& d, int n, int stage, cudaStream_t st) {
+    k_fwd_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
   };
   o.state_cols = [](const Dev& d, cudaStream_t st) {
     k_state_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d);
@@ -116,6 +116,10 @@ Ops make_ops() {
       launch_clusters<W::C>(k_window_adj<N, V>, d.B, W::THREADS, W::SMEM, st, d, k1, k0, sources);
     };
   }
+  o.make_symbols = [](const Dev& d, double nu, cudaStream_t st) {
+    k_make_symbols<N, V><<<dim3((G::Kr * G::Kc + 255) / 256), 256, 0, st>>>((ModeSym*)d.symF, (ModeSym*)d.symA,
+                                                                          (double*)d.k2, (double*)d.nuk2, nu);
+  };
   o.make_mult = [](const Dev& d, double* mult, const int* kind, const double* param, const double* table, const double* nu,
                    cudaStream_t st) {
     k_make_mult<N, V><<<dim3((G::Kr * G::Kc + 255) / 256, d.B), 256, 0, st>>>(mult, kind, param, table, nu);

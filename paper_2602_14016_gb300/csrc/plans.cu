@@ -18,18 +18,14 @@ int cached_plan(int n, int B) {
   return it == g_plan_choice.end() ? 0 : it->second;
 }
 
-// Switches the context's pass kernels to plan variant v: launchers, folded
-// twiddle table, shared-memory attributes.  A captured graph holds the old
+// Switches the context's pass kernels to plan variant v: launchers, twiddle
+// tables, shared-memory attributes.  A captured graph holds the old
 // kernels and is dropped; a stored forward trajectory is invalidated.
 static da_status set_plan(da_ctx* c, int v) {
   const Ops* o = da::ops_for(c->n, v);
   if (!o) return fail(c, DA_EINVAL, "plan variant out of range (da_plan_count)");
   if (o == c->ops) return DA_OK;
-  std::vector<double> fold(o->fold_doubles);
-  o->fold_table(fold.data());
-  DA_TRY_CUDA(c, cudaMemcpy((void*)c->dev.fold, fold.data(), fold.size() * sizeof(double), cudaMemcpyHostToDevice));
-  std::vector<int4> fxtw(o->fx_entries);
-  o->fx_table(fxtw.data());
+  const std::vector<int4>& fxtw = o->fx_table();
   DA_TRY_CUDA(c, cudaMemcpy((void*)c->dev.fxtw, fxtw.data(), fxtw.size() * sizeof(int4), cudaMemcpyHostToDevice));
   DA_TRY_CUDA(c, o->setup());
   c->ops = o;
@@ -58,7 +54,7 @@ extern "C" da_status da_plan_flops(int n, int variant, double* inverse, double* 
 
 extern "C" da_status da_set_plan(da_ctx* c, int variant) {
   if (!c) return fail(c, DA_EINVAL, "ctx must not be NULL");
-  // the folded table and the launchers change under any work in flight
+  // the twiddle tables and the launchers change under any work in flight
   DA_TRY_CUDA(c, cudaDeviceSynchronize());
   return set_plan(c, variant);
 }
@@ -100,7 +96,7 @@ static da_status tuning_steps(da_ctx* c, int steps, cudaStream_t st) {
     const int k = store ? i % d.traj_steps : 0;
     for (int j = 1; j <= 4; ++j) {
       o->fwd_rows(d, k, j, store ? da::F_STORE : 0, st);
-      o->fwd_cols(d, k, j, 0, st);
+      o->fwd_cols(d, k, j, st);
     }
     if (store)
       for (int j = 4; j >= 1; --j) {

@@ -106,7 +106,7 @@ struct Win {
   }
   __device__ __forceinline__ RowLoad take_row() {
     const q2* M = rowbuf + (pair * 2 + x.f) * 2 * G::Kc;
-    return load_row<P>(M, M + G::Kc, rowexp, x);
+    return load_row<P>(M, M + G::Kc, rowexp, rowexp + G::Kc, x);
   }
   // The transformed row in src, twice its two fields, to the columns' owners.
   __device__ __forceinline__ void send_row(int e) {

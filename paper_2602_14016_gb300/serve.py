@@ -78,12 +78,12 @@ def context_bytes(n: int, nsteps: int, px: int, every: int, ckpt_every: int, bat
     nt = nsteps // every
     comp = batch * Kr * Kc * 16
     b = 6 * comp + batch * 4 * n * Kc * 16 + 3 * batch * nt * px * px * 2 * 8 + comp // 2
-    b += n * 16 + 64 * 16 + batch * (8 + 4 + 8) + batch * 8 + Kr * Kc * 72 + batch * (4 * 4 + 8)
-    if ckpt_every == 0:
-        b += batch * nsteps * 8 * n * n * 8
-    else:
-        kk = min(ckpt_every, nsteps)
-        b += batch * kk * 8 * n * n * 8 + ((nsteps + kk - 1) // kk) * comp
+    b += 2 * n * 16 + 64 * 16 + batch * (8 + 4 + 8) + batch * 8 + Kr * Kc * 112 + batch * (4 * 4 + 8)
+    b += batch * (2 * Kc + n) * 4  # exponents of the mixed fields
+    kk = nsteps if ckpt_every == 0 else min(ckpt_every, nsteps)
+    b += batch * kk * 4 * n * (2 * n * 8 + 4)  # stage fields and their exponents
+    if ckpt_every:
+        b += ((nsteps + kk - 1) // kk) * comp
     slots = memory + 1
     # optimiser: vector banks, device scalars and costs, argument tables
     b += batch * (5 + 2 * slots) * n * n * 8 + batch * 7 * 8 + (3 * batch + batch * memory) * 4
