@@ -9,6 +9,8 @@
 #include <cmath>
 #include <cstdio>
 #include <string>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "../../include/da.h"
@@ -171,6 +173,31 @@ da_status dalloc(da_ctx* c, T** p, size_t count) {
   *p = static_cast<T*>(v);
   return DA_OK;
 }
+
+// Arrays of a context that share one device allocation (a cudaMalloc costs the
+// host 0.1 ms): add each, then alloc sets their pointers, 256 bytes aligned.
+class DeviceGroup {
+ public:
+  template <typename T>
+  void add(T** p, size_t count) {
+    *p = nullptr;
+    parts_.push_back({reinterpret_cast<void**>(const_cast<std::remove_const_t<T>**>(p)), total_});
+    bytes_ += count * sizeof(T);
+    total_ += (count * sizeof(T) + 255) / 256 * 256;
+  }
+  da_status alloc(da_ctx* c) {
+    char* base = nullptr;
+    da_status r = dalloc(c, &base, total_);
+    if (r) return r;
+    c->bytes -= total_ - bytes_;  // what the arrays hold, not the padding
+    for (auto& p : parts_) *p.first = base + p.second;
+    return DA_OK;
+  }
+
+ private:
+  std::vector<std::pair<void**, size_t>> parts_;
+  size_t total_ = 0, bytes_ = 0;
+};
 
 // Whether global step k of the evaluation window can be an observation step
 // of some member (every member's window is a whole number of observation

@@ -91,42 +91,38 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
 
   const size_t B = c->B, N = n, comp = B * ops->Kr * ops->Kc, P2 = (size_t)c->P * c->P;
   da_status s = DA_OK;
+  DeviceGroup group;
   auto A = [&](da_status st) {
     if (s == DA_OK) s = st;
   };
-  A(dalloc(c, &d.W, comp));
-  A(dalloc(c, &d.Acc, comp));
-  A(dalloc(c, &d.Y, comp));
-  A(dalloc(c, &d.KB, comp));
-  A(dalloc(c, &d.LamBar, comp));
-  A(dalloc(c, &d.Sum, comp));
-  A(dalloc(c, &d.Mx, B * 2 * N * ops->Kc));
-  A(dalloc(c, &d.Mn, B * 2 * N * ops->Kc));
-  A(dalloc(c, &d.eX, B * 2 * ops->Kc));
-  A(dalloc(c, &d.eN, B * N));
-  A(dalloc(c, &d.obs, B * c->nt * P2 * 2));
-  A(dalloc(c, (double**)&d.mobs, B * c->nt * P2 * 2));
-  A(dalloc(c, &d.res, B * c->nt * P2 * 2));
-  A(dalloc(c, &d.J, B));
-  A(dalloc(c, (double**)&d.mult, comp));
+  group.add(&d.W, comp);
+  group.add(&d.Acc, comp);
+  group.add(&d.Y, comp);
+  group.add(&d.KB, comp);
+  group.add(&d.LamBar, comp);
+  group.add(&d.Sum, comp);
+  group.add(&d.Mx, B * 2 * N * ops->Kc);
+  group.add(&d.Mn, B * 2 * N * ops->Kc);
+  group.add(&d.eX, B * 2 * ops->Kc);
+  group.add(&d.eN, B * N);
+  group.add(&d.obs, B * c->nt * P2 * 2);
+  group.add((double**)&d.mobs, B * c->nt * P2 * 2);
+  group.add(&d.res, B * c->nt * P2 * 2);
+  group.add(&d.J, B);
+  group.add((double**)&d.mult, comp);
   size_t fx_max = 0;  // room for the twiddle tables of any plan variant
   for (int v = 0; v < da::plan_count(n); ++v) fx_max = std::max(fx_max, (size_t)da::ops_for(n, v)->fx_entries);
-  A(dalloc(c, (int4**)&d.fxtw, fx_max));
-  A(dalloc(c, (double2**)&d.twP, (size_t)64));
-  A(dalloc(c, (da::ModeSym**)&d.symF, comp / B));
-  A(dalloc(c, (da::ModeSym**)&d.symA, comp / B));
-  A(dalloc(c, (double**)&d.nuk2, comp / B));
-  A(dalloc(c, (double**)&d.k2, comp / B));
-  A(dalloc(c, &c->d_mstart, B));
-  A(dalloc(c, &c->d_mnt, B));
-  A(dalloc(c, &c->d_mpx, B));
-  A(dalloc(c, &c->d_mforce, B));
-  A(dalloc(c, &c->d_mnu, B));
-  d.mstart = c->d_mstart;
-  d.mnt = c->d_mnt;
-  d.mpx = c->d_mpx;
-  d.mforce = c->d_mforce;
-  d.mnu = c->d_mnu;
+  group.add((int4**)&d.fxtw, fx_max);
+  group.add((double2**)&d.twP, (size_t)64);
+  group.add((da::ModeSym**)&d.symF, comp / B);
+  group.add((da::ModeSym**)&d.symA, comp / B);
+  group.add((double**)&d.nuk2, comp / B);
+  group.add((double**)&d.k2, comp / B);
+  group.add(&c->d_mstart, B);
+  group.add(&c->d_mnt, B);
+  group.add(&c->d_mpx, B);
+  group.add(&c->d_mforce, B);
+  group.add(&c->d_mnu, B);
   // stage-field store: the whole window, or one checkpoint segment
   if (c->ckpt == 0) {
     d.traj_steps = c->nsteps;
@@ -137,10 +133,16 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
   }
   if (c->ckpt >= 0) {
     A(dalloc(c, &d.traj, B * (size_t)d.traj_steps * 4 * N * N));
-    A(dalloc(c, &d.eT, B * (size_t)d.traj_steps * 4 * N));
+    group.add(&d.eT, B * (size_t)d.traj_steps * 4 * N);
   }
-  A(dalloc(c, &c->d_kind, B));
-  A(dalloc(c, &c->d_param, B));
+  group.add(&c->d_kind, B);
+  group.add(&c->d_param, B);
+  A(group.alloc(c));
+  d.mstart = c->d_mstart;
+  d.mnt = c->d_mnt;
+  d.mpx = c->d_mpx;
+  d.mforce = c->d_mforce;
+  d.mnu = c->d_mnu;
   bool any_table = false;
   for (int b = 0; b < c->B; ++b) any_table |= kernels[b].kind == DA_KERNEL_TABLE;
   if (any_table) A(dalloc(c, &c->d_table, B * N * (N / 2 + 1)));
