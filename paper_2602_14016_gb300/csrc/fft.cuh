@@ -124,7 +124,7 @@ template <> struct Plan<256, 0> { using two = Radices<4, 4, 4, 4>; using one = R
 template <> struct Plan<256, 1> { using two = Radices<8, 8, 4>; using one = Radices<8, 8, 4>; static constexpr int threads = 64; };
 template <> struct Plan<256, 2> { using two = Radices<4, 4, 4, 4>; using one = Radices<4, 4, 4, 4>; static constexpr int threads = 64; };
 template <> struct Plan<512, 0> { using two = Radices<8, 8, 8>; using one = Radices<8, 8, 8>; static constexpr int threads = 128; };
-template <> struct Plan<512, 1> { using two = Radices<8, 4, 4, 4>; using one = Radices<8, 4, 4, 4>; static constexpr int threads = 256; };
+template <> struct Plan<512, 1> { using two = Radices<8, 4, 4, 4>; using one = Radices<8, 4, 4, 4>; static constexpr int threads = 128; };
 template <> struct Plan<512, 2> { using two = Radices<8, 8, 8>; using one = Radices<8, 8, 8>; static constexpr int threads = 64; };
 template <> struct Plan<1024, 0> { using two = Radices<16, 8, 8>; using one = Radices<16, 8, 8>; static constexpr int threads = 256; };
 template <> struct Plan<1024, 1> { using two = Radices<16, 4, 4, 4>; using one = Radices<16, 4, 4, 4>; static constexpr int threads = 256; };

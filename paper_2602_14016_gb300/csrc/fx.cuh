@@ -284,11 +284,6 @@ struct FxPlanOf {
   static constexpr int GROWTH2 = Growth<R1, typename TailRadices<fwd>::type>::most(0);  // the others
   static constexpr int BITS_FWD = 62 - GROWTH;
   static constexpr int SEQ = N + N / 8;  // q2 of one buffer of a sequence
-  // Threads of several warps read one buffer and write another (one barrier a
-  // stage); a warp alone works in place, since its barriers cost nothing and
-  // half the shared memory lets more of its kind run.
-  static constexpr bool PING = TPS > 32;
-  static constexpr int BUFS = PING ? 2 : 1;
   static constexpr int WARPS = (TPS + 31) / 32;
 };
 
@@ -563,52 +558,39 @@ struct Bfly {
   __device__ static __forceinline__ bool active(int t) { return NB >= P::TPS || t < NB; }
 };
 
-// Inputs i + m NB of butterfly i, out of src; Z: inputs left out.
+// Inputs i + m NB of butterfly i, out of buf; Z: inputs left out.
 template <typename P, int R, int Z = 0>
-__device__ __forceinline__ void fx_load(q2* a, const q2* src, int i) {
-  const q2* s = src + pad(i);
+__device__ __forceinline__ void fx_load(q2* a, const q2* buf, int i) {
+  const q2* s = buf + pad(i);
 #pragma unroll
   for (int m = 0; m < R; ++m)
     if (!((Z >> m) & 1)) a[m] = s[pad(m * (P::N / R))];
 }
 
-// Outputs of butterfly i of the stage with sub-length L, into dst.
+// Outputs of butterfly i of the stage with sub-length L, into buf.
 template <typename P, int R, int L>
-__device__ __forceinline__ void fx_store(const q2* a, q2* dst, int i) {
+__device__ __forceinline__ void fx_store(const q2* a, q2* buf, int i) {
   const int k = i & (L - 1);
-  q2* d = dst + pad((i - k) * R + k);
+  q2* d = buf + pad((i - k) * R + k);
 #pragma unroll
   for (int m = 0; m < R; ++m) d[pad(m * L)] = a[m];
 }
 
-// src and dst are the same buffer where P works in place.
-template <typename P>
-__device__ __forceinline__ void swap_bufs(q2*& a, q2*& b) {
-  if constexpr (P::PING) {
-    q2* c = a;
-    a = b;
-    b = c;
-  }
-}
-// Between a stage's loads and its stores in place.
-template <typename P>
-__device__ __forceinline__ void in_place_sync(int id) {
-  if constexpr (!P::PING) seq_sync<P::TPS>(id);
-}
-
-// Middle stages with sub-lengths from L on: src -> dst, sync, swap.  SHR: the
+// Middle stages with sub-lengths from L on, in place: every thread holds its
+// butterflies in registers across a barrier of the sequence (two buffers and one
+// barrier a stage measured the same from 128 to 1024 points).  SHR: the
 // first of them starts with a right shift by r.
 template <typename P, int S, int L, bool SHR>
-__device__ __forceinline__ void fx_middle(q2*&, q2*&, const int4*, int, int, int, Radices<>) {}
+__device__ __forceinline__ void fx_middle(q2*, const int4*, int, int, int, Radices<>) {}
 template <typename P, int S, int L, bool SHR, int R, int... Rs>
-__device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int t, int id, int r, Radices<R, Rs...>) {
+__device__ __forceinline__ void fx_middle(q2* buf, const int4* T, int t, int id, int r, Radices<R, Rs...>) {
   using B = Bfly<P, R>;
   q2 a[B::POINTS];
   if (B::active(t)) {
 #pragma unroll
     for (int jb = 0; jb < B::J; ++jb) {
       const int i = t + jb * P::TPS;
-      fx_load<P, R>(a + jb * R, src, i);
+      fx_load<P, R>(a + jb * R, buf, i);
       if constexpr (SHR) {
         if (r > 0) {
 #pragma unroll
@@ -616,30 +598,25 @@ __device__ __forceinline__ void fx_middle(q2*& src, q2*& dst, const int4* T, int
         }
       }
       fx_butterfly<R, S, L, 0>(a + jb * R, T, i & (L - 1));
-      if constexpr (P::PING) fx_store<P, R, L>(a + jb * R, dst, i);
-    }
-  }
-  if constexpr (!P::PING) {
-    seq_sync<P::TPS>(id);
-    if (B::active(t)) {
-#pragma unroll
-      for (int jb = 0; jb < B::J; ++jb) fx_store<P, R, L>(a + jb * R, dst, t + jb * P::TPS);
     }
   }
   seq_sync<P::TPS>(id);
-  swap_bufs<P>(src, dst);
-  fx_middle<P, S, L * R, false>(src, dst, T + (R - 1) * L, t, id, r, Radices<Rs...>{});
+  if (B::active(t)) {
+#pragma unroll
+    for (int jb = 0; jb < B::J; ++jb) fx_store<P, R, L>(a + jb * R, buf, t + jb * P::TPS);
+  }
+  seq_sync<P::TPS>(id);
+  fx_middle<P, S, L * R, false>(buf, T + (R - 1) * L, t, id, r, Radices<Rs...>{});
 }
 
-// Inverse transform (S = +1) of the sequence in src, zero outside the band
+// Inverse transform (S = +1) of the sequence in buf, zero outside the band
 // KB: the inputs are shifted right by pre (left by
 // -pre) first,
 // and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
 // is left in registers: out[jb R + m] is position t + jb TPS + m N / R for R
-// the last radix.  dst is free afterwards if it is another buffer than src;
-// src is not before the next sync.
+// the last radix.  buf is not free before the next sync.
 template <typename P, int KB>
-__device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, int t, int id, int pre, q2* out) {
+__device__ __forceinline__ void fx_inverse(q2* buf, const int4* tw, int t, int id, int pre, q2* out) {
   using I = typename P::inv;
   constexpr int R1 = FirstRadix<I>::value, RL = LastRadix<I>::value;
   constexpr int Z = gap_common(P::N, R1, KB);  // inputs in the gap for every butterfly
@@ -652,7 +629,7 @@ __device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, i
 #pragma unroll
     for (int jb = 0; jb < B1::J; ++jb) {
       q2* b = a + jb * R1;
-      fx_load<P, R1, Z>(b, src, t + jb * P::TPS);
+      fx_load<P, R1, Z>(b, buf, t + jb * P::TPS);
       if (pre > 0) {
 #pragma unroll
         for (int m = 0; m < R1; ++m)
@@ -665,22 +642,21 @@ __device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, i
       qdftR<R1, +1, Z>(b);
     }
   }
-  in_place_sync<P>(id);
+  seq_sync<P::TPS>(id);
   if (B1::active(t)) {
 #pragma unroll
-    for (int jb = 0; jb < B1::J; ++jb) fx_store<P, R1, 1>(a + jb * R1, dst, t + jb * P::TPS);
+    for (int jb = 0; jb < B1::J; ++jb) fx_store<P, R1, 1>(a + jb * R1, buf, t + jb * P::TPS);
   }
   seq_sync<P::TPS>(id);
-  swap_bufs<P>(src, dst);
   using Mid = typename InitRadices<typename TailRadices<I>::type>::type;
-  fx_middle<P, +1, R1, false>(src, dst, T, t, id, 0, Mid{});
+  fx_middle<P, +1, R1, false>(buf, T, t, id, 0, Mid{});
   constexpr int L = P::N / RL;
   if (BL::active(t)) {
     const int4* Tl = T + P::ENTRIES_INV - (RL - 1) * L;
 #pragma unroll
     for (int jb = 0; jb < BL::J; ++jb) {
       const int i = t + jb * P::TPS;
-      fx_load<P, RL>(out + jb * RL, src, i);
+      fx_load<P, RL>(out + jb * RL, buf, i);
       fx_butterfly<RL, +1, L, 0>(out + jb * RL, Tl, i);
     }
   }
@@ -690,10 +666,10 @@ __device__ __forceinline__ void fx_inverse(q2*& src, q2*& dst, const int4* tw, i
 // position t + jb TPS + m N / R for R the first radix.  MEASURE: the inputs
 // leave room for the first stage only, and a shift measured after it makes
 // room for the others, with SPARE bits of the result free; the shift is
-// returned.  The result, times 2^-SHIFT, is left in src, in natural order,
+// returned.  The result, times 2^-SHIFT, is left in buf, in natural order,
 // synchronised; only the band KB is formed.
 template <typename P, int KB, bool MEASURE, int SPARE>
-__device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4* tw, int t, int id, int* scratch) {
+__device__ __forceinline__ int fx_forward(q2* in, q2* buf, const int4* tw, int t, int id, int* scratch) {
   using F = typename P::fwd;
   using Tail = typename TailRadices<F>::type;
   constexpr int R1 = FirstRadix<F>::value, RL = LastRadix<F>::value, L = P::N / RL;
@@ -701,7 +677,7 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
   using B1 = Bfly<P, R1>;
   using BL = Bfly<P, RL>;
   int big = 0, r = 0;
-  in_place_sync<P>(id);  // the registers were loaded from this buffer
+  seq_sync<P::TPS>(id);  // the registers may have been loaded from this buffer
   if (B1::active(t)) {
 #pragma unroll
     for (int jb = 0; jb < B1::J; ++jb) {
@@ -711,16 +687,15 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
 #pragma unroll
         for (int m = 0; m < R1; ++m) big = max_mag(big, a[m]);
       }
-      fx_store<P, R1, 1>(a, dst, t + jb * P::TPS);
+      fx_store<P, R1, 1>(a, buf, t + jb * P::TPS);
     }
   }
   if constexpr (MEASURE) big = seq_max_put<P::TPS>(big, t, scratch);
   seq_sync<P::TPS>(id);
-  swap_bufs<P>(src, dst);
   if constexpr (MEASURE) r = max(0, bits64(seq_max_get<P::TPS>(big, scratch)) - (62 - SPARE - P::GROWTH2));
   using Mid = typename InitRadices<Tail>::type;
   constexpr bool MIDDLE = L > R1;  // there are middle stages
-  fx_middle<P, -1, R1, MEASURE && MIDDLE>(src, dst, tw, t, id, r, Mid{});
+  fx_middle<P, -1, R1, MEASURE && MIDDLE>(buf, tw, t, id, r, Mid{});
   q2 a[BL::POINTS];
   if (BL::active(t)) {
     const int4* Tl = tw + P::ENTRIES - (RL - 1) * L;
@@ -728,7 +703,7 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
     for (int jb = 0; jb < BL::J; ++jb) {
       const int i = t + jb * P::TPS;
       q2* b = a + jb * RL;
-      fx_load<P, RL>(b, src, i);
+      fx_load<P, RL>(b, buf, i);
       if constexpr (MEASURE && !MIDDLE) {
         if (r > 0) {
 #pragma unroll
@@ -738,18 +713,17 @@ __device__ __forceinline__ int fx_forward(q2* in, q2*& src, q2*& dst, const int4
       fx_butterfly<RL, -1, L, 0>(b, Tl, i);
     }
   }
-  in_place_sync<P>(id);
+  seq_sync<P::TPS>(id);
   if (BL::active(t)) {
 #pragma unroll
     for (int jb = 0; jb < BL::J; ++jb) {
-      q2* d = dst + pad(t + jb * P::TPS);
+      q2* d = buf + pad(t + jb * P::TPS);
 #pragma unroll
       for (int m = 0; m < RL; ++m)
         if (!((C >> m) & 1)) d[pad(m * L)] = a[jb * RL + m];
     }
   }
   seq_sync<P::TPS>(id);
-  swap_bufs<P>(src, dst);
   return r;
 }
 

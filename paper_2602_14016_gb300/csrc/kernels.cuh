@@ -142,7 +142,7 @@ struct Geo {
   // passes that run the integer transforms: the buffers of two sequences,
   // scratch of the reductions (Place), and probe sums (adjoint column passes)
   static constexpr int SCRATCH = ((3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS + 3) / 4 * 4;
-  static constexpr size_t SMEM_FX = sizeof(q2) * (2 * FxPlan<N, V>::BUFS * FxPlan<N, V>::SEQ) + sizeof(int) * SCRATCH;
+  static constexpr size_t SMEM_FX = sizeof(q2) * (2 * FxPlan<N, V>::SEQ) + sizeof(int) * SCRATCH;
   static constexpr size_t SMEM_FXP = SMEM_FX + sizeof(double2) * 2 * PMAX;
   // Column passes: small grids leave most of the chip idle, so a warp's own
   // latency counts, and they load their epilogue inputs before the transforms
@@ -224,26 +224,25 @@ __global__ void k_half_to_compact(const double2* __restrict__ in, double2* __res
 // ---------------------------------------------------------------------------
 
 // A thread's place in a column pass: sequence f of its column, thread t of
-// the sequence and pt of the column's PT threads; the buffers of its sequence
-// and of the column's first sequence (the other's lie OTHER further); scratch of
+// the sequence and pt of the column's PT threads; the buffer of its sequence
+// (the other's lies OTHER away); scratch of
 // the sequence's reductions (three of WARPS ints) and of the column's (two of
 // PAIR ints).  In a row pass the two sequences are rows.
 template <typename P_>
 struct Place {
   using P = P_;
   static constexpr int PT = 2 * P::TPS;
-  static constexpr int OTHER = P::BUFS * P::SEQ;
+  static constexpr int OTHER = P::SEQ;
   static constexpr int PAIR = PT > 32 ? 2 * (PT / 32) : 0;
   static constexpr int SCRATCH = 2 * 3 * P::WARPS + 2 * PAIR;  // ints of the pair
   int t, f, pt;
-  q2 *src, *dst;
+  q2* src;
   int *scratch, *pscratch;
   // pair: index of the pair of sequences in the CTA; thread: index in the pair
   __device__ __forceinline__ Place(q2* bufs, int* ints, int pair, int thread) : pt(thread) {
     f = thread / P::TPS;
     t = thread - f * P::TPS;
     src = bufs + (pair * 2 + f) * OTHER;
-    dst = P::PING ? src + P::SEQ : src;
     int* s = ints + pair * SCRATCH;
     scratch = s + f * 3 * P::WARPS;
     pscratch = s + 2 * 3 * P::WARPS;
@@ -363,7 +362,7 @@ __device__ __forceinline__ int finish_columns(const ColumnPut<P>& c, Place<P>& x
   constexpr int R = LastRadix<typename P::inv>::value;
   using B = Bfly<P, R>;
   q2 out[B::POINTS];
-  fx_inverse<P, G::K>(x.src, x.dst, tw, x.t, x.f, pre, out);
+  fx_inverse<P, G::K>(x.src, tw, x.t, x.f, pre, out);
   if (B::active(x.t)) {
 #pragma unroll
     for (int jb = 0; jb < B::J; ++jb)
@@ -441,7 +440,7 @@ __device__ __forceinline__ int forward_columns(const q2* __restrict__ M, const i
       for (int j = 0; j < B::POINTS; ++j) v[j] = ShiftRight(-sh)(v[j]);
     }
   }
-  const int r = fx_forward<P, G::K, MEASURE, 1>(v, x.src, x.dst, tw, x.t, x.f, x.scratch + P::WARPS);
+  const int r = fx_forward<P, G::K, MEASURE, 1>(v, x.src, tw, x.t, x.f, x.scratch + P::WARPS);
   if constexpr (MEASURE && COMMON) {  // results of two shifts: bring both to the larger one
     if (x.t == 0) x.scratch[0] = r;
     pair_sync<P>();
@@ -681,7 +680,7 @@ struct RowPoints {
 template <typename P, int BITS, typename Between>
 __device__ __forceinline__ int row_fields(const RowLoad& in, Place<P>& x, const int4* tw, q2* z, Between between) {
   using RP = RowPoints<P>;
-  fx_inverse<P, Geo<P::N>::K>(x.src, x.dst, tw, x.t, x.f, in.pre, z);
+  fx_inverse<P, Geo<P::N>::K>(x.src, tw, x.t, x.f, in.pre, z);
   between();
   int m = 0;
   if (RP::B::active(x.t)) {
@@ -771,7 +770,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
   if constexpr (OBS) {
     if (flags & F_OBS_ONLY) return;  // the final state: probes only
   }
-  const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+  const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, d.fxtw, x.t, x.f, x.scratch);
   store_row_pair<N, V>(d, bm, y0, x, 2 * ex + 64 + P::SHIFT + r);
 }
 
@@ -815,7 +814,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_r2c_rows(Dev d, const do
 #pragma unroll
     for (int j = 0; j < B::POINTS; ++j) z[j] = mkq(double_to_fx(v[j].x, e), double_to_fx(v[j].y, e));
   }
-  const int r = fx_forward<P, G::K, MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch + P::WARPS);
+  const int r = fx_forward<P, G::K, MEASURE, 1>(z, x.src, d.fxtw, x.t, x.f, x.scratch + P::WARPS);
   q2* M = d.Mn + (size_t)bm * G::Kc * 2 * N + y0;
   for (int kx = x.t; kx < G::Kc; kx += P::TPS) {
     const q2 zk = x.src[pad(kx)], zm = x.src[pad((N - kx) & (N - 1))];
@@ -855,8 +854,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d) {
       if (rr >= G::Kr) break;
       put_stage_columns(put, j, d.symF[kx * G::Kr + rr], w0(rr, x.first(x.src)));
     }
-    swap_bufs<P>(x.src, x.dst);
-    finish_to_mixed(d, put, x, bm, kx);
+      finish_to_mixed(d, put, x, bm, kx);
   } else {
     for (int rr = x.t; rr < G::Kr; rr += P::TPS) w0(rr, x.src);
   }
@@ -908,7 +906,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_spec_to_mixed(Dev d, con
   const int pre = inv_shift<P, 60>(seq_sum_get<P::TPS>(sum, x.scratch + P::WARPS));
   using RP = RowPoints<P>;
   q2 z[RP::POINTS];
-  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, pre, z);
+  fx_inverse<P, G::K>(x.src, d.fxtw, x.t, x.f, pre, z);
   q2* M = d.Mx + (size_t)bm * 2 * N * G::Kc + kx;
   if (RP::B::active(x.t)) {
 #pragma unroll
@@ -931,7 +929,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_c2r_rows(Dev d, double* 
   const int* eX = d.eX + (size_t)bm * 2 * G::Kc;
   const RowLoad in = load_row<P>(M, M + G::Kc, eX, eX, x);
   q2 z[RP::POINTS];
-  fx_inverse<P, G::K>(x.src, x.dst, d.fxtw, x.t, x.f, in.pre, z);
+  fx_inverse<P, G::K>(x.src, d.fxtw, x.t, x.f, in.pre, z);
   const int e = clamp_exp(in.e + in.pre + P::SHIFT_INV);
   double* r0 = out + ((size_t)bm * N + y0) * N;
   if (RP::B::active(x.t)) {
@@ -1000,7 +998,6 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
     d.Y[idx] = yv[t];
     put_stage_columns(put, t, mc[t], yv[t]);
   }
-  swap_bufs<P>(x.src, x.dst);
   finish_to_mixed(d, put, x, bm, kx);
 }
 
@@ -1144,7 +1141,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
     for (int j = 0; j < RP::POINTS; ++j) z[j] = rho_products(uv[j], z[j]);
   }
   const int eT = d.eT[trow];
-  const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+  const int r = fx_forward<P, Geo<N>::K, RowBits<P>::MEASURE, 1>(z, x.src, d.fxtw, x.t, x.f, x.scratch);
   store_row_pair<N, V>(d, bm, y0, x, clamp_exp(ex + eT) + 64 + P::SHIFT + r);
 }
 
@@ -1210,7 +1207,6 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
     put_adjoint_columns(put, t, mc[t], kbv[t]);
   }
   if (stage == 1 && n == mw.start) return;  // the member's first step: lambda_0 stays in LamBar
-  swap_bufs<P>(x.src, x.dst);
   finish_to_mixed(d, put, x, bm, kx);
 }
 

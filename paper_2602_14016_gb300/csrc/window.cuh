@@ -43,7 +43,7 @@ struct WinGeo {
   static constexpr int SLOTS = ROWS;  // sequences a CTA works on at once
   static_assert(!SUPPORTED || (2 * COLS <= SLOTS && SLOTS % 2 == 0), "columns fit the rows' slots");
   static constexpr int THREADS = SLOTS * TPS;
-  static constexpr int WORK = SLOTS * P::BUFS * P::SEQ, ROWBUF = ROWS * 2 * G::Kc, COLBUF = COLS * 2 * N;  // q2
+  static constexpr int WORK = SLOTS * P::SEQ, ROWBUF = ROWS * 2 * G::Kc, COLBUF = COLS * 2 * N;  // q2
   static constexpr int INTS = 2 * G::Kc + N + SLOTS / 2 * X::SCRATCH;
   static constexpr size_t SMEM = sizeof(q2) * (WORK + ROWBUF + COLBUF + COLS * 2 * G::PMAX) + sizeof(int) * INTS;
 };
@@ -97,7 +97,6 @@ struct Win {
 
   // This pair's columns to the rows' owners.
   __device__ __forceinline__ void send_columns(const ColumnPut<P>& put, const int4* tw) {
-    swap_bufs<P>(x.src, x.dst);
     const int e = finish_columns<P>(put, x, tw, [&](int y, q2 z) {
       if (column) on(rowbuf + ((y % W::ROWS) * 2 + x.f) * G::Kc + kx, y / W::ROWS)[0] = z;
     });
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(WinGeo<N, V>::THREADS) k_window_fwd(Dev d, int
         }
       }
       if (n == k1) break;  // the final state: probes only
-      const int r = fx_forward<P, G::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+      const int r = fx_forward<P, G::K, RowBits<P>::MEASURE, 1>(z, x.src, d.fxtw, x.t, x.f, x.scratch);
       w.send_row(2 * ex + 64 + P::SHIFT + r);
       Wn::sync();
       // column pass
@@ -267,7 +266,7 @@ __global__ void __launch_bounds__(WinGeo<N, V>::THREADS) k_window_adj(Dev d, int
 #pragma unroll
         for (int j = 0; j < RP::POINTS; ++j) z[j] = rho_products(uv[j], z[j]);
       }
-      const int r = fx_forward<P, G::K, RowBits<P>::MEASURE, 1>(z, x.src, x.dst, d.fxtw, x.t, x.f, x.scratch);
+      const int r = fx_forward<P, G::K, RowBits<P>::MEASURE, 1>(z, x.src, d.fxtw, x.t, x.f, x.scratch);
       w.send_row(clamp_exp(ex + eT) + 64 + P::SHIFT + r);
       Wn::sync();
       // column pass
