@@ -6,6 +6,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <string>
@@ -84,6 +85,10 @@ struct da_ctx {
   unsigned long long sp_launches = 0;
   int sp_key = -1;
   double *sp_lbuf = nullptr, *sp_member = nullptr, *sp_mean = nullptr;
+  // the batch's parts but the first run their RK stages on these streams (Parts)
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> side_done;
+  cudaEvent_t side_go = nullptr;
   // event timing of one kernel class
   int timed_class = 0;
   std::vector<cudaEvent_t> ev;
@@ -210,6 +215,67 @@ inline bool obs_step_host(const da_ctx* c, int k) { return k % c->obs.every == 0
 inline bool whole_windows(const da_ctx* c) {
   return c->ops->window_fwd && c->B <= c->ops->window_batch && c->timed_class == 0;
 }
+
+// Parts that a batch's RK stages are split into, each a chain of kernels on a
+// stream of its own: a pass ends with SMs that have nothing left to do while
+// its last rows and columns finish, and begins with loads that nothing covers;
+// the other parts' passes fill both.  From two thirds of the resident threads
+// on (768 an SM): us for a stage pass of all members, replayed as a graph, in one part and in
+// three: 256^2 on 128 threads, batch 5 (0.70 of 152 x 768) 9.86 and 9.21, 7 11.3 and 10.2, 10
+// 16.3 and 12.1, 16 23.3 and 18.6; 512^2 batch 4 23.2 and 18.4; 1024^2 batch 2
+// 46.3 and 39.3 (two parts).  Below the line a part no longer fills its own
+// launches: 256^2 batch 4 (0.56) 8.65 and 8.69, on 64 threads batch 7 (0.49) 11.4
+// and 12.0; 128^2 batch 8 (0.56) 6.6 and 6.9; 64^2 batch 24 (0.42) 5.3 and 5.9.
+// More than three parts change nothing.
+constexpr int kMaxParts = 3;
+constexpr int kSplitThreads = 152 * 512;
+inline int batch_parts(const Ops& o, int B) {
+  return (long long)B * (o.n / 2) * o.threads >= kSplitThreads ? std::min(B, kMaxParts) : 1;
+}
+
+// The batch of a context in parts between fork and join: part p's stage passes
+// are launched with dev(p) on stream(p).  The first part runs on the caller's
+// stream, which the others wait for in fork and which waits for them in join,
+// so that to the caller all of it is on that stream, captured or not.
+class Parts {
+ public:
+  Parts(da_ctx* c, cudaStream_t st) : c_(c), st_(st), n_(c->timed_class == 0 ? batch_parts(*c->ops, c->B) : 1) {}
+  ~Parts() { join(); }
+  int count() const { return n_; }
+  int begin(int p) const { return (int)((long long)c_->B * p / n_); }
+  Dev dev(int p) const {
+    Dev d = c_->dev;
+    d.b0 = begin(p);
+    d.B = begin(p + 1) - d.b0;
+    return d;
+  }
+  cudaStream_t stream(int p) const { return p == 0 ? st_ : c_->side[p - 1]; }
+  da_status fork() {
+    if (n_ == 1 || forked_) return DA_OK;
+    DA_TRY_CUDA(c_, cudaEventRecord(c_->side_go, st_));
+    forked_ = true;
+    for (int p = 1; p < n_; ++p) DA_TRY_CUDA(c_, cudaStreamWaitEvent(stream(p), c_->side_go, 0));
+    return DA_OK;
+  }
+  da_status join() {
+    if (!forked_) return DA_OK;
+    forked_ = false;
+    cudaError_t e = cudaSuccess;
+    for (int p = 1; p < n_; ++p) {
+      cudaError_t ep = cudaEventRecord(c_->side_done[p - 1], stream(p));
+      if (ep == cudaSuccess) ep = cudaStreamWaitEvent(st_, c_->side_done[p - 1], 0);
+      if (e == cudaSuccess) e = ep;
+    }
+    DA_TRY_CUDA(c_, e);
+    return DA_OK;
+  }
+
+ private:
+  da_ctx* c_;
+  cudaStream_t st_;
+  int n_;
+  bool forked_ = false;
+};
 
 // Sets the evaluation window for the members marked in `live` (all members
 // with a non-empty window if live is NULL): eval_steps = the longest live

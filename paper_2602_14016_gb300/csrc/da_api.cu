@@ -183,6 +183,15 @@ extern "C" da_status da_create(da_ctx** out, const da_grid* grid, double nu, con
                      cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(d.obs, 0, B * c->nt * P2 * 2 * sizeof(double));
   if (e == cudaSuccess) e = ops->setup();
+  int parts = 1;  // of any plan variant
+  for (int v = 0; v < da::plan_count(n); ++v) parts = std::max(parts, batch_parts(*da::ops_for(n, v), c->B));
+  c->side.assign(parts - 1, nullptr);
+  c->side_done.assign(parts - 1, nullptr);
+  if (parts > 1 && e == cudaSuccess) e = cudaEventCreateWithFlags(&c->side_go, cudaEventDisableTiming);
+  for (cudaStream_t& q : c->side)
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking);
+  for (cudaEvent_t& v : c->side_done)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     g_create_error = std::string("setup: ") + cudaGetErrorString(e);
     da_destroy(c);
@@ -248,6 +257,11 @@ extern "C" void da_destroy(da_ctx* c) {
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->gstream) cudaStreamDestroy(c->gstream);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
+  if (c->side_go) cudaEventDestroy(c->side_go);
+  for (cudaEvent_t e : c->side_done)
+    if (e) cudaEventDestroy(e);
+  for (cudaStream_t q : c->side)
+    if (q) cudaStreamDestroy(q);
   for (void* p : c->allocs) cudaFree(p);
   if (c->lb_host) cudaFreeHost(c->lb_host);
   delete c;
@@ -275,6 +289,38 @@ extern "C" da_status da_set_observations(da_ctx* c, const double* m, void* strea
   DA_TRY_CUDA(c, cudaMemcpyAsync((void*)c->dev.mobs, m, bytes, cudaMemcpyDefault, (cudaStream_t)stream));
   c->have_obs = true;
   return DA_OK;
+}
+
+// The four RK stages of step k, part by part.
+static da_status forward_step(da_ctx* c, const Parts& parts, int k, int store_flag, int obs_flag) {
+  for (int j = 1; j <= 4; ++j)
+    for (int p = 0; p < parts.count(); ++p) {
+      const Dev d = parts.dev(p);
+      const cudaStream_t st = parts.stream(p);
+      {
+        Timed t(c, 1, st);
+        c->ops->fwd_rows(d, k, j, store_flag | (j == 1 ? obs_flag : 0), st);
+      }
+      Timed t(c, 2, st);
+      c->ops->fwd_cols(d, k, j, st);
+    }
+  return check_launch(c, 8 * parts.count());
+}
+
+// ... and of its adjoint, last stage first.
+static da_status adjoint_step(da_ctx* c, const Parts& parts, int k, int flags) {
+  for (int j = 4; j >= 1; --j)
+    for (int p = 0; p < parts.count(); ++p) {
+      const Dev d = parts.dev(p);
+      const cudaStream_t st = parts.stream(p);
+      {
+        Timed t(c, 3, st);
+        c->ops->adj_rows(d, k, j, st);
+      }
+      Timed t(c, 4, st);
+      c->ops->adj_cols(d, k, j, j == 1 ? flags : 0, st);
+    }
+  return check_launch(c, 8 * parts.count());
 }
 
 // Forward window from control s.  With storage, the stage fields of every
@@ -312,22 +358,20 @@ static da_status run_forward(da_ctx* c, const double* s, bool gather, cudaStream
     c->have_fwd = store;
     return DA_OK;
   }
+  Parts parts(c, st);
+  if ((r = parts.fork())) return r;
   for (int k = 0; k < E; ++k) {
     if (c->ckpt > 0 && store && k % K == 0)
-      DA_TRY_CUDA(c, cudaMemcpyAsync(c->ckpt_buf + (size_t)(k / K) * comp, d.W, comp * sizeof(double2),
-                                     cudaMemcpyDeviceToDevice, st));
+      for (int p = 0; p < parts.count(); ++p) {
+        const size_t at = comp / c->B * parts.begin(p), to = comp / c->B * parts.begin(p + 1);
+        DA_TRY_CUDA(c, cudaMemcpyAsync(c->ckpt_buf + (size_t)(k / K) * comp + at, d.W + at, (to - at) * sizeof(double2),
+                                       cudaMemcpyDeviceToDevice, parts.stream(p)));
+      }
     const int obs_flag = (gather && obs_step_host(c, k)) ? da::F_OBS : 0;
     const int store_flag = (store && k >= d.seg0) ? da::F_STORE : 0;
-    for (int j = 1; j <= 4; ++j) {
-      {
-        Timed t(c, 1, st);
-        o->fwd_rows(d, k, j, store_flag | (j == 1 ? obs_flag : 0), st);
-      }
-      Timed t(c, 2, st);
-      o->fwd_cols(d, k, j, st);
-    }
-    if ((r = check_launch(c, 8))) return r;
+    if ((r = forward_step(c, parts, k, store_flag, obs_flag))) return r;
   }
+  if ((r = parts.join())) return r;
   if (gather && obs_step_host(c, E)) {
     o->fwd_rows(d, E, 1, da::F_OBS_ONLY, st);
     if ((r = check_launch(c))) return r;
@@ -345,8 +389,13 @@ struct SpectraOut {
   double* scratch = nullptr; // [B][nshell]
 };
 
+// Whether spectra are recorded after step k of the sweep.
+static bool records(const da_ctx* c, const SpectraOut* sp, int k) {
+  return sp && sp->every > 0 && (c->nsteps - k) % sp->every == 0;
+}
+
 static da_status record_spectra(da_ctx* c, const SpectraOut* sp, int k, cudaStream_t st) {
-  if (!sp || sp->every <= 0 || (c->nsteps - k) % sp->every) return DA_OK;
+  if (!records(c, sp, k)) return DA_OK;
   const int slot = (c->nsteps - k) / sp->every;
   const int nsave = c->nsteps / sp->every + 1;
   const int nmodes = c->ops->Kr * c->ops->Kc;
@@ -383,6 +432,7 @@ static da_status run_adjoint(da_ctx* c, bool sources, cudaStream_t st, const Spe
   const size_t comp = (size_t)c->B * o->Kr * o->Kc;
   const bool whole = whole_windows(c);
   da_status r;
+  Parts parts(c, st);
   for (int seg = nseg - 1; seg >= 0; --seg) {
     const int k0 = seg * K, k1 = std::min(k0 + K, E);
     if (whole) {
@@ -410,34 +460,25 @@ static da_status run_adjoint(da_ctx* c, bool sources, cudaStream_t st, const Spe
       d.seg0 = k0;
       o->state_cols(d, st);
       if ((r = check_launch(c))) return r;
-      for (int k = k0; k < k1; ++k) {
-        for (int j = 1; j <= 4; ++j) {
-          {
-            Timed t(c, 1, st);
-            o->fwd_rows(d, k, j, da::F_STORE, st);
-          }
-          Timed t(c, 2, st);
-          o->fwd_cols(d, k, j, st);
-        }
-        if ((r = check_launch(c, 8))) return r;
-      }
+      if ((r = parts.fork())) return r;
+      for (int k = k0; k < k1; ++k)
+        if ((r = forward_step(c, parts, k, da::F_STORE, 0))) return r;
+      if ((r = parts.join())) return r;
       o->adj_init(d, da::INIT_RESUME, st);
       if ((r = check_launch(c))) return r;
     }
     d.seg0 = k0;
+    if ((r = parts.fork())) return r;
     for (int k = k1 - 1; k >= k0; --k) {
-      for (int j = 4; j >= 1; --j) {
-        const int flags = (j == 1 && sources && obs_step_host(c, k)) ? da::F_SRC : 0;
-        {
-          Timed t(c, 3, st);
-          o->adj_rows(d, k, j, st);
-        }
-        Timed t(c, 4, st);
-        o->adj_cols(d, k, j, flags, st);
+      const int flags = sources && obs_step_host(c, k) ? da::F_SRC : 0;
+      if ((r = adjoint_step(c, parts, k, flags))) return r;
+      if (records(c, sp, k)) {  // reads every part
+        if ((r = parts.join())) return r;
+        if ((r = record_spectra(c, sp, k, st))) return r;
+        if ((r = parts.fork())) return r;
       }
-      if ((r = check_launch(c, 8))) return r;
-      if ((r = record_spectra(c, sp, k, st))) return r;
     }
+    if ((r = parts.join())) return r;
   }
   // the stored segment is now the first one; a later vjp must rerun the forward
   c->have_fwd = c->ckpt == 0;

@@ -90,6 +90,7 @@ struct __align__(16) ModeSym {
 // Everything a kernel needs, passed by value.
 struct Dev {
   int B, nsteps, every, include_t0, px, nt;  // nsteps: the evaluation's window (global steps)
+  int b0;                                    // first member of an RK stage pass (else 0), which works on B
   double dt, nu;
   int force;
   double amp;
@@ -738,7 +739,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, i
   using RP = RowPoints<P>;
   extern __shared__ double2 sm[];
   Place<P> x = pass_place<N, V>(sm);
-  const int bm = blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
+  const int bm = d.b0 + blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;  // the member's window has not begun
   constexpr int Kc = Geo<N>::Kc;
@@ -956,7 +957,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
   using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
   Place<P> x = pass_place<N, V>(sm);
-  const int kx = blockIdx.x, bm = blockIdx.y;
+  const int kx = blockIdx.x, bm = d.b0 + blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
   // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
@@ -1122,7 +1123,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
   using RP = RowPoints<P>;
   extern __shared__ double2 sm[];
   Place<P> x = pass_place<N, V>(sm);
-  const int bm = blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
+  const int bm = d.b0 + blockIdx.y, y0 = 2 * blockIdx.x, y = y0 + x.f;
   if (d.ragged && n < d.mstart[bm]) return;
   constexpr int Kc = Geo<N>::Kc;
   const q2* MA = d.Mx + ((size_t)bm * 2 * N + y) * Kc;
@@ -1158,7 +1159,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
   extern __shared__ double2 sm[];
   Place<P> x = pass_place<N, V>(sm);
   double2 *Tu = pass_probe_sums<N, V>(sm), *Tv = Tu + G::PMAX;
-  const int kx = blockIdx.x, bm = blockIdx.y;
+  const int kx = blockIdx.x, bm = d.b0 + blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
   // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)

@@ -92,21 +92,29 @@ static da_status tuning_steps(da_ctx* c, int steps, cudaStream_t st) {
     }
     return DA_OK;
   }
+  Parts parts(c, st);
+  da_status r = parts.fork();
+  if (r) return r;
   for (int i = 0; i < steps; ++i) {
     const int k = store ? i % d.traj_steps : 0;
-    for (int j = 1; j <= 4; ++j) {
-      o->fwd_rows(d, k, j, store ? da::F_STORE : 0, st);
-      o->fwd_cols(d, k, j, st);
-    }
-    if (store)
-      for (int j = 4; j >= 1; --j) {
-        o->adj_rows(d, k, j, st);
-        o->adj_cols(d, k, j, 0, st);
+    for (int j = 1; j <= 4; ++j)
+      for (int p = 0; p < parts.count(); ++p) {
+        Dev dp = parts.dev(p);
+        dp.ragged = 0;
+        o->fwd_rows(dp, k, j, store ? da::F_STORE : 0, parts.stream(p));
+        o->fwd_cols(dp, k, j, parts.stream(p));
       }
-    da_status r = check_launch(c, store ? 16 : 8);
-    if (r) return r;
+    if (store)
+      for (int j = 4; j >= 1; --j)
+        for (int p = 0; p < parts.count(); ++p) {
+          Dev dp = parts.dev(p);
+          dp.ragged = 0;
+          o->adj_rows(dp, k, j, parts.stream(p));
+          o->adj_cols(dp, k, j, 0, parts.stream(p));
+        }
+    if ((r = check_launch(c, (store ? 16 : 8) * parts.count()))) return r;
   }
-  return DA_OK;
+  return parts.join();
 }
 
 extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_per_step) {
