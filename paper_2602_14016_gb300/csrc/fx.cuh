@@ -371,11 +371,15 @@ struct Shift {
 
 // The threads of one sequence: TPS of them, whole warps or an aligned part of
 // one.  Threads of several sequences share a warp where TPS < 32; they run in
-// lockstep.  id: the sequence's index in the CTA.
+// lockstep.  id: the sequence's index in the CTA, 0 or 1 where TPS > 32.  The
+// barriers are named by constants: one named by a register reserves all 16 of
+// a CTA's, and an SM has 64 (256^2 on 128 threads: 4 CTAs of the 10 that the
+// registers allow).
 template <int TPS>
 __device__ __forceinline__ void seq_sync(int id) {
   if constexpr (TPS <= 32) __syncwarp();
-  else asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "n"(TPS) : "memory");
+  else if (id == 0) asm volatile("bar.sync 1, %0;" ::"n"(TPS) : "memory");
+  else asm volatile("bar.sync 2, %0;" ::"n"(TPS) : "memory");
 }
 
 // Reductions over a sequence: put leaves each warp's part in scratch (TPS/32
