@@ -219,15 +219,15 @@ inline bool whole_windows(const da_ctx* c) {
 // Parts that a batch's RK stages are split into, each a chain of kernels on a
 // stream of its own: a pass ends with SMs that have nothing left to do while
 // its last rows and columns finish, and begins with loads that nothing covers;
-// the other parts' passes fill both.  From two thirds of the resident threads
-// on (768 an SM): us for a stage pass of all members, replayed as a graph, in one part and in
-// three: 256^2 on 128 threads, batch 5 (0.70 of 152 x 768) 9.86 and 9.21, 7 11.3 and 10.2, 10
-// 16.3 and 12.1, 16 23.3 and 18.6; 512^2 batch 4 23.2 and 18.4; 1024^2 batch 2
-// 46.3 and 39.3 (two parts).  Below the line a part no longer fills its own
-// launches: 256^2 batch 4 (0.56) 8.65 and 8.69, on 64 threads batch 7 (0.49) 11.4
-// and 12.0; 128^2 batch 8 (0.56) 6.6 and 6.9; 64^2 batch 24 (0.42) 5.3 and 5.9.
-// More than three parts change nothing.
-constexpr int kMaxParts = 3;
+// the other parts' passes fill both.  From 512 threads an SM on: us for a stage
+// pass of all members, replayed as a graph, in one part and in four: 256^2 on 128
+// threads, batch 5 (539 threads an SM) 8.60 and 8.37, 7 9.93 and 9.68, 8 12.0 and
+// 10.3, 16 20.6 and 16.0; on 64 threads batch 16 19.8 and 17.5; 512^2 batch 3 17.6
+// and 15.8 (three parts); 128^2 batch 16 9.08 and 8.12; 1024^2 batch 2 49.5 and
+// 43.4 (two parts).  Below the line there is little to gain and four times the
+// launches: 512^2 batch 2 (431) 14.0 and 13.5, 128^2 batch 8 6.6 and 6.9.  Three
+// parts: 0 to 4 % more (256^2 batch 7 9.88, 16 16.0); six: batch 7 9.4, but 16 17.3.
+constexpr int kMaxParts = 4;
 constexpr int kSplitThreads = 152 * 512;
 inline int batch_parts(const Ops& o, int B) {
   return (long long)B * (o.n / 2) * o.threads >= kSplitThreads ? std::min(B, kMaxParts) : 1;
@@ -246,6 +246,7 @@ class Parts {
   Dev dev(int p) const {
     Dev d = c_->dev;
     d.b0 = begin(p);
+    d.early = n_ == 1;
     d.B = begin(p + 1) - d.b0;
     return d;
   }

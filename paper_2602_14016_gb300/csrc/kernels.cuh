@@ -91,6 +91,7 @@ struct __align__(16) ModeSym {
 struct Dev {
   int B, nsteps, every, include_t0, px, nt;  // nsteps: the evaluation's window (global steps)
   int b0;                                    // first member of an RK stage pass (else 0), which works on B
+  int early;                                 // launchers: column passes of an undivided batch may load early
   double dt, nu;
   int force;
   double amp;
@@ -145,13 +146,26 @@ struct Geo {
   static constexpr int SCRATCH = ((3 * 2 + 2 * 4) * FxPlan<N, V>::WARPS + 3) / 4 * 4;
   static constexpr size_t SMEM_FX = sizeof(q2) * (2 * FxPlan<N, V>::SEQ) + sizeof(int) * SCRATCH;
   static constexpr size_t SMEM_FXP = SMEM_FX + sizeof(double2) * 2 * PMAX;
-  // Column passes: small grids leave most of the chip idle, so a warp's own
-  // latency counts, and they load their epilogue inputs before the transforms
-  // (about 60 more registers a thread); larger ones hide it behind other
-  // warps, at 768 threads an SM or more (256^2, batch 16: 28.9 us a column
-  // pass with the loads up front at 153 registers, 20.6 us without at 80).
-  static constexpr bool PREFETCH = N <= 128;
-  static constexpr int COL_CTAS = PREFETCH ? 1 : 768 / THREADS;
+  // Column passes load their epilogue inputs before the transforms (EARLY:
+  // about 60 more registers a thread) where a warp's own latency counts, and
+  // after them, at 768 threads an SM or more, where other warps hide it.  us a
+  // stage pass by captured graphs, early / late: 256^2 1 member 4.99 / 5.13, 3
+  // members 7.01 / 7.22, 16 members 17.0 / 16.0; 512^2 1 member 10.1 / 10.6, 2
+  // members 16.0 / 14.0, 4 members in parts 20.8 / 19.0; 1024^2 1 member 34.3 / 29.2;
+  // 128^2 on 64 threads 8 members 6.06 / 6.19, on 128 threads 4 members 5.28 / 4.91.
+  // So: early where a whole, undivided batch is at most 256 threads an SM
+  // (early_columns); on 64 threads and fewer up to 128^2 always, on 128 never.
+  static constexpr int EARLY_CTAS = N > 128 ? 152 * 256 / THREADS : THREADS < 128 ? 1 << 30 : 0;
+  static constexpr int COL_CTAS = 768 / THREADS;
+  // Row passes: registers for 768 threads an SM on plans of up to 128 threads;
+  // for 512 on radix-16 plans, whose rows took up to 178 registers and left
+  // room for one CTA of 256 threads (1024^2 plan 0: 35.9 -> 33.1 us a pass; for
+  // 768 they spill: 38.5); free on 1024^2 plan 2 (28.9, for 1 CTA or 512 29.2).  256^2: 1
+  // member 5.39 -> 5.15, 7 members 10.0 -> 9.8, 16 members 15.7 -> 16.0.
+  static constexpr int ROW_CTAS = N <= 128                        ? 1
+                                  : THREADS <= 128                ? 768 / THREADS
+                                  : FirstRadix<typename Plan<N, V>::two>::value == 16 ? 512 / THREADS
+                                                                  : 0;
 };
 
 __device__ __forceinline__ int ky_of_row(int r, int K) { return r <= K ? r : r - (2 * K + 1); }
@@ -734,7 +748,7 @@ __device__ __forceinline__ size_t stored_row(const Dev& d, int bm, int n, int st
 // each row (packed as P + i Q) and their forward transforms along x into
 // Mn.  OBS: with the probe gather.  grid (N/2, B).
 template <int N, int V, bool OBS>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_fwd_rows(Dev d, int n, int stage, int flags) {
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::ROW_CTAS) k_fwd_rows(Dev d, int n, int stage, int flags) {
   using P = FxPlan<N, V>;
   using RP = RowPoints<P>;
   extern __shared__ double2 sm[];
@@ -951,8 +965,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_c2r_rows(Dev d, double* 
 // k_j = -n_hat - nu k^2 y_j + f_hat, the RK4 update, and the inverse column
 // transforms of u and v of the next stage state.  Acc holds k1 + 2 k2 +
 // 2 k3 (+ k4).  grid (Kc, B).
-template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd_cols(Dev d, int n, int stage) {
+template <int N, int V, bool EARLY>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, EARLY ? 1 : Geo<N, V>::COL_CTAS) k_fwd_cols(Dev d, int n, int stage) {
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
@@ -960,7 +974,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
   const int kx = blockIdx.x, bm = d.b0 + blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
-  // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
+  // the epilogue's inputs for this thread's modes (EARLY: loaded before the transforms)
   ColumnPut<P> put;
   double2 yv[put.MT], wv[put.MT], accv[put.MT];
   ModeSym mc[put.MT];
@@ -977,7 +991,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
     }
   };
   const int e = forward_columns<P>(d.Mn + (((size_t)bm * G::Kc + kx) * 2 + x.f) * N, d.eN + bm * N, x, d.fxtw, [&] {
-    if constexpr (G::PREFETCH) {
+    if constexpr (EARLY) {
 #pragma unroll
       for (int t = 0; t < put.MT; ++t) load_inputs(t);
     }
@@ -988,7 +1002,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_fwd
   for (int t = 0; t < put.MT; ++t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr >= G::Kr) break;
-    if constexpr (!G::PREFETCH) load_inputs(t);
+    if constexpr (!EARLY) load_inputs(t);
     const int ky = ky_of_row(rr, G::K);
     const int qi = pad(ky & (N - 1));
     const size_t idx = cidx<N>(bm, rr, kx);
@@ -1118,7 +1132,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_init(Dev d, int mode
 // row packed as rho_u + i rho_v), and their forward transforms along x into
 // Mn (twice, as in the forward row pass).  grid (N/2, B).
 template <int N, int V = 0>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, int stage) {
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::ROW_CTAS) k_adj_rows(Dev d, int n, int stage) {
   using P = FxPlan<N, V>;
   using RP = RowPoints<P>;
   extern __shared__ double2 sm[];
@@ -1152,8 +1166,8 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_adj_rows(Dev d, int n, i
 // stage 1), and the inverse column transforms of a, b of the next kbar.
 // SRC: with the observation source, which few steps have and whose code would
 // double the kernel.  grid (Kc, B).
-template <int N, int V, bool SRC>
-__global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj_cols(Dev d, int n, int stage) {
+template <int N, int V, bool SRC, bool EARLY>
+__global__ void __launch_bounds__(Geo<N, V>::THREADS, EARLY ? 1 : Geo<N, V>::COL_CTAS) k_adj_cols(Dev d, int n, int stage) {
   using G = Geo<N, V>;
   using P = FxPlan<N, V>;
   extern __shared__ double2 sm[];
@@ -1162,7 +1176,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
   const int kx = blockIdx.x, bm = d.b0 + blockIdx.y;
   const MemberWindow mw = member_window(d, bm);
   if (n < mw.start) return;
-  // the epilogue's inputs for this thread's modes (G::PREFETCH: loaded early)
+  // the epilogue's inputs for this thread's modes (EARLY: loaded before the transforms)
   ColumnPut<P> put;
   double2 kbv[put.MT], lbv[put.MT], sumv[put.MT];
   ModeSym mc[put.MT];
@@ -1180,7 +1194,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
   };
   const int slot = SRC ? obs_slot(d, n - mw.start) : -1;
   const int e = forward_columns<P>(d.Mn + (((size_t)bm * G::Kc + kx) * 2 + x.f) * N, d.eN + bm * N, x, d.fxtw, [&] {
-    if constexpr (G::PREFETCH) {
+    if constexpr (EARLY) {
 #pragma unroll
       for (int t = 0; t < put.MT; ++t) load_inputs(t);
     }
@@ -1193,7 +1207,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS, Geo<N, V>::COL_CTAS) k_adj
   for (int t = 0; t < put.MT; ++t) {
     const int rr = threadIdx.x + t * G::THREADS;
     if (rr >= G::Kr) break;
-    if constexpr (!G::PREFETCH) load_inputs(t);
+    if constexpr (!EARLY) load_inputs(t);
     const int ky = ky_of_row(rr, G::K);
     const int qi = pad(ky & (N - 1));
     const size_t idx = cidx<N>(bm, rr, kx);

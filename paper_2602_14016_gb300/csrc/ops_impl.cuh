@@ -22,6 +22,24 @@ inline void launch_clusters(void (*f)(A...), int members, int threads, size_t sm
   cudaLaunchKernelEx(&c, f, args...);
 }
 
+// The column kernels that a batch may run (Geo::EARLY_CTAS): those of one kind
+// are not built where no batch, or every batch, loads early.
+template <int N, int V>
+struct Columns {
+  using G = Geo<N, V>;
+  static constexpr bool SOME_EARLY = G::EARLY_CTAS >= G::Kc, ALL_EARLY = N <= 128 && SOME_EARLY;
+  static bool early(const Dev& d) {
+    return ALL_EARLY || (SOME_EARLY && d.early && (long long)d.B * G::Kc <= G::EARLY_CTAS);
+  }
+  static auto fwd(const Dev& d) {
+    return early(d) ? k_fwd_cols<N, V, SOME_EARLY> : k_fwd_cols<N, V, ALL_EARLY>;
+  }
+  template <bool SRC>
+  static auto adj(const Dev& d) {
+    return early(d) ? k_adj_cols<N, V, SRC, SOME_EARLY> : k_adj_cols<N, V, SRC, ALL_EARLY>;
+  }
+};
+
 template <int N, int V>
 Ops make_ops() {
   using G = Geo<N, V>;
@@ -48,12 +66,15 @@ Ops make_ops() {
     set((const void*)k_ctrl_cols<N, V, true>);
     set((const void*)k_fwd_rows<N, V, false>);
     set((const void*)k_fwd_rows<N, V, true>);
-    set((const void*)k_fwd_cols<N, V>);
+    set((const void*)k_fwd_cols<N, V, Columns<N, V>::ALL_EARLY>);
+    set((const void*)k_fwd_cols<N, V, Columns<N, V>::SOME_EARLY>);
     set((const void*)k_state_cols<N, V>);
     set((const void*)k_adj_init<N, V>, G::SMEM_FXP);
     set((const void*)k_adj_rows<N, V>);
-    set((const void*)k_adj_cols<N, V, false>, G::SMEM_FXP);
-    set((const void*)k_adj_cols<N, V, true>, G::SMEM_FXP);
+    set((const void*)k_adj_cols<N, V, false, Columns<N, V>::ALL_EARLY>, G::SMEM_FXP);
+    set((const void*)k_adj_cols<N, V, true, Columns<N, V>::ALL_EARLY>, G::SMEM_FXP);
+    set((const void*)k_adj_cols<N, V, false, Columns<N, V>::SOME_EARLY>, G::SMEM_FXP);
+    set((const void*)k_adj_cols<N, V, true, Columns<N, V>::SOME_EARLY>, G::SMEM_FXP);
     if constexpr (WinGeo<N, V>::SUPPORTED) {
       for (const void* f : {(const void*)k_window_fwd<N, V>, (const void*)k_window_adj<N, V>}) {
         set(f, WinGeo<N, V>::SMEM);
@@ -88,7 +109,7 @@ Ops make_ops() {
       k_fwd_rows<N, V, false><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage, flags);
   };
   o.fwd_cols = [](const Dev& d, int n, int stage, cudaStream_t st) {
-    k_fwd_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
+    Columns<N, V>::fwd(d)<<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
   };
   o.state_cols = [](const Dev& d, cudaStream_t st) {
     k_state_cols<N, V><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FX, st>>>(d);
@@ -100,8 +121,9 @@ Ops make_ops() {
     k_adj_rows<N, V><<<dim3(N / 2, d.B), G::THREADS, G::SMEM_FX, st>>>(d, n, stage);
   };
   o.adj_cols = [](const Dev& d, int n, int stage, int flags, cudaStream_t st) {
-    if (flags & F_SRC) k_adj_cols<N, V, true><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
-    else k_adj_cols<N, V, false><<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
+    using C = Columns<N, V>;
+    const auto f = flags & F_SRC ? C::template adj<true>(d) : C::template adj<false>(d);
+    f<<<dim3(G::Kc, d.B), G::THREADS, G::SMEM_FXP, st>>>(d, n, stage);
   };
   o.window_batch = 0;
   o.window_fwd = nullptr;

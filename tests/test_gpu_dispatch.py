@@ -106,3 +106,15 @@ def test_caller_captures_an_evaluation(api, n, plan, B):
     got = [t.clone() for t in out]
     ctx.close()
     assert same(got, want)
+
+
+# batches on both sides of the line up to which column passes load their inputs early
+@pytest.mark.parametrize("n,plan,few,many", [(256, 0, 3, 4), (256, 1, 7, 8), (512, 0, 1, 2), (512, 2, 3, 4)])
+def test_members_do_not_depend_on_their_batch(api, n, plan, few, many):
+    out = []
+    for B in (few, many):
+        ctx, s, lam = make(api, n, plan, B, 2, 1, forced=True)
+        ctx.set_observations(torch.full((B, ctx.nt, 16, 2), 0.25, dtype=torch.float64, device="cuda"))
+        out.append([t[:few].clone() for t in results(ctx, s, lam, spectra=False)])
+        ctx.close()
+    assert same(*out)
