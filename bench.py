@@ -79,7 +79,8 @@ def fp64_probe(kinds=(0, 1, 2, 3), iters: int = 100000) -> dict:
 
 
 def fp64_peak(probe: dict, sms: int) -> dict:
-    """Roofline denominator of the FP64-bound pass kernels, derived from unit
+    """Denominator of the pass kernels' nominal FP64 flops (their transforms run on
+    integers, so that the fraction can exceed 1), derived from unit
     counts and clocks: SMs x DFMA per clock per SM x 2 flop x maximum SM clock.
     The DFMA rate per SM is the probe's best DFMA rate rounded to a whole
     number of operations per clock (the pipe issues whole operations)."""
@@ -119,7 +120,7 @@ def src_hash() -> str:
 def hbm_fraction(traffic, avg_ms):
     """DRAM bandwidth the dominant kernel uses (measured bytes per launch over
     its launch time) against the measured HBM copy peak: the %HBM view of a
-    kernel whose bound is the FP64 pipe."""
+    kernel whose bound is arithmetic."""
     if traffic is None or not avg_ms:
         return None
     peak, src = 6800.0, "fallback"

@@ -1,7 +1,7 @@
 /*
  * da.h -- C ABI of the GB300 cost-and-gradient library for preconditioned
  * adjoint data assimilation of 2D incompressible Navier-Stokes turbulence
- * (vorticity form, periodic box [0, 2pi)^2, FP64 throughout).
+ * (vorticity form, periodic box [0, 2pi)^2, FP64 in and out).
  *
  * What it computes (Ke, You & Wang, "Preconditioned Adjoint Data
  * Assimilation for Two-Dimensional Decaying and Forced Turbulence"):
@@ -399,8 +399,8 @@ da_status da_omega_from_control_static(int n, double nu, const da_kernel* kernel
                                        void* stream, const char** message);
 
 /* FP64 throughput probe, a measurement utility (the paper has no
- * counterpart): the pass kernels are bound by FP64 arithmetic, and this
- * probe measures the pipe's issue rate that bounds them.  Runs 8 independent
+ * counterpart): the issue rate of the pipe that bounds FP64 transforms, the
+ * denominator of the pass kernels' nominal flops.  Runs 8 independent
  * dependency chains per thread of one operation -- kind 0: DFMA with a
  * register multiplicand and a constant addend; 1: DFMA with three register
  * operands; 2: DADD; 3: DMUL -- on 4 CTAs of 256 threads per SM, iters x 32

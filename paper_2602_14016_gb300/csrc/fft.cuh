@@ -23,7 +23,6 @@ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ double2 conjd(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 
 // (S i) * a, S = +-1
@@ -98,7 +97,7 @@ struct Radices {};
 
 // Plans: for each size N, a few variants V of the radix list used for two
 // concurrent transforms (the pass kernels; `two`) and for a single transform
-// (`one`), with the CTA width they run on.  Wide radices keep the FP64
+// (`one`), with the CTA width they run on.  Wide radices keep the
 // instruction count low; narrow ones and wider CTAs keep more warps in
 // flight.  A stage with more butterflies than threads gives each thread
 // several.  Variant 0 is the default; the autotuner (da_autotune) times the
@@ -109,11 +108,10 @@ template <> struct Plan<16, 0> { using two = Radices<4, 4>; using one = Radices<
 template <> struct Plan<32, 0> { using two = Radices<4, 8>; using one = Radices<4, 8>; static constexpr int threads = 32; };
 template <> struct Plan<64, 0> { using two = Radices<4, 4, 4>; using one = Radices<4, 4, 4>; static constexpr int threads = 32; };
 template <> struct Plan<64, 1> { using two = Radices<8, 8>; using one = Radices<8, 8>; static constexpr int threads = 32; };
-// Radix-2 plans: 1.2x the FP64 instructions of the radix-4 ones, but each
-// thread's chain is about half as long (34 instead of 60 instructions per
-// 64-point transform).  On GB300 a lone warp issues one FP64 instruction per
-// ~67 SM clocks whatever its active lanes, so the small grids at small
-// batches, whose pass kernels are bound by that chain, run faster on them.
+// Radix-2 plans: more instructions than the radix-4 ones, but a shorter chain a
+// thread.  Small grids at small batches, whose pass kernels are bound by that
+// chain, run faster on them: 128^2, one member, 5.3 us a pass on plan 0 and 4.2
+// on plan 3; 24 members 9.2 and 9.5.
 template <> struct Plan<32, 1> { using two = Radices<2, 2, 2, 2, 2>; using one = Radices<2, 2, 2, 2, 2>; static constexpr int threads = 32; };
 template <> struct Plan<64, 2> { using two = Radices<2, 2, 2, 2, 2, 2>; using one = Radices<2, 2, 2, 2, 2, 2>; static constexpr int threads = 64; };
 template <> struct Plan<128, 0> { using two = Radices<4, 4, 8>; using one = Radices<4, 4, 8>; static constexpr int threads = 64; };
@@ -204,14 +202,10 @@ __device__ __forceinline__ void run_stages(double2* buf, const double2* tw, Radi
 // transforms are read back only on the band q <= K, q >= N - K.  Input m of
 // butterfly i of the first stage is x[i + m N/R]; output m of butterfly k of
 // the last stage is y[k + m N/R].  Where that position lies in the gap for
-// all 32 lanes of a warp, the warp skips the load and the additions the zero
-// would enter (first stage), or neither forms nor stores the output (last
-// stage; the buffer keeps whatever it held there).  The tests are per warp
-// because GB300's FP64 pipe spends the same time on a warp instruction
-// whatever its active lanes: only whole warp instructions saved count.  A
-// warp covers 32 consecutive butterflies of one sequence when N/R is a
-// multiple of 32; otherwise only the positions in the gap for every
-// butterfly are skipped.
+// every butterfly, the load and the additions the zero would enter (first
+// stage), or the output's forming and storing (last stage), are left out
+// (gap_common).  The nominal flop counts (da_plan_flops) also leave out what
+// lies in the gap for all 32 lanes of a warp (GapMask).
 
 // positions lo..hi all in the gap of band kb (kb < 0: no band)
 __host__ __device__ constexpr bool in_gap(int n, int kb, int lo, int hi) {

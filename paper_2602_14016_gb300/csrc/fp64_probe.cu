@@ -1,6 +1,6 @@
 // fp64_probe.cu -- FP64 pipe throughput probe (da_fp64_probe of
-// include/da.h): the measurement behind the roofline denominator of the pass
-// kernels, which are bound by FP64 arithmetic rather than by HBM.
+// include/da.h): the measurement behind the denominator of the pass kernels'
+// nominal flops.  Their transforms run on integers because of it (fx.cuh).
 //
 // Every thread runs 8 independent dependency chains of one FP64 operation
 // for `iters` x 4 rounds; 4 CTAs of 256 threads per SM keep 32 warps per SM

@@ -11,17 +11,17 @@
 // Error.  A sequence enters a forward transform normalised so that its
 // largest component has 62 - log2 G bits, G the largest growth of a component
 // over the stages, or over the first stage only where that leaves two bits
-// more: the second stage then starts with a measured shift.  A sequence enters an inverse transform, whose inputs are
-// spectra with few large coefficients, normalised by the sum of its
-// components' magnitudes, which bounds every partial sum (inv_shift).  Every
-// rounding is at most one unit, against results whose root mean square is
+// more: the second stage then starts with a measured shift.  A sequence enters
+// an inverse transform, whose inputs are spectra with few large coefficients,
+// normalised by the sum of its components' magnitudes, which bounds every
+// partial sum (inv_shift).  Every rounding is at most one unit, against results whose root mean square is
 // 2^54 units or more on the fields of the path (FP64's roundings are 2^-53 of
 // the values themselves).
 //
 // Stages are those of fft.cuh (Stockham, mixed radix, in place, R points per
 // butterfly in registers).  The inverse transform runs the plan's radices in
 // reverse, so its last radix is the forward transform's first, and the row
-// passes hand the data over in registers (fx_turn).  A twiddled stage of
+// passes hand the data over in registers.  A twiddled stage of
 // radix 4 or 8 scales by 1/4, one of radix 2 by 1/2: the twiddles are 62-bit
 // integers, and no shift follows the product.
 #pragma once
@@ -614,9 +614,7 @@ __device__ __forceinline__ void fx_middle(q2* buf, const int4* T, int t, int id,
 }
 
 // Inverse transform (S = +1) of the sequence in buf, zero outside the band
-// KB: the inputs are shifted right by pre (left by
-// -pre) first,
-// and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
+// KB: the inputs are shifted right by pre (left by -pre) first, and the result is the transform times 2^-SHIFT_INV, of at most 60 bits.  It
 // is left in registers: out[jb R + m] is position t + jb TPS + m N / R for R
 // the last radix.  buf is not free before the next sync.
 template <typename P, int KB>

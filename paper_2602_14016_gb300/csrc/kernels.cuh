@@ -30,7 +30,7 @@
 // A forward RK stage is two kernels: a ROW pass (inverse transforms along x
 // of the packed mixed rows -> u, v; stage-field store; probe gather; the
 // products u v and v^2 - u^2; their forward transforms along x, handed over
-// in registers: fx_turn) and a COLUMN
+// in registers) and a COLUMN
 // pass (forward transforms along y of the two products, the advection term,
 // RK epilogue with viscosity, forcing and the stage update, then the
 // inverse column transforms of the next stage's u and v).  The adjoint
@@ -39,8 +39,8 @@
 // applied once, to the spectral coefficients before the column transform.
 // Every inverse transform here reads a sequence that is zero in the gap
 // K < q < N - K, and every forward transform is read back only on the band
-// q <= K, q >= N - K: the transforms are band-limited (KIN / KOUT = K) and
-// skip that work where whole warps allow.
+// q <= K, q >= N - K: the transforms are band-limited and skip the inputs and
+// outputs that lie in the gap for every butterfly of a stage.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(Geo<N, V>::THREADS) k_ctrl_cols(Dev d) {
       if (rr >= G::Kr) break;
       put_stage_columns(put, j, d.symF[kx * G::Kr + rr], w0(rr, x.first(x.src)));
     }
-      finish_to_mixed(d, put, x, bm, kx);
+    finish_to_mixed(d, put, x, bm, kx);
   } else {
     for (int rr = x.t; rr < G::Kr; rr += P::TPS) w0(rr, x.src);
   }
