@@ -337,9 +337,13 @@ inline const std::vector<int4>& fx_table() {
 // Exponents and conversions
 // ---------------------------------------------------------------------------
 
-// Exponent of an all-zero sequence, and of one that holds an infinity or a
-// NaN; sums of two exponents are brought back to these by clamp_exp.
-constexpr int kZeroExp = -100000, kBadExp = 100000;
+// Exponent of an all-zero sequence (or symbol), and of one that holds an
+// infinity or a NaN, whose integers are all zero.  Ordinary exponents and those
+// of symbols are a few thousand at most, so that a mark plus any of them stays
+// beyond half the mark, and clamp_exp brings it back.  The sum of the two marks
+// lies beyond half the bad one: zero times NaN is NaN.
+constexpr int kZeroExp = -100000, kBadExp = 400000;
+static_assert(kBadExp + kZeroExp - 10000 > kBadExp / 2, "a bad sequence stays bad in a product with a zero one");
 
 __device__ __forceinline__ int clamp_exp(int e) { return e < kZeroExp / 2 ? kZeroExp : e > kBadExp / 2 ? kBadExp : e; }
 
@@ -458,7 +462,7 @@ __device__ __forceinline__ double pow2_double(int e) {  // 2^e, -1022 <= e <= 10
 // The scaling where 2^e is not an ordinary double: in steps, each within a
 // double's range.  Out of line: states in the ordinary range never come here.
 static __device__ __noinline__ double fx_scale_far(double d, int e) {
-  if (e >= kBadExp) return __hiloint2double(0x7ff80000, 0);
+  if (e > kBadExp / 2) return __hiloint2double(0x7ff80000, 0);
   if (d == 0.0) return 0.0;
   int left = max(min(e, 2200), -2200);
   while (left != 0) {
