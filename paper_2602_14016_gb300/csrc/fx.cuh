@@ -337,11 +337,12 @@ inline const std::vector<int4>& fx_table() {
 // Exponents and conversions
 // ---------------------------------------------------------------------------
 
-// Exponent of an all-zero sequence (or symbol), and of one that holds an
-// infinity or a NaN, whose integers are all zero.  Ordinary exponents and those
-// of symbols are a few thousand at most, so that a mark plus any of them stays
-// beyond half the mark, and clamp_exp brings it back.  The sum of the two marks
-// lies beyond half the bad one: zero times NaN is NaN.
+// Exponent of a symbol that vanishes or of values that are not there, and of a
+// sequence that holds an infinity or a NaN, whose integers are all zero (zeros
+// that are data have the exponent of subnormals).  Ordinary exponents are a few
+// thousand at most, so that a mark plus any of them stays beyond half the mark,
+// and clamp_exp brings it back.  The sum of the two marks lies beyond half the
+// bad one: zero times NaN is NaN.
 constexpr int kZeroExp = -100000, kBadExp = 400000;
 static_assert(kBadExp + kZeroExp - 10000 > kBadExp / 2, "a bad sequence stays bad in a product with a zero one");
 
@@ -497,25 +498,26 @@ __device__ __forceinline__ i64 fx_pair_sum(const FxPair& c, i64 p, i64 q) {
   return mul_hi2(Words(p), Words(c.ah, c.al), Words(q), SG > 0 ? Words(c.bh, c.bl) : Words(-c.bh, -c.bl));
 }
 
-// Biased exponent field of a double (0: zero or subnormal, 2047: not finite).
+// Biased exponent field of a double (0: zero or subnormal, whose unit is that
+// of field 1; 2047: not finite).
 __device__ __forceinline__ int exp_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
 
 // Exponent e for a sequence whose largest exponent field is f, so that every
 // component has at most BITS bits: |d| < 2^(f - 1022) = 2^(BITS + e).
 template <int BITS>
 __device__ __forceinline__ int exp_for(int f) {
-  return f == 0 ? kZeroExp : f == 2047 ? kBadExp : f - 1022 - BITS;
+  return f == 2047 ? kBadExp : max(f, 1) - 1022 - BITS;
 }
 
 // d / 2^e as an integer, rounded towards zero; e from exp_for<BITS> (BITS <=
-// 62).  Subnormals count as zero.
+// 62).
 __device__ __forceinline__ i64 double_to_fx(double d, int e) {
   const int hi = __double2hiint(d), lo = __double2loint(d);
   const int f = (hi >> 20) & 0x7ff;
-  // 53-bit significand m, value m 2^(f - 1075): m 2^9 >> r
-  const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
-  const int r = (int)min((unsigned)(9 - (f - 1075 - e)), 63u);
-  const i64 q = f == 0 ? 0 : (m << 9) >> r;
+  // significand m of 53 bits (of a subnormal: fewer), value m 2^(max(f, 1) - 1075): m 2^9 >> r
+  const i64 m = ((i64)((hi & 0xfffff) | (f ? 0x100000 : 0)) << 32) | (unsigned)lo;
+  const int r = (int)min((unsigned)(9 - (max(f, 1) - 1075 - e)), 63u);
+  const i64 q = (m << 9) >> r;
   return hi < 0 ? -q : q;
 }
 
