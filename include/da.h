@@ -210,15 +210,16 @@ da_status da_set_plan(da_ctx* ctx, int variant);
 
 /* Autotuner: for each plan variant of the context's n, runs one warm-up and
  * `steps` timed RK steps of the forward and (when stage fields are stored)
- * adjoint pass kernels over the context's own batch, on zeroed working
- * buffers, timed with CUDA events; switches the context to the fastest and
- * records the choice for later contexts of the same n and batch in this
- * process.  chosen (nullable): HOST int, the variant taken; ms_per_step
+ * adjoint pass kernels over the context's own batch, on a smooth field in its
+ * working buffers, replayed as a graph (of at most 32 steps; more are rounded
+ * up to whole graphs) and timed with CUDA events; switches the context to the
+ * fastest and records the choice for later contexts of the same n and batch in
+ * this process.  chosen (nullable): HOST int, the variant taken; ms_per_step
  * (nullable): HOST double[da_plan_count(n)], the measured milliseconds per
  * step of each variant.  Synchronous (it first waits for all work on the
- * device, then runs on the legacy default stream); it overwrites the context's state and
- * stored trajectory, so call it before the evaluations (observations set by
- * da_set_observations are kept).  DA_EINVAL for steps < 1. */
+ * device, then runs on the legacy default stream); it overwrites the context's
+ * state and stored trajectory, so call it before the evaluations (observations
+ * set by da_set_observations are kept).  DA_EINVAL for steps < 1. */
 da_status da_autotune(da_ctx* ctx, int steps, int* chosen, double* ms_per_step);
 
 /* Nominal flops of one band-limited transform of n points as the pass

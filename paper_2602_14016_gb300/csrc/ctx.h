@@ -278,6 +278,10 @@ class Parts {
   bool forked_ = false;
 };
 
+// The RK stages of step k and of its adjoint, part by part (da_api.cu).
+da_status forward_step(da_ctx* c, const Parts& parts, int k, int store_flag, int obs_flag);
+da_status adjoint_step(da_ctx* c, const Parts& parts, int k, int flags);
+
 // Sets the evaluation window for the members marked in `live` (all members
 // with a non-empty window if live is NULL): eval_steps = the longest live
 // window, each live member end-aligned in it, the others idle; uploads the

@@ -292,7 +292,7 @@ extern "C" da_status da_set_observations(da_ctx* c, const double* m, void* strea
 }
 
 // The four RK stages of step k, part by part.
-static da_status forward_step(da_ctx* c, const Parts& parts, int k, int store_flag, int obs_flag) {
+da_status forward_step(da_ctx* c, const Parts& parts, int k, int store_flag, int obs_flag) {
   for (int j = 1; j <= 4; ++j)
     for (int p = 0; p < parts.count(); ++p) {
       const Dev d = parts.dev(p);
@@ -308,7 +308,7 @@ static da_status forward_step(da_ctx* c, const Parts& parts, int k, int store_fl
 }
 
 // ... and of its adjoint, last stage first.
-static da_status adjoint_step(da_ctx* c, const Parts& parts, int k, int flags) {
+da_status adjoint_step(da_ctx* c, const Parts& parts, int k, int flags) {
   for (int j = 4; j >= 1; --j)
     for (int p = 0; p < parts.count(); ++p) {
       const Dev d = parts.dev(p);

@@ -73,48 +73,115 @@ static da_status clear_state(da_ctx* c, cudaStream_t st) {
   return DA_OK;
 }
 
-// `steps` RK steps of the pass kernels (forward, and the adjoint when the
-// context stores stage fields) over whatever the working buffers hold.
+// A state and an adjoint field of ordinary size for the tuning passes, real and
+// even in k, slow enough (velocities of 1e-3) to stay so over any tuning run:
+// values that are zero or not finite take another path in the conversions.
+__global__ void k_tuning_fields(double2* W, double2* LamBar, double amp, int Kr, int Kc) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Kr * Kc; i += gridDim.x * blockDim.x) {
+    const int kx = i / Kr, r = i - kx * Kr, ky = r < Kc ? r : r - Kr;
+    const double2 v = make_double2(i == 0 ? 0.0 : amp / (1 + kx * kx + ky * ky), 0.0);
+    W[(size_t)blockIdx.y * Kr * Kc + i] = LamBar[(size_t)blockIdx.y * Kr * Kc + i] = v;
+  }
+}
+
+// `steps` RK steps of the context's batch as an evaluation runs them (its
+// route, its parts; forward, and the adjoint when the context stores stage
+// fields), in windows that the store holds.
 static da_status tuning_steps(da_ctx* c, int steps, cudaStream_t st) {
   const Ops* o = c->ops;
-  c->dev.seg0 = 0;
-  Dev d = c->dev;
-  d.ragged = 0;  // every member works, whatever windows a ragged batch holds
-  const bool store = d.traj != nullptr;
-  if (whole_windows(c)) {
-    const int most = store ? d.traj_steps : steps;
-    for (int i = 0; i < steps; i += most) {
-      const int k = std::min(most, steps - i);
-      o->window_fwd(d, 0, k, store ? da::W_STORE : 0, st);
-      if (store) o->window_adj(d, k, 0, 0, st);
-      da_status r = check_launch(c, store ? 2 : 1);
-      if (r) return r;
-    }
-    return DA_OK;
-  }
+  const Dev& d = c->dev;
+  const bool store = d.traj != nullptr, whole = whole_windows(c);
+  const int most = store ? d.traj_steps : steps;
   Parts parts(c, st);
-  da_status r = parts.fork();
-  if (r) return r;
-  for (int i = 0; i < steps; ++i) {
-    const int k = store ? i % d.traj_steps : 0;
-    for (int j = 1; j <= 4; ++j)
-      for (int p = 0; p < parts.count(); ++p) {
-        Dev dp = parts.dev(p);
-        dp.ragged = 0;
-        o->fwd_rows(dp, k, j, store ? da::F_STORE : 0, parts.stream(p));
-        o->fwd_cols(dp, k, j, parts.stream(p));
-      }
-    if (store)
-      for (int j = 4; j >= 1; --j)
-        for (int p = 0; p < parts.count(); ++p) {
-          Dev dp = parts.dev(p);
-          dp.ragged = 0;
-          o->adj_rows(dp, k, j, parts.stream(p));
-          o->adj_cols(dp, k, j, 0, parts.stream(p));
-        }
-    if ((r = check_launch(c, (store ? 16 : 8) * parts.count()))) return r;
+  da_status r = DA_OK;
+  for (int i = 0; i < steps; i += most) {
+    const int n = std::min(most, steps - i);
+    if (whole) {
+      o->window_fwd(d, 0, n, store ? da::W_STORE : 0, st);
+    } else {
+      o->state_cols(d, st);
+      if ((r = parts.fork())) return r;
+      for (int k = 0; k < n; ++k)
+        if ((r = forward_step(c, parts, k, store ? da::F_STORE : 0, 0))) return r;
+      if ((r = parts.join())) return r;
+    }
+    if ((r = check_launch(c))) return r;
+    if (!store) continue;
+    o->adj_init(d, da::INIT_LAMBAR, st);
+    if (whole) {
+      o->window_adj(d, n, 0, 0, st);
+    } else {
+      if ((r = parts.fork())) return r;
+      for (int k = n - 1; k >= 0; --k)
+        if ((r = adjoint_step(c, parts, k, 0))) return r;
+      if ((r = parts.join())) return r;
+    }
+    if ((r = check_launch(c, whole ? 2 : 1))) return r;
   }
-  return parts.join();
+  return DA_OK;
+}
+
+// The tuning steps as a graph, captured on cap; *exec stays NULL where another
+// thread's device-wide calls broke every capture (da_cost_grad's note on that).
+static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t cap, cudaGraphExec_t* exec,
+                                unsigned long long* launches) {
+  for (int attempt = 0; attempt < 4; ++attempt) {
+    cudaGraph_t g = nullptr;
+    const unsigned long long l0 = c->launches;
+    DA_TRY_CUDA(c, cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+    da_status r = tuning_steps(c, steps, cap);
+    cudaError_t e = cudaStreamEndCapture(cap, &g);
+    *launches = c->launches - l0;
+    c->launches = l0;
+    if (!r && e == cudaSuccess) {
+      e = cudaGraphInstantiate(exec, g, 0);
+      cudaGraphDestroy(g);
+      if (e != cudaSuccess) *exec = nullptr;
+      DA_TRY_CUDA(c, e);
+      return DA_OK;
+    }
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();
+    if (e != cudaErrorStreamCaptureInvalidated && (r != DA_ECUDA || e == cudaSuccess))
+      return r ? r : fail(c, DA_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+  }
+  return DA_OK;
+}
+
+// Milliseconds of a step on the context's plan, replayed as a graph of at most
+// 32 steps unless whole windows run in one kernel.  Launched directly, the 16
+// launches of a step (64 of a batch in four parts) would be what is timed, 2.5
+// us each, wherever a pass takes less: 256^2, batch 5, 0.173 ms a step where
+// evaluations take 0.140, and batch 2 0.147 where they take 0.105.
+static da_status time_plan(da_ctx* c, int steps, cudaStream_t st, cudaStream_t cap, cudaEvent_t e0, cudaEvent_t e1,
+                           float* ms) {
+  cudaGraphExec_t exec = nullptr;
+  unsigned long long launches = 0;
+  const int part = std::min(steps, 32), parts = (steps + part - 1) / part;
+  da_status r = tuning_steps(c, 1, st);  // warm-up
+  if (r) return r;
+  if (!whole_windows(c) && (r = capture_tuning(c, part, cap, &exec, &launches))) return r;
+  auto run = [&]() -> da_status {
+    if (exec) DA_TRY_CUDA(c, cudaGraphUpload(exec, st));
+    DA_TRY_CUDA(c, cudaEventRecord(e0, st));
+    for (int j = 0; j < parts; ++j) {
+      if (exec) {
+        DA_TRY_CUDA(c, cudaGraphLaunch(exec, st));
+        c->launches += launches;
+      } else {
+        da_status q = tuning_steps(c, part, st);
+        if (q) return q;
+      }
+    }
+    DA_TRY_CUDA(c, cudaEventRecord(e1, st));
+    DA_TRY_CUDA(c, cudaEventSynchronize(e1));
+    DA_TRY_CUDA(c, cudaEventElapsedTime(ms, e0, e1));
+    *ms /= part * parts;
+    return DA_OK;
+  };
+  r = run();
+  if (exec) cudaGraphExecDestroy(exec);
+  return r;
 }
 
 extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_per_step) {
@@ -123,10 +190,9 @@ extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_p
   // the tuning passes overwrite the working state: let every evaluation in
   // flight on any stream finish first
   DA_TRY_CUDA(c, cudaDeviceSynchronize());
-  // the device is idle now; the tuning runs on the legacy default stream
-  // (creating a stream of its own here was measured to leave later
-  // evaluations in the process about 1 % slower)
-  cudaStream_t st = nullptr;
+  // the device is idle now; the tuning runs on the legacy default stream, which
+  // cannot be captured: that takes a stream of its own
+  cudaStream_t st = nullptr, cap = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   da_status r = DA_OK;
   int best = 0;
@@ -136,29 +202,36 @@ extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_p
   };
   cuda(cudaEventCreate(&e0), "event");
   cuda(cudaEventCreate(&e1), "event");
+  cuda(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "stream");
+  // every member works, whatever windows a ragged batch holds, on the routes
+  // that evaluations take, whatever is being timed
+  const int ragged = c->dev.ragged, timed = c->timed_class;
+  c->dev.ragged = 0;
+  c->timed_class = 0;
+  c->dev.seg0 = 0;
+  const int modes = c->ops->Kr * c->ops->Kc;
   for (int v = 0; r == DA_OK && v < da::plan_count(c->n); ++v) {
     if ((r = set_plan(c, v))) break;
     if ((r = clear_state(c, st))) break;
-    if ((r = tuning_steps(c, 1, st))) break;  // warm-up
-    cuda(cudaEventRecord(e0, st), "event record");
-    if (r || (r = tuning_steps(c, steps, st))) break;
-    cuda(cudaEventRecord(e1, st), "event record");
-    cuda(cudaEventSynchronize(e1), "event synchronize");
+    k_tuning_fields<<<dim3((modes + 255) / 256, c->B), 256, 0, st>>>(c->dev.W, c->dev.LamBar, 1e-3 * c->n * c->n,
+                                                                  c->ops->Kr, c->ops->Kc);
     float ms = 0.f;
-    cuda(cudaEventElapsedTime(&ms, e0, e1), "event elapsed time");
-    if (r) break;
-    ms /= steps;
+    if ((r = check_launch(c))) break;
+    if ((r = time_plan(c, steps, st, cap, e0, e1, &ms))) break;
     if (ms_per_step) ms_per_step[v] = ms;
     if (v == 0 || ms < best_ms) {
       best = v;
       best_ms = ms;
     }
   }
+  c->dev.ragged = ragged;
+  c->timed_class = timed;
   if (r == DA_OK) r = set_plan(c, best);
   if (r == DA_OK) r = clear_state(c, st);
   if (r == DA_OK) cuda(cudaStreamSynchronize(st), "stream synchronize");
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
+  if (cap) cudaStreamDestroy(cap);
   if (r) return r;
   {
     std::lock_guard<std::mutex> lock(g_plan_mu);
