@@ -277,8 +277,9 @@ class CoBatchServer:
     members that finished.  A retired member takes no part in later steps; it
     keeps its slot until another job needs one, so that retiring costs no
     blocking call between steps (idling a slot waits for the stream and
-    uploads its tables).  `peak_members` of a run's summary is the most member
-    slots that were held at once, retired members included.
+    uploads its tables).  `peak_running` of a run's summary is the most members
+    of a pool that ran at once, `peak_members` the most slots of a pool that
+    were held at once, retired members included.
     Plan variant `plan` on every pool, so a job's result equals its result in
     a batch-1 context on that variant; plan=None lets the autotuner pick each
     pool's variant for its slot count (results then equal the batch-1 ones to
@@ -309,7 +310,7 @@ class CoBatchServer:
                     ctx.set_member(b, 0)
                 self.pools[n] = {"ctx": ctx, "slots": p["slots"], "stream": torch.cuda.Stream(device),
                                  "jobs": [None] * p["slots"], "held": set(), "steps": 0}
-        self.peak_members = 0
+        self.peak_members = self.peak_running = 0
 
     @staticmethod
     def pool_bytes(n: int, nsteps: int, px: int, every: int, ckpt_every: int, slots: int) -> int:
@@ -340,6 +341,7 @@ class CoBatchServer:
                                            torch.from_numpy(j.m[0]), stream=st)
                             ctx.lbfgs_start(b, torch.from_numpy(j.s0[0]).to(ctx.device), j.iters, stream=st)
                         busy = sum(x is not None for x in slots)
+                        self.peak_running = max(self.peak_running, busy)
                         self.peak_members = max(self.peak_members, busy + len(held))
                         remaining = len(queue)
                     if busy == 0:
@@ -385,7 +387,7 @@ class CoBatchServer:
             th.join()
         if errors:
             raise RuntimeError(f"pool failures: {errors}")
-        return summarize(jobs, peak_members=self.peak_members,
+        return summarize(jobs, peak_members=self.peak_members, peak_running=self.peak_running,
                          steps={int(n): p["steps"] for n, p in self.pools.items()})
 
     def close(self):
