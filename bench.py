@@ -91,21 +91,38 @@ def fp64_peak(probe: dict, sms: int) -> dict:
             "probe_best_dfma_per_clk_per_sm": best, "sm_max_mhz": mhz, "clock_source": src,
             "source": "derived: SMs x DFMA/clk/SM (da_fp64_probe, this run) x 2 flop x max SM clock"}
 
-# DRAM bytes (read + write) per launch of each pass kernel at this workload
-# (256^2, batch 7), from one ncu capture of the same launch configuration on
-# a 40-step window (per-launch data are the same for any window length);
-# valid only for the kernel sources they were taken from.
-TRAFFIC = {"src_hash": "ebf205b24a74b487", "adj_rows": 12301312, "adj_cols": 10530816, "fwd_rows": 4977152,
-           "fwd_cols": 10495744}
+# DRAM bytes (read + write) and warp instructions per launch of each pass kernel
+# at this workload (256^2, batch 7 undivided, plan 0), from one ncu capture of
+# the same launch configuration on a 40-step window (per-launch data are the
+# same for any window length); valid only for the kernel sources they were
+# taken from.
+COUNTERS = {"src_hash": "ce0e624bf079f5d5",
+            "adj_rows": {"dram_bytes": 12321792, "warp_inst": 5857152},
+            "adj_cols": {"dram_bytes": 9102080, "warp_inst": 4222064},
+            "fwd_rows": {"dram_bytes": 4975872, "warp_inst": 5749632},
+            "fwd_cols": {"dram_bytes": 10760448, "warp_inst": 4274550}}
+
+
+def issue_roofline(counters, avg_ms, sms: int):
+    """What bounds the pass kernels, whose transforms are 64-bit integer
+    arithmetic: the warp instructions of a launch over its time against four a
+    clock per SM at the maximum SM clock."""
+    mhz, src = sm_max_mhz()
+    peak = sms * 4 * mhz / 1e3
+    if counters is None or not avg_ms:
+        return None
+    rate = counters["warp_inst"] / (avg_ms * 1e-3) / 1e9
+    return {"bound": "issue", "achieved": rate, "peak": peak, "unit": "G warp instructions/s", "frac": rate / peak,
+            "warp_inst_per_launch": counters["warp_inst"], "clock_source": src}
 
 
 def src_hash() -> str:
     """Hash of the sources of the pass kernels and their launch configuration
-    (kernels, FFT engine, launchers, instantiations), with comments and blank
-    space removed: what the measured traffic figures depend on.  Host code
+    (kernels, FFT engines, launchers, instantiations), with comments and blank
+    space removed: what the measured counters depend on.  Host code
     that only orders launches is left out."""
     csrc = os.path.join(ROOT, "paper_2602_14016_gb300", "csrc")
-    files = [os.path.join(csrc, f) for f in ("kernels.cuh", "fft.cuh", "ops.h", "ops_impl.cuh")]
+    files = [os.path.join(csrc, f) for f in ("kernels.cuh", "fft.cuh", "fx.cuh", "ops.h", "ops_impl.cuh")]
     files += glob.glob(os.path.join(csrc, "inst_n*.cu"))
     h = hashlib.sha256()
     for p in sorted(files):
@@ -134,12 +151,12 @@ def hbm_fraction(traffic, avg_ms):
 
 
 def pass_flops(n: int, batch: int, variant: int = 0) -> dict:
-    """Algorithmic FP64 flops per launch of each pass kernel: the nominal
-    count of the transforms it performs plus its pointwise arithmetic.  A
-    transform counts 5 n log2 n less the operations the kernels skip on the
-    gap of the 2/3 rule under this plan variant (da_plan_flops: zero inputs
-    of an inverse transform's first stage, unused outputs of a forward
-    transform's last stage)."""
+    """Algorithmic flops per launch of each pass kernel, as if in FP64: the
+    nominal count of the transforms it performs plus its pointwise arithmetic.
+    A transform counts 5 n log2 n less what FP64 stages of this plan variant
+    could skip on the gap of the 2/3 rule (da_plan_flops: zero inputs of an
+    inverse transform's first stage, unused outputs of a forward transform's
+    last stage)."""
     from paper_2602_14016_gb300 import api
 
     K = (n - 1) // 3
@@ -396,7 +413,11 @@ def run_gpu(args):
     probe = fp64_probe((0, 1), iters=50000)
     peak = fp64_peak(probe, torch.cuda.get_device_properties(device).multi_processor_count)
     peak_gflops = peak["gflops"]
-    traffic = TRAFFIC.get(dom) if (TRAFFIC.get("src_hash") == src_hash() and n == 256 and B == 7) else None
+    same = COUNTERS["src_hash"] == src_hash() and n == 256 and B == 7 and plan == 0
+    counters = COUNTERS[dom] if same else None
+    traffic = counters["dram_bytes"] if same else None
+    nominal = {"flops_per_launch": pf, "achieved": achieved, "peak": peak_gflops, "unit": "GFLOP/s",
+               "frac": achieved / peak_gflops}
     cpu = cpu_baseline(args) if args.cpu_baseline else None
     line = {
         "metric": METRIC,
@@ -419,9 +440,11 @@ def run_gpu(args):
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(s_host.numel() * 8),
                 "d2h_bytes_per_step": int(J_host.numel() * 8 + g_host.numel() * 8)},
         "gpu_launches": int(launches),
-        "roofline": {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": peak_gflops,
-                     "unit": "GFLOP/s", "frac": achieved / peak_gflops, "traffic": traffic,
-                     "flops_per_launch": pf, "avg_launch_ms": avg_ms, "launches_timed": dom_n,
+        # the nominal flops against the FP64 peak say nothing of the integer kernels'
+        # bound; they stand in only where the counters are of other sources or sizes
+        "roofline": {"kernel": dom, "traffic": traffic, "nominal_fp64": nominal,
+                     **(issue_roofline(counters, avg_ms, peak["sms"]) or {"bound": "fp64 nominal", **nominal}),
+                     "avg_launch_ms": avg_ms, "launches_timed": dom_n,
                      "timed_in": "roofline pass of the same workload, direct launches, CUDA events per launch",
                      "roofline_pass_ms_per_step": roof_pass_ms,
                      "class_ms_warmup": {k: v[0] for k, v in class_ms.items()},

@@ -65,7 +65,7 @@ def _ptr(t: torch.Tensor | None) -> ctypes.c_void_p | None:
 
 def plan_flops(n: int, variant: int = 0) -> tuple[float, float]:
     """Nominal flops of one band-limited (inverse, forward) transform of n
-    points as the pass kernels run it under plan `variant` (da_plan_flops)."""
+    points with the radices of plan `variant` (da_plan_flops)."""
     lib = N.load()
     inv, fwd = ctypes.c_double(), ctypes.c_double()
     st = lib.da_plan_flops(int(n), int(variant), ctypes.byref(inv), ctypes.byref(fwd))

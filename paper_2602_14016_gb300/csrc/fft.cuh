@@ -1,14 +1,13 @@
 // fft.cuh -- radix plans and gap masks of the integer FFT engine (fx.cuh), and
 // an FP64 shared-memory FFT for the allocation-free control map.
 //
-// A CTA transforms a batch of F complex sequences of length N held in shared
-// memory, with a mixed-radix Stockham auto-sort algorithm: stage s with
+// A CTA transforms a complex sequence of length N held in shared memory, with a mixed-radix Stockham auto-sort algorithm: stage s with
 // radix R and current sub-length L loads the R points x[i + m N/R] of
 // butterfly i, twiddles them by W_{LR}^{m (i mod L)}, applies an R-point DFT
 // in registers and stores them to y[(i - i mod L) R + i mod L + m L].  After
 // the last stage (L = N) the output is in natural order.  The FP64 stages work
 // in place: every thread holds its butterfly in registers across a barrier.
-// fft_batch takes a plain table of W_N^t = exp(-2 pi i t / N) (conjugated for
+// fft_sequence takes a plain table of W_N^t = exp(-2 pi i t / N) (conjugated for
 // the inverse sign); the allocation-free control map has static scratch and no
 // context to keep the integer engine's tables.
 #pragma once
@@ -138,27 +137,22 @@ struct PlanInfo {
   static constexpr int THREADS = Plan<N, V>::threads;
 };
 
-// One in-place Stockham stage on F sequences of N points stored back to back
-// in `buf`: every thread loads the R points of each of its butterflies,
-// twiddles and transforms them in registers, waits for all loads, then
-// stores.
-template <int N, int R, int S, int F>
+// One in-place Stockham stage on the N points in `buf`: every thread loads the
+// R points of each of its butterflies, twiddles and transforms them in
+// registers, waits for all loads, then stores.
+template <int N, int R, int S>
 __device__ __forceinline__ void stockham_stage(double2* buf, int L, const double2* __restrict__ tw) {
-  constexpr int NB = N / R, T = PlanInfo<N>::THREADS, TOT = F * NB, J = (TOT + T - 1) / T;
+  constexpr int NB = N / R, T = PlanInfo<N>::THREADS, J = (NB + T - 1) / T;
   double2 a[J][R];
-  int base[J], dst[J];
+  int dst[J];
 #pragma unroll
   for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * T;
-    base[jb] = 0;
+    const int i = threadIdx.x + jb * T;
     dst[jb] = 0;
-    if (TOT % T == 0 || u < TOT) {
-      const int f = u / NB;
-      const int i = u - f * NB;
+    if (NB % T == 0 || i < NB) {
       const int k = i & (L - 1);
-      base[jb] = f * N;
 #pragma unroll
-      for (int m = 0; m < R; ++m) a[jb][m] = buf[base[jb] + i + m * NB];
+      for (int m = 0; m < R; ++m) a[jb][m] = buf[i + m * NB];
       if (L > 1) {
         const int step = N / (L * R);
 #pragma unroll
@@ -175,22 +169,22 @@ __device__ __forceinline__ void stockham_stage(double2* buf, int L, const double
   __syncthreads();
 #pragma unroll
   for (int jb = 0; jb < J; ++jb) {
-    const int u = threadIdx.x + jb * T;
-    if (TOT % T == 0 || u < TOT) {
+    const int i = threadIdx.x + jb * T;
+    if (NB % T == 0 || i < NB) {
 #pragma unroll
-      for (int m = 0; m < R; ++m) buf[base[jb] + dst[jb] + m * L] = a[jb][m];
+      for (int m = 0; m < R; ++m) buf[dst[jb] + m * L] = a[jb][m];
     }
   }
   __syncthreads();
 }
 
-template <int N, int S, int F, int L>
+template <int N, int S, int L>
 __device__ __forceinline__ void run_stages(double2*, const double2*, Radices<>) {}
 
-template <int N, int S, int F, int L, int R, int... Rs>
+template <int N, int S, int L, int R, int... Rs>
 __device__ __forceinline__ void run_stages(double2* buf, const double2* tw, Radices<R, Rs...>) {
-  stockham_stage<N, R, S, F>(buf, L, tw);
-  run_stages<N, S, F, L * R>(buf, tw, Radices<Rs...>{});
+  stockham_stage<N, R, S>(buf, L, tw);
+  run_stages<N, S, L * R>(buf, tw, Radices<Rs...>{});
 }
 
 // ---------------------------------------------------------------------------
@@ -205,7 +199,8 @@ __device__ __forceinline__ void run_stages(double2* buf, const double2* tw, Radi
 // every butterfly, the load and the additions the zero would enter (first
 // stage), or the output's forming and storing (last stage), are left out
 // (gap_common).  The nominal flop counts (da_plan_flops) also leave out what
-// lies in the gap for all 32 lanes of a warp (GapMask).
+// lies in the gap for all 32 lanes of a warp (GapMask), which FP64 stages can
+// skip and the integer stages of fx.cuh do not.
 
 // positions lo..hi all in the gap of band kb (kb < 0: no band)
 __host__ __device__ constexpr bool in_gap(int n, int kb, int lo, int hi) {
@@ -283,11 +278,14 @@ template <int R, int R2, int... Rs> struct InitRadices<Radices<R, R2, Rs...>> {
 template <typename P> struct TailRadices;
 template <int R, int... Rs> struct TailRadices<Radices<R, Rs...>> { using type = Radices<Rs...>; };
 
-// Host side: flops of one band-limited transform of N points under Plan<N,
-// V> as the pass kernels run it: the nominal 5 N log2 N less the operations
-// the gap tests skip (a real addition or multiplication counts one, an FMA
-// two).  Inverse: the zero inputs of the first stage; forward: the unformed
-// outputs of the last (two FMAs each).
+// Host side: nominal flops of one band-limited transform of N points under
+// Plan<N, V>: 5 N log2 N less the FP64 operations that warp-wide gap tests
+// would skip in the list's first stage (inverse) and last stage (forward); a
+// real addition or multiplication counts one, an FMA two.  A measure of the
+// work, the same whatever arithmetic does it: the pass kernels run integer
+// stages, whose inverse begins with the list's last radix.  Inverse: the zero
+// inputs of the first stage; forward: the unformed outputs of the last (two
+// FMAs each).
 
 // flops a zero mask z saves in the untwiddled r-point DFT (dft2/4/8/16):
 // every add_z / sub_z with a known-zero operand saves one complex addition
@@ -314,16 +312,12 @@ inline double band_transform_flops(bool inverse) {
   return 5.0 * N * std::log2((double)N) - saved;
 }
 
-// Transform, in place, F (1 or 2) sequences of N points stored back to back
-// in buf.  Called by every thread of a CTA of PlanInfo<N>::THREADS threads,
-// with buf already synchronised; returns after a final __syncthreads().
-template <int N, int S, int F>
-__device__ __forceinline__ void fft_batch(double2* buf, const double2* tw) {
-  static_assert(F == 1 || F == 2, "batches of one or two transforms");
-  if constexpr (F == 1)
-    run_stages<N, S, F, 1>(buf, tw, typename Plan<N>::one{});
-  else
-    run_stages<N, S, F, 1>(buf, tw, typename Plan<N>::two{});
+// Transform, in place, the N points in buf.  Called by every thread of a CTA of
+// PlanInfo<N>::THREADS threads, with buf already synchronised; returns after a
+// final __syncthreads().
+template <int N, int S>
+__device__ __forceinline__ void fft_sequence(double2* buf, const double2* tw) {
+  run_stages<N, S, 1>(buf, tw, typename Plan<N>::one{});
 }
 
 }  // namespace da

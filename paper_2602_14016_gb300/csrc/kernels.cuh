@@ -154,14 +154,20 @@ struct Geo {
   // members 16.0 / 14.0, 4 members in parts 20.8 / 19.0; 1024^2 1 member 34.3 / 29.2;
   // 128^2 on 64 threads 8 members 6.06 / 6.19, on 128 threads 4 members 5.28 / 4.91.
   // So: early where a whole, undivided batch is at most 256 threads an SM
-  // (early_columns); on 64 threads and fewer up to 128^2 always, on 128 never.
+  // (Columns::early); on 64 threads and fewer up to 128^2 always, on 128 never.
+  // 768 threads an SM leave 80 registers, and the late kernels spill (ptxas, bytes
+  // stored a thread, without / with the observation source): forward 256^2 32 to
+  // 76, 512^2 92 to 332, 1024^2 88 to 148; adjoint 256^2 0 to 80 / 84 to 136,
+  // 512^2 60 to 272 / 136 to 656, 1024^2 64 to 144 / 144 to 664, 128^2 on 128
+  // threads 0 / 52.  Bounds between 512 and 768 have not been measured.
   static constexpr int EARLY_CTAS = N > 128 ? 152 * 256 / THREADS : THREADS < 128 ? 1 << 30 : 0;
   static constexpr int COL_CTAS = 768 / THREADS;
   // Row passes: registers for 768 threads an SM on plans of up to 128 threads;
   // for 512 on radix-16 plans, whose rows took up to 178 registers and left
-  // room for one CTA of 256 threads (1024^2 plan 0: 35.9 -> 33.1 us a pass; for
-  // 768 they spill: 38.5); free on 1024^2 plan 2 (28.9, for 1 CTA or 512 29.2).  256^2: 1
-  // member 5.39 -> 5.15, 7 members 10.0 -> 9.8, 16 members 15.7 -> 16.0.
+  // room for one CTA of 256 threads (1024^2 plan 0: 35.9 -> 33.1 us a pass, with
+  // adj_rows spilling 188 to 260 bytes a thread; for 768 38.5); free on 1024^2
+  // plan 2 (28.9, for 1 CTA or 512 29.2).  256^2: 1 member 5.39 -> 5.15, 7
+  // members 10.0 -> 9.8, 16 members 15.7 -> 16.0.
   static constexpr int ROW_CTAS = N <= 128                        ? 1
                                   : THREADS <= 128                ? 768 / THREADS
                                   : FirstRadix<typename Plan<N, V>::two>::value == 16 ? 512 / THREADS

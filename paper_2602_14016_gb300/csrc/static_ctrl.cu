@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(Geo<N>::THREADS) k_rows(const double* __restri
   const double* r0 = s + (size_t)y0 * N;
   for (int x = threadIdx.x; x < N; x += blockDim.x) a[x] = make_double2(r0[x], r0[N + x]);
   __syncthreads();
-  fft_batch<N, -1, 1>(a, tw);
+  fft_sequence<N, -1>(a, tw);
   double2* M = rows + (size_t)y0 * G::Kc;
   for (int kx = threadIdx.x; kx < G::Kc; kx += blockDim.x) {
     double2 A, Bv;
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(Geo<N>::THREADS) k_cols(const double2* __restr
   load_tw<N>(tw, tw256);
   for (int y = threadIdx.x; y < N; y += blockDim.x) a[y] = rows[(size_t)y * G::Kc + kx];
   __syncthreads();
-  fft_batch<N, -1, 1>(a, tw);
+  fft_sequence<N, -1>(a, tw);
   const double2* r = a;
   for (int q = threadIdx.x; q < N; q += blockDim.x) {
     const int ky = q < N / 2 ? q : q - N;
