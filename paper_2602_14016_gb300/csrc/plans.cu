@@ -121,10 +121,13 @@ static da_status tuning_steps(da_ctx* c, int steps, cudaStream_t st) {
   return DA_OK;
 }
 
-// The tuning steps as a graph, captured on cap; *exec stays NULL where another
-// thread's device-wide calls broke every capture (da_cost_grad's note on that).
-static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t cap, cudaGraphExec_t* exec,
+// The tuning steps as a graph, captured on *cap_stream (made on first use); *exec stays
+// NULL where another thread's device-wide calls broke every capture
+// (da_cost_grad's note on that).
+static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t* cap_stream, cudaGraphExec_t* exec,
                                 unsigned long long* launches) {
+  if (!*cap_stream) DA_TRY_CUDA(c, cudaStreamCreateWithFlags(cap_stream, cudaStreamNonBlocking));
+  const cudaStream_t cap = *cap_stream;
   for (int attempt = 0; attempt < 4; ++attempt) {
     cudaGraph_t g = nullptr;
     const unsigned long long l0 = c->launches;
@@ -153,7 +156,7 @@ static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t cap, cudaGrap
 // launches of a step (64 of a batch in four parts) would be what is timed, 2.5
 // us each, wherever a pass takes less: 256^2, batch 5, 0.173 ms a step where
 // evaluations take 0.140, and batch 2 0.147 where they take 0.105.
-static da_status time_plan(da_ctx* c, int steps, cudaStream_t st, cudaStream_t cap, cudaEvent_t e0, cudaEvent_t e1,
+static da_status time_plan(da_ctx* c, int steps, cudaStream_t st, cudaStream_t* cap, cudaEvent_t e0, cudaEvent_t e1,
                            float* ms) {
   cudaGraphExec_t exec = nullptr;
   unsigned long long launches = 0;
@@ -191,7 +194,7 @@ extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_p
   // flight on any stream finish first
   DA_TRY_CUDA(c, cudaDeviceSynchronize());
   // the device is idle now; the tuning runs on the legacy default stream, which
-  // cannot be captured: that takes a stream of its own
+  // cannot be captured: that takes a stream of its own (cap)
   cudaStream_t st = nullptr, cap = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   da_status r = DA_OK;
@@ -202,7 +205,6 @@ extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_p
   };
   cuda(cudaEventCreate(&e0), "event");
   cuda(cudaEventCreate(&e1), "event");
-  cuda(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "stream");
   // every member works, whatever windows a ragged batch holds, on the routes
   // that evaluations take, whatever is being timed
   const int ragged = c->dev.ragged, timed = c->timed_class;
@@ -217,7 +219,7 @@ extern "C" da_status da_autotune(da_ctx* c, int steps, int* chosen, double* ms_p
                                                                   c->ops->Kr, c->ops->Kc);
     float ms = 0.f;
     if ((r = check_launch(c))) break;
-    if ((r = time_plan(c, steps, st, cap, e0, e1, &ms))) break;
+    if ((r = time_plan(c, steps, st, &cap, e0, e1, &ms))) break;
     if (ms_per_step) ms_per_step[v] = ms;
     if (v == 0 || ms < best_ms) {
       best = v;
