@@ -227,6 +227,9 @@ inline bool whole_windows(const da_ctx* c) {
 // 43.4 (two parts).  Below the line there is little to gain and four times the
 // launches: 512^2 batch 2 (431) 14.0 and 13.5, 128^2 batch 8 6.6 and 6.9.  Three
 // parts: 0 to 4 % more (256^2 batch 7 9.88, 16 16.0); six: batch 7 9.4, but 16 17.3.
+// These are replays: launched directly, a divided batch takes its launches' time
+// where that is longer (256^2 batch 5, forward: 1600 launches in 4.2 ms, 10.5 us
+// a pass of all members).
 constexpr int kMaxParts = 4;
 constexpr int kSplitThreads = 152 * 512;
 inline int batch_parts(const Ops& o, int B) {
