@@ -106,6 +106,13 @@ inline void drop_graphs(da_ctx* c) {
   c->cg_cache.clear();
 }
 
+// A captured sequence made ready for replay, and its replay.  A graph holds 2.5 KB
+// of device memory a launch, which no context counts: where the device has not
+// that much left, the evaluations captured before give theirs up, and if that is
+// not enough *exec becomes NULL with DA_OK, and the caller launches directly.
+da_status instantiate_graph(da_ctx* c, cudaGraph_t g, cudaGraphExec_t* exec);
+da_status launch_graph(da_ctx* c, cudaGraphExec_t* exec, cudaStream_t st);
+
 // Message of the last failed da_create (no context to hold it).
 extern std::string g_create_error;
 

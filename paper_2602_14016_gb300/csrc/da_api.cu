@@ -660,6 +660,33 @@ extern "C" da_status da_set_graphs(da_ctx* c, int enable) {
   return DA_OK;
 }
 
+da_status instantiate_graph(da_ctx* c, cudaGraph_t g, cudaGraphExec_t* exec) {
+  cudaError_t e = cudaGraphInstantiate(exec, g, 0);
+  if (e == cudaErrorMemoryAllocation && !c->cg_cache.empty()) {
+    cudaGetLastError();
+    drop_graphs(c);
+    e = cudaGraphInstantiate(exec, g, 0);
+  }
+  if (e == cudaSuccess) return DA_OK;
+  *exec = nullptr;
+  if (e != cudaErrorMemoryAllocation)
+    return fail(c, DA_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  cudaGetLastError();
+  return DA_OK;
+}
+
+da_status launch_graph(da_ctx* c, cudaGraphExec_t* exec, cudaStream_t st) {
+  const cudaError_t e = cudaGraphLaunch(*exec, st);
+  if (e == cudaErrorMemoryAllocation) {  // its first launch puts it on the device
+    cudaGetLastError();
+    cudaGraphExecDestroy(*exec);
+    *exec = nullptr;
+    return DA_OK;
+  }
+  DA_TRY_CUDA(c, e);
+  return DA_OK;
+}
+
 extern "C" da_status da_cost_grad(da_ctx* c, const double* s, double* J, double* grad_s, void* stream) {
   if (!c || !s) return fail(c, DA_EINVAL, "ctx and s must not be NULL");
   if (!c->have_obs) return fail(c, DA_EINVAL, "no observations: call da_set_observations first");
@@ -700,24 +727,32 @@ da_status cost_grad_members(da_ctx* c, const double* s, double* J, double* grad_
           return r ? r : fail(c, DA_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
         direct = true;
       } else {
-        e = cudaGraphInstantiate(&ex, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return fail(c, DA_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-        if (c->cg_cache.size() >= kMaxCapturedEvals) {  // evict the oldest
-          cudaGraphExecDestroy(c->cg_cache.front().exec);
-          c->cg_cache.erase(c->cg_cache.begin());
-        }
-        c->cg_cache.push_back({c->eval_steps, ex, c->launches - l0});
+        const unsigned long long nodes = c->launches - l0;
         c->launches = l0;
-        ce = &c->cg_cache.back();
+        r = instantiate_graph(c, g, &ex);
+        cudaGraphDestroy(g);
+        if (r) return r;
+        direct = !ex;
+        if (ex) {
+          if (c->cg_cache.size() >= kMaxCapturedEvals) {  // evict the oldest
+            cudaGraphExecDestroy(c->cg_cache.front().exec);
+            c->cg_cache.erase(c->cg_cache.begin());
+          }
+          c->cg_cache.push_back({c->eval_steps, ex, nodes});
+          ce = &c->cg_cache.back();
+        }
       }
     }
-    if (direct) {
-      if ((r = enqueue_cost_grad(c, c->sbuf, c->gbuf, c->gstream))) return r;
-    } else {
-      DA_TRY_CUDA(c, cudaGraphLaunch(ce->exec, c->gstream));
-      c->launches += ce->launches;
+    if (!direct) {
+      if ((r = launch_graph(c, &ce->exec, c->gstream))) return r;
+      if (ce->exec) {
+        c->launches += ce->launches;
+      } else {
+        c->cg_cache.erase(c->cg_cache.begin() + (ce - c->cg_cache.data()));
+        direct = true;
+      }
     }
+    if (direct && (r = enqueue_cost_grad(c, c->sbuf, c->gbuf, c->gstream))) return r;
     c->have_fwd = c->ckpt == 0;
     DA_TRY_CUDA(c, cudaEventRecord(c->ev_out, c->gstream));
     DA_TRY_CUDA(c, cudaStreamWaitEvent(st, c->ev_out, 0));
@@ -874,17 +909,15 @@ extern "C" da_status da_adjoint_spectra(da_ctx* c, const double* s, const double
       return r;
     }
     if (e != cudaSuccess) return fail(c, DA_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&c->sp_exec, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-      c->sp_exec = nullptr;
-      return fail(c, DA_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    }
     c->sp_launches = c->launches - l0;
     c->launches = l0;
+    r = instantiate_graph(c, g, &c->sp_exec);
+    cudaGraphDestroy(g);
+    if (r) return r;
   }
-  DA_TRY_CUDA(c, cudaGraphLaunch(c->sp_exec, c->gstream));
-  c->launches += c->sp_launches;
+  if (c->sp_exec && (r = launch_graph(c, &c->sp_exec, c->gstream))) return r;
+  if (c->sp_exec) c->launches += c->sp_launches;
+  else if ((r = enqueue_spectra(c, c->sbuf, c->sp_lbuf, sp, c->gstream))) return r;
   c->have_fwd = c->ckpt == 0;
   DA_TRY_CUDA(c, cudaEventRecord(c->ev_out, c->gstream));
   DA_TRY_CUDA(c, cudaStreamWaitEvent(st, c->ev_out, 0));

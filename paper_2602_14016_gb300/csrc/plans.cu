@@ -121,10 +121,11 @@ static da_status tuning_steps(da_ctx* c, int steps, cudaStream_t st) {
   return DA_OK;
 }
 
-// The tuning steps as a graph, captured on *cap_stream (made on first use); *exec stays
-// NULL where another thread's device-wide calls broke every capture
-// (da_cost_grad's note on that).
-static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t* cap_stream, cudaGraphExec_t* exec,
+// The tuning steps as a graph that is on the device, captured on *cap_stream
+// (made on first use); *exec stays NULL where another thread's device-wide calls
+// broke every capture (da_cost_grad's note on that) or the device has no memory
+// for it.
+static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t st, cudaStream_t* cap_stream, cudaGraphExec_t* exec,
                                 unsigned long long* launches) {
   if (!*cap_stream) DA_TRY_CUDA(c, cudaStreamCreateWithFlags(cap_stream, cudaStreamNonBlocking));
   const cudaStream_t cap = *cap_stream;
@@ -137,11 +138,14 @@ static da_status capture_tuning(da_ctx* c, int steps, cudaStream_t* cap_stream, 
     *launches = c->launches - l0;
     c->launches = l0;
     if (!r && e == cudaSuccess) {
-      e = cudaGraphInstantiate(exec, g, 0);
+      r = instantiate_graph(c, g, exec);
       cudaGraphDestroy(g);
-      if (e != cudaSuccess) *exec = nullptr;
-      DA_TRY_CUDA(c, e);
-      return DA_OK;
+      if (*exec && cudaGraphUpload(*exec, st) != cudaSuccess) {
+        cudaGetLastError();
+        cudaGraphExecDestroy(*exec);
+        *exec = nullptr;
+      }
+      return r;
     }
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
@@ -163,18 +167,14 @@ static da_status time_plan(da_ctx* c, int steps, cudaStream_t st, cudaStream_t* 
   const int part = std::min(steps, 32), parts = (steps + part - 1) / part;
   da_status r = tuning_steps(c, 1, st);  // warm-up
   if (r) return r;
-  if (!whole_windows(c) && (r = capture_tuning(c, part, cap, &exec, &launches))) return r;
+  if (!whole_windows(c) && (r = capture_tuning(c, part, st, cap, &exec, &launches))) return r;
   auto run = [&]() -> da_status {
-    if (exec) DA_TRY_CUDA(c, cudaGraphUpload(exec, st));
     DA_TRY_CUDA(c, cudaEventRecord(e0, st));
     for (int j = 0; j < parts; ++j) {
-      if (exec) {
-        DA_TRY_CUDA(c, cudaGraphLaunch(exec, st));
-        c->launches += launches;
-      } else {
-        da_status q = tuning_steps(c, part, st);
-        if (q) return q;
-      }
+      da_status q = exec ? launch_graph(c, &exec, st) : DA_OK;
+      if (exec) c->launches += launches;
+      else if (!q) q = tuning_steps(c, part, st);
+      if (q) return q;
     }
     DA_TRY_CUDA(c, cudaEventRecord(e1, st));
     DA_TRY_CUDA(c, cudaEventSynchronize(e1));
